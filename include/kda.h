@@ -211,10 +211,11 @@ kda_status_t kda_layer_decode_step(const void *q_c, const void *k_c, const void 
  *     L = sum_t <d_o_t, o_t> + <dS_T, S_T>
  *
  * it returns dL/dq, dL/dk, dL/dv, dL/dlog_alpha, dL/dbeta and dL/dS0.  The forward pass is
- * recomputed inside (nothing has to be kept from kda_chunk_fwd): a first sweep stores the state at
- * the start of every block of 8 tokens, a reverse sweep recomputes one block at a time (in shared
- * memory) and runs the adjoint through
- * it token by token; fp32 arithmetic throughout.
+ * recomputed inside (nothing has to be kept from kda_chunk_fwd), in the chunkwise form of Section 3.1:
+ * per-chunk quantities of all chunks at once, the recurrences of the state and of its adjoint over
+ * the chunks, then the gradients of all chunks at once.  Heads in which some chunk's log decay
+ * leaves [-40, 1] run token by token instead (any decay is exact there).  Inputs of the matrix
+ * products keep 22 significant bits, sums are fp32.
  *
  *   q, k [T_total,H,dk], v, d_o [T_total,H,dv]   device, element type `dt` (KDA_F32 or KDA_BF16)
  *   log_alpha [T_total,H,dk], beta [T_total,H]   fp32 device
@@ -222,10 +223,9 @@ kda_status_t kda_layer_decode_step(const void *q_c, const void *k_c, const void 
  *   dq, dk, dlog_alpha [T_total,H,dk], dv [T_total,H,dv], dbeta [T_total,H]   fp32 device, written
  *   dS0 [n_seqs,H,dk,dv] fp32 device, written, or NULL
  *   cu_seqlens_dev / cu_seqlens_host, n_seqs, total_tokens, H, scale: as in kda_chunk_fwd
- *   workspace: device memory, 256-byte aligned, at least kda_chunk_bwd_workspace_bytes(...) (chunk
- *              states at the start of every block of 8 tokens and the
- *              per-slice shares of the gradients that are summed over dv; about 0.45 MB per token
- *              at H = 32).  Its first 256 bytes hold the status word that kda_check_status reads.
+ *   workspace: device memory, 256-byte aligned, at least kda_chunk_bwd_workspace_bytes(...) (the
+ *              chunk tiles, or for the token-sequential form the states of every eighth token and
+ *              per-slice shares of the gradients; about 0.45 MB per token at H = 32).  Its first 256 bytes hold the status word that kda_check_status reads.
  * Only dk = dv = 128 and chunk = 64.  Asynchronous on `cuda_stream`; nothing is allocated; results
  * are deterministic (fixed summation order).  Errors: KDA_ERR_INVALID_ARG, KDA_ERR_UNSUPPORTED,
  * KDA_ERR_WORKSPACE, KDA_ERR_CUDA.

@@ -16,9 +16,7 @@
 // state at the start of every block of 8 tokens, the reverse sweep recomputes one block at a time into
 // shared memory (8 decayed states of this slice, 128 KB) and runs the adjoint through it.  All
 // arithmetic is fp32 FMA; q, k, v, d_o may be stored as bf16.
-#include <vector>
-
-#include "kda_common.cuh"
+#include "kda_bwd.cuh"
 
 namespace kda {
 namespace {
@@ -43,6 +41,7 @@ struct BwdArgs {
     float* ckpt;        // [total_chunks * 8][H][128][128]: state at the start of every block of 8 tokens
     float* part_q; float* part_k; float* part_g;   // [kSlices][T][H][128]
     float* part_b;      // [kSlices][T][H]
+    const int* seq_heads;   // [H]: heads this form has to do
     int n_seqs, H;
     int64_t total_tokens, seq_len, chunks_per_seq;
     float scale;
@@ -103,6 +102,7 @@ __global__ void __launch_bounds__(kThreads, 1) kda_bwd_sweep(BwdArgs a)
     extern __shared__ __align__(16) float sm[];
     const int t = threadIdx.x, lane = t & 31, rg = t >> 5;
     const int slice = blockIdx.x, h = blockIdx.y, n = blockIdx.z;
+    if (!a.seq_heads[h]) return;
     const int col = slice * NS + lane;
     const int i0 = rg * kRows;                 // first of this thread's rows
 
@@ -269,10 +269,15 @@ __global__ void __launch_bounds__(kThreads, 1) kda_bwd_sweep(BwdArgs a)
 __global__ void kda_bwd_reduce(const float* __restrict__ part_q, const float* __restrict__ part_k,
                                const float* __restrict__ part_g, const float* __restrict__ part_b,
                                float* __restrict__ dq, float* __restrict__ dk, float* __restrict__ dg,
-                               float* __restrict__ dbeta, size_t n_vec, size_t n_tok)
+                               float* __restrict__ dbeta, size_t n_vec, size_t n_tok,
+                               const int* __restrict__ seq_heads, int H)
 {
+    int any = 0;
+    for (int h = threadIdx.x; h < H; h += blockDim.x) any |= seq_heads[h];
+    if (!__syncthreads_or(any)) return;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec / 4; i += stride) {
+        if (!seq_heads[i / (kD / 4) % H]) continue;
         float4 sq = make_float4(0.f, 0.f, 0.f, 0.f), sk = sq, sg = sq;
 #pragma unroll
         for (int s = 0; s < kSlices; ++s) {
@@ -288,6 +293,7 @@ __global__ void kda_bwd_reduce(const float* __restrict__ part_q, const float* __
         reinterpret_cast<float4*>(dg)[i] = sg;
     }
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_tok; i += stride) {
+        if (!seq_heads[i % H]) continue;
         float s = 0.f;
 #pragma unroll
         for (int sl = 0; sl < kSlices; ++sl) s += part_b[sl * n_tok + i];
@@ -296,7 +302,7 @@ __global__ void kda_bwd_reduce(const float* __restrict__ part_q, const float* __
 }
 
 struct BwdLayout {
-    size_t off_table, off_ckpt, off_pq, off_pk, off_pg, off_pb, total;
+    size_t off_table, off_heads, off_ckpt, off_pq, off_pk, off_pg, off_pb, total;
 };
 BwdLayout bwd_layout(int64_t T, int n_seqs, int H)
 {
@@ -304,7 +310,9 @@ BwdLayout bwd_layout(int64_t T, int n_seqs, int H)
     const size_t chunks = (size_t)((T + kC - 1) / kC + n_seqs);
     const size_t vec = (size_t)T * H * kD * sizeof(float);
     L.off_table = sizeof(WsHeader);
-    L.off_ckpt = L.off_table + align_up((size_t)(n_seqs + 1) * sizeof(int32_t));
+    L.off_heads = L.off_table + align_up((size_t)(n_seqs + 1) * sizeof(int32_t));
+    L.off_ckpt = L.off_heads + align_up((size_t)H * sizeof(int));
+    static_assert(bt::kFloats <= kBlocksPerChunk * kD * kD, "the chunk form's tiles fit where the sequential form keeps its states");
     L.off_pq = L.off_ckpt + align_up(chunks * kBlocksPerChunk * H * kD * kD * sizeof(float));
     L.off_pk = L.off_pq + align_up(kSlices * vec);
     L.off_pg = L.off_pk + align_up(kSlices * vec);
@@ -357,21 +365,25 @@ kda_status_t kda_chunk_bwd(const void* q, const void* k, const void* v, const fl
     for (const void* p : ptrs)
         if (!aligned16(p)) return fail(KDA_ERR_INVALID_ARG, "kda_chunk_bwd: pointer %p is not 16-byte "
                                        "aligned", p);
-    int64_t seq_len = 0, chunks_per_seq = 0;
+    int64_t seq_len = 0, chunks_per_seq = 0, n_chunks = 0;
     if (cu_seqlens_host) {
         if (cu_seqlens_host[0] != 0 || (int64_t)cu_seqlens_host[n_seqs] != total_tokens)
             return fail(KDA_ERR_INVALID_ARG, "kda_chunk_bwd: cu_seqlens must start at 0 and end at "
                         "total_tokens");
-        for (int n = 0; n < n_seqs; ++n)
+        for (int n = 0; n < n_seqs; ++n) {
             if (cu_seqlens_host[n + 1] < cu_seqlens_host[n])
                 return fail(KDA_ERR_INVALID_ARG, "kda_chunk_bwd: cu_seqlens decreases at %d", n);
+            n_chunks += ((int64_t)cu_seqlens_host[n + 1] - cu_seqlens_host[n] + kC - 1) / kC;
+        }
     } else {
         if (total_tokens % n_seqs != 0)
             return fail(KDA_ERR_INVALID_ARG, "kda_chunk_bwd: total_tokens not divisible by n_seqs for an "
                         "equal-length batch");
         seq_len = total_tokens / n_seqs;
         chunks_per_seq = (seq_len + kC - 1) / kC;
+        n_chunks = chunks_per_seq * n_seqs;
     }
+    if (n_chunks > 0x7fffffff) return fail(KDA_ERR_INVALID_ARG, "kda_chunk_bwd: too many chunks");
     const BwdLayout L = bwd_layout(total_tokens, n_seqs, H);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) || workspace_bytes < L.total)
         return fail(KDA_ERR_WORKSPACE, "kda_chunk_bwd: workspace must be 256-byte aligned and at least %zu "
@@ -380,8 +392,17 @@ kda_status_t kda_chunk_bwd(const void* q, const void* k, const void* v, const fl
     char* ws = static_cast<char*>(workspace);
     WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
     int32_t* chunk_cu_dev = reinterpret_cast<int32_t*>(ws + L.off_table);
-    kda_status_t rc = launch_prep(hdr, cu_seqlens_dev, chunk_cu_dev, n_seqs, st);
+    BwdChunkArgs ca;
+    ca.q = q; ca.k = k; ca.v = v; ca.d_o = d_o; ca.log_alpha = log_alpha; ca.beta = beta; ca.S0 = S0; ca.dS_T = dS_T;
+    ca.dq = dq; ca.dk = dk_out; ca.dv = dv_out; ca.dg = dlog_alpha; ca.db = dbeta; ca.dS0 = dS0;
+    ca.cu_seqlens = cu_seqlens_dev; ca.chunk_cu = cu_seqlens_dev ? chunk_cu_dev : nullptr;
+    ca.tiles = reinterpret_cast<float*>(ws + L.off_ckpt);
+    ca.seq_heads = reinterpret_cast<int*>(ws + L.off_heads);
+    ca.n_seqs = n_seqs; ca.H = H; ca.seq_len = seq_len; ca.chunks_per_seq = chunks_per_seq; ca.n_chunks = n_chunks;
+    ca.scale = scale;
+    kda_status_t rc = launch_bwd_chunk(ca, dt, hdr, chunk_cu_dev, st);
     if (rc != KDA_OK) return rc;
+    // heads with a chunk that decays too fast for the chunk form (normally none: these return at once)
     {
         DeviceLock lk;
         if (!lk.st) return lk.rc;
@@ -402,6 +423,7 @@ kda_status_t kda_chunk_bwd(const void* q, const void* k, const void* v, const fl
     a.part_k = reinterpret_cast<float*>(ws + L.off_pk);
     a.part_g = reinterpret_cast<float*>(ws + L.off_pg);
     a.part_b = reinterpret_cast<float*>(ws + L.off_pb);
+    a.seq_heads = ca.seq_heads;
     a.n_seqs = n_seqs; a.H = H; a.total_tokens = total_tokens; a.seq_len = seq_len;
     a.chunks_per_seq = chunks_per_seq; a.scale = scale;
     if (total_tokens > 0 || dS0) {
@@ -416,7 +438,7 @@ kda_status_t kda_chunk_bwd(const void* q, const void* k, const void* v, const fl
         const size_t n_vec = (size_t)total_tokens * H * kD, n_tok = (size_t)total_tokens * H;
         ProfScope ps(PROF_INTRA, st);
         kda_bwd_reduce<<<1184, 256, 0, st>>>(a.part_q, a.part_k, a.part_g, a.part_b, dq, dk_out, dlog_alpha,
-                                             dbeta, n_vec, n_tok);
+                                             dbeta, n_vec, n_tok, a.seq_heads, H);
         count_launch();
         KDA_CUDA_TRY(cudaGetLastError());
     }

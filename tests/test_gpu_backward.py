@@ -104,3 +104,22 @@ def test_backward_argument_errors():
         K.kda_chunk_bwd(z, z, z, z, b, None, z, None, z.clone(), z.clone(), z.clone(), z.clone(), b.clone(), None,
                         None, None, 1, 64, 1, 128, 128, 64, 1.0, K.KDA_F32, ws)
     assert ei.value.code == 3
+
+
+@pytest.mark.parametrize("lens,dtype", [([200, 63], torch.float32), ([65, 128, 1], torch.bfloat16)])
+def test_backward_fast_decay_heads(oracle_mod, lens, dtype):
+    """Heads whose decay leaves the range of the chunk form (log decay below -40 in some chunk) go through
+    the token-sequential kernels, the others through the chunk form, in the same call: head 0 stays
+    inside, head 1 leaves the range in every chunk, head 2 in one token, head 3 comes close (-38)."""
+    d = inputs.chunk_inputs(lens, H=4, dtype=dtype, seed=33, s0_std=0.05)
+    la = d["log_alpha"]
+    la[:, 1] *= 60.0
+    la[40, 2, 7] = -45.0
+    la[:, 3] = -38.0 / 64
+    d_o, dS_T = cotangents(d, 33, dtype)
+    out = run_bwd(d, d_o, dS_T)
+    ref = oracle_bwd(oracle_mod, d, d_o, dS_T)
+    for n in NAMES:
+        x, y = to_np32(out[n]), ref[n]
+        for h in range(4):      # (a decay ratio of head 3 carries up to 38 * 2^-24 = 2.3e-6)
+            assert rel_l2(x[:, h], y[:, h]) <= TOL, (n, h)
