@@ -1,4 +1,6 @@
-"""ctypes binding of ``include/kda.h``: argument marshalling only.
+"""Python binding of ``include/kda.h``: argument marshalling only (ctypes; for the calls a program makes
+every step the native marshalling of ``csrc/marshal.cpp`` comes first and leaves to ctypes what is not
+plain, e.g. arguments that have to raise).
 
 Every function has the name and argument order of its C entry point; tensors are ``torch`` tensors
 (used for device memory and streams only) whose ``data_ptr()`` is passed through.  Nothing is
@@ -21,6 +23,7 @@ _STATUS = {0: "KDA_OK", 1: "KDA_ERR_INVALID_ARG", 2: "KDA_ERR_UNSUPPORTED", 3: "
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_HERE, "libkda_b200.so")
 _lib = None
+_fast = None     # native marshalling, bound to _lib
 
 
 class KdaError(RuntimeError):
@@ -35,7 +38,7 @@ def library_path() -> str:
 
 def load():
     """Loads the CUDA library (built by ``paper_2510_26692_b200.build``); raises if it is absent."""
-    global _lib
+    global _lib, _fast
     if _lib is not None:
         return _lib
     if not os.path.exists(_LIB_PATH):
@@ -108,6 +111,11 @@ def load():
     lib.kda_version.restype = ctypes.c_char_p
     lib.kda_set_chunk_path.restype = i32
     lib.kda_set_chunk_path.argtypes = [i32]
+    from . import _marshal
+    _marshal.bind(*(ctypes.cast(f, vp).value for f in (
+        lib.kda_decode_step, lib.kda_decode_multi, lib.kda_layer_decode_step, lib.kda_chunk_fwd, lib.kda_layer_fwd,
+        lib.kda_chunk_bwd)))
+    _fast = _marshal
     _lib = lib
     return lib
 
@@ -185,6 +193,15 @@ def kda_chunk_fwd(q, k, v, log_alpha, beta, S0, o, S_T, cu_seqlens_dev, cu_seqle
                   stream=None):
     """``kda_chunk_fwd`` of ``include/kda.h``; device tensors, ``cu_seqlens_host`` a CPU int32
     tensor.  Asynchronous on ``stream`` (default: torch's current stream)."""
+    if _lib is None:
+        load()
+    rc = _fast.chunk_fwd(
+        q, k, v, log_alpha, beta, S0, o, S_T, cu_seqlens_dev, cu_seqlens_host, n_seqs, total_tokens, H, dk, dv,
+        chunk, scale, dt, workspace, workspace_bytes, stream)
+    if rc == 0:
+        return
+    if rc is not None:
+        _check(rc)
     f32 = torch.float32
     et = torch.bfloat16 if dt == KDA_BF16 else torch.float32
     if workspace_bytes is None:
@@ -236,6 +253,15 @@ def kda_chunk_bwd(q, k, v, log_alpha, beta, S0, d_o, dS_T, dq, dk_out, dv_out, d
                   workspace, workspace_bytes=None, stream=None):
     """``kda_chunk_bwd`` of ``include/kda.h``: gradients of the prefill operator (fp32 outputs).
     Asynchronous on ``stream``."""
+    if _lib is None:
+        load()
+    rc = _fast.chunk_bwd(
+        q, k, v, log_alpha, beta, S0, d_o, dS_T, dq, dk_out, dv_out, dlog_alpha, dbeta, dS0, cu_seqlens_dev,
+        cu_seqlens_host, n_seqs, total_tokens, H, dk, dv, chunk, scale, dt, workspace, workspace_bytes, stream)
+    if rc == 0:
+        return
+    if rc is not None:
+        _check(rc)
     f32 = torch.float32
     et = torch.bfloat16 if dt == KDA_BF16 else torch.float32
     if workspace_bytes is None:
@@ -272,6 +298,15 @@ def kda_layer_fwd(q_c, k_c, v, g_a, b_pre, g_o, A_log, dt_bias, rms_weight, l2_e
                   workspace_bytes=None, stream=None):
     """``kda_layer_fwd`` of ``include/kda.h``: the operator with L2Norm, decay function, beta
     sigmoid, head-wise RMSNorm and output gate, from bf16 pre-activations.  Asynchronous."""
+    if _lib is None:
+        load()
+    rc = _fast.layer_fwd(
+        q_c, k_c, v, g_a, b_pre, g_o, A_log, dt_bias, rms_weight, l2_eps, rms_eps, S0, y, S_T, cu_seqlens_dev,
+        cu_seqlens_host, n_seqs, total_tokens, H, dk, dv, chunk, scale, workspace, workspace_bytes, stream)
+    if rc == 0:
+        return
+    if rc is not None:
+        _check(rc)
     f32, bf = torch.float32, torch.bfloat16
     if workspace_bytes is None:
         workspace_bytes = workspace.numel() * workspace.element_size()
@@ -291,6 +326,15 @@ def kda_layer_decode_step(q_c, k_c, v, g_a, b_pre, g_o, A_log, dt_bias, rms_weig
                           state_slot, y, n_seqs, H, dk, dv, scale, stream=None):
     """``kda_layer_decode_step`` of ``include/kda.h``: one decode token per sequence with the layer's
     element-wise stages inside the kernel (bf16 activations, fp32 state in place)."""
+    if _lib is None:
+        load()
+    rc = _fast.layer_decode_step(
+        q_c, k_c, v, g_a, b_pre, g_o, A_log, dt_bias, rms_weight, l2_eps, rms_eps, S, state_slot, y, n_seqs, H, dk,
+        dv, scale, stream)
+    if rc == 0:
+        return
+    if rc is not None:
+        _check(rc)
     f32, bf = torch.float32, torch.bfloat16
     rc = load().kda_layer_decode_step(
         _ptr(q_c, True, bf, "q_c"), _ptr(k_c, True, bf, "k_c"), _ptr(v, True, bf, "v"), _ptr(g_a, True, bf, "g_a"),
@@ -329,6 +373,14 @@ def kda_chunk_fwd_static(q, k, v, log_alpha, beta, S0, o, S_T, cu_seqlens_dev, c
 def kda_decode_step(q, k, v, log_alpha, beta, S, state_slot, o, n_seqs, H, dk, dv, scale, dt,
                     stream=None):
     """``kda_decode_step`` of ``include/kda.h``; ``S`` is updated in place."""
+    if _lib is None:
+        load()
+    rc = _fast.decode_step(
+        q, k, v, log_alpha, beta, S, state_slot, o, n_seqs, H, dk, dv, scale, dt, stream)
+    if rc == 0:
+        return
+    if rc is not None:
+        _check(rc)
     f32 = torch.float32
     et = torch.bfloat16 if dt == KDA_BF16 else torch.float32
     rc = load().kda_decode_step(
@@ -343,6 +395,14 @@ def kda_decode_step(q, k, v, log_alpha, beta, S, state_slot, o, n_seqs, H, dk, d
 def kda_decode_multi(q, k, v, log_alpha, beta, S, state_slot, o, n_seqs, n_tokens, H, dk, dv, scale,
                      dt, stream=None):
     """``kda_decode_multi`` of ``include/kda.h``: ``n_tokens`` tokens per sequence, ``S`` in place."""
+    if _lib is None:
+        load()
+    rc = _fast.decode_multi(
+        q, k, v, log_alpha, beta, S, state_slot, o, n_seqs, n_tokens, H, dk, dv, scale, dt, stream)
+    if rc == 0:
+        return
+    if rc is not None:
+        _check(rc)
     f32 = torch.float32
     et = torch.bfloat16 if dt == KDA_BF16 else torch.float32
     rc = load().kda_decode_multi(
