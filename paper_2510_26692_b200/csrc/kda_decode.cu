@@ -10,6 +10,7 @@
 // four columns 4l..4l+3 of each: every warp-level access is one fully coalesced 512-byte row, and
 // all 16 loads of a thread are issued before the first use (64 KiB in flight per CTA).
 #include "kda_common.cuh"
+#include "kda_ptx.cuh"
 
 namespace kda {
 namespace {
@@ -58,35 +59,67 @@ struct DecodeLayer {
     float l2_eps, rms_eps;
 };
 
-template <typename T, bool kLayer>
-__global__ void __launch_bounds__(256, 2)
+// Columns of the state never mix, so a state may also be cut into column slices of NC columns with a CTA
+// each (decode_cols() says when): the lanes of a warp then cover 128 / NC rows at once.  The layer mode's
+// RMSNorm needs the whole output row, so it keeps whole states.
+template <typename T, bool kLayer, int NC>
+__global__ void __launch_bounds__(256, kD / NC * 2)
 kda_decode_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                   const float* __restrict__ log_alpha, const float* __restrict__ beta, float* S,
                   const int32_t* __restrict__ slot, T* __restrict__ o, int H, float scale, DecodeLayer lay)
 {
+    static_assert(!kLayer || NC == kD, "the output stage needs the whole row");
+    constexpr int kSlices = kD / NC;
+    constexpr int LPR = NC / 4;              // lanes per row
+    constexpr int RPW = 32 / LPR;            // rows of one warp-level access
+    constexpr int NX = kD / (8 * RPW);       // rows per thread
     __shared__ float s_a[kD], s_k[kD], s_q[kD];
-    __shared__ float4 s_red[2][8][32];
-    const int item = blockIdx.x;
+    __shared__ float4 s_red[2][8][LPR];
+    const int item = blockIdx.x / kSlices, slice = blockIdx.x - item * kSlices;
     const int n = item / H, h = item - n * H;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int col = slice * NC + (lane % LPR) * 4, row0 = warp * RPW + lane / LPR;
+    ptx::grid_dep_wait();                    // (launched before the preceding kernel has ended)
+    ptx::grid_dep_launch();
     const size_t sl = slot ? (size_t)slot[n] : (size_t)n;
-    float* Sp = S + (sl * H + h) * (size_t)(kD * kD) + lane * 4;
+    float* Sp = S + (sl * H + h) * (size_t)(kD * kD) + col;
 
-    float4 x[16];
-#pragma unroll
-    for (int m = 0; m < 16; ++m) x[m] = ld_stream(Sp + (size_t)(warp + 8 * m) * kD);
-
+    // the vectors first: their arithmetic is done by the time the state has arrived
     const size_t vec = (size_t)item * kD;
+    const float b_in = beta[item];
+    const float4 vv = IO<T>::load4(v + vec + col);
+    float4 w4 = make_float4(0.f, 0.f, 0.f, 0.f), g4 = w4;   // for the output stage
+    float kv_in = 0.f, qv_in = 0.f, g_in = 0.f, bias_in = 0.f, rate_in = 0.f;
+    if (t < kD) {
+        kv_in = to_f<T>(k[vec + t]);
+        qv_in = to_f<T>(q[vec + t]);
+        if (kLayer) {
+            g_in = to_f<T>(reinterpret_cast<const T*>(log_alpha)[vec + t]);
+            bias_in = lay.dt_bias[(size_t)h * kD + t];
+            rate_in = lay.A_log[h];
+        } else {
+            g_in = log_alpha[vec + t];
+        }
+    }
+    if (kLayer && warp == 0) {
+        w4 = *reinterpret_cast<const float4*>(lay.rms_weight + col);
+        g4 = IO<T>::load4(reinterpret_cast<const T*>(lay.g_o) + vec + col);
+    }
+    asm volatile("" ::: "memory");
+    float4 x[NX];
+#pragma unroll
+    for (int m = 0; m < NX; ++m) x[m] = ld_stream(Sp + (size_t)(row0 + 8 * RPW * m) * kD);
+
     if (t < kD) {
         if (kLayer) {
-            const float z = to_f<T>(reinterpret_cast<const T*>(log_alpha)[vec + t]) + lay.dt_bias[(size_t)h * kD + t];
+            const float z = g_in + bias_in;
             const float sp = fmaxf(z, 0.f) + log1pf(expf(-fabsf(z)));
-            s_a[t] = expf(-expf(lay.A_log[h]) * sp);
+            s_a[t] = expf(-expf(rate_in) * sp);
         } else {
-            s_a[t] = expf(log_alpha[vec + t]);
+            s_a[t] = expf(g_in);
         }
-        s_k[t] = to_f<T>(k[vec + t]);
-        s_q[t] = to_f<T>(q[vec + t]);
+        s_k[t] = kv_in;
+        s_q[t] = qv_in;
     }
     __syncthreads();
 
@@ -115,52 +148,78 @@ kda_decode_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __r
 
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f), s = p;
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
-        const int row = warp + 8 * m;
+    for (int m = 0; m < NX; ++m) {
+        const int row = row0 + 8 * RPW * m;
         const float a = s_a[row], kk = kLayer ? s_k[row] * rk : s_k[row], qq = kLayer ? s_q[row] * rq : s_q[row];
         x[m].x *= a; x[m].y *= a; x[m].z *= a; x[m].w *= a;
         p.x += kk * x[m].x; p.y += kk * x[m].y; p.z += kk * x[m].z; p.w += kk * x[m].w;
         s.x += qq * x[m].x; s.y += qq * x[m].y; s.z += qq * x[m].z; s.w += qq * x[m].w;
     }
-    s_red[0][warp][lane] = p;
-    s_red[1][warp][lane] = s;
+#pragma unroll
+    for (int ofs = LPR; ofs < 32; ofs <<= 1) {
+        p.x += __shfl_xor_sync(0xffffffffu, p.x, ofs); p.y += __shfl_xor_sync(0xffffffffu, p.y, ofs);
+        p.z += __shfl_xor_sync(0xffffffffu, p.z, ofs); p.w += __shfl_xor_sync(0xffffffffu, p.w, ofs);
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, ofs); s.y += __shfl_xor_sync(0xffffffffu, s.y, ofs);
+        s.z += __shfl_xor_sync(0xffffffffu, s.z, ofs); s.w += __shfl_xor_sync(0xffffffffu, s.w, ofs);
+    }
+    if (lane < LPR) {
+        s_red[0][warp][lane] = p;
+        s_red[1][warp][lane] = s;
+    }
     __syncthreads();
-    p = s_red[0][0][lane];
-    s = s_red[1][0][lane];
+    p = s_red[0][0][lane % LPR];
 #pragma unroll
     for (int w = 1; w < 8; ++w) {   // fixed order: bitwise reproducible
-        float4 a = s_red[0][w][lane], b = s_red[1][w][lane];
+        const float4 a = s_red[0][w][lane % LPR];
         p.x += a.x; p.y += a.y; p.z += a.z; p.w += a.w;
-        s.x += b.x; s.y += b.y; s.z += b.z; s.w += b.w;
     }
-    const float bt = kLayer ? 1.f / (1.f + expf(-beta[item])) : beta[item];
-    float4 vv = IO<T>::load4(v + vec + lane * 4);
-    float4 r = make_float4(vv.x - p.x, vv.y - p.y, vv.z - p.z, vv.w - p.w);
-    if (warp == 0) {
-        const float c = bt * qk;
-        float4 ov = make_float4(scale * (s.x + c * r.x), scale * (s.y + c * r.y),
-                                scale * (s.z + c * r.z), scale * (s.w + c * r.w));
-        if (kLayer) {   // head-wise RMSNorm over the 128 values of the row (4 per lane), weight, sigmoid gate
-            float ss = ov.x * ov.x + ov.y * ov.y + ov.z * ov.z + ov.w * ov.w;
+    const float bt = kLayer ? 1.f / (1.f + expf(-b_in)) : b_in;
+    const float4 r = make_float4(vv.x - p.x, vv.y - p.y, vv.z - p.z, vv.w - p.w);
 #pragma unroll
-            for (int ofs = 16; ofs > 0; ofs >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, ofs);
+    for (int m = 0; m < NX; ++m) {
+        const int row = row0 + 8 * RPW * m;
+        const float c = kLayer ? bt * s_k[row] * rk : bt * s_k[row];
+        x[m].x += c * r.x; x[m].y += c * r.y; x[m].z += c * r.z; x[m].w += c * r.w;
+        st_stream(Sp + (size_t)row * kD, x[m]);
+    }
+    // output row: warp 0 (its lanes below LPR)
+    float4 ov = make_float4(0.f, 0.f, 0.f, 0.f);
+    float ss = 0.f;
+    if (warp == 0) {
+        s = s_red[1][0][lane % LPR];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) {
+            const float4 b = s_red[1][w][lane % LPR];
+            s.x += b.x; s.y += b.y; s.z += b.z; s.w += b.w;
+        }
+        const float c = bt * qk;
+        ov = make_float4(scale * (s.x + c * r.x), scale * (s.y + c * r.y),
+                         scale * (s.z + c * r.z), scale * (s.w + c * r.w));
+        if (kLayer) {
+            ss = ov.x * ov.x + ov.y * ov.y + ov.z * ov.z + ov.w * ov.w;
+#pragma unroll
+            for (int ofs = LPR / 2; ofs > 0; ofs >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, ofs);
+        }
+        if (kLayer) {   // head-wise RMSNorm over the 128 values of the row (4 per lane), weight, sigmoid gate
             const float rstd = rsqrtf(ss * (1.f / kD) + lay.rms_eps);
-            const float4 w4 = *reinterpret_cast<const float4*>(lay.rms_weight + lane * 4);
-            const float4 g4 = IO<T>::load4(reinterpret_cast<const T*>(lay.g_o) + vec + lane * 4);
             ov.x *= rstd * w4.x / (1.f + expf(-g4.x));
             ov.y *= rstd * w4.y / (1.f + expf(-g4.y));
             ov.z *= rstd * w4.z / (1.f + expf(-g4.z));
             ov.w *= rstd * w4.w / (1.f + expf(-g4.w));
         }
-        IO<T>::store4(o + vec + lane * 4, ov);
+        IO<T>::store4(o + vec + col, ov);
     }
-#pragma unroll
-    for (int m = 0; m < 16; ++m) {
-        const int row = warp + 8 * m;
-        const float c = kLayer ? bt * s_k[row] * rk : bt * s_k[row];
-        x[m].x += c * r.x; x[m].y += c * r.y; x[m].z += c * r.z; x[m].w += c * r.w;
-        st_stream(Sp + (size_t)row * kD, x[m]);
-    }
+}
+
+// State columns per CTA of a call over `items` (sequence, head) pairs: half states, four CTAs per SM, have the
+// finer first and last wave; whole states win where one wave of two per SM holds the call (n_sm * 2 items)
+// and, by the fewer barriers per byte, in long streams.  Measured (us a step, whole / half): 32 states 3.4 /
+// 3.1, 96: 4.3 / 3.8, 160: 6.0 / 5.4, 288: 5.8 / 6.0, 512: 14.0 / 13.2, 1184: 27.8 / 26.4, 2048: 44.6 / 42.9,
+// 8192: 165.1 / 165.9.
+inline int decode_cols(int64_t items, int n_sm)
+{
+    if (items <= n_sm + n_sm / 2) return 64;
+    return items <= 2 * n_sm || items > 40 * n_sm ? kD : 64;
 }
 
 // Multi-token decode: the same recurrence for T consecutive tokens of each sequence (speculative
@@ -250,6 +309,8 @@ kda_decode_multi_kernel(const T* __restrict__ q, const T* __restrict__ k, const 
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
+    ptx::grid_dep_wait();      // (launched before the preceding kernel has ended)
+    ptx::grid_dep_launch();
     int item = blockIdx.x;
     if (item < n_items) fetch(item);
     for (; item < n_items; item += gridDim.x) {
@@ -366,25 +427,56 @@ kda_decode_multi_kernel(const T* __restrict__ q, const T* __restrict__ k, const 
 
 }  // namespace
 
+namespace {
+kda_status_t sm_count(int* n_sm)
+{
+    DeviceLock lk;
+    if (!lk.st) return lk.rc;
+    if (lk.st->n_sm == 0) {
+        int dev = 0;
+        KDA_CUDA_TRY(cudaGetDevice(&dev));
+        KDA_CUDA_TRY(cudaDeviceGetAttribute(&lk.st->n_sm, cudaDevAttrMultiProcessorCount, dev));
+    }
+    *n_sm = lk.st->n_sm;
+    return KDA_OK;
+}
+template <typename T, bool kLayer>
+kda_status_t launch_decode_t(const void* q, const void* k, const void* v, const float* log_alpha, const float* beta,
+                             float* S, const int32_t* slot, void* o, int n_seqs, int H, float scale,
+                             const DecodeLayer& lay, cudaStream_t st)
+{
+    ProfScope ps(PROF_DECODE, st);
+    int nc = kD;
+    if (!kLayer) {
+        int n_sm = 0;
+        if (const kda_status_t rc = sm_count(&n_sm)) return rc;
+        nc = decode_cols((int64_t)n_seqs * H, n_sm);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((size_t)n_seqs * H * (kD / nc)));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    auto kern = nc == kD ? kda_decode_kernel<T, kLayer, kD> : kda_decode_kernel<T, kLayer, kLayer ? kD : 64>;
+    KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, (const T*)q, (const T*)k, (const T*)v, log_alpha, beta, S, slot, (T*)o, H,
+                                    scale, lay));
+    count_launch();
+    return KDA_OK;
+}
+}  // namespace
+
 kda_status_t launch_decode(const void* q, const void* k, const void* v, const float* log_alpha,
                            const float* beta, float* S, const int32_t* slot, void* o, int n_seqs,
                            int H, float scale, kda_dtype_t dt, cudaStream_t st)
 {
     if (n_seqs == 0) return KDA_OK;
-    const unsigned grid = (unsigned)((size_t)n_seqs * H);
-    ProfScope ps(PROF_DECODE, st);
-    if (dt == KDA_BF16) {
-        using T = __nv_bfloat16;
-        kda_decode_kernel<T, false><<<grid, 256, 0, st>>>((const T*)q, (const T*)k, (const T*)v,
-                                                          log_alpha, beta, S, slot, (T*)o, H, scale, DecodeLayer());
-    } else {
-        kda_decode_kernel<float, false><<<grid, 256, 0, st>>>((const float*)q, (const float*)k,
-                                                              (const float*)v, log_alpha, beta, S, slot,
-                                                              (float*)o, H, scale, DecodeLayer());
-    }
-    count_launch();
-    KDA_CUDA_TRY(cudaGetLastError());
-    return KDA_OK;
+    if (dt == KDA_BF16)
+        return launch_decode_t<__nv_bfloat16, false>(q, k, v, log_alpha, beta, S, slot, o, n_seqs, H, scale, DecodeLayer(), st);
+    return launch_decode_t<float, false>(q, k, v, log_alpha, beta, S, slot, o, n_seqs, H, scale, DecodeLayer(), st);
 }
 
 kda_status_t launch_layer_decode(const void* q_c, const void* k_c, const void* v, const void* g_a,
@@ -393,18 +485,11 @@ kda_status_t launch_layer_decode(const void* q_c, const void* k_c, const void* v
                                  const int32_t* slot, void* y, int n_seqs, int H, float scale, cudaStream_t st)
 {
     if (n_seqs == 0) return KDA_OK;
-    using T = __nv_bfloat16;
     DecodeLayer lay;
     lay.A_log = A_log; lay.dt_bias = dt_bias; lay.g_o = g_o; lay.rms_weight = rms_weight;
     lay.l2_eps = l2_eps; lay.rms_eps = rms_eps;
-    const unsigned grid = (unsigned)((size_t)n_seqs * H);
-    ProfScope ps(PROF_DECODE, st);
-    kda_decode_kernel<T, true><<<grid, 256, 0, st>>>((const T*)q_c, (const T*)k_c, (const T*)v,
-                                                     reinterpret_cast<const float*>(g_a), b_pre, S, slot, (T*)y, H,
-                                                     scale, lay);
-    count_launch();
-    KDA_CUDA_TRY(cudaGetLastError());
-    return KDA_OK;
+    return launch_decode_t<__nv_bfloat16, true>(q_c, k_c, v, reinterpret_cast<const float*>(g_a), b_pre, S, slot, y, n_seqs,
+                                                H, scale, lay, st);
 }
 
 kda_status_t launch_decode_multi(const void* q, const void* k, const void* v, const float* log_alpha,
@@ -435,14 +520,23 @@ kda_status_t launch_decode_multi(const void* q, const void* k, const void* v, co
     const int n_items = n_seqs * H;
     const unsigned grid = (unsigned)(n_items < 2 * n_sm ? n_items : 2 * n_sm);   // persistent, two CTAs per SM
     ProfScope ps(PROF_DECODE, st);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = dt == KDA_BF16 ? MultiSmem<__nv_bfloat16>::kTotal : MultiSmem<float>::kTotal;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
     if (dt == KDA_BF16) {
         using T = __nv_bfloat16;
-        kda_decode_multi_kernel<T><<<grid, 256, MultiSmem<T>::kTotal, st>>>((const T*)q, (const T*)k, (const T*)v, log_alpha,
-                                                                  beta, S, slot, (T*)o, H, n_tok, scale, n_items);
+        KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kda_decode_multi_kernel<T>, (const T*)q, (const T*)k, (const T*)v, log_alpha,
+                                        beta, S, slot, (T*)o, H, n_tok, scale, n_items));
     } else {
-        kda_decode_multi_kernel<float><<<grid, 256, MultiSmem<float>::kTotal, st>>>((const float*)q, (const float*)k,
-                                                                      (const float*)v, log_alpha, beta, S, slot,
-                                                                      (float*)o, H, n_tok, scale, n_items);
+        KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kda_decode_multi_kernel<float>, (const float*)q, (const float*)k,
+                                        (const float*)v, log_alpha, beta, S, slot, (float*)o, H, n_tok, scale, n_items));
     }
     count_launch();
     KDA_CUDA_TRY(cudaGetLastError());
