@@ -28,7 +28,8 @@
  *     kda_check_status as KDA_ERR_GATE_RANGE.
  *   - dt selects the storage type of q, k, v and o (fp32 or bf16).  Gates, beta and states are
  *     always fp32.  dt = KDA_BF16 runs the contractions on bf16 tensor cores with fp32
- *     accumulation; dt = KDA_F32 runs everything in fp32 FMA arithmetic.
+ *     accumulation; dt = KDA_F32 keeps fp32 accuracy throughout: matrix products take
+ *     operands of 22 significant bits (two tf32 parts) with fp32 sums, everything else is fp32.
  *   - Supported shapes: dk = dv = 128, chunk = 64.  Anything else returns KDA_ERR_UNSUPPORTED;
  *     there is no fallback path of any kind.
  *   - Unless a parameter says "host", every pointer is a DEVICE pointer, 16-byte aligned, owned by
@@ -247,8 +248,8 @@ kda_status_t kda_chunk_bwd(const void *q, const void *k, const void *v, const fl
  *     S_t = (Diag(exp(g_t)) + b_t a_t^T) S_{t-1} + k_t v_t^T ,      o_t = scale * S_t^T q_t
  *
  * (a_t is contracted with the state the previous token left; with a = alpha . k, b = -beta k and
- * the key beta k this is Eq. 1).  fp32 storage and arithmetic only, in the same two-kernel FMA
- * style as kda_chunk_fwd with dt = KDA_F32, so that the two run times compare like with like.
+ * the key beta k this is Eq. 1).  fp32 storage and FMA arithmetic only, as two
+ * kernels like kda_chunk_fwd with dt = KDA_F32 (whose products run on the tensor cores).
  *
  *   q, k, a, b, g  [T_total, H, dk] fp32 device;  v, o [T_total, H, dv] fp32 device
  *   S0, S_T, cu_seqlens_dev, cu_seqlens_host, n_seqs, total_tokens, H, scale: as in kda_chunk_fwd

@@ -111,7 +111,7 @@ bool shape_ok(int dk, int dv, int chunk, kda_dtype_t dt)
 
 size_t tile_bytes(kda_dtype_t dt)
 {
-    return dt == KDA_BF16 ? tc_tile_bytes() : simt_tile_bytes();
+    return dt == KDA_BF16 ? tc_tile_bytes() : f32_tile_bytes();
 }
 
 struct WsLayout {
@@ -462,7 +462,7 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
         if (dt == KDA_BF16)
             rc = launch_chunk_tc(a, ws + L.off_tiles, n_begin, n_count, hdr, tc_clears && first, st);
         else
-            rc = launch_chunk_simt(a, dt, ws + L.off_tiles, n_begin, n_count, hdr, st);
+            rc = launch_chunk_f32(a, ws + L.off_tiles, n_begin, n_count, hdr, st);
         if (rc != KDA_OK) return rc;
         g0 = g1;
         first = false;

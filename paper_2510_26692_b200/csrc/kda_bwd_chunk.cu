@@ -94,20 +94,6 @@ constexpr int kFloats = VEC + 128 + 64 + 512;
 constexpr size_t kSmem1 = (size_t)p1::kFloats * 4;
 static_assert(kSmem1 <= 232448, "fits the shared memory of one SM");
 
-// rows of a 16 MT x 8 NT fragment block to a row-major array
-template <int MT, int NT, typename F>
-__device__ __forceinline__ void each_pair(const float (&acc)[MT][NT][4], int lane, F f) {
-    const int g = lane >> 2, c = lane & 3;
-#pragma unroll
-    for (int m = 0; m < MT; ++m)
-#pragma unroll
-        for (int n = 0; n < NT; ++n) {
-            f(16 * m + g, 8 * n + 2 * c, acc[m][n][0], acc[m][n][1]);
-            f(16 * m + g + 8, 8 * n + 2 * c, acc[m][n][2], acc[m][n][3]);
-        }
-}
-__device__ __forceinline__ void st2(float* p, float x, float y) { *reinterpret_cast<float2*>(p) = make_float2(x, y); }
-
 template <typename T>
 __global__ void __launch_bounds__(kT1, 1) kda_bwd_intra(BwdChunkArgs a)
 {
@@ -208,49 +194,7 @@ __global__ void __launch_bounds__(kT1, 1) kda_bwd_intra(BwdChunkArgs a)
     }
     __syncthreads();
 
-    // T' = (I + B Diag(beta))^-1: 16 x 16 diagonal blocks by substitution, then two doublings
-    // [T11 0; T21 T22] with T21 = -T22 (L21 T11); the inner product sits in the empty upper triangle of sB
-    if (t < 64) {
-        const int b0 = t & 48, j = t & 15;
-        float x[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            float s0 = i == j ? 1.f : 0.f, s1 = 0.f;
-#pragma unroll
-            for (int m = 0; m < i; ++m) {
-                const float l = sB[(b0 + i) * LM + b0 + m];
-                if (m & 1) s1 = fmaf(-l, x[m], s1); else s0 = fmaf(-l, x[m], s0);
-            }
-            x[i] = s0 + s1;
-            sT[(b0 + i) * LM + b0 + j] = x[i];
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int s = 16; s < 64; s *= 2) {
-        for (int idx = t; idx < 32 * s; idx += kT1) {
-            const int j = idx % s, i = (idx / s) % s, c0 = idx / (s * s) * 2 * s, r0 = c0 + s;
-            float x0 = 0.f, x1 = 0.f;
-#pragma unroll 8
-            for (int m = 0; m < s; m += 2) {
-                x0 = fmaf(sB[(r0 + i) * LM + c0 + m], sT[(c0 + m) * LM + c0 + j], x0);
-                x1 = fmaf(sB[(r0 + i) * LM + c0 + m + 1], sT[(c0 + m + 1) * LM + c0 + j], x1);
-            }
-            sB[(c0 + i) * LM + r0 + j] = x0 + x1;
-        }
-        __syncthreads();
-        for (int idx = t; idx < 32 * s; idx += kT1) {
-            const int j = idx % s, i = (idx / s) % s, c0 = idx / (s * s) * 2 * s, r0 = c0 + s;
-            float x0 = 0.f, x1 = 0.f;
-#pragma unroll 8
-            for (int m = 0; m < s; m += 2) {
-                x0 = fmaf(sT[(r0 + i) * LM + r0 + m], sB[(c0 + m) * LM + r0 + j], x0);
-                x1 = fmaf(sT[(r0 + i) * LM + r0 + m + 1], sB[(c0 + m + 1) * LM + r0 + j], x1);
-            }
-            sT[(r0 + i) * LM + c0 + j] = -(x0 + x1);
-        }
-        __syncthreads();
-    }
+    invert_unit_lower<kT1, LM>(sB, sT, t);      // T' = (I + B Diag(beta))^-1
     for (int idx = t; idx < 64 * 64; idx += kT1) tile[bt::T + idx] = sT[(idx >> 6) * LM + (idx & 63)];
 
     // W' = T' K^, U' = T' V, P^T dO: warps 2 x 8, 32 x 16 entries each; the triangles bound the sums
@@ -297,12 +241,6 @@ template <int NS> struct ChainSmem {
     static constexpr size_t kBytes = (size_t)(ST + 128 * LS) * 4;
 };
 static_assert(ChainSmem<64>::kBytes <= 232448, "fits the shared memory of one SM");
-
-__device__ __forceinline__ void cp16(float* dst, const float* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 template <int NS, bool kFwd>
 __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, float* sm, int n, int h, int col0)
@@ -723,7 +661,8 @@ kda_status_t launch_bwd_chunk(const BwdChunkArgs& a, kda_dtype_t dt, WsHeader* h
     }
     {
         ProfScope ps(PROF_INTER, st);
-        const bool narrow = (int64_t)a.n_seqs * a.H * 4 <= 148;   // 64-column slices would leave half the SMs idle
+        // one CTA per SM (shared memory): 32-column slices only while they fit one wave
+        const bool narrow = (int64_t)a.n_seqs * a.H * 8 <= 148;
         if (narrow) kda_bwd_chain<32><<<dim3(8, (unsigned)a.H, (unsigned)a.n_seqs), kT2, ChainSmem<32>::kBytes, st>>>(a);
         else kda_bwd_chain<64><<<dim3(4, (unsigned)a.H, (unsigned)a.n_seqs), kT2, ChainSmem<64>::kBytes, st>>>(a);
     }

@@ -176,9 +176,9 @@ kda_status_t launch_decode_multi(const void* q, const void* k, const void* v, co
                                  const float* beta, float* S, const int32_t* slot, void* o, int n_seqs,
                                  int n_tok, int H, float scale, kda_dtype_t dt, cudaStream_t st);
 
-// fp32 FMA path (also accepts bf16 storage): per-tile scratch size and pass launcher
-size_t simt_tile_bytes();
-kda_status_t launch_chunk_simt(const ChunkArgs& a, kda_dtype_t dt, void* tiles, int n_begin,
+// fp32 path: per-tile scratch size and pass launcher
+size_t f32_tile_bytes();
+kda_status_t launch_chunk_f32(const ChunkArgs& a, void* tiles, int n_begin,
                                int n_count, WsHeader* hdr, cudaStream_t st);
 
 // bf16 tensor-core path (tcgen05 + bulk copies): per-tile scratch size and pass launcher

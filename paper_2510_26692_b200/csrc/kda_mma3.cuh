@@ -14,14 +14,11 @@
 namespace kda {
 namespace mma3 {
 
-__device__ __forceinline__ uint32_t tf32_rn(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return r;
-}
+// Rounding to nearest (ties away) by an integer addition on the bit pattern; the tensor core ignores the 13
+// low bits.  (cvt.rna.tf32 gives the same and is several times slower to issue.)
 __device__ __forceinline__ void split(float x, uint32_t& hi, uint32_t& lo) {
-    hi = tf32_rn(x);
-    lo = tf32_rn(x - __uint_as_float(hi));
+    hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+    lo = __float_as_uint(x - __uint_as_float(hi)) + 0x1000u;
 }
 __device__ __forceinline__ void mma8(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
     asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -103,6 +100,76 @@ __device__ __forceinline__ void zero(float (&acc)[MT][NT][4]) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) acc[m][n][j] = 0.f;
 }
+
+// f(row, column, x, y) for every pair of neighbouring columns that this lane holds of a fragment block
+template <int MT, int NT, typename F>
+__device__ __forceinline__ void each_pair(const float (&acc)[MT][NT][4], int lane, F f) {
+    const int g = lane >> 2, c = lane & 3;
+#pragma unroll
+    for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            f(16 * m + g, 8 * n + 2 * c, acc[m][n][0], acc[m][n][1]);
+            f(16 * m + g + 8, 8 * n + 2 * c, acc[m][n][2], acc[m][n][3]);
+        }
+}
+__device__ __forceinline__ void st2(float* p, float x, float y) { *reinterpret_cast<float2*>(p) = make_float2(x, y); }
+
+// T = (I + L)^-1 of a strictly lower triangular 64 x 64 L (row pitch LD, its upper triangle is overwritten), by
+// kThreads threads; T has to be zero above the diagonal blocks on entry.  16 x 16 diagonal blocks by
+// substitution (one column per thread), then two doublings [T11 0; T21 T22], T21 = -T22 (L21 T11), whose
+// inner product sits in the empty upper triangle of L.  fp32 FMA: the chain of dependent products is
+// what the result's accuracy rests on.  Ends with a barrier.
+template <int kThreads, int LD>
+__device__ __forceinline__ void invert_unit_lower(float* __restrict__ L, float* __restrict__ T, int t) {
+    if (t < 64) {
+        const int b0 = t & 48, j = t & 15;
+        float x[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            float s0 = i == j ? 1.f : 0.f, s1 = 0.f;
+#pragma unroll
+            for (int m = 0; m < i; ++m) {
+                const float l = L[(b0 + i) * LD + b0 + m];
+                if (m & 1) s1 = fmaf(-l, x[m], s1); else s0 = fmaf(-l, x[m], s0);
+            }
+            x[i] = s0 + s1;
+            T[(b0 + i) * LD + b0 + j] = x[i];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int s = 16; s < 64; s *= 2) {
+        for (int idx = t; idx < 32 * s; idx += kThreads) {
+            const int j = idx % s, i = (idx / s) % s, c0 = idx / (s * s) * 2 * s, r0 = c0 + s;
+            float x0 = 0.f, x1 = 0.f;
+#pragma unroll 8
+            for (int m = 0; m < s; m += 2) {
+                x0 = fmaf(L[(r0 + i) * LD + c0 + m], T[(c0 + m) * LD + c0 + j], x0);
+                x1 = fmaf(L[(r0 + i) * LD + c0 + m + 1], T[(c0 + m + 1) * LD + c0 + j], x1);
+            }
+            L[(c0 + i) * LD + r0 + j] = x0 + x1;
+        }
+        __syncthreads();
+        for (int idx = t; idx < 32 * s; idx += kThreads) {
+            const int j = idx % s, i = (idx / s) % s, c0 = idx / (s * s) * 2 * s, r0 = c0 + s;
+            float x0 = 0.f, x1 = 0.f;
+#pragma unroll 8
+            for (int m = 0; m < s; m += 2) {
+                x0 = fmaf(T[(r0 + i) * LD + r0 + m], L[(c0 + m) * LD + r0 + j], x0);
+                x1 = fmaf(T[(r0 + i) * LD + r0 + m + 1], L[(c0 + m + 1) * LD + r0 + j], x1);
+            }
+            T[(r0 + i) * LD + c0 + j] = -(x0 + x1);
+        }
+        __syncthreads();
+    }
+}
+
+__device__ __forceinline__ void cp16(float* dst, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 }  // namespace mma3
 }  // namespace kda
