@@ -399,8 +399,8 @@ kda_status_t kda_chunk_bwd(const void* q, const void* k, const void* v, const fl
     ca.tiles = reinterpret_cast<float*>(ws + L.off_ckpt);
     ca.seq_heads = reinterpret_cast<int*>(ws + L.off_heads);
     ca.n_seqs = n_seqs; ca.H = H; ca.seq_len = seq_len; ca.chunks_per_seq = chunks_per_seq; ca.n_chunks = n_chunks;
-    ca.scale = scale;
-    kda_status_t rc = launch_bwd_chunk(ca, dt, hdr, chunk_cu_dev, st);
+    ca.scale = scale; ca.hdr = hdr; ca.wait_limit_ns = wait_limit_ns();
+    kda_status_t rc = launch_bwd_chunk(ca, dt, chunk_cu_dev, st);
     if (rc != KDA_OK) return rc;
     // heads with a chunk that decays too fast for the chunk form (normally none: these return at once)
     {

@@ -15,8 +15,10 @@ struct BwdChunkArgs {
     float* tiles;                                                    // [chunks][H][kBwdTile]
     int* seq_heads;   // [H]: 1 = a chunk of this head decays too fast for the chunkwise form
     int n_seqs, H;
+    WsHeader* hdr;
     int64_t seq_len, chunks_per_seq, n_chunks;
     float scale;
+    unsigned long long wait_limit_ns;
 };
 
 // Scratch tile (floats), written by the first kernel unless stated otherwise
@@ -35,6 +37,33 @@ constexpr int GC = B + 64 * 64;      // [128] e^(G_C)
 constexpr int kFloats = GC + 128;
 }  // namespace bt
 
-kda_status_t launch_bwd_chunk(const BwdChunkArgs& a, kda_dtype_t dt, WsHeader* hdr, int32_t* chunk_cu_dev, cudaStream_t st);
+// first token, valid tokens (1..64) and sequence of global chunk g
+struct BwdLoc { int64_t tok0; int len; int n; };
+__device__ __forceinline__ BwdLoc bwd_locate(const BwdChunkArgs& a, int64_t g) {
+    BwdLoc L;
+    int64_t c;
+    int64_t b, e;
+    if (a.cu_seqlens == nullptr) {
+        L.n = (int)(g / a.chunks_per_seq);
+        c = g - (int64_t)L.n * a.chunks_per_seq;
+        b = (int64_t)L.n * a.seq_len; e = b + a.seq_len;
+    } else {
+        int lo = 0, hi = a.n_seqs - 1;   // last n with chunk_cu[n] <= g
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if ((int64_t)a.chunk_cu[mid] <= g) lo = mid; else hi = mid - 1;
+        }
+        L.n = lo;
+        c = g - a.chunk_cu[lo];
+        b = a.cu_seqlens[lo]; e = a.cu_seqlens[lo + 1];
+    }
+    L.tok0 = b + c * kC;
+    L.len = (e - L.tok0) < kC ? (int)(e - L.tok0) : kC;
+
+    return L;
+}
+
+kda_status_t launch_bwd_out(const BwdChunkArgs& a, kda_dtype_t dt, cudaStream_t st);
+kda_status_t launch_bwd_chunk(const BwdChunkArgs& a, kda_dtype_t dt, int32_t* chunk_cu_dev, cudaStream_t st);
 
 }  // namespace kda

@@ -28,32 +28,6 @@ using namespace mma3;
 // every decay ratio carries a relative error of up to kRange 2^-24 = 2.4e-6.
 constexpr float kRange = 40.f;
 
-struct BLoc { int64_t tok0; int len; int n; int first, last; };
-__device__ __forceinline__ BLoc locate(const BwdChunkArgs& a, int64_t g) {
-    BLoc L;
-    int64_t c, nc;
-    int64_t b, e;
-    if (a.cu_seqlens == nullptr) {
-        L.n = (int)(g / a.chunks_per_seq);
-        c = g - (int64_t)L.n * a.chunks_per_seq;
-        nc = a.chunks_per_seq;
-        b = (int64_t)L.n * a.seq_len; e = b + a.seq_len;
-    } else {
-        int lo = 0, hi = a.n_seqs - 1;   // last n with chunk_cu[n] <= g
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if ((int64_t)a.chunk_cu[mid] <= g) lo = mid; else hi = mid - 1;
-        }
-        L.n = lo;
-        c = g - a.chunk_cu[lo];
-        nc = a.chunk_cu[lo + 1] - a.chunk_cu[lo];
-        b = a.cu_seqlens[lo]; e = a.cu_seqlens[lo + 1];
-    }
-    L.tok0 = b + c * kC;
-    L.len = (e - L.tok0) < kC ? (int)(e - L.tok0) : kC;
-    L.first = c == 0; L.last = c + 1 == nc;
-    return L;
-}
 template <typename T> __device__ __forceinline__ float ldf(const T* p);
 template <> __device__ __forceinline__ float ldf<float>(const float* p) { return *p; }
 template <> __device__ __forceinline__ float ldf<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
@@ -101,7 +75,7 @@ __global__ void __launch_bounds__(kT1, 1) kda_bwd_intra(BwdChunkArgs a)
     extern __shared__ __align__(16) float sm[];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int h = blockIdx.y;
-    const BLoc loc = locate(a, blockIdx.x);
+    const BwdLoc loc = bwd_locate(a, blockIdx.x);
     float* tile = a.tiles + ((size_t)blockIdx.x * a.H + h) * bt::kFloats;
     float* sKG = sm + p1::KG; float* sKI = sm + p1::KI; float* sQG = sm + p1::QG;
     float* sV = sm + p1::V; float* sDO = sm + p1::DO;
@@ -373,270 +347,9 @@ __global__ void __launch_bounds__(kT2, 1) kda_bwd_chain(BwdChunkArgs a)
     else chain_run<NS, false>(a, sm, n, h, slice * NS);
 }
 
-// ---- gradients ---------------------------------------------------------------------------------------
-constexpr int kT3 = 512;
-namespace p3 {
-constexpr int DO = 0;                            // [64][LR] d_o, later dP (first 64 x LM)
-constexpr int DV = DO + 64 * LR;                 // [64][LR] dV,  later dB (first 64 x LM)
-constexpr int R = DV + 64 * LR;                  // [64][LR] r
-constexpr int BIG = R + 64 * LR;                 // two 64-row halves of S, then of Lam [2][64][LR] | dX [64][LC]
-constexpr int DX = BIG + 2 * 64 * LR;            //   later Q, K^, K_ [3][64][LC]; at the end dQ, dK^, dK_ [3][64][LR]
-constexpr int T = BIG + 3 * 64 * LC;             // [64][72] beta T'
-constexpr int LT = 72;
-constexpr int VEC = T + 64 * LT;                 // beta[64], e^(G_m)[128], e^(G_C - G_m)[128], d G_C [2][128], dbeta [9][64], [4][128]
-constexpr int kFloats = VEC + 64 + 128 + 128 + 256 + 9 * 64 + 512;
-static_assert(DX + 64 * LC <= T, "dX fits before T'");
-}  // namespace p3
-constexpr size_t kSmem3 = (size_t)p3::kFloats * 4;
-static_assert(kSmem3 <= 232448, "fits the shared memory of one SM");
-
-template <typename T>
-__global__ void __launch_bounds__(kT3, 1) kda_bwd_out(BwdChunkArgs a)
-{
-    constexpr bool kX = sizeof(T) == 2;
-    extern __shared__ __align__(16) float sm[];
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int h = blockIdx.y;
-    if (a.seq_heads[h]) return;
-    const BLoc loc = locate(a, blockIdx.x);
-    const float* tile = a.tiles + ((size_t)blockIdx.x * a.H + h) * bt::kFloats;
-    float* sDO = sm + p3::DO; float* sDV = sm + p3::DV; float* sR = sm + p3::R; float* sBig = sm + p3::BIG;
-    float* sDX = sm + p3::DX; float* sT = sm + p3::T;
-    float* sBeta = sm + p3::VEC; float* sEm = sBeta + 64; float* sEc = sEm + 128; float* sGC = sEc + 128;
-    float* sDb = sGC + 256; float* sSeg = sDb + 9 * 64;
-
-    // half hf of a state (S or Lam): rows 32 x + 16 hf + y go to buffer row 16 x + y, so that both halves
-    // of the product below give a warp neighbouring columns
-    auto fetch_half = [&](const float* src, int hf) {
-        float* dst = sBig + hf * 64 * LR;
-        for (int idx = t; idx < 64 * 32; idx += kT3) {
-            const int r = idx >> 5, x = (idx & 31) * 4;
-            cp16(dst + r * LR + x, src + (32 * (r >> 4) + 16 * hf + (r & 15)) * kD + x);
-        }
-        cp_commit();
-    };
-    for (int idx = t; idx < 64 * 32; idx += kT3) {
-        const int r = idx >> 5, x = (idx & 31) * 4;
-        cp16(sDX + r * LC + x, tile + bt::X + r * kD + x);
-        cp16(sR + r * LR + x, tile + bt::R + r * kD + x);
-    }
-    cp_commit();
-    fetch_half(tile + bt::S, 0);
-    fetch_half(tile + bt::S, 1);
-    for (int idx = t; idx < 64 * 16; idx += kT3) {
-        const int r = idx >> 4, x = (idx & 15) * 4;
-        const float b = r < loc.len ? a.beta[(size_t)(loc.tok0 + r) * a.H + h] : 0.f;
-        const float4 v = *reinterpret_cast<const float4*>(tile + bt::T + r * 64 + x);
-        *reinterpret_cast<float4*>(sT + r * p3::LT + x) = make_float4(b * v.x, b * v.y, b * v.z, b * v.w);
-        if (x == 0) sBeta[r] = b;
-    }
-    for (int idx = t; idx < 64 * 32; idx += kT3) {
-        const int r = idx >> 5, x = (idx & 31) * 4;
-        float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < loc.len && a.d_o)
-            y = IO<T>::load4(reinterpret_cast<const T*>(a.d_o) + ((size_t)(loc.tok0 + r) * a.H + h) * kD + x);
-        *reinterpret_cast<float4*>(sDO + r * LR + x) = y;
-    }
-    if (t < 128) {
-        const float gc = tile[bt::G + 63 * kD + t];
-        const float e = expf(0.5f * gc);
-        sEm[t] = e;
-        sEc[t] = e;     // G_m = G_C / 2
-    }
-    asm volatile("cp.async.wait_group 2;" ::: "memory");
-    __syncthreads();
-
-    // dV = (beta T')^T dX: warps 2 x 8, 32 x 16 entries each
-    {
-        const int r0 = (w >> 3) * 32, c0 = (w & 7) * 16;
-        float acc[2][2][4];
-        zero(acc);
-        gemm<0, 2, true, false, false, false>(acc, sT + r0, p3::LT, sDX + c0, LC, r0, 64, lane);
-        each_pair(acc, lane, [&](int i, int j, float x, float y) {
-            i += r0; j += c0;
-            st2(sDV + i * LR + j, x, y);
-            if (i < loc.len) st2(a.dv + ((size_t)(loc.tok0 + i) * a.H + h) * kD + j, x, y);
-        });
-        // r_j . dX_j: 8 threads per row
-        const int row = t >> 3, e = (t & 7) * 4;
-        float s = 0.f;
-#pragma unroll
-        for (int x = 0; x < 128; x += 32) {
-            const float4 u = *reinterpret_cast<const float4*>(sR + row * LR + x + e);
-            const float4 v = *reinterpret_cast<const float4*>(sDX + row * LC + x + e);
-            s += u.x * v.x + u.y * v.y + u.z * v.z + u.w * v.w;
-        }
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if ((t & 7) == 0) sDb[row] = s;
-    }
-    cp_wait0();
-    __syncthreads();
-
-    // [d_o ; dV] S^T: warps 4 x 4, 32 x 32 entries each
-    const int mi = w >> 2, ni = w & 3;
-    float acc[2][4][4];
-    zero(acc);
-    gemm<0, 2, false, true, kX, false>(acc, sDO + mi * 32 * LR, LR, sBig + 16 * ni * LR, LR, 0, mi < 2 ? kD : 0, lane);
-    gemm<2, 2, false, true, kX, false>(acc, sDO + mi * 32 * LR, LR, sBig + (64 + 16 * ni) * LR, LR, 0, mi < 2 ? kD : 0, lane);
-    gemm<0, 2, false, true, false, false>(acc, sDO + mi * 32 * LR, LR, sBig + 16 * ni * LR, LR, 0, mi < 2 ? 0 : kD, lane);
-    gemm<2, 2, false, true, false, false>(acc, sDO + mi * 32 * LR, LR, sBig + (64 + 16 * ni) * LR, LR, 0, mi < 2 ? 0 : kD, lane);
-    __syncthreads();
-    fetch_half(tile + bt::L, 0);
-    fetch_half(tile + bt::L, 1);
-    // e^(G_C) rowsum(S Lam): warp w takes rows 8 w .. 8 w + 7
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int r = 8 * w + j;
-        const float4 u = *reinterpret_cast<const float4*>(tile + bt::S + r * kD + lane * 4);
-        const float4 v = *reinterpret_cast<const float4*>(tile + bt::L + r * kD + lane * 4);
-        float s = u.x * v.x + u.y * v.y + u.z * v.z + u.w * v.w;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) sGC[r] = s * tile[bt::GC + r];
-    }
-    // Gram matrices [d_o ; dV] r^T: warps 4 x 4, 32 x 16 entries each
-    float gr[2][2][4];
-    zero(gr);
-    const int gr0 = (mi & 1) * 32, gc0 = ni * 16;
-    if (gc0 < gr0 + 32) {
-        if (mi < 2) gemm<0, 2, false, true, kX, false>(gr, sDO + mi * 32 * LR, LR, sR + gc0 * LR, LR, 0, kD, lane);
-        else gemm<0, 2, false, true, false, false>(gr, sDO + mi * 32 * LR, LR, sR + gc0 * LR, LR, 0, kD, lane);
-    }
-    {
-        const float sgn = mi < 2 ? 1.f : -1.f;
-#pragma unroll
-        for (int m = 0; m < 2; ++m)
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[m][nt][j] *= sgn * sEm[32 * ni + 8 * nt + 2 * (lane & 3) + (j & 1)];
-    }
-    cp_wait0();
-    __syncthreads();
-
-    // r Lam^T, rows scaled by beta and columns by e^(G_C - G_m): warps 4 x 4, 16 x 32 entries each
-    float ak[1][4][4];
-    zero(ak);
-    gemm<0, 2, false, true, false, false>(ak, sR + mi * 16 * LR, LR, sBig + 16 * ni * LR, LR, 0, kD, lane);
-    gemm<2, 2, false, true, false, false>(ak, sR + mi * 16 * LR, LR, sBig + (64 + 16 * ni) * LR, LR, 0, kD, lane);
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            ak[0][nt][j] *= sBeta[16 * mi + 8 * (j >> 1) + (lane >> 2)] * sEc[32 * ni + 8 * nt + 2 * (lane & 3) + (j & 1)];
-    // dbeta's share sum_i B_ij (dV_i . r_j), then the masked and scaled Gram matrices to shared memory
-    {
-        float cs[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-        float* dst = mi < 2 ? sDO : sDV;
-        const int strict = mi < 2 ? 0 : 1;
-        const float sgn = mi < 2 ? 1.f : -1.f;
-        __syncthreads();      // d_o, dV, r and Lam are no longer read
-#pragma unroll
-        for (int m = 0; m < 2; ++m)
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                    const int i = gr0 + 16 * m + 8 * hf + (lane >> 2), j = gc0 + 8 * nt + 2 * (lane & 3);
-                    float x = gr[m][nt][2 * hf], y = gr[m][nt][2 * hf + 1];
-                    x = j + strict <= i ? x : 0.f;
-                    y = j + 1 + strict <= i ? y : 0.f;
-                    if (mi >= 2) {
-                        const float2 b = *reinterpret_cast<const float2*>(tile + bt::B + i * 64 + j);
-                        cs[nt][0] = fmaf(b.x, x, cs[nt][0]);
-                        cs[nt][1] = fmaf(b.y, y, cs[nt][1]);
-                    }
-                    st2(dst + i * LM + j, sgn * sBeta[j] * x, sgn * sBeta[j + 1] * y);
-                }
-        if (mi >= 2) {
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    float s = cs[nt][e];
-                    s += __shfl_xor_sync(0xffffffffu, s, 4);
-                    s += __shfl_xor_sync(0xffffffffu, s, 8);
-                    s += __shfl_xor_sync(0xffffffffu, s, 16);
-                    if (lane < 4) sDb[64 * (mi - 1) + gc0 + 8 * nt + 2 * lane + e] = s;
-                }
-        }
-    }
-    // gated operands: thread = channel c of 16 consecutive tokens
-    const int c = t & 127, seg = t >> 7;
-    float* sQG = sBig; float* sKG = sBig + 64 * LC; float* sKI = sBig + 2 * 64 * LC;
-    const T* kp = reinterpret_cast<const T*>(a.k);
-    const T* qp = reinterpret_cast<const T*>(a.q);
-    const float gm = 0.5f * tile[bt::G + 63 * kD + c];
-#pragma unroll 4
-    for (int i = 0; i < 16; ++i) {
-        const int r = seg * 16 + i;
-        const size_t off = ((size_t)(loc.tok0 + r) * a.H + h) * kD + c;
-        const bool in = r < loc.len;
-        const float G = tile[bt::G + r * kD + c];
-        const float kk = in ? ldf<T>(kp + off) : 0.f, qq = in ? ldf<T>(qp + off) : 0.f;
-        const float e1 = expf(G - gm), e2 = expf(gm - G);
-        sQG[r * LC + c] = a.scale * qq * e1;
-        sKG[r * LC + c] = kk * e1;
-        sKI[r * LC + c] = kk * e2;
-    }
-    __syncthreads();
-    if (t < 64 && t < loc.len) a.db[(size_t)(loc.tok0 + t) * a.H + h] = sDb[t] - (sDb[64 + t] + sDb[128 + t]);
-    // sum_i K~_i (beta r Lam^T)_i: per warp over its 16 rows
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int cc = 32 * ni + 8 * nt + 2 * (lane & 3) + e, r = 16 * mi + (lane >> 2);
-            float s = ak[0][nt][e] * sKI[r * LC + cc] + ak[0][nt][2 + e] * sKI[(r + 8) * LC + cc];
-            s += __shfl_xor_sync(0xffffffffu, s, 4);
-            s += __shfl_xor_sync(0xffffffffu, s, 8);
-            s += __shfl_xor_sync(0xffffffffu, s, 16);
-            if (lane < 4) sSeg[mi * 128 + cc] = s;
-        }
-    // dQ += dP K_, dK^ += dB K_ ; dK_ += dP^T Q + dB^T K^
-    gemm<0, 4, false, false, false, false>(acc, (mi < 2 ? sDO : sDV) + gr0 * LM, LM, sKI + 32 * ni, LC, 0, gr0 + 32, lane);
-    gemm<0, 4, true, false, false, false>(ak, sDO + 16 * mi, LM, sQG + 32 * ni, LC, 16 * mi, 64, lane);
-    gemm<0, 4, true, false, false, false>(ak, sDV + 16 * mi, LM, sKG + 32 * ni, LC, 16 * mi, 64, lane);
-    __syncthreads();
-    each_pair(acc, lane, [&](int i, int j, float x, float y) { st2(sBig + (32 * mi + i) * LR + 32 * ni + j, x, y); });
-    each_pair(ak, lane, [&](int i, int j, float x, float y) { st2(sBig + (128 + 16 * mi + i) * LR + 32 * ni + j, x, y); });
-    if (t < 128) {
-        sGC[t] += (sSeg[t] + sSeg[128 + t]) + (sSeg[256 + t] + sSeg[384 + t]);
-    }
-    __syncthreads();
-    float dG[16], run = 0.f;
-#pragma unroll
-    for (int i = 15; i >= 0; --i) {
-        const int r = seg * 16 + i;
-        const size_t off = ((size_t)(loc.tok0 + r) * a.H + h) * kD + c;
-        const bool in = r < loc.len;
-        const float G = tile[bt::G + r * kD + c];
-        const float kk = in ? ldf<T>(kp + off) : 0.f, qq = in ? ldf<T>(qp + off) : 0.f;
-        const float e1 = expf(G - gm), e2 = expf(gm - G);
-        const float dq = a.scale * e1 * sBig[r * LR + c];
-        const float dk1 = e1 * sBig[(64 + r) * LR + c], dk2 = e2 * sBig[(128 + r) * LR + c];
-        if (in) {
-            a.dq[off] = dq;
-            a.dk[off] = dk1 + dk2;
-        }
-        run += fmaf(qq, dq, kk * (dk1 - dk2));
-        dG[i] = run;
-    }
-    sSeg[seg * 128 + c] = run;      // (read above by other threads only before the barrier)
-    __syncthreads();
-    float base = sGC[c];
-    for (int s = 3; s > seg; --s) base += sSeg[s * 128 + c];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const int r = seg * 16 + i;
-        if (r < loc.len) a.dg[((size_t)(loc.tok0 + r) * a.H + h) * kD + c] = dG[i] + base;
-    }
-}
-
 }  // namespace
 
-kda_status_t launch_bwd_chunk(const BwdChunkArgs& a, kda_dtype_t dt, WsHeader* hdr, int32_t* chunk_cu_dev, cudaStream_t st)
+kda_status_t launch_bwd_chunk(const BwdChunkArgs& a, kda_dtype_t dt, int32_t* chunk_cu_dev, cudaStream_t st)
 {
     {
         DeviceLock lk;
@@ -645,14 +358,12 @@ kda_status_t launch_bwd_chunk(const BwdChunkArgs& a, kda_dtype_t dt, WsHeader* h
             const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
             KDA_CUDA_TRY(cudaFuncSetAttribute(kda_bwd_intra<float>, attr, (int)kSmem1));
             KDA_CUDA_TRY(cudaFuncSetAttribute(kda_bwd_intra<__nv_bfloat16>, attr, (int)kSmem1));
-            KDA_CUDA_TRY(cudaFuncSetAttribute(kda_bwd_out<float>, attr, (int)kSmem3));
-            KDA_CUDA_TRY(cudaFuncSetAttribute(kda_bwd_out<__nv_bfloat16>, attr, (int)kSmem3));
             KDA_CUDA_TRY(cudaFuncSetAttribute(kda_bwd_chain<64>, attr, (int)ChainSmem<64>::kBytes));
             KDA_CUDA_TRY(cudaFuncSetAttribute(kda_bwd_chain<32>, attr, (int)ChainSmem<32>::kBytes));
             lk.st->attr_done[15] = true;
         }
     }
-    kda_bwd_prep<<<1, 256, 0, st>>>(hdr, a.cu_seqlens, chunk_cu_dev, a.n_seqs, a.seq_heads, a.H);
+    kda_bwd_prep<<<1, 256, 0, st>>>(a.hdr, a.cu_seqlens, chunk_cu_dev, a.n_seqs, a.seq_heads, a.H);
     const dim3 grid((unsigned)a.n_chunks, (unsigned)a.H);
     if (a.n_chunks > 0) {
         ProfScope ps(PROF_INTRA, st);
@@ -666,14 +377,9 @@ kda_status_t launch_bwd_chunk(const BwdChunkArgs& a, kda_dtype_t dt, WsHeader* h
         if (narrow) kda_bwd_chain<32><<<dim3(8, (unsigned)a.H, (unsigned)a.n_seqs), kT2, ChainSmem<32>::kBytes, st>>>(a);
         else kda_bwd_chain<64><<<dim3(4, (unsigned)a.H, (unsigned)a.n_seqs), kT2, ChainSmem<64>::kBytes, st>>>(a);
     }
-    if (a.n_chunks > 0) {
-        ProfScope ps(PROF_INTRA, st);
-        if (dt == KDA_BF16) kda_bwd_out<__nv_bfloat16><<<grid, kT3, kSmem3, st>>>(a);
-        else kda_bwd_out<float><<<grid, kT3, kSmem3, st>>>(a);
-    }
-    count_launch(a.n_chunks > 0 ? 4 : 2);
+    count_launch(a.n_chunks > 0 ? 3 : 2);
     KDA_CUDA_TRY(cudaGetLastError());
-    return KDA_OK;
+    return a.n_chunks > 0 ? launch_bwd_out(a, dt, st) : KDA_OK;
 }
 
 }  // namespace kda
