@@ -383,7 +383,7 @@ kda_status_t kda_chunk_bwd(const void* q, const void* k, const void* v, const fl
         chunks_per_seq = (seq_len + kC - 1) / kC;
         n_chunks = chunks_per_seq * n_seqs;
     }
-    if (n_chunks > 0x7fffffff) return fail(KDA_ERR_INVALID_ARG, "kda_chunk_bwd: too many chunks");
+    if (n_chunks * H > 0x7fffffff) return fail(KDA_ERR_INVALID_ARG, "kda_chunk_bwd: too many chunks");
     const BwdLayout L = bwd_layout(total_tokens, n_seqs, H);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) || workspace_bytes < L.total)
         return fail(KDA_ERR_WORKSPACE, "kda_chunk_bwd: workspace must be 256-byte aligned and at least %zu "

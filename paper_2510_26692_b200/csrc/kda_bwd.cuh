@@ -19,23 +19,34 @@ struct BwdChunkArgs {
     int64_t seq_len, chunks_per_seq, n_chunks;
     float scale;
     unsigned long long wait_limit_ns;
+    int n_sm;
 };
 
-// Scratch tile (floats), written by the first kernel unless stated otherwise
+// Scratch tile (floats), written by the first kernel unless stated otherwise.  K^, K_ and Q are relative to the
+// middle G_m of the chunk's log decay (K^ = k e^(G - G_m), K_ = k e^(G_m - G)); the chains restore the true
+// scale on the state.  "rf" = rows fastest: element (row, c) of a matrix with R rows at float
+// ((c / 4) R + row) 4 + c % 4, which a thread per row reads and writes in whole 16-byte pieces beside its
+// neighbours'.
 namespace bt {
-constexpr int W = 0;                 // [64][128] W' = T' K^      (K^ = k e^G, T' = (I + StrictTril(K^ K~^T) Diag(beta))^-1)
-constexpr int R = W + 64 * 128;      // [64][128] U' = T' V, replaced by r = U' - W' S by the forward chain
-constexpr int X = R + 64 * 128;      // [64][128] Tril(Q K^T)^T dO, replaced by dX = .. + K~ Lam by the backward chain
-constexpr int KT = X + 64 * 128;     // [64][128] K~ = k e^(G_C - G)
-constexpr int N = KT + 64 * 128;     // [128][128] Q^T dO
-constexpr int S = N + 128 * 128;     // [128][128] state entering the chunk (forward chain)
-constexpr int L = S + 128 * 128;     // [128][128] adjoint of the state leaving the chunk (backward chain)
+constexpr int WI = 0;                // W' = T' K^ [64][128] as a split image (kda_split3.cuh), T' = (I + B Diag(beta))^-1
+constexpr int KI = WI + 12288;       // K_ [64][128] as a split image
+constexpr int R = KI + 12288;        // [64][128] rf: U' = T' V, replaced by r = U' - W' S by the forward chain
+constexpr int X = R + 64 * 128;      // [64][128] rf: P^T dO, replaced by dX = P^T dO + K~ Lam by the backward chain
+constexpr int N = X + 64 * 128;      // [128][128] rf: Q^T dO
+constexpr int S = N + 128 * 128;     // [128][128] rf: state entering the chunk (forward chain)
+constexpr int L = S + 128 * 128;     // [128][128] rf: adjoint of the state leaving the chunk (backward chain)
 constexpr int G = L + 128 * 128;     // [64][128] cumulative log decay
 constexpr int T = G + 64 * 128;      // [64][64] T'
-constexpr int B = T + 64 * 64;       // [64][64] StrictTril(K^ K~^T)
+constexpr int B = T + 64 * 64;       // [64][64] B = StrictTril(K^ K_^T)
 constexpr int GC = B + 64 * 64;      // [128] e^(G_C)
-constexpr int kFloats = GC + 128;
+constexpr int EM = GC + 128;         // [128] e^(G_m), also e^(G_C - G_m)
+constexpr int kFloats = EM + 128;
 }  // namespace bt
+__device__ __forceinline__ int rf(int rows, int row, int c) { return ((c >> 2) * rows + row) * 4 + (c & 3); }
+
+// Largest decay of a chunk taken in chunk form.  The cumulative sum is rounded to 2^-24 of its size, so
+// every decay ratio carries a relative error of up to kBwdRange 2^-24 = 2.4e-6.
+constexpr float kBwdRange = 40.f;
 
 // first token, valid tokens (1..64) and sequence of global chunk g
 struct BwdLoc { int64_t tok0; int len; int n; };
@@ -59,11 +70,67 @@ __device__ __forceinline__ BwdLoc bwd_locate(const BwdChunkArgs& a, int64_t g) {
     }
     L.tok0 = b + c * kC;
     L.len = (e - L.tok0) < kC ? (int)(e - L.tok0) : kC;
-
     return L;
 }
 
+// The per-chunk kernels hold one CTA per SM whose loads, products and stores take turns, so HBM idles while
+// the tensor core works and the other way round.  Each CTA therefore asks for what the CTA n_sm places
+// further on will read (likely the next on its SM) to come into L2 while it works itself: 148 tiles are
+// 45 MB of the 126 MB.
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {   // 16-byte aligned, multiple of 16
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+// Tiles in the order of memory, heads fastest: the CTAs that run together then read and write whole rows of
+// the token-major tensors (a head's share of a row is 256 or 512 bytes).
+__device__ __forceinline__ void bwd_tile(const BwdChunkArgs& a, int64_t id, int64_t& g, int& h) {
+    g = (int64_t)((uint32_t)id / (uint32_t)a.H);
+    h = (int)(id - g * a.H);
+}
+// tile of the CTA n_sm places further on; false if there is none
+__device__ __forceinline__ bool bwd_next(const BwdChunkArgs& a, int64_t& g, int& h) {
+    const int64_t id = (int64_t)blockIdx.x + a.n_sm;
+    if (id >= gridDim.x) return false;
+    bwd_tile(a, id, g, h);
+    return true;
+}
+
+// Eight consecutive elements as they are stored.  The loads are volatile so that they stay where they are
+// written, ahead of the stores and waits that they overlap; `in` = false gives zeros.
+template <typename T> struct Raw8 { uint32_t w[2 * sizeof(T)]; };
+__device__ __forceinline__ void ldraw4(uint32_t* w, const void* p) {
+    asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(p));
+}
+// the same for data that this kernel itself overwrites later
+__device__ __forceinline__ void ldraw4_w(uint32_t* w, const void* p) {
+    asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void ldraw(Raw8<float>& r, const float* p, bool in = true) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) r.w[e] = 0u;
+    if (in) { ldraw4(r.w, p); ldraw4(r.w + 4, p + 4); }
+}
+__device__ __forceinline__ void ldraw(Raw8<__nv_bfloat16>& r, const __nv_bfloat16* p, bool in = true) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) r.w[e] = 0u;
+    if (in) ldraw4(r.w, p);
+}
+// (row, c .. c + 7) of an rf matrix
+__device__ __forceinline__ void ldraw_rf(Raw8<float>& r, const float* m, int rows, int row, int c) {
+    ldraw4(r.w, m + rf(rows, row, c));
+    ldraw4(r.w + 4, m + rf(rows, row, c + 4));
+}
+__device__ __forceinline__ void to_f(const Raw8<float>& r, float (&x)[8]) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) x[e] = __uint_as_float(r.w[e]);
+}
+__device__ __forceinline__ void to_f(const Raw8<__nv_bfloat16>& r, float (&x)[8]) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { x[2 * e] = __uint_as_float(r.w[e] << 16); x[2 * e + 1] = __uint_as_float(r.w[e] & 0xffff0000u); }
+}
+
+kda_status_t launch_bwd_intra(const BwdChunkArgs& a, kda_dtype_t dt, cudaStream_t st);
+kda_status_t launch_bwd_chain(const BwdChunkArgs& a, cudaStream_t st);
 kda_status_t launch_bwd_out(const BwdChunkArgs& a, kda_dtype_t dt, cudaStream_t st);
-kda_status_t launch_bwd_chunk(const BwdChunkArgs& a, kda_dtype_t dt, int32_t* chunk_cu_dev, cudaStream_t st);
+kda_status_t launch_bwd_chunk(BwdChunkArgs a, kda_dtype_t dt, int32_t* chunk_cu_dev, cudaStream_t st);
 
 }  // namespace kda

@@ -25,22 +25,22 @@ constexpr uint32_t O_DX = O_RA + 3 * 8192;                    // dX beside T'
 constexpr uint32_t O_LAM0 = O_RB + 3 * 16384;                 // Lam, v columns 0-63, beside r
 constexpr uint32_t O_LAM1 = O_RA;                             // Lam, v columns 64-127; then K_
 constexpr uint32_t O_DPB = O_RA + 3 * 16384;                  // [dP ; dB]
-// fp32 vectors (floats from O_VEC): beta[64] dbeta[64] gm[128] sGC[128] colsum[2][64] seg[4][128], then barriers
-constexpr int V_BETA = 0, V_DB = 64, V_GM = 128, V_GC = 256, V_CS = 384, V_SEG = 512, V_BAR = 1024;
+// fp32 vectors (floats from O_VEC): beta[64] gm[128] dbeta[8][64] sGC[4][128] colsum[2][64] seg[4][128], then barriers
+constexpr int V_BETA = 0, V_GM = 64, V_DB = 192, V_GC = 704, V_CS = 1216, V_SEG = 1344, V_BAR = 1856;
 constexpr uint32_t kSmem = O_VEC + V_BAR * 4 + 64 + 1024;     // + alignment slack
 static_assert(4 * 64 * LR * 4 <= O_VEC, "the staged accumulators fit over the images");
 static_assert(kSmem <= 232448, "fits the shared memory of one SM");
 constexpr uint32_t C_P2 = 0, C_P4 = 128, C_P1 = 192, C_P6 = 256, C_P3 = 384;   // TMEM columns (P1: 192-319, read before P6)
 
-__device__ __forceinline__ void ld8(const float* p, float (&x)[8]) {
-    const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
-    x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+__device__ __forceinline__ float ldv(const float* p, bool in) {
+    float x = 0.f;
+    if (in) asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(x) : "l"(p));
+    return x;
 }
-__device__ __forceinline__ void ld8(const __nv_bfloat16* p, float (&x)[8]) {
-    const uint4 a = *reinterpret_cast<const uint4*>(p);
-    const uint32_t w[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) { x[2 * e] = __uint_as_float(w[e] << 16); x[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u); }
+__device__ __forceinline__ float ldv(const __nv_bfloat16* p, bool in) {
+    unsigned short x = 0;
+    if (in) asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(x) : "l"(p));
+    return __uint_as_float((uint32_t)x << 16);
 }
 
 template <typename T>
@@ -48,7 +48,8 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int h = blockIdx.y;
+    int64_t chunk; int h;
+    bwd_tile(a, blockIdx.x, chunk, h);
     if (a.seq_heads[h]) return;
     uint8_t* sm = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
     float* vec = reinterpret_cast<float*>(sm + O_VEC);
@@ -56,8 +57,8 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     float* sCs = vec + V_CS; float* sSeg = vec + V_SEG;
     uint64_t* bar = reinterpret_cast<uint64_t*>(vec + V_BAR);   // one per group of MMAs, each used once
     uint32_t* slot = reinterpret_cast<uint32_t*>(bar + 6);
-    const BwdLoc loc = bwd_locate(a, blockIdx.x);
-    const float* tile = a.tiles + ((size_t)blockIdx.x * a.H + h) * bt::kFloats;
+    const BwdLoc loc = bwd_locate(a, chunk);
+    const float* tile = a.tiles + (size_t)blockIdx.x * bt::kFloats;
 
     if (w == 0) {
         ptx::tmem_alloc(slot, 512);
@@ -81,39 +82,66 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         ptx::tc_fence_after();
     };
     // unit u of a matrix with 128 columns: row u >> 4, columns 8 (u & 15) .. + 7
-    const int c8 = (t & 15) * 8, row0 = t >> 4;      // rows row0 + 32 j
+    const int c8 = (t & 15) * 8, row0 = t >> 4;      // token tensors: rows row0 + 32 j
+    const int ra = t & 63, ca = (t >> 6) * 8;        // rf matrices of 64 rows: columns ca + 64 j
+    const int rs = t & 127, cs = (t >> 7) * 8;       // and of 128 rows: columns cs + 32 j
     auto tok_off = [&](int r) { return ((size_t)(loc.tok0 + r) * a.H + h) * kD; };
 
     // ---- P1: dV -----------------------------------------------------------------------------------------
-    float xs[4][8];     // S now, Lam later
-#pragma unroll
-    for (int j = 0; j < 4; ++j) ld8(tile + bt::S + (row0 + 32 * j) * kD + c8, xs[j]);
+    Raw8<float> xs[4], rr[2];     // S now, Lam later; r
     {
+        Raw8<float> xt, xx[2];
         const int r = t >> 3, x = (t & 7) * 8;
-        float v[8];
-        ld8(tile + bt::T + r * 64 + x, v);
+        ldraw(xt, tile + bt::T + r * 64 + x);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) ldraw_rf(xx[j], tile + bt::X, 64, ra, ca + 64 * j);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) ldraw_rf(rr[j], tile + bt::R, 64, ra, ca + 64 * j);
         const float b = r < loc.len ? a.beta[(size_t)(loc.tok0 + r) * a.H + h] : 0.f;
+        const float gl = tile[bt::G + 63 * kD + (t & 127)];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ldraw_rf(xs[j], tile + bt::S, 128, rs, cs + 32 * j);
+        float v[8], u[8];
+        to_f(xt, v);
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] *= b;
         put8<64, 1>(sm + O_RA, r, x, v);
         if (x == 0) sBeta[r] = b;
+        if (t < 128) sGm[t] = 0.5f * gl;
+        float s = 0.f;      // share of r_j . dX_j
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            to_f(xx[j], v);
+            to_f(rr[j], u);
+            put8<64, 2>(sm + O_DX, ra, ca + 64 * j, v);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) s = fmaf(v[e], u[e], s);
+        }
+        sDb[t] = s;         // [8][64]
     }
-    float rr[2][8];
+    Raw8<float> lam[4];
+    Raw8<T> dd[2];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int r = row0 + 32 * j;
-        float v[8];
-        ld8(tile + bt::X + r * kD + c8, v);
-        ld8(tile + bt::R + r * kD + c8, rr[j]);
-        put8<64, 2>(sm + O_DX, r, c8, v);
-        float s = 0.f;      // r_j . dX_j
+    for (int j = 0; j < 4; ++j) ldraw_rf(lam[j], tile + bt::L, 128, rs, cs + 32 * j);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) s = fmaf(v[e], rr[j][e], s);
-#pragma unroll
-        for (int o = 1; o < 16; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if ((t & 15) == 0) sDb[r] = s;
+    for (int j = 0; j < 2; ++j)
+        ldraw(dd[j], static_cast<const T*>(a.d_o) + tok_off(row0 + 32 * j) + c8, row0 + 32 * j < loc.len && a.d_o);
+    {   // see prefetch_l2; the token vectors by 64 threads, a row each
+        int64_t ng; int nh;
+        if ((t & ~63) == 448 && bwd_next(a, ng, nh)) {
+            const float* nt = a.tiles + ((size_t)ng * a.H + nh) * bt::kFloats;
+            const int r = t & 63;
+            if (r == 0) prefetch_l2(nt + bt::R, 2 * 64 * kD * 4);
+            if (r == 1) prefetch_l2(nt + bt::S, (bt::kFloats - bt::S) * 4);
+            const BwdLoc nl = bwd_locate(a, ng);
+            if (r < nl.len) {
+                const size_t off = ((size_t)(nl.tok0 + r) * a.H + nh) * kD;
+                prefetch_l2(static_cast<const T*>(a.k) + off, kD * sizeof(T));
+                prefetch_l2(static_cast<const T*>(a.q) + off, kD * sizeof(T));
+                if (a.d_o) prefetch_l2(static_cast<const T*>(a.d_o) + off, kD * sizeof(T));
+            }
+        }
     }
-    if (t < 128) sGm[t] = 0.5f * tile[bt::G + 63 * kD + t];
     publish();
     const uint32_t tm = *slot;
     const uint32_t mnA = ptx::kIdescAMajorMN, mnB = ptx::kIdescBMajorMN;
@@ -122,31 +150,22 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         ptx::umma_commit(&bar[0]);
     }
     // meanwhile: e^(G_m) S, and its dot products with Lam
-    float dd[2][8];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int r = row0 + 32 * j;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) dd[j][e] = 0.f;
-        if (r < loc.len && a.d_o) ld8(reinterpret_cast<const T*>(a.d_o) + tok_off(r) + c8, dd[j]);
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int r = row0 + 32 * j;
-        const float em = expf(sGm[r]);
-        float v[8], l[8];
-        ld8(tile + bt::L + r * kD + c8, l);
+    {
+        const float em = expf(sGm[rs]);
         float s = 0.f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            s = fmaf(xs[j][e], l[e], s);
-            v[e] = em * xs[j][e];
-            xs[j][e] = l[e];
-        }
-        put8<128, 2>(sm + O_RB, r, c8, v);
+        for (int j = 0; j < 4; ++j) {
+            float v[8], l[8];
+            to_f(xs[j], v);
+            to_f(lam[j], l);
 #pragma unroll
-        for (int o = 1; o < 16; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if ((t & 15) == 0) sGC[r] = s * tile[bt::GC + r];
+            for (int e = 0; e < 8; ++e) {
+                s = fmaf(v[e], l[e], s);
+                v[e] *= em;
+            }
+            put8<128, 2>(sm + O_RB, rs, cs + 32 * j, v);
+        }
+        sGC[t] = s * em * em;      // [4][128]; (G_m = G_C / 2)
     }
     wait(0);
     // dV: rows = TMEM lanes 0-63 (warps of quadrants 0 and 1), 32 columns each
@@ -172,7 +191,11 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         }
     }
 #pragma unroll
-    for (int j = 0; j < 2; ++j) put8<128, 2>(sm + O_RA, row0 + 32 * j, c8, dd[j]);
+    for (int j = 0; j < 2; ++j) {
+        float v[8];
+        to_f(dd[j], v);
+        put8<128, 2>(sm + O_RA, row0 + 32 * j, c8, v);
+    }
     publish();
 
     // ---- P2, then P4 and the first half of P3 ---------------------------------------------------------------
@@ -180,35 +203,42 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         mma6<8>(tm + C_P2, k_major<128, 2>(sm + O_RA), k_major<128, 2>(sm + O_RB), ptx::umma_idesc_bf16(128, 128), false);
         ptx::umma_commit(&bar[1]);
     }
+    // the gated operands' inputs, requested while the tensor core works
+    Raw8<T> kr[2], qr[2];
+    Raw8<float> gr[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int r = row0 + 32 * j;
+        ldraw(kr[j], static_cast<const T*>(a.k) + tok_off(r) + c8, r < loc.len);
+        ldraw(qr[j], static_cast<const T*>(a.q) + tok_off(r) + c8, r < loc.len);
+        ldraw(gr[j], tile + bt::G + r * kD + c8);
+    }
     wait(1);
 #pragma unroll
-    for (int j = 0; j < 2; ++j) put8<64, 2>(sm + O_RB, row0 + 32 * j, c8, rr[j]);
-    if (c8 < 64)
+    for (int j = 0; j < 2; ++j) {
+        float v[8];
+        to_f(rr[j], v);
+        put8<64, 2>(sm + O_RB, ra, ca + 64 * j, v);
+    }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) put8<128, 1>(sm + O_LAM0, row0 + 32 * j, c8, xs[j]);
+    for (int j = 0; j < 2; ++j) {
+        float v[8];
+        to_f(lam[j], v);
+        put8<128, 1>(sm + O_LAM0, rs, cs + 32 * j, v);
+    }
     publish();
     if (t == 0) {
         mma6<8>(tm + C_P4, k_major<128, 2>(sm + O_RA), k_major<64, 2>(sm + O_RB), ptx::umma_idesc_bf16(128, 64), false);
         ptx::umma_commit(&bar[2]);
         mma6<4>(tm + C_P3, k_major<64, 2>(sm + O_RB), k_major<128, 1>(sm + O_LAM0), ptx::umma_idesc_bf16(128, 128), false);
     }
-    // the gated operands' inputs, requested while the tensor core works
-    float kk[2][8], qq[2][8], gg[2][8];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int r = row0 + 32 * j;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) kk[j][e] = qq[j][e] = 0.f;
-        if (r < loc.len) {
-            ld8(reinterpret_cast<const T*>(a.k) + tok_off(r) + c8, kk[j]);
-            ld8(reinterpret_cast<const T*>(a.q) + tok_off(r) + c8, qq[j]);
-        }
-        ld8(tile + bt::G + r * kD + c8, gg[j]);
-    }
     wait(2);
-    if (c8 >= 64)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) put8<128, 1>(sm + O_LAM1, row0 + 32 * j, c8 - 64, xs[j]);
+    for (int j = 2; j < 4; ++j) {
+        float v[8];
+        to_f(lam[j], v);
+        put8<128, 1>(sm + O_LAM1, rs, cs + 32 * j - 64, v);
+    }
     {   // masked and scaled Gram matrices; columns j0 .. j0 + 15 of row lane + 32 quad of [dP ; dB]
         const int R = quad * 32 + lane, i = R & 63, j0 = (w >> 2) * 16;
         const bool isB = quad >= 2;
@@ -254,19 +284,27 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         mma6<4>(tm + C_P3, k_major<64, 2>(sm + O_RB + 8192), k_major<128, 1>(sm + O_LAM1), ptx::umma_idesc_bf16(128, 128), true);
         ptx::umma_commit(&bar[3]);
     }
-    if (t < loc.len) a.db[(size_t)(loc.tok0 + t) * a.H + h] = sDb[t] + (sCs[t] + sCs[64 + t]);
-    // gates in place of G: exp(G - G_m), exp(G_m - G)
-    float e1[2][8];
+    if (t < loc.len) {
+        float s = sCs[t] + sCs[64 + t];
 #pragma unroll
-    for (int j = 0; j < 2; ++j)
+        for (int j = 0; j < 8; ++j) s += sDb[j * 64 + t];
+        a.db[(size_t)(loc.tok0 + t) * a.H + h] = s;
+    }
+    // gated operands: exp(G - G_m), exp(G_m - G)
+    float kk[2][8], qq[2][8], gg[2][8];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        to_f(kr[j], kk[j]);
+        to_f(qr[j], qq[j]);
+        to_f(gr[j], gg[j]);
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const float x = gg[j][e] - sGm[c8 + e];
-            e1[j][e] = expf(x);
+            const float x = gg[j][e] - sGm[c8 + e], f1 = expf(x);
             gg[j][e] = kk[j][e] * expf(-x);          // K_
-            kk[j][e] *= e1[j][e];                    // K^
-            qq[j][e] *= a.scale * e1[j][e];          // Q
+            kk[j][e] *= f1;                          // K^
+            qq[j][e] *= a.scale * f1;                // Q
         }
+    }
     wait(3);
 
     // ---- P5, P6 -------------------------------------------------------------------------------------------
@@ -293,6 +331,17 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     // the column pass's inputs: thread = channel c of 16 consecutive tokens
     const int c = t & 127, seg = t >> 7;
     const float gm = sGm[c];
+    const T* kp = static_cast<const T*>(a.k);
+    const T* qp = static_cast<const T*>(a.q);
+    float kv[16], qv[16], gv[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int r = seg * 16 + i;
+        const bool in = r < loc.len;
+        kv[i] = ldv(kp + tok_off(r) + c, in);
+        qv[i] = ldv(qp + tok_off(r) + c, in);
+        gv[i] = ldv(tile + bt::G + r * kD + c, true);
+    }
     wait(4);
     {
         uint32_t y[32];
@@ -319,8 +368,6 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     }
     ptx::tc_fence_before();
     __syncthreads();
-    const T* kp = reinterpret_cast<const T*>(a.k);
-    const T* qp = reinterpret_cast<const T*>(a.q);
     const float ec = expf(gm);        // e^(G_C - G_m): G_m = G_C / 2
     float dG[16], run = 0.f, gsum = 0.f;
 #pragma unroll
@@ -328,8 +375,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         const int r = seg * 16 + i;
         const size_t off = tok_off(r) + c;
         const bool in = r < loc.len;
-        const float x = tile[bt::G + r * kD + c] - gm;
-        const float kv = in ? (float)kp[off] : 0.f, qv = in ? (float)qp[off] : 0.f;
+        const float x = gv[i] - gm;
         const float f1 = expf(x), f2 = expf(-x);
         const float dq = a.scale * f1 * stage[r * LR + c];
         const float p3 = ec * f2 * stage[(192 + r) * LR + c];       // e^(G_C - G) (beta r Lam^T)
@@ -338,8 +384,8 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
             a.dq[off] = dq;
             a.dk[off] = dk1 + dk2;
         }
-        gsum = fmaf(kv, p3, gsum);
-        run += fmaf(qv, dq, kv * (dk1 - dk2));
+        gsum = fmaf(kv[i], p3, gsum);
+        run += fmaf(qv[i], dq, kv[i] * (dk1 - dk2));
         dG[i] = run;
     }
     // d G_C: all segments' sums of K~ dK~ and e^(G_C) rowsum(S Lam)
@@ -347,7 +393,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     sSeg[seg * 128 + c] = run;
     sSum[seg * 128 + c] = gsum;
     __syncthreads();
-    float base = sGC[c] + ((sSum[c] + sSum[128 + c]) + (sSum[256 + c] + sSum[384 + c]));
+    float base = ((sGC[c] + sGC[128 + c]) + (sGC[256 + c] + sGC[384 + c])) + ((sSum[c] + sSum[128 + c]) + (sSum[256 + c] + sSum[384 + c]));
     for (int s = 3; s > seg; --s) base += sSeg[s * 128 + c];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -372,7 +418,7 @@ kda_status_t launch_bwd_out(const BwdChunkArgs& a, kda_dtype_t dt, cudaStream_t 
             lk.st->attr_done[14] = true;
         }
     }
-    const dim3 grid((unsigned)a.n_chunks, (unsigned)a.H);
+    const dim3 grid((unsigned)(a.n_chunks * a.H));
     ProfScope ps(PROF_INTRA, st);
     if (dt == KDA_BF16) kda_bwd_out<__nv_bfloat16><<<grid, kT, kSmem, st>>>(a);
     else kda_bwd_out<float><<<grid, kT, kSmem, st>>>(a);
