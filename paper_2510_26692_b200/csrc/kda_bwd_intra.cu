@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
         mma6<4>(tm + C_X, mn_major<64, 1>(sm + O_RP), mn_major<64, 2>(sm + O_RK), idesc, false);
         ptx::umma_commit(&bar[1]);
     }
-    mma3::invert_unit_lower<kT, LM>(sL, sT, t);
+    mma3::invert_unit_lower<LM>(sL, sT, t);
     wait(1);
     {   // T' to the tile and as image; V
         const int r = t >> 3, x0 = (t & 7) * 8;

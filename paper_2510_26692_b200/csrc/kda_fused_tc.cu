@@ -75,8 +75,8 @@ constexpr uint32_t E_A = 65536;         // fp32 [64][LDT]: L, X below the diagon
 constexpr uint32_t E_TD = E_A + 64 * LDT * 4;     // fp32 4 x [16][LDD]: diagonal blocks of T; scan exchange [8][128] before
 constexpr uint32_t E_TD_BYTES = 4096;
 constexpr uint32_t E_BETA = E_TD + E_TD_BYTES;    // 64 fp32
-constexpr uint32_t E_DESC = E_BETA + 256;         // two tile descriptors
-constexpr uint32_t E_BAR = E_DESC + 128;          // 8-byte words: mma barrier, K barrier, abort word, Q barrier,
+constexpr uint32_t E_DESC = E_BETA + 256;         // three tile descriptors: this tile, the next, the one after
+constexpr uint32_t E_BAR = E_DESC + 192;          // 8-byte words: mma barrier, K barrier, abort word, Q barrier,
                                                   // (first engine) TMEM slot, V barrier
 constexpr uint32_t E_KS = (E_BAR + 64 + 1023) / 1024 * 1024;   // raw k of the NEXT tile [2 K-halves][64][64] bf16
 constexpr uint32_t E_NORM = E_KS + 16384;         // layer mode: 1 / |k_i|, 1 / |q_i| (64 fp32 each)
@@ -222,7 +222,7 @@ struct TileDesc {
     uint32_t need;                   // the ring position is free once every progress word has reached this
     int pad[3];
 };
-static_assert(sizeof(TileDesc) == 64, "two descriptors fit the 128 bytes reserved");
+static_assert(sizeof(TileDesc) == 64, "three descriptors fit the 192 bytes reserved");
 
 // Hands out production indices in increasing order to whichever engine asks next (a slow engine
 // then delays one tile, not every tile of a fixed share).  The counter lives in the workspace header
@@ -272,9 +272,8 @@ __device__ bool describe_tile(const FusedArgs& f, uint32_t i, TileDesc* d)
     d->len = rem < kC ? (int)rem : kC;
     return true;
 }
-// The scheduler thread's look-ahead state: the request for the index after next is in flight while
-// a tile is worked on, and so is a first look at the progress of the next tile's consumers; neither
-// value is touched before it is needed, so the round trips cost nothing.
+// The service thread's look-ahead state: the request for the next index is in flight while a tile is
+// worked on, and so is a look at the progress of the next tile's consumers.
 struct SchedState {
     unsigned long long pending;             // return value of the counter request in flight
     unsigned long long seen[kSlices];       // progress words of the next tile's consumers, read a tile early
@@ -291,23 +290,23 @@ __device__ void next_tile(const FusedArgs& f, SchedState& ss, TileDesc* d)
         ss.pending = atomicAdd(ctr, 1ull);
         if (describe_tile(f, i, d)) break;
     }
-#pragma unroll
-    for (int sl = 0; sl < kSlices; ++sl) ss.seen[sl] = d->need > 0 ? ptx::ld_acquire_gpu(d->consumed + sl) : 0ull;
 }
-// Waits (bounded) until the chain roles have finished with the previous occupant of the tile's ring
-// position.  Runs in ONE thread, at a point where its engine holds no unfinished tile and has
-// published every finished one: a producer that waited for its consumers while sitting on a tile
-// they need would deadlock.
-__device__ void wait_slot_free(const FusedArgs& f, const TileDesc& d, const SchedState& ss,
-                               volatile uint32_t* abort_word)
+// Whether the look taken a tile ago settles that the previous occupant of the tile's ring position has been
+// consumed by every chain role.
+__device__ bool slot_seen_free(const FusedArgs& f, const TileDesc& d, const SchedState& ss)
 {
-    if (d.need == 0) return;
+    bool ok = true;
+    for (int sl = 0; sl < kSlices; ++sl) ok = ok && (uint32_t)(ss.seen[sl] >> 32) == f.epoch && (uint32_t)ss.seen[sl] >= d.need;
+    return ok || d.need == 0;
+}
+// Waits (bounded) for that.  Runs in ONE thread, whose engine has published every finished tile: a
+// producer that waited for its consumers while sitting on a tile they need would deadlock.
+__device__ void wait_slot_free(const FusedArgs& f, const TileDesc& d, volatile uint32_t* abort_word)
+{
     uint64_t t0 = 0;
     for (int sl = 0; sl < kSlices; ++sl) {
-        unsigned long long v = ss.seen[sl];   // the look taken a tile ago usually settles it
         for (;;) {
-            if ((uint32_t)(v >> 32) == f.epoch && (uint32_t)v >= d.need) break;
-            v = ptx::ld_acquire_gpu(d.consumed + sl);
+            const unsigned long long v = ptx::ld_acquire_gpu(d.consumed + sl);
             if ((uint32_t)(v >> 32) == f.epoch && (uint32_t)v >= d.need) break;
             if (t0 == 0) t0 = ptx::globaltimer_ns();
             if (*abort_word || call_aborted(f)) { *abort_word = 1; return; }
@@ -319,7 +318,6 @@ __device__ void wait_slot_free(const FusedArgs& f, const TileDesc& d, const Sche
             ptx::nanosleep(100);
         }
     }
-    ptx::fence_proxy_async_all();   // the consumers' bulk reads of the position precede our writes
 }
 
 // ====================================================================================================
@@ -352,8 +350,13 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 {
     constexpr bool has_q = kHasQ;
     constexpr int kNW = 8, kRPT = 8;
-    constexpr int kBulkThread = 128;   // lane 0 of warp 4 issues every bulk copy; thread 0 the MMAs
-    constexpr int kSchedThread = 32;   // lane 0 of warp 1 finds the next tile
+    // Lane 0 of warp 7 issues every bulk copy, finds the tiles and talks to the chains (thread 0 issues the
+    // MMAs).  What takes it about a microsecond -- publishing a tile, looking at flags -- it does during the
+    // blocked substitution, which warps 6 and 7 have no part in: on any other path all eight warps would
+    // wait for it (publishing at the top of the next tile and looking for tiles beside the first MMA group:
+    // 11.2 us a tile).
+    constexpr int kServiceThread = 224;
+    constexpr int kInvWarps = 6;       // warps of the blocked substitution
     constexpr int kMma2Thread = 64;    // lane 0 of warp 2 issues half of the second MMA group
     const ChunkArgs& a = f.a;
     float* sA = reinterpret_cast<float*>(smem + E_A);
@@ -369,6 +372,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 
     const int warp = te >> 5, lane = te & 31;
     auto ebar = [&]() { ptx::named_bar_sync(bar_id, kEngThreads); };
+    auto inv_bar = [&]() { ptx::named_bar_sync(bar_id + 2, kInvWarps * 32); };
 
     // thread (w, c4) owns rows 8w..8w+7 and channels 4c4..4c4+3 in the gating phase
     const int c4 = lane, d0 = c4 * 4, i0 = warp * kRPT;
@@ -445,22 +449,26 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
     uint32_t next_static = first;
     bool stores_pending = false;   // (bulk thread) the previous tile's staging may still be read out
     int cur = 0;
-    unsigned long long* pending_ready = nullptr;   // bulk thread: flag of the tile whose stores are in flight
+    unsigned long long* pending_ready = nullptr;   // service thread: flag of the last finished tile, not yet published
     unsigned long long pending_val = 0;
-
-    if (te == kSchedThread) {
+    auto find_tile = [&](TileDesc* d) {   // (service thread)
         if (kFused) {
-            ss.pending = tag(f.epoch, fetch_index(f));
-            next_tile(f, ss, &desc[0]);
+            next_tile(f, ss, d);
         } else {
-            static_tile(f, next_static, &desc[0]);
+            static_tile(f, next_static, d);
             next_static += stride;
         }
+    };
+    if (te == kServiceThread) {
+        if (kFused) ss.pending = tag(f.epoch, fetch_index(f));
+        find_tile(&desc[0]);
+        if (desc[0].len > 0) find_tile(&desc[1]);
+        else desc[1].len = 0;
     }
     ebar();
     if (desc[0].len > 0 && !*abort_word) {
         prefetch_regs(desc[0]);
-        if (te == kBulkThread) {
+        if (te == kServiceThread) {
             request_k(desc[0]);
             if (has_q) request_q(desc[0]);
             request_v(desc[0]);
@@ -497,24 +505,19 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             for (int e = 0; e < 4; ++e) G[r][e] = fmaf(G[r][e], kLog2e, G[r - 1][e]);
         *reinterpret_cast<float4*>(sTot + warp * kD + d0) =
             make_float4(G[kRPT - 1][0], G[kRPT - 1][1], G[kRPT - 1][2], G[kRPT - 1][3]);
-        if (!kFused && te == kBulkThread && stores_pending) ptx::bulk_wait_read0();   // staging read out
-        if (kFused && te == kBulkThread && pending_ready) {
-            // The previous tile is complete in global memory: hand it to the chain roles.  (This also
-            // means its W' / U staging has been read out: the buffers are written again below.)  It
-            // has to happen before this engine may wait for a ring position: a producer that waits
-            // for its consumers while holding back a tile they need would deadlock.
-            ptx::bulk_wait_all0();
-            ptx::fence_proxy_async_all();
-            ptx::st_release_gpu(pending_ready, pending_val);
-            pending_ready = nullptr;
+        if (te == kServiceThread) {
+            if (stores_pending) ptx::bulk_wait_read0();   // the previous tile's W' / U staging has been read out
+            if (kFused && !slot_seen_free(f, D, ss)) {
+                if (pending_ready) {      // publish before waiting
+                    ptx::bulk_wait_all0();
+                    ptx::fence_proxy_async_all();
+                    ptx::st_release_gpu(pending_ready, pending_val);
+                    pending_ready = nullptr;
+                }
+                wait_slot_free(f, D, abort_word);
+            }
+            if (kFused) ptx::fence_proxy_async_all();   // the consumers' bulk reads of the position precede our writes
         }
-#ifdef KDA_FUSED_TIMING
-        const uint64_t ts0_ = te == kSchedThread ? ptx::globaltimer_ns() : 0;
-#endif
-        if (kFused && te == kSchedThread) wait_slot_free(f, D, ss, abort_word);
-#ifdef KDA_FUSED_TIMING
-        if (te == kSchedThread) atomicAdd(&f.hdr->pad[11], (int)((ptx::globaltimer_ns() - ts0_) >> 4));
-#endif
         ptx::cp_async_wait_all();             // beta
         if (kLayer && te < kC)                // (each of these threads copied its own element)
             sBeta[te] = te < D.len ? 1.f / (1.f + __expf(-sBeta[te])) : 0.f;
@@ -657,7 +660,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         KT_MARK(te == 0, 3);   // gating
 
         // ---- a2 + a5: [Kg ; Qg] Ki^T --------------------------------------------------------------------
-        if (te == kBulkThread) {
+        if (te == kServiceThread) {
             // Q' (rows 64-127 of both K-halves of the operand image) and K' are tile contents as they are
             if (has_q) {
                 ptx::bulk_s2g(tile + tc::OFF_QW + 8192, smem + E_KQ + 8192, 8192);
@@ -676,27 +679,20 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             ptx::umma_commit(mma_bar);
         }
         if (te == kMma2Thread) ptx::umma_commit(mma_bar);   // (the barrier counts both issuing threads)
-        if (te == kSchedThread) {
-            if (kFused) {
-                next_tile(f, ss, &desc[cur ^ 1]);
-            } else {
-                static_tile(f, next_static, &desc[cur ^ 1]);
-                next_static += stride;
-            }
-        }
-        if (!ptx::mbar_wait(mma_bar, 0, f.a.wait_limit_ns)) timed_out = true;
-        // Q' and K' have been read out of shared memory by now: Aqk goes over the Q' rows next
-        if (te == kBulkThread) ptx::bulk_wait_read0();
-        ebar();
-        ptx::tc_fence_after();
-        KT_MARK(te == 0, 4);   // MMA A
-        const TileDesc Dn = desc[cur ^ 1];
+        const int nxt = cur == 2 ? 0 : cur + 1, nxt2 = nxt == 2 ? 0 : nxt + 1;
+        const TileDesc Dn = desc[nxt];
         const bool has_next = Dn.len > 0 && !*abort_word;
         if (has_next) {
             prefetch_regs(Dn);   // the next tile's log alpha: its registers are free since the gating loop
-            if (te == kBulkThread) request_k(Dn);   // the staging buffer was read by the gating loop
+            if (te == kServiceThread) request_k(Dn);   // the staging buffer was read by the gating loop
             pend_k = true;
         }
+        if (!ptx::mbar_wait(mma_bar, 0, f.a.wait_limit_ns)) timed_out = true;
+        // Q' and K' have been read out of shared memory by now: Aqk goes over the Q' rows next
+        if (te == kServiceThread) ptx::bulk_wait_read0();
+        ebar();
+        ptx::tc_fence_after();
+        KT_MARK(te == 0, 4);   // MMA A
         {
             const int q4 = warp & 3, c0 = (warp >> 2) * 32;
             const int Rr = q4 * 32 + lane;
@@ -735,9 +731,32 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         ptx::fence_async_smem();
         ptx::tc_fence_before();
         ebar();
-        if (te == kBulkThread && has_q) {
-            ptx::bulk_s2g(tile + tc::OFF_AQ, smem + E_AQ, 8192);
-            ptx::bulk_commit();
+        if (te == kServiceThread) {
+            if (has_q) {
+                ptx::bulk_s2g(tile + tc::OFF_AQ, smem + E_AQ, 8192);
+                ptx::bulk_commit();
+            }
+            if (kFused && has_next && Dn.need > 0)
+#pragma unroll
+                for (int sl = 0; sl < kSlices; ++sl) ss.seen[sl] = ptx::ld_relaxed_gpu(Dn.consumed + sl);
+            if (has_q) {   // the Aqk staging has been read out: the next tile's q may land over it
+                ptx::bulk_wait_read0();
+                if (has_next) request_q(Dn);
+            }
+            if (kFused) {
+                // the previous tile's stores are complete (at most the one or two groups of this tile are not)
+                if (pending_ready) {
+                    if (has_q) ptx::bulk_wait_all<2>();
+                    else ptx::bulk_wait_all<1>();
+                    ptx::fence_proxy_async_all();
+                }
+                ptx::fence_acq_rel_gpu();   // orders the looks taken above and the publication
+                if (pending_ready) ptx::st_relaxed_gpu(pending_ready, pending_val);
+                pending_ready = nullptr;
+            }
+            if (has_next) find_tile(&desc[nxt2]);
+            else desc[nxt2].len = 0;
+            ptx::bulk_wait_read0();        // K' has been read out: the Mm image goes there
         }
         KT_MARK(te == 0, 5);   // A read-out
 
@@ -754,13 +773,19 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             for (int r = 0; r < 16; ++r) {
                 float s = (r == c) ? 1.f : 0.f;
 #pragma unroll
-                for (int m = 0; m < r; ++m) s -= Lb[r * LDT + m] * x[m];
+                for (int m4 = 0; m4 < r; m4 += 4) {
+                    const float4 l4 = *reinterpret_cast<const float4*>(Lb + r * LDT + m4);
+                    const float l[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (m4 + e < r) s -= l[e] * x[m4 + e];
+                }
                 x[r] = s;
             }
 #pragma unroll
             for (int r = 0; r < 16; ++r) blkD(I)[r * LDD + c] = x[r];
         }
-        ebar();
+        if (warp < kInvWarps) inv_bar();
         // X_IM = T_II L_IM for the six sub-diagonal blocks (one warp each, in place), then
         // T_IJ = - sum_{M=J..I-1} X_IM T_MJ in three dependency stages; the terms of a sum that do not
         // depend on blocks still being computed are taken early (kept, un-negated, in the block's place).
@@ -779,7 +804,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             block16_mma(acc2, blkA(I, M), LDT, blkD(M), LDD, lane);
             block16_store(blkA(M, I), acc2, (I - M == 1) ? -1.f : 1.f, LDT, lane);
         }
-        ebar();
+        if (warp < kInvWarps) inv_bar();
         if (warp < 3) {
             // warp 0: T20 (M = 1), warp 1: T31 (M = 2), warp 2: P30 += X31 T10
             const int I = warp == 0 ? 2 : 3, J = warp == 1 ? 1 : 0, M = warp == 1 ? 2 : 1;
@@ -788,18 +813,12 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             block16_mma(acc, blkA(I, M), LDT, blkA(J, M), LDT, lane);
             block16_store(blkA(J, I), acc, warp < 2 ? -1.f : 1.f, LDT, lane);
         }
-        ebar();
+        if (warp < kInvWarps) inv_bar();
         if (warp == 0) {
             float acc[2][4];
             block16_load(acc, blkA(0, 3), LDT, lane);
             block16_mma(acc, blkA(3, 2), LDT, blkA(0, 2), LDT, lane);
             block16_store(blkA(0, 3), acc, -1.f, LDT, lane);
-        }
-        // K' (overwritten by the Mm image) and the Aqk staging have been read out: the next tile's q
-        // may land over the Aqk staging
-        if (te == kBulkThread) {
-            ptx::bulk_wait_read0();
-            if (has_next && has_q) request_q(Dn);
         }
         if (has_next) pend_q = has_q;
         if (!ptx::mbar_wait(bar_v, tma_parity, f.a.wait_limit_ns)) timed_out = true;   // v has landed
@@ -868,7 +887,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         if (!ptx::mbar_wait(mma_bar, 1, f.a.wait_limit_ns)) timed_out = true;
         KT_MARK(te == 0, 7);   // Mm + MMA B
         if (has_next) {   // V and beta are free: the next tile's may land
-            if (te == kBulkThread) request_v(Dn);
+            if (te == kServiceThread) request_v(Dn);
             request_beta(Dn);
             pend_v = true;
         }
@@ -909,7 +928,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         ptx::tc_fence_before();
         if (timed_out) *abort_word = 1;
         ebar();
-        if (te == kBulkThread) {
+        if (te == kServiceThread) {
             ptx::bulk_s2g(tile + tc::OFF_QW, smem + E_KI, 8192);
             ptx::bulk_s2g(tile + tc::OFF_QW + tc::QW_HALF, smem + E_KI + 8192, 8192);
             ptx::bulk_s2g(tile + tc::OFF_U, smem + E_A, 16384);
@@ -922,13 +941,13 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 #ifdef KDA_FUSED_TIMING
         if (te == 0) kt_acc_[9] += 16;   // tiles
 #endif
-        cur ^= 1;
+        cur = nxt;
     }   // tile loop
     KT_FLUSH(te == 0, f.hdr, 0, 10);
 
     if (timed_out) report_timeout(f, 10);
     if (out_of_range) atomicOr(&f.hdr->flags, 1);
-    if (te == kBulkThread) {
+    if (te == kServiceThread) {
         ptx::bulk_wait_all0();   // shared memory must outlive the reads of every bulk store
         if (kFused && pending_ready && !timed_out && !*abort_word) {
             ptx::fence_proxy_async_all();
