@@ -1,6 +1,7 @@
 // C ABI of the KDA library: argument validation, workspace carving, pass scheduling.  Every step
 // of the computation runs in the kernels of the other translation units; this file only decides
 // what to launch.
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <cstdarg>
@@ -131,25 +132,12 @@ int64_t max_chunks(int64_t total_tokens, int n_seqs)
     return (total_tokens + kC - 1) / kC + n_seqs;
 }
 
-// ---- fused bf16 path: workspace = header | flag words | round table | ring of tiles ---------------------
-constexpr int kSlotCap = 64;      // upper bound of concurrently running (sequence, head) chains
-constexpr int kRingMax = 16;      // tiles per chain the engines may run ahead
-constexpr size_t kFlagBytes = (size_t)kSlotCap * kRingMax * 8 + (size_t)kSlotCap * 4 * 8;
-struct FusedLayout {
-    size_t off_ready, off_consumed, off_table, off_ring;
-};
-FusedLayout fused_layout(int64_t J)
-{
-    FusedLayout L;
-    L.off_ready = sizeof(WsHeader);
-    L.off_consumed = L.off_ready + (size_t)kSlotCap * kRingMax * 8;
-    L.off_table = L.off_ready + kFlagBytes;
-    L.off_ring = L.off_table + align_up((size_t)(J + 1) * sizeof(uint32_t));
-    return L;
-}
-// Call counter that tags the flag words of the fused kernel.  It starts at a value drawn per process:
-// device memory handed from one process to the next may still hold the flag words of the earlier
-// one, and a counter that restarted at 1 could meet its own tags there.
+// ---- fused bf16 path: workspace = header | ring of tiles ------------------------------------------------
+constexpr size_t kFusedRing = sizeof(WsHeader);
+constexpr int kSlotCap = 64, kRingMax = 16;   // bounds of fused_plan
+// Call counter of the tensor-core kernels, by which a call that gave up marks itself in the header.  It starts at a
+// value drawn per process: device memory handed from one process to the next may still hold the mark of an
+// earlier one.
 uint32_t epoch_seed()
 {
     std::random_device rd;
@@ -157,6 +145,11 @@ uint32_t epoch_seed()
     return (uint32_t)rd() ^ (uint32_t)(t * 0x9E3779B97F4A7C15ull >> 32);
 }
 std::atomic<uint32_t> g_epoch{epoch_seed()};
+uint32_t next_epoch()
+{
+    const uint32_t e = g_epoch.fetch_add(1, std::memory_order_relaxed) + 1;
+    return e ? e : g_epoch.fetch_add(1, std::memory_order_relaxed) + 1;   // never 0
+}
 
 // Schedule of the fused kernel: Q chains run side by side (one round), each with a ring of R tiles;
 // n_prod counts the production indices, a round taking (longest chain) x (chains of the round).
@@ -168,7 +161,7 @@ FusedPlan fused_plan(const std::vector<int64_t>& chunk_cu, int n_seqs, int H, in
 {
     FusedPlan P{0, 0, 0, 0};
     const int64_t J = (int64_t)n_seqs * H;
-    int Qmax = fused_max_slots(n_sm);
+    int Qmax = n_sm / 4;
     if (Qmax > kSlotCap) Qmax = kSlotCap;
     if (Qmax < 1 || avail_tiles < 2 || J < 1) return P;
     // whole sequences per round when the heads of one fit, so that the chains of a round have
@@ -191,7 +184,7 @@ FusedPlan fused_plan(const std::vector<int64_t>& chunk_cu, int n_seqs, int H, in
     return P;
 }
 std::atomic<int> g_chunk_path{0};
-std::atomic<int> g_fuse_output{1};  // kda_layer_fwd: 1 = output stage inside the inter-chunk kernel when possible   // 0 = automatic, 1 = always two kernels, 2 = always the fused kernel
+std::atomic<int> g_fuse_output{1};  // kda_layer_fwd: 1 = output stage inside the chains, 0 = a pass of its own
 
 }  // namespace
 }  // namespace kda
@@ -250,7 +243,7 @@ size_t kda_chunk_fwd_min_workspace_bytes(int64_t total_tokens, int n_seqs, int H
     // fp32: state scratch + one tile per head (the call then walks the chunks one at a time).
     // bf16: what the fused kernel needs -- header, flag words, round table and a ring of two tiles.
     if (dt != KDA_BF16) return ws_layout(n_seqs, H).fixed + align_up((size_t)H * tile_bytes(dt));
-    return fused_layout((int64_t)n_seqs * H).off_ring + 2 * tc_tile_bytes();
+    return kFusedRing + 2 * tc_tile_bytes();
 }
 
 size_t kda_chunk_fwd_workspace_bytes(int64_t total_tokens, int n_seqs, int H, int dk, int dv,
@@ -264,7 +257,7 @@ size_t kda_chunk_fwd_workspace_bytes(int64_t total_tokens, int n_seqs, int H, in
     if (dt == KDA_BF16) {
         // never below a full ring for the fused kernel (the path of a capped workspace)
         const int64_t J = (int64_t)n_seqs * H;
-        const size_t ring = fused_layout(J).off_ring + (size_t)(J < kSlotCap ? J : kSlotCap) * kRingMax * tc_tile_bytes();
+        const size_t ring = kFusedRing + (size_t)(J < kSlotCap ? J : kSlotCap) * kRingMax * tc_tile_bytes();
         if (want < ring) want = ring;
     }
     return want < lo ? lo : want;
@@ -283,6 +276,60 @@ struct LayerMode {
     const float* rms_weight = nullptr;
     float rms_eps = 0.f;
 };
+
+// Whether a bf16 call runs as the fused kernel (kda_set_chunk_path).
+bool use_fused(int n_seqs, int H, int64_t total_chunks, size_t workspace_bytes, bool layer, bool has_q)
+{
+    const int mode = g_chunk_path.load(std::memory_order_relaxed);
+    if (mode != 0) return mode == 2 && (!layer || workspace_bytes >= kFusedRing + 2 * tc_tile_bytes());
+    const size_t fixed = ws_layout(n_seqs, H).fixed, row = (size_t)H * tc_tile_bytes();
+    const bool one_pass = workspace_bytes >= fixed && (int64_t)((workspace_bytes - fixed) / row) >= total_chunks;
+    if (layer && workspace_bytes < kFusedRing + 2 * tc_tile_bytes()) return false;
+    return !one_pass || (int64_t)n_seqs * H <= (layer ? 37 : 148);
+}
+
+// Cluster shape, number of clusters and ring depth of a call of the fused kernel.
+kda_status_t fused_schedule(FusedArgs& f, const std::vector<int64_t>& chunk_cu, int64_t avail, bool has_q)
+{
+    const int H = f.a.H, n_seqs = f.a.n_seqs;
+    auto len = [&](int n) { return chunk_cu[n + 1] - chunk_cu[n]; };
+    int most[2];
+    const kda_status_t rc = fused_max_clusters(most);
+    if (rc != KDA_OK) return rc;
+    if (most[0] < 1 && most[1] < 1) return fail(KDA_ERR_UNSUPPORTED, "kda_chunk_fwd: the device holds no cluster of the fused kernel");
+    // Two or three engine CTAs per chain: microseconds a tile costs the chain and an engine (measured), times the
+    // tiles of the most loaded cluster.
+    const double chain = has_q ? 1.5 : 1.3, engine = f.a.gate_rate ? 9.5 : has_q ? 8.0 : 7.5;
+    double best = 0.;
+    for (int i = 0; i < 2; ++i) {
+        if (most[i] < 1) continue;
+        const int nc = f.J < most[i] ? f.J : most[i];
+        int64_t tiles = 0;
+        if (f.J <= 4096) {
+            std::vector<int64_t> load((size_t)nc, 0);
+            for (int j = 0; j < f.J; ++j) {
+                const int r = j / nc, c = j - r * nc, n = f.ordered ? f.order[j / H] : j / H;
+                load[(size_t)((r & 1) ? nc - 1 - c : c)] += len(n);
+            }
+            tiles = *std::max_element(load.begin(), load.end());
+        } else {
+            tiles = (chunk_cu[n_seqs] * H + nc - 1) / nc;
+        }
+        const double per = engine / (2 * (2 + i)) > chain ? engine / (2 * (2 + i)) : chain;
+        const double t = per * (double)tiles + engine;
+        if (f.n_clusters == 0 || t < best) {
+            best = t;
+            f.n_clusters = nc;
+            f.cluster_size = 3 + i;
+        }
+    }
+    f.n_eng = 2 * (f.cluster_size - 1);
+    if (avail < f.n_eng) f.n_eng = (int)avail;          // (avail >= 2)
+    if ((int64_t)f.n_clusters * f.n_eng > avail) f.n_clusters = (int)(avail / f.n_eng);
+    const int64_t per = avail / ((int64_t)f.n_clusters * f.n_eng);
+    f.depth = (int)(per < FusedArgs::kMaxDepth ? per : FusedArgs::kMaxDepth);
+    return KDA_OK;
+}
 
 kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const float* log_alpha,
                             const float* beta, const float* S0, void* o, float* S_T,
@@ -342,76 +389,42 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
         return fail(KDA_ERR_INVALID_ARG, "kda_chunk_fwd: too many chunks");
 
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    // bf16: two paths.  With room for every tile of the call, the intra-chunk stage runs as one
-    // kernel over all SMs followed by the inter-chunk kernel (fastest on this device).  With less
-    // room, one fused cooperative kernel hands the tiles over through a small ring that stays in L2
-    // instead of walking the chunks in several passes.
-    bool fused = false;
+    FusedArgs f = {};
     if (dt == KDA_BF16) {
-        const int mode = g_chunk_path.load(std::memory_order_relaxed);
-        const WsLayout L2p = ws_layout(n_seqs, H);
-        const bool one_pass = workspace_bytes >= L2p.fixed &&
-                              (int64_t)((workspace_bytes - L2p.fixed) / ((size_t)H * tc_tile_bytes())) >= total_chunks;
-        fused = !lm.rate && (mode == 2 || (mode == 0 && !one_pass));
+        f.a.n_seqs = n_seqs; f.a.H = H; f.a.cu_seqlens = cu_seqlens_dev;
+        f.J = n_seqs * H;
+        f.ordered = cu_seqlens_dev != nullptr && n_seqs > 1 && n_seqs <= FusedArgs::kMaxOrder;
+        if (f.ordered) {
+            for (int n = 0; n < n_seqs; ++n) f.order[n] = (uint16_t)n;
+            std::stable_sort(f.order, f.order + n_seqs, [&](uint16_t x, uint16_t y) {
+                return chunk_cu[x + 1] - chunk_cu[x] > chunk_cu[y + 1] - chunk_cu[y];
+            });
+        }
+        f.epoch = next_epoch();
     }
-    if (fused) {
-        // ---- one fused cooperative kernel ----
-        const int64_t J = (int64_t)n_seqs * H;
-        const FusedLayout FL = fused_layout(J);
+    if (dt == KDA_BF16 && use_fused(n_seqs, H, total_chunks, workspace_bytes, lm.rate != nullptr, q && o)) {
         const size_t tbf = tc_tile_bytes();
-        if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) ||
-            workspace_bytes < FL.off_ring + 2 * tbf)
+        if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) || workspace_bytes < kFusedRing + 2 * tbf)
             return fail(KDA_ERR_WORKSPACE, "kda_chunk_fwd: workspace must be 256-byte aligned and at "
-                        "least %zu bytes (got %zu)", FL.off_ring + 2 * tbf, workspace_bytes);
-        if (J > 0x3fffffff) return fail(KDA_ERR_INVALID_ARG, "kda_chunk_fwd: n_seqs*H too large");
+                        "least %zu bytes (got %zu)", kFusedRing + 2 * tbf, workspace_bytes);
+        if ((int64_t)n_seqs * H > 0x3fffffff) return fail(KDA_ERR_INVALID_ARG, "kda_chunk_fwd: n_seqs*H too large");
         char* wsb = static_cast<char*>(workspace);
-        WsHeader* hdrf = reinterpret_cast<WsHeader*>(wsb);
+        f.hdr = reinterpret_cast<WsHeader*>(wsb);
         if (!o && !S_T) {   // nothing observable to produce: only leave a clean status word
-            KDA_CUDA_TRY(cudaMemsetAsync(hdrf, 0, sizeof(WsHeader), st));
+            KDA_CUDA_TRY(cudaMemsetAsync(f.hdr, 0, sizeof(WsHeader), st));
             return KDA_OK;
         }
-        int n_sm = 0;
-        {
-            DeviceLock lk;
-            if (!lk.st) return lk.rc;
-            if (lk.st->n_sm == 0) {
-                int dev = 0;
-                KDA_CUDA_TRY(cudaGetDevice(&dev));
-                KDA_CUDA_TRY(cudaDeviceGetAttribute(&lk.st->n_sm, cudaDevAttrMultiProcessorCount, dev));
-            }
-            n_sm = lk.st->n_sm;
-        }
-        const int64_t avail = (int64_t)((workspace_bytes - FL.off_ring) / tbf);
-        const FusedPlan P = fused_plan(chunk_cu, n_seqs, H, avail, n_sm);
-        if (P.Q < 1) return fail(KDA_ERR_UNSUPPORTED, "kda_chunk_fwd: the device has too few SMs");
-        const int64_t Q = P.Q, R = P.R, n_rounds = P.n_rounds;
-        const uint64_t n_prod = P.n_prod;
-        if (n_prod > 0x7fffffffull)
-            return fail(KDA_ERR_UNSUPPORTED, "kda_chunk_fwd: too many (chunk, head) tiles in one call");
-        FusedArgs f;
         f.a.q = q; f.a.k = k; f.a.v = v; f.a.log_alpha = log_alpha; f.a.beta = beta;
         f.a.S_in = S0; f.a.S_out = S_T; f.a.o = o;
-        f.a.cu_seqlens = cu_seqlens_dev; f.a.chunk_cu = nullptr;
-        f.a.n_seqs = n_seqs; f.a.H = H; f.a.total_tokens = total_tokens; f.a.seq_len = seq_len;
-        f.a.chunks_per_seq = chunks_per_seq; f.a.g0 = 0; f.a.g1 = total_chunks; f.a.scale = scale;
+        f.a.total_tokens = total_tokens; f.a.seq_len = seq_len; f.a.chunks_per_seq = chunks_per_seq;
+        f.a.g0 = 0; f.a.g1 = total_chunks; f.a.scale = scale;
         f.a.wait_limit_ns = wait_limit_ns();
-        f.ring = wsb + FL.off_ring;
-        f.ready = reinterpret_cast<unsigned long long*>(wsb + FL.off_ready);
-        f.consumed = reinterpret_cast<unsigned long long*>(wsb + FL.off_consumed);
-        f.round_base = cu_seqlens_dev ? reinterpret_cast<const uint32_t*>(wsb + FL.off_table) : nullptr;
-        f.hdr = hdrf;
-        f.Q = (int)Q; f.R = (int)R; f.J = (int)J; f.n_rounds = (int)n_rounds;
-        f.n_prod = (uint32_t)n_prod;
-        uint32_t ep = g_epoch.fetch_add(1, std::memory_order_relaxed) + 1;
-        if (ep == 0) ep = g_epoch.fetch_add(1, std::memory_order_relaxed) + 1;
-        f.epoch = ep;
-        f.n_chain_cta = (int)(fused_slices() * Q);
-        kda_status_t rcf = KDA_OK;
-        if (cu_seqlens_dev)
-            rcf = launch_fused_prep(hdrf, cu_seqlens_dev, reinterpret_cast<uint32_t*>(wsb + FL.off_table),
-                                    n_seqs, H, (int)Q, (int)n_rounds, st);
+        f.a.gate_rate = lm.rate; f.a.gate_bias = lm.bias; f.a.l2_eps = lm.l2_eps;
+        f.a.out_gate = lm.out_gate; f.a.rms_weight = lm.rms_weight; f.a.rms_eps = lm.rms_eps;
+        f.ring = wsb + kFusedRing;
+        const kda_status_t rcf = fused_schedule(f, chunk_cu, (int64_t)((workspace_bytes - kFusedRing) / tbf), q && o);
         if (rcf != KDA_OK) return rcf;
-        return launch_fused_tc(f, q != nullptr && o != nullptr, cu_seqlens_dev == nullptr, st);
+        return launch_fused_tc(f, q != nullptr && o != nullptr, st);
     }
 
     const WsLayout L = ws_layout(n_seqs, H);
@@ -459,9 +472,15 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
             while (n_end < n_seqs && chunk_cu[n_end] < g1) ++n_end;
             n_count = n_end - n_begin;
         }
-        if (dt == KDA_BF16)
-            rc = launch_chunk_tc(a, ws + L.off_tiles, n_begin, n_count, hdr, tc_clears && first, st);
-        else
+        if (dt == KDA_BF16) {
+            rc = launch_intra_tc(a, ws + L.off_tiles, hdr, tc_clears && first, st);
+            f.a = a;
+            f.ring = ws + L.off_tiles;
+            f.hdr = hdr;
+            f.n_begin = n_begin;
+            f.ordered = f.ordered && n_count == n_seqs;
+            if (rc == KDA_OK && n_count > 0) rc = launch_chain_tc(f, n_count, st);
+        } else
             rc = launch_chunk_f32(a, ws + L.off_tiles, n_begin, n_count, hdr, st);
         if (rc != KDA_OK) return rc;
         g0 = g1;
@@ -522,10 +541,9 @@ kda_status_t kda_layer_fwd(const void* q_c, const void* k_c, const void* v, cons
                                        "aligned", p);
     LayerMode lm;
     lm.rate = A_log; lm.bias = dt_bias; lm.l2_eps = l2_eps;
-    // The output stage runs inside the inter-chunk kernel when the device can hold the clusters this
-    // needs (the slices of a row exchange their sums of squares), else as a pass of its own.
+    // The output stage runs where the output rows are formed, unless a pass of its own is asked for.
     const bool fuse_out = y && total_tokens > 0 && n_seqs > 0 && g_fuse_output.load(std::memory_order_relaxed) &&
-                          inter_can_fuse_epilogue((int64_t)n_seqs * H);
+                          (int64_t)n_seqs * H <= 37;
     if (fuse_out) {
         lm.out_gate = g_o; lm.rms_weight = rms_weight; lm.rms_eps = rms_eps;
     }

@@ -37,7 +37,7 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
     uint64_t* x_ready = s_ready + 1;     // 4 warps: beta r or -beta dX written
     volatile uint32_t* abort_word = reinterpret_cast<volatile uint32_t*>(x_ready + 1);
     uint32_t* slot = const_cast<uint32_t*>(abort_word) + 1;
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int t = threadIdx.x, lane = t & 31, w = ptx::warp_uniform(t >> 5);
     int64_t g0, nc, tok_begin, tok_end;
     if (a.cu_seqlens) {
         g0 = a.chunk_cu[n]; nc = a.chunk_cu[n + 1] - g0;
@@ -67,7 +67,7 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tm = *slot;
+    const uint32_t tm = (uint32_t)ptx::warp_uniform((int)*slot);
     // false once any wait of the CTA has run out
     auto wait = [&](uint64_t* bar, int64_t phase) {
         if (!ptx::mbar_wait(bar, (uint32_t)phase & 1u, a.wait_limit_ns)) *abort_word = 1;
@@ -92,18 +92,18 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
             }
         }
     } else if (w == 8) {
-        if (lane == 0) {
-            const uint32_t id1 = ptx::umma_idesc_bf16(128, NS) | ptx::kIdescBMajorMN, id2 = id1 | ptx::kIdescAMajorMN;
-            for (int64_t i = 0; i < nc; ++i) {
-                if (!wait(s_ready, i) || !wait(&fullA[i & 1], i >> 1)) break;
-                ptx::tc_fence_after();
-                mma6<8>(tm + C_1, k_major<64, 2>(sm + O_A + (i & 1) * kImg), mn_major<128, 1>(sm + O_S), id1, false);
-                ptx::umma_commit(m1);
-                if (!wait(x_ready, i) || !wait(fullB, i)) break;
-                ptx::tc_fence_after();
-                mma6<4>(tm + C_2, mn_major<64, 2>(sm + O_B), mn_major<64, 1>(sm + O_X), id2, false);
-                ptx::umma_commit(m2);
-            }
+        const uint32_t id1 = ptx::umma_idesc_bf16(128, NS) | ptx::kIdescBMajorMN, id2 = id1 | ptx::kIdescAMajorMN;
+        for (int64_t i = 0; i < nc; ++i) {
+            if (!wait(s_ready, i) || !wait(&fullA[i & 1], i >> 1)) break;
+            __syncwarp();
+            ptx::tc_fence_after();
+            mma6<8>(tm + C_1, k_major<64, 2>(sm + O_A + (i & 1) * kImg), mn_major<128, 1>(sm + O_S), id1, false);
+            ptx::umma_commit(m1);
+            if (!wait(x_ready, i) || !wait(fullB, i)) break;
+            __syncwarp();
+            ptx::tc_fence_after();
+            mma6<4>(tm + C_2, mn_major<64, 2>(sm + O_B), mn_major<64, 1>(sm + O_X), id2, false);
+            ptx::umma_commit(m2);
         }
     } else {
         const int quad = w & 3, row = quad * 32 + lane, ch = (w >> 2) * 32;

@@ -31,7 +31,7 @@ template <typename T>
 __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int t = threadIdx.x, lane = t & 31, w = ptx::warp_uniform(t >> 5);
     int64_t chunk; int h;
     bwd_tile(a, blockIdx.x, chunk, h);
     uint8_t* sm = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -152,10 +152,10 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
         }
     }
     publish();
-    const uint32_t tm = *slot;
+    const uint32_t tm = (uint32_t)ptx::warp_uniform((int)*slot);
     const uint32_t mnA = ptx::kIdescAMajorMN, mnB = ptx::kIdescBMajorMN;
     constexpr int kCopy = 64;      // the thread that issues the bulk copies
-    if (t == 0) {
+    if (w == 0) {
         mma6<8>(tm + C_A, k_major<128, 2>(sm + O_RQ), k_major<64, 2>(sm + O_RK), ptx::umma_idesc_bf16(128, 64), false);
         ptx::umma_commit(&bar[0]);
     }
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
         put8<64, 2>(sm + O_RK, row0 + 32 * j, c8, x);
     }
     publish();
-    if (t == 0) {
+    if (w == 0) {
         const uint32_t idesc = ptx::umma_idesc_bf16(128, 128) | mnA | mnB;
         mma6<4>(tm + C_N, mn_major<128, 2>(sm + O_RQ, 64), mn_major<64, 2>(sm + O_RK), idesc, false);
         mma6<4>(tm + C_X, mn_major<64, 1>(sm + O_RP), mn_major<64, 2>(sm + O_RK), idesc, false);
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
         }
     }
     publish();
-    if (t == 0) {
+    if (w == 0) {
         const uint32_t idesc = ptx::umma_idesc_bf16(128, 128) | mnB;
         mma6<4>(tm + C_W, k_major<64, 1>(sm + O_RP), mn_major<128, 2>(sm + O_RQ), idesc, false);
         ptx::umma_commit(&bar[2]);

@@ -47,7 +47,7 @@ template <typename T>
 __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int t = threadIdx.x, lane = t & 31, w = ptx::warp_uniform(t >> 5);
     int64_t chunk; int h;
     bwd_tile(a, blockIdx.x, chunk, h);
     if (a.seq_heads[h]) return;
@@ -143,9 +143,9 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         }
     }
     publish();
-    const uint32_t tm = *slot;
+    const uint32_t tm = (uint32_t)ptx::warp_uniform((int)*slot);
     const uint32_t mnA = ptx::kIdescAMajorMN, mnB = ptx::kIdescBMajorMN;
-    if (t == 0) {
+    if (w == 0) {
         mma6<4>(tm + C_P1, mn_major<64, 1>(sm + O_RA), mn_major<64, 2>(sm + O_DX), ptx::umma_idesc_bf16(128, 128) | mnA | mnB, false);
         ptx::umma_commit(&bar[0]);
     }
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     publish();
 
     // ---- P2, then P4 and the first half of P3 ---------------------------------------------------------------
-    if (t == 0) {
+    if (w == 0) {
         mma6<8>(tm + C_P2, k_major<128, 2>(sm + O_RA), k_major<128, 2>(sm + O_RB), ptx::umma_idesc_bf16(128, 128), false);
         ptx::umma_commit(&bar[1]);
     }
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         put8<128, 1>(sm + O_LAM0, rs, cs + 32 * j, v);
     }
     publish();
-    if (t == 0) {
+    if (w == 0) {
         mma6<8>(tm + C_P4, k_major<128, 2>(sm + O_RA), k_major<64, 2>(sm + O_RB), ptx::umma_idesc_bf16(128, 64), false);
         ptx::umma_commit(&bar[2]);
         mma6<4>(tm + C_P3, k_major<64, 2>(sm + O_RB), k_major<128, 1>(sm + O_LAM0), ptx::umma_idesc_bf16(128, 128), false);
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         }
     }
     publish();
-    if (t == 0) {
+    if (w == 0) {
         mma6<4>(tm + C_P3, k_major<64, 2>(sm + O_RB + 8192), k_major<128, 1>(sm + O_LAM1), ptx::umma_idesc_bf16(128, 128), true);
         ptx::umma_commit(&bar[3]);
     }
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         put8<128, 2>(sm + O_RB, 64 + r, c8, kk[j]);
     }
     publish();
-    if (t == 0) {
+    if (w == 0) {
         mma6<4>(tm + C_P2, k_major<128, 1>(sm + O_DPB), mn_major<64, 2>(sm + O_LAM1), ptx::umma_idesc_bf16(128, 128) | mnB, true);
         mma6<8>(tm + C_P6, mn_major<128, 1>(sm + O_DPB), mn_major<128, 2>(sm + O_RB), ptx::umma_idesc_bf16(128, 128) | mnA | mnB, false);
         ptx::umma_commit(&bar[4]);

@@ -81,26 +81,22 @@ struct ChunkArgs {
     float rms_eps = 0.f;
 };
 
-// Work description of the fused bf16 chunk-forward kernel (one cooperative launch per call).
-//
-// Jobs are (sequence, head) pairs in natural order j = n * H + h.  Q of them run at a time ("round"
-// r covers jobs [r Q, (r + 1) Q)); slot q of a round is served by the chain CTAs 2 q and 2 q + 1
-// (one 64-column slice of the state each); the other CTAs run two intra-chunk engines each.  The intra-chunk engines of all CTAs
-// produce the tiles of a round chunk by chunk (production index = base_r + c * Q_r + q) into a ring
-// of R tiles per slot; `ready` holds (epoch << 32 | production index + 1) per ring position and
-// `consumed` (epoch << 32 | number of production indices the slice has finished with) per chain
-// role, so nothing has to be cleared between calls.
+// Work description of the fused bf16 chunk-forward kernel and of the two kernels of the two-kernel schedule.
+// Jobs are (sequence, head) pairs.  Fused: a cluster of CTAs works through a fixed share of them (job_info in
+// kda_fused_tc.cu), its engines handing tiles to its chain through a ring of n_eng * depth tiles.
 struct FusedArgs {
-    ChunkArgs a;                     // g0, g1 unused
-    char* ring;                      // [Q][R] tiles
-    unsigned long long* ready;       // [Q * R]
-    unsigned long long* consumed;    // [Q * fused_slices()]
-    const uint32_t* round_base;      // packed batches: [n_rounds + 1] production index base per round; else nullptr
+    ChunkArgs a;                     // (g0, g1: two-kernel schedule)
+    char* ring;                      // [n_clusters][n_eng][depth] tiles; two-kernel schedule: all tiles of the pass
     WsHeader* hdr;
-    int Q, R, J, n_rounds;
-    uint32_t n_prod;                 // production indices in total (equal lengths; packed: round_base[n_rounds])
+    uint32_t n_prod;                 // two-kernel schedule: tiles of the pass
     uint32_t epoch;                  // call id, never 0
-    int n_chain_cta;                 // chain CTAs: fused_slices() per slot
+    int J;                           // jobs
+    int n_clusters, cluster_size;    // CTAs of a cluster: one chain, the others two engines each
+    int n_eng, depth;                // engines in use per cluster, ring positions of an engine (1 .. kMaxDepth)
+    int n_begin;                     // two-kernel schedule: first sequence of the pass
+    int ordered;                     // order[] holds the sequences, longest first
+    static constexpr int kMaxDepth = 4, kMaxOrder = 256;
+    uint16_t order[kMaxOrder];
 };
 
 // ---- dtype helpers ------------------------------------------------------------------------------
@@ -181,22 +177,13 @@ size_t f32_tile_bytes();
 kda_status_t launch_chunk_f32(const ChunkArgs& a, void* tiles, int n_begin,
                                int n_count, WsHeader* hdr, cudaStream_t st);
 
-// bf16 tensor-core path (tcgen05 + bulk copies): per-tile scratch size and pass launcher
+// bf16 tensor-core path (tcgen05 + bulk copies): per-tile scratch size, the two kernels of a pass, the fused kernel
 size_t tc_tile_bytes();
-kda_status_t launch_chunk_tc(const ChunkArgs& a, void* tiles, int n_begin, int n_count,
-                             WsHeader* hdr, bool clear_status, cudaStream_t st);
-bool inter_can_fuse_epilogue(int64_t groups);
+kda_status_t launch_intra_tc(const ChunkArgs& a, void* tiles, WsHeader* hdr, bool clear_status, cudaStream_t st);
+kda_status_t launch_chain_tc(const FusedArgs& f, int n_count, cudaStream_t st);
+kda_status_t fused_max_clusters(int (&n)[2]);   // resident clusters of 3 and of 4 CTAs
+kda_status_t launch_fused_tc(const FusedArgs& f, bool has_q, cudaStream_t st);
 unsigned long long wait_limit_ns();   // KDA_WAIT_LIMIT_MS (1 .. 600000) in ns, default 1 s
-kda_status_t make_plain_tmap(CUtensorMap* tm, const void* base, int64_t total_tokens, int H, int cols, int rows);
-
-// fused bf16 path: workspace bytes besides the ring (flags and round table), and the launcher
-size_t fused_fixed_bytes(int n_seqs, int H);
-int fused_max_slots(int n_sm);
-int fused_slices();
-kda_status_t launch_fused_tc(FusedArgs f, bool has_q, bool clear_status, cudaStream_t st);
-kda_status_t launch_fused_prep(WsHeader* hdr, const int32_t* cu_seqlens, uint32_t* round_base, int n_seqs,
-                               int H, int Q, int n_rounds, cudaStream_t st);
-
 // ---- per-device library state ---------------------------------------------------------------------
 // Everything the library caches about a device (SM count, which kernels already carry their
 // dynamic-shared-memory attribute, helper streams) lives in one slot per device ordinal, created
@@ -207,7 +194,7 @@ struct DeviceState {
     int n_sm = 0;
     bool attr_done[kAttrSlots] = {};
     cudaStream_t copy_in = nullptr, copy_out = nullptr;
-    int max_clusters = -1;   // resident 4-CTA clusters of the inter-chunk kernel with the output stage (-1: not asked yet)
+    int fused_clusters[2] = {0, 0};   // resident clusters of 3 and of 4 CTAs of the fused kernel
 };
 // Locks the table and returns the slot of the calling thread's current device (nullptr + error set
 // on failure); the lock is released by ~DeviceLock.

@@ -45,6 +45,9 @@ namespace {
 
 constexpr int kThreads = 512;
 constexpr int kEngThreads = 256;
+// Lane 0 of an engine's warp 7 issues every bulk copy, finds the tiles and talks to the chain (warps 0 and 2 issue
+// the MMAs); what it can it does during the blocked substitution, which warps 6 and 7 have no part in.
+constexpr int kServiceThread = 224;
 constexpr int LDT = 68;                                   // padded fp32 row of the 64x64 matrix
 constexpr int LDD = 16;                                   // padded fp32 row of a 16x16 diagonal block
 constexpr float kLog2e = 1.4426950408889634f;
@@ -76,32 +79,28 @@ constexpr uint32_t E_TD = E_A + 64 * LDT * 4;     // fp32 4 x [16][LDD]: diagona
 constexpr uint32_t E_TD_BYTES = 4096;
 constexpr uint32_t E_BETA = E_TD + E_TD_BYTES;    // 64 fp32
 constexpr uint32_t E_DESC = E_BETA + 256;         // three tile descriptors: this tile, the next, the one after
-constexpr uint32_t E_BAR = E_DESC + 192;          // 8-byte words: mma barrier, K barrier, abort word, Q barrier,
+constexpr uint32_t E_CUR = E_DESC + 192;          // the service thread's EngineCursor
+constexpr int kMaxDepth = FusedArgs::kMaxDepth;   // ring positions of an engine
+constexpr uint32_t E_BAR = E_CUR + 64;          // 8-byte words: mma barrier, K barrier, abort word, Q barrier,
                                                   // (first engine) TMEM slot, V barrier
-constexpr uint32_t E_KS = (E_BAR + 64 + 1023) / 1024 * 1024;   // raw k of the NEXT tile [2 K-halves][64][64] bf16
+constexpr uint32_t E_KS = (E_BAR + 96 + 1023) / 1024 * 1024;   // raw k of the NEXT tile [2 K-halves][64][64] bf16
 constexpr uint32_t E_NORM = E_KS + 16384;         // layer mode: 1 / |k_i|, 1 / |q_i| (64 fp32 each)
-constexpr uint32_t E_BYTES = E_NORM + 1024;
+constexpr uint32_t E_GV = E_NORM + 512;           // gamma^C and exp(G_m) on their way to the tile
+constexpr uint32_t E_BYTES = (E_GV + tc::GV_BYTES + 1023) / 1024 * 1024;
 static_assert(E_TD_BYTES >= 8 * 128 * 4 && E_TD_BYTES >= 4 * 16 * LDD * 4, "scan exchange and diagonal blocks fit");
 
 // ---- shared-memory map of a chain CTA (bytes from the 1024-aligned base) -----------------------------
-constexpr int NS = 64;                             // state columns per chain CTA
-constexpr int kSlices = kD / NS;                   // chain CTAs per (sequence, head)
-constexpr int kStagesAB = 2, kStagesG = 3;
-constexpr uint32_t C_QW = 0;                       // [2 K-halves][128][64]: rows 0-63 W', 64-127 Q'
-constexpr uint32_t C_KT = 32768;                   // K': [2 dk-halves][64 tokens][64], MN-major A operand
-constexpr uint32_t C_AQ = 49152;                   // Aqk [64][64]; used as rows 64-127 of a 128-row operand
-constexpr uint32_t C_U = 57344;                    // two [64 tokens][32] blocks of U
-constexpr uint32_t C_UBYTES = (NS / 32) * tc::U_BLOCK;
-constexpr uint32_t C_STAGE = C_U + C_UBYTES;
-constexpr uint32_t C_SBF = kStagesAB * C_STAGE;    // B operand of MMA1, MN-major: [128 dk rows][128 B] = bf16(exp(G_m) . S)
-constexpr uint32_t C_VN = C_SBF + 128 * 128;       // B operand of MMA2, MN-major: [64 token rows][128 B] = V_new
-constexpr uint32_t C_GV = C_VN + 64 * 128;         // [3] x (gamma^C | exp(G_m) | exp(G_C - G_m))
-constexpr uint32_t C_BAR = C_GV + kStagesG * tc::GV_BYTES;
-constexpr uint32_t C_BYTES = C_BAR + 256;
+constexpr int kStages = 3;                         // tiles on their way or in work
+constexpr uint32_t C_STAGE = (tc::TILE_BYTES + 1023) / 1024 * 1024;
+constexpr uint32_t C_SSQ = kStages * C_STAGE;      // output stage: [2][64][4] fp32 row sums of squares
+constexpr uint32_t C_BAR = C_SSQ + 2048;
+constexpr uint32_t C_BYTES = C_BAR + 512;
 constexpr uint32_t kSmemBytes = 2 * E_BYTES > C_BYTES ? 2 * E_BYTES : C_BYTES;
-static_assert(C_STAGE % 1024 == 0 && E_BYTES % 1024 == 0, "operand images stay 1024-byte aligned");
+static_assert(E_BYTES % 1024 == 0, "operand images stay 1024-byte aligned");
 static_assert(kSmemBytes <= 232448, "fits the shared memory of one SM");
-constexpr uint32_t kTmemCols = 512;                // two engines of 256 columns, or one chain of 384
+constexpr uint32_t kTmemCols = 512;                // two engines of 256 columns, or one chain
+// TMEM columns of a chain: D1 of two chunks, D3, the bf16 state and V_new (A operands, two values a column)
+constexpr uint32_t T_D1 = 0, T_D3 = 256, T_S = 384, T_VN = 448;
 
 // loads that the compiler may not sink below their issue point (register prefetch of the next tile)
 __device__ __forceinline__ void ld_nc_f4(const float* p, float& a, float& b, float& c, float& d) {
@@ -109,11 +108,9 @@ __device__ __forceinline__ void ld_nc_f4(const float* p, float& a, float& b, flo
                  : "=f"(a), "=f"(b), "=f"(c), "=f"(d)
                  : "l"(p));
 }
-__device__ __forceinline__ uint32_t to_tf32(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return r;
-}
+// rounding to tf32 (to nearest, ties away) by an addition on the bit pattern: the tensor core ignores the 13 low
+// bits (cvt.rna.tf32 gives the same and issues several times slower)
+__device__ __forceinline__ uint32_t to_tf32(float x) { return __float_as_uint(x) + 0x1000u; }
 // 16x16 block products of the forward substitution on the warp-level tensor path (mma.sync
 // m16n8k8, tf32 inputs rounded to nearest, fp32 accumulation): acc += A * B with A, B 16x16 fp32
 // blocks in shared memory (row strides lda, ldb floats).
@@ -168,26 +165,20 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     return *reinterpret_cast<uint32_t*>(&p);
 }
 
-// ---- job / round geometry (the same formulas on the producing and the consuming side) --------------
-struct RoundInfo {
-    uint32_t base;   // production index of (chunk 0, slot 0) of the round
-    int Qr;          // jobs in the round
-};
-__device__ __forceinline__ RoundInfo round_info(const FusedArgs& f, int r) {
-    RoundInfo R;
-    R.base = f.round_base ? f.round_base[r] : (uint32_t)r * (uint32_t)f.a.chunks_per_seq * (uint32_t)f.Q;
-    const int left = f.J - r * f.Q;
-    R.Qr = left < f.Q ? left : f.Q;
-    return R;
-}
+// ---- jobs: (sequence, head) pairs, dealt out to the clusters ------------------------------------------
 struct JobInfo {
     int n, h, nch;
     int64_t tok_begin, tok_end;
+    int64_t tile0;                // two-kernel schedule: index of the first tile (then every H-th)
 };
-__device__ __forceinline__ JobInfo job_info(const FusedArgs& f, int j) {
-    JobInfo I;
-    I.n = j / f.a.H;
-    I.h = j - I.n * f.a.H;
+// Job number r of cluster cid; false past its last.  Sequences come longest first (f.order) and the
+// clusters take turns back and forth, so that their loads stay close to each other.
+__device__ __forceinline__ bool job_info(const FusedArgs& f, int cid, int r, JobInfo& I) {
+    const int64_t jr = (int64_t)r * f.n_clusters + ((r & 1) ? f.n_clusters - 1 - cid : cid);
+    if (jr >= f.J) return false;
+    const int rank = (int)jr / f.a.H;
+    I.h = (int)jr - rank * f.a.H;
+    I.n = f.ordered ? (int)f.order[rank] : rank;
     if (f.a.cu_seqlens) {
         I.tok_begin = f.a.cu_seqlens[I.n];
         I.tok_end = f.a.cu_seqlens[I.n + 1];
@@ -196,10 +187,29 @@ __device__ __forceinline__ JobInfo job_info(const FusedArgs& f, int j) {
         I.tok_end = I.tok_begin + f.a.seq_len;
     }
     I.nch = (int)((I.tok_end - I.tok_begin + kC - 1) / kC);
-    return I;
+    return true;
 }
-__device__ __forceinline__ unsigned long long tag(uint32_t epoch, uint32_t x) {
-    return ((unsigned long long)epoch << 32) | x;
+// The one job of a chain CTA of the two-kernel schedule: the chunks that the pass has of its (sequence, head).
+__device__ __forceinline__ bool pass_job(const FusedArgs& f, int id, int r, JobInfo& I) {
+    if (r > 0) return false;
+    const ChunkArgs& a = f.a;
+    const int rank = id / a.H;
+    I.n = f.ordered ? (int)f.order[rank] : f.n_begin + rank;
+    I.h = id - rank * a.H;
+    int64_t cb, ce, tok0;
+    if (a.cu_seqlens) {
+        cb = a.chunk_cu[I.n]; ce = a.chunk_cu[I.n + 1];
+        tok0 = a.cu_seqlens[I.n]; I.tok_end = a.cu_seqlens[I.n + 1];
+    } else {
+        cb = (int64_t)I.n * a.chunks_per_seq; ce = cb + a.chunks_per_seq;
+        tok0 = (int64_t)I.n * a.seq_len; I.tok_end = tok0 + a.seq_len;
+    }
+    const int64_t first = cb < a.g0 ? a.g0 : cb;
+    if (ce > a.g1) ce = a.g1;
+    I.nch = ce > first ? (int)(ce - first) : 0;
+    I.tok_begin = tok0 + (first - cb) * kC;
+    I.tile0 = (first - a.g0) * a.H + I.h;
+    return true;
 }
 __device__ __forceinline__ bool call_aborted(const FusedArgs& f) {
     return *reinterpret_cast<volatile unsigned int*>(&f.hdr->abort_epoch) == f.epoch;
@@ -210,114 +220,42 @@ __device__ __forceinline__ void report_timeout(const FusedArgs& f, int where) {
     __threadfence();
 }
 
-// One (chunk, head) tile as the engine's scheduler thread hands it to the other 255 threads.
+// One (chunk, head) tile as the engine's service thread hands it to the other 255 threads.
 struct TileDesc {
     long long tok0;                  // first token of the chunk
-    char* tile;                      // ring position
-    unsigned long long* ready;       // its flag word
-    unsigned long long ready_val;
-    const unsigned long long* consumed;   // the four progress words of the slot's chain roles
+    char* tile;                      // where it goes
     int h;
     int len;                         // valid tokens, 1..64; 0 = no more tiles for this engine
-    uint32_t need;                   // the ring position is free once every progress word has reached this
-    int pad[3];
+    int pad[10];
 };
 static_assert(sizeof(TileDesc) == 64, "three descriptors fit the 192 bytes reserved");
 
-// Hands out production indices in increasing order to whichever engine asks next (a slow engine
-// then delays one tile, not every tile of a fixed share).  The counter lives in the workspace header
-// and carries the call id in its upper half, so a value left by an earlier call is recognised and
-// replaced by the first asker instead of having to be cleared.
-__device__ __forceinline__ uint32_t fetch_index(const FusedArgs& f)
-{
-    unsigned long long* ctr = reinterpret_cast<unsigned long long*>(&f.hdr->pad[40]);
-    for (;;) {
-        const unsigned long long v = *reinterpret_cast<volatile unsigned long long*>(ctr);
-        if ((uint32_t)(v >> 32) == f.epoch) return (uint32_t)atomicAdd(ctr, 1ull);
-        if (atomicCAS(ctr, v, tag(f.epoch, 1u)) == v) return 0u;
-    }
-}
-// Describes the tile with production index i; false if there is no tile at that index (a shorter
-// sequence of the round, or past the end).
-__device__ bool describe_tile(const FusedArgs& f, uint32_t i, TileDesc* d)
+// The tiles of a cluster are numbered through its jobs; engine e of E makes tiles e, e + E, ..., its m-th
+// tile in position m % depth of its own share of the cluster's ring.
+struct EngineCursor {
+    int cid, e;
+    int r, c, m;                     // job, chunk inside it, tiles handed out so far
+    uint32_t ready;                  // shared::cluster address of the chain's barriers of this engine's positions
+    int done, published;             // tiles finished, and announced to the chain
+};
+static_assert(sizeof(EngineCursor) <= 64, "fits the 64 bytes reserved");
+__device__ void cluster_tile(const FusedArgs& f, EngineCursor& k, TileDesc* d)
 {
     d->len = 0;
-    if (i >= f.n_prod) return false;
-    int r;
-    if (f.round_base) {
-        int lo = 0, hi = f.n_rounds - 1;   // last round with base <= i
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (f.round_base[mid] <= i) lo = mid; else hi = mid - 1;
-        }
-        r = lo;
-    } else {
-        r = (int)(i / ((uint32_t)f.a.chunks_per_seq * (uint32_t)f.Q));
+    JobInfo J;
+    for (;;) {
+        if (!job_info(f, k.cid, k.r, J)) return;
+        if (k.c < J.nch) break;
+        k.c -= J.nch;
+        ++k.r;
     }
-    const RoundInfo R = round_info(f, r);
-    const uint32_t il = i - R.base;
-    const int c = (int)(il / (uint32_t)R.Qr), q = (int)(il - (uint32_t)c * (uint32_t)R.Qr);
-    const JobInfo J = job_info(f, r * f.Q + q);
-    if (c >= J.nch) return false;
-    const int pos = q * f.R + c % f.R;
-    d->tok0 = J.tok_begin + (int64_t)c * kC;
+    d->tok0 = J.tok_begin + (int64_t)k.c * kC;
     const int64_t rem = J.tok_end - d->tok0;
-    d->tile = f.ring + (size_t)pos * tc::TILE_BYTES;
-    d->ready = f.ready + pos;
-    d->ready_val = tag(f.epoch, i + 1u);
-    d->consumed = f.consumed + q * kSlices;
-    // the ring position was last used by chunk c - R of this job, or by the slot's job of an earlier round
-    d->need = c >= f.R ? i - (uint32_t)f.R * (uint32_t)R.Qr + 1u : R.base;
+    d->tile = f.ring + (size_t)((k.cid * f.n_eng + k.e) * f.depth + k.m % f.depth) * tc::TILE_BYTES;
     d->h = J.h;
     d->len = rem < kC ? (int)rem : kC;
-    return true;
-}
-// The service thread's look-ahead state: the request for the next index is in flight while a tile is
-// worked on, and so is a look at the progress of the next tile's consumers.
-struct SchedState {
-    unsigned long long pending;             // return value of the counter request in flight
-    unsigned long long seen[kSlices];       // progress words of the next tile's consumers, read a tile early
-};
-// The engine's next tile: takes the index requested a tile ago, requests the one after it, skips
-// indices without a tile.  ONE thread.
-__device__ void next_tile(const FusedArgs& f, SchedState& ss, TileDesc* d)
-{
-    unsigned long long* ctr = reinterpret_cast<unsigned long long*>(&f.hdr->pad[40]);
-    for (;;) {
-        // (the counter carries this call's id since the engine's first request)
-        const uint32_t i = (uint32_t)(ss.pending >> 32) == f.epoch ? (uint32_t)ss.pending : 0xffffffffu;
-        if (i >= f.n_prod) { d->len = 0; return; }
-        ss.pending = atomicAdd(ctr, 1ull);
-        if (describe_tile(f, i, d)) break;
-    }
-}
-// Whether the look taken a tile ago settles that the previous occupant of the tile's ring position has been
-// consumed by every chain role.
-__device__ bool slot_seen_free(const FusedArgs& f, const TileDesc& d, const SchedState& ss)
-{
-    bool ok = true;
-    for (int sl = 0; sl < kSlices; ++sl) ok = ok && (uint32_t)(ss.seen[sl] >> 32) == f.epoch && (uint32_t)ss.seen[sl] >= d.need;
-    return ok || d.need == 0;
-}
-// Waits (bounded) for that.  Runs in ONE thread, whose engine has published every finished tile: a
-// producer that waited for its consumers while sitting on a tile they need would deadlock.
-__device__ void wait_slot_free(const FusedArgs& f, const TileDesc& d, volatile uint32_t* abort_word)
-{
-    uint64_t t0 = 0;
-    for (int sl = 0; sl < kSlices; ++sl) {
-        for (;;) {
-            const unsigned long long v = ptx::ld_acquire_gpu(d.consumed + sl);
-            if ((uint32_t)(v >> 32) == f.epoch && (uint32_t)v >= d.need) break;
-            if (t0 == 0) t0 = ptx::globaltimer_ns();
-            if (*abort_word || call_aborted(f)) { *abort_word = 1; return; }
-            if (ptx::globaltimer_ns() - t0 > f.a.wait_limit_ns) {
-                *abort_word = 1;
-                report_timeout(f, 20);
-                return;
-            }
-            ptx::nanosleep(100);
-        }
-    }
+    k.c += f.n_eng;
+    ++k.m;
 }
 
 // ====================================================================================================
@@ -334,10 +272,6 @@ __device__ bool static_tile(const FusedArgs& f, uint32_t idx, TileDesc* d)
     const ChunkLoc L = locate_chunk(f.a, f.a.g0 + gl);
     d->tok0 = L.tok0;
     d->tile = f.ring + (size_t)idx * tc::TILE_BYTES;
-    d->ready = nullptr;
-    d->ready_val = 0;
-    d->consumed = nullptr;
-    d->need = 0;
     d->h = (int)(idx - gl * (uint32_t)f.a.H);
     d->len = L.len;
     return true;
@@ -350,14 +284,8 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 {
     constexpr bool has_q = kHasQ;
     constexpr int kNW = 8, kRPT = 8;
-    // Lane 0 of warp 7 issues every bulk copy, finds the tiles and talks to the chains (thread 0 issues the
-    // MMAs).  What takes it about a microsecond -- publishing a tile, looking at flags -- it does during the
-    // blocked substitution, which warps 6 and 7 have no part in: on any other path all eight warps would
-    // wait for it (publishing at the top of the next tile and looking for tiles beside the first MMA group:
-    // 11.2 us a tile).
-    constexpr int kServiceThread = 224;
     constexpr int kInvWarps = 6;       // warps of the blocked substitution
-    constexpr int kMma2Thread = 64;    // lane 0 of warp 2 issues half of the second MMA group
+    constexpr int kMma2Warp = 2;       // issues half of the second MMA group (warp 0 the rest)
     const ChunkArgs& a = f.a;
     float* sA = reinterpret_cast<float*>(smem + E_A);
     float* sTd = reinterpret_cast<float*>(smem + E_TD);
@@ -368,9 +296,10 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
     uint64_t* bar_k = mma_bar + 1;   // raw k has landed in the staging buffer
     uint64_t* bar_q = mma_bar + 3;   // raw q has landed in rows 64-127 of the operand image
     uint64_t* bar_v = mma_bar + 5;   // v has landed
+    uint64_t* bar_free = mma_bar + 6;   // [depth] (kFused) the chain has read a ring position
     volatile uint32_t* abort_word = reinterpret_cast<volatile uint32_t*>(mma_bar + 2);
 
-    const int warp = te >> 5, lane = te & 31;
+    const int warp = ptx::warp_uniform(te >> 5), lane = te & 31;
     auto ebar = [&]() { ptx::named_bar_sync(bar_id, kEngThreads); };
     auto inv_bar = [&]() { ptx::named_bar_sync(bar_id + 2, kInvWarps * 32); };
 
@@ -445,22 +374,24 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
     bool timed_out = false, out_of_range = false;
     bool pend_k = false, pend_q = false, pend_v = false;   // (thread 0) requests not yet waited for
     uint32_t tma_parity = 0;
-    SchedState ss = {};   // (scheduler thread)
     uint32_t next_static = first;
-    bool stores_pending = false;   // (bulk thread) the previous tile's staging may still be read out
     int cur = 0;
-    unsigned long long* pending_ready = nullptr;   // service thread: flag of the last finished tile, not yet published
-    unsigned long long pending_val = 0;
+    EngineCursor& cursor = *reinterpret_cast<EngineCursor*>(smem + E_CUR);   // (service thread, kFused)
+    auto publish = [&]() {
+        if (cursor.published == cursor.done) return;
+        ptx::bulk_wait_all0();           // the tile's stores are performed
+        ptx::mbar_arrive_cluster_relaxed(cursor.ready + (uint32_t)(cursor.published % f.depth) * 8u);
+        ++cursor.published;
+    };
     auto find_tile = [&](TileDesc* d) {   // (service thread)
         if (kFused) {
-            next_tile(f, ss, d);
+            cluster_tile(f, cursor, d);
         } else {
             static_tile(f, next_static, d);
             next_static += stride;
         }
     };
     if (te == kServiceThread) {
-        if (kFused) ss.pending = tag(f.epoch, fetch_index(f));
         find_tile(&desc[0]);
         if (desc[0].len > 0) find_tile(&desc[1]);
         else desc[1].len = 0;
@@ -471,17 +402,17 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         if (te == kServiceThread) {
             request_k(desc[0]);
             if (has_q) request_q(desc[0]);
-            request_v(desc[0]);
         }
         request_beta(desc[0]);
-        pend_k = pend_v = true;
+        pend_k = true;
         pend_q = has_q;
     }
     KT_DECL(10);
     while (true) {
-        const TileDesc D = desc[cur];
-        if (D.len == 0 || *abort_word) break;
-        char* tile = D.tile;
+        // (the descriptors are read where they are used: registers are short)
+        const TileDesc& D = desc[cur];
+        const int d_len = D.len;
+        if (d_len == 0 || *abort_word) break;
         KT_MARK(te == 0, 0);   // loop overhead
 
         if (kLayer) {
@@ -493,7 +424,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
                 for (int e = 0; e < 4; ++e) {
                     const float x = G[r][e] + bias[e];
                     const float sp = fmaxf(x, 0.f) + __logf(1.f + __expf(-fabsf(x)));
-                    G[r][e] = (i0 + r < D.len) ? nr * sp : 0.f;
+                    G[r][e] = (i0 + r < d_len) ? nr * sp : 0.f;
                 }
         }
         // ---- a1: cumulative log-decay, in the log2 domain (exponentials below are bare ex2) ---------
@@ -505,22 +436,9 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             for (int e = 0; e < 4; ++e) G[r][e] = fmaf(G[r][e], kLog2e, G[r - 1][e]);
         *reinterpret_cast<float4*>(sTot + warp * kD + d0) =
             make_float4(G[kRPT - 1][0], G[kRPT - 1][1], G[kRPT - 1][2], G[kRPT - 1][3]);
-        if (te == kServiceThread) {
-            if (stores_pending) ptx::bulk_wait_read0();   // the previous tile's W' / U staging has been read out
-            if (kFused && !slot_seen_free(f, D, ss)) {
-                if (pending_ready) {      // publish before waiting
-                    ptx::bulk_wait_all0();
-                    ptx::fence_proxy_async_all();
-                    ptx::st_release_gpu(pending_ready, pending_val);
-                    pending_ready = nullptr;
-                }
-                wait_slot_free(f, D, abort_word);
-            }
-            if (kFused) ptx::fence_proxy_async_all();   // the consumers' bulk reads of the position precede our writes
-        }
         ptx::cp_async_wait_all();             // beta
         if (kLayer && te < kC)                // (each of these threads copied its own element)
-            sBeta[te] = te < D.len ? 1.f / (1.f + __expf(-sBeta[te])) : 0.f;
+            sBeta[te] = te < d_len ? 1.f / (1.f + __expf(-sBeta[te])) : 0.f;
         ebar();
         KT_MARK(te == 0, 1);   // scan + publish + slot wait
         if (*abort_word) break;
@@ -539,16 +457,13 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         // |G_i - G_ref| <= |G_C| / 2 for every row whatever the distribution of the decay over the chunk
 #pragma unroll
         for (int e = 0; e < 4; ++e) gref[e] = 0.5f * glast[e];
-        // the true scales exp(G_C), exp(G_m) and exp(G_C - G_m) go to the tile as fp32 vectors; the
-        // chain applies them to the state in fp32
+        float em[4];   // exp(G_m) = exp(G_C - G_m)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) em[e] = ex2(gref[e]);
         if (warp == 0) {
-            *reinterpret_cast<float4*>(tile + tc::OFF_GV + d0 * 4) =
+            *reinterpret_cast<float4*>(smem + E_GV + d0 * 4) =
                 make_float4(ex2(glast[0]), ex2(glast[1]), ex2(glast[2]), ex2(glast[3]));
-            *reinterpret_cast<float4*>(tile + tc::OFF_GV + 512 + d0 * 4) =
-                make_float4(ex2(gref[0]), ex2(gref[1]), ex2(gref[2]), ex2(gref[3]));
-            *reinterpret_cast<float4*>(tile + tc::OFF_GV + 1024 + d0 * 4) =
-                make_float4(ex2(glast[0] - gref[0]), ex2(glast[1] - gref[1]), ex2(glast[2] - gref[2]),
-                            ex2(glast[3] - gref[3]));
+            *reinterpret_cast<float4*>(smem + E_GV + 512 + d0 * 4) = make_float4(em[0], em[1], em[2], em[3]);
             // a channel that decays by more than e^-160 inside this chunk leaves the range of the
             // two-factor form: flag it (the clamp below keeps everything finite)
             if (fminf(fminf(glast[0], glast[1]), fminf(glast[2], glast[3])) < -2.f * kClamp2) out_of_range = true;
@@ -594,7 +509,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 #pragma unroll
             for (int r = 0; r < kRPT; ++r)
                 if (lane == r) {   // (rows past the end of the sequence are zeroed below: keep their factor finite)
-                    const bool in = i0 + r < D.len;
+                    const bool in = i0 + r < d_len;
                     sNorm[i0 + r] = in ? rsqrtf(ssk[r] + a.l2_eps) : 0.f;
                     sNorm[kC + i0 + r] = in ? rsqrtf(ssq[r] + a.l2_eps) : 0.f;
                 }
@@ -614,7 +529,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
                 uint2 k2 = *reinterpret_cast<const uint2*>(smem + E_KS + hf * 8192 + o2);
                 uint2 q2 = make_uint2(0u, 0u);
                 if (has_q) q2 = *reinterpret_cast<const uint2*>(pk + 8192);
-                if (i >= D.len) k2 = q2 = make_uint2(0u, 0u);
+                if (i >= d_len) k2 = q2 = make_uint2(0u, 0u);
                 const float kf[4] = {__uint_as_float(k2.x << 16), __uint_as_float(k2.x & 0xffff0000u),
                                      __uint_as_float(k2.y << 16), __uint_as_float(k2.y & 0xffff0000u)};
                 const float qf[4] = {__uint_as_float(q2.x << 16), __uint_as_float(q2.x & 0xffff0000u),
@@ -646,6 +561,9 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
                         make_uint2(pack_bf16(oqg[0], oqg[1]), pack_bf16(oqg[2], oqg[3]));
                 *reinterpret_cast<uint2*>(smem + E_KI + hf * E_KI_HALF + o2) =
                     make_uint2(pack_bf16(oki[0], oki[1]), pack_bf16(oki[2], oki[3]));
+                if (has_q)   // what the chain reads: scale Q exp(G), over the raw k that this thread has just read
+                    *reinterpret_cast<uint2*>(smem + E_KS + hf * 8192 + o2) =
+                        make_uint2(pack_bf16(oqg[0] * em[0], oqg[1] * em[1]), pack_bf16(oqg[2] * em[2], oqg[3] * em[3]));
             }
         };
         {
@@ -661,15 +579,26 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 
         // ---- a2 + a5: [Kg ; Qg] Ki^T --------------------------------------------------------------------
         if (te == kServiceThread) {
-            // Q' (rows 64-127 of both K-halves of the operand image) and K' are tile contents as they are
-            if (has_q) {
-                ptx::bulk_s2g(tile + tc::OFF_QW + 8192, smem + E_KQ + 8192, 8192);
-                ptx::bulk_s2g(tile + tc::OFF_QW + tc::QW_HALF + 8192, smem + E_KQ + E_KQ_HALF + 8192, 8192);
+            if (kFused) {
+                publish();               // (before any wait: the chain may need that tile to go on)
+                const int m = cursor.done;
+                if (m >= f.depth) {
+                    const uint64_t t0 = ptx::globaltimer_ns();
+                    while (!ptx::mbar_try(&bar_free[m % f.depth], (uint32_t)(m / f.depth - 1) & 1u)) {
+                        if (*abort_word || call_aborted(f)) { *abort_word = 1; break; }
+                        if (ptx::globaltimer_ns() - t0 > f.a.wait_limit_ns) { timed_out = true; *abort_word = 1; break; }
+                    }
+                }
             }
-            ptx::bulk_s2g(tile + tc::OFF_KI, smem + E_KI, 16384);
+            if (has_q) {
+                ptx::bulk_s2g(D.tile + tc::OFF_QW + 8192, smem + E_KS, 8192);
+                ptx::bulk_s2g(D.tile + tc::OFF_QW + tc::QW_HALF + 8192, smem + E_KS + 8192, 8192);
+            }
+            ptx::bulk_s2g(D.tile + tc::OFF_KI, smem + E_KI, 16384);
+            ptx::bulk_s2g(D.tile + tc::OFF_GV, smem + E_GV, tc::GV_BYTES);
             ptx::bulk_commit();
         }
-        if (te == 0) {
+        if (warp == 0) {
             const uint32_t idesc = ptx::umma_idesc_bf16(128, 64);
             const uint32_t a0 = ptx::smem_u32(smem + E_KQ), b0 = ptx::smem_u32(smem + E_KI);
 #pragma unroll
@@ -678,18 +607,23 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
                                ptx::umma_desc_sw128(b0 + (k >> 2) * E_KI_HALF + (k & 3) * 32), idesc, k > 0);
             ptx::umma_commit(mma_bar);
         }
-        if (te == kMma2Thread) ptx::umma_commit(mma_bar);   // (the barrier counts both issuing threads)
+        if (warp == kMma2Warp) ptx::umma_commit(mma_bar);   // (the barrier counts both issuing warps)
         const int nxt = cur == 2 ? 0 : cur + 1, nxt2 = nxt == 2 ? 0 : nxt + 1;
-        const TileDesc Dn = desc[nxt];
+        const TileDesc& Dn = desc[nxt];
         const bool has_next = Dn.len > 0 && !*abort_word;
         if (has_next) {
             prefetch_regs(Dn);   // the next tile's log alpha: its registers are free since the gating loop
-            if (te == kServiceThread) request_k(Dn);   // the staging buffer was read by the gating loop
             pend_k = true;
         }
         if (!ptx::mbar_wait(mma_bar, 0, f.a.wait_limit_ns)) timed_out = true;
-        // Q' and K' have been read out of shared memory by now: Aqk goes over the Q' rows next
-        if (te == kServiceThread) ptx::bulk_wait_read0();
+        // everything staged for bulk stores has been read out of shared memory (this tile's Q and K', the previous
+        // tile's W and U^T): the next k goes over Q, v over W, L over U^T
+        if (te == kServiceThread) {
+            ptx::bulk_wait_read0();
+            request_v(D);
+            if (has_next) request_k(Dn);
+        }
+        pend_v = true;
         ebar();
         ptx::tc_fence_after();
         KT_MARK(te == 0, 4);   // MMA A
@@ -733,30 +667,15 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         ebar();
         if (te == kServiceThread) {
             if (has_q) {
-                ptx::bulk_s2g(tile + tc::OFF_AQ, smem + E_AQ, 8192);
+                ptx::bulk_s2g(D.tile + tc::OFF_AQ, smem + E_AQ, 8192);
                 ptx::bulk_commit();
             }
-            if (kFused && has_next && Dn.need > 0)
-#pragma unroll
-                for (int sl = 0; sl < kSlices; ++sl) ss.seen[sl] = ptx::ld_relaxed_gpu(Dn.consumed + sl);
             if (has_q) {   // the Aqk staging has been read out: the next tile's q may land over it
                 ptx::bulk_wait_read0();
                 if (has_next) request_q(Dn);
             }
-            if (kFused) {
-                // the previous tile's stores are complete (at most the one or two groups of this tile are not)
-                if (pending_ready) {
-                    if (has_q) ptx::bulk_wait_all<2>();
-                    else ptx::bulk_wait_all<1>();
-                    ptx::fence_proxy_async_all();
-                }
-                ptx::fence_acq_rel_gpu();   // orders the looks taken above and the publication
-                if (pending_ready) ptx::st_relaxed_gpu(pending_ready, pending_val);
-                pending_ready = nullptr;
-            }
             if (has_next) find_tile(&desc[nxt2]);
             else desc[nxt2].len = 0;
-            ptx::bulk_wait_read0();        // K' has been read out: the Mm image goes there
         }
         KT_MARK(te == 0, 5);   // A read-out
 
@@ -824,9 +743,9 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         if (!ptx::mbar_wait(bar_v, tma_parity, f.a.wait_limit_ns)) timed_out = true;   // v has landed
         pend_v = false;
         tma_parity ^= 1;
-        if (D.len < kC) {   // short last chunk: rows past the end hold other tokens' v; zero them
-            for (int idx = te; idx < (kC - D.len) * 16; idx += kEngThreads) {
-                const int j = D.len + (idx >> 4), c16 = idx & 15;
+        if (d_len < kC) {   // short last chunk: rows past the end hold other tokens' v; zero them
+            for (int idx = te; idx < (kC - d_len) * 16; idx += kEngThreads) {
+                const int j = d_len + (idx >> 4), c16 = idx & 15;
                 *reinterpret_cast<uint4*>(smem + E_V + (c16 >> 3) * E_V_BLOCK + j * 128 +
                                           (((c16 & 7) ^ (j & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
             }
@@ -863,7 +782,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         ptx::fence_async_smem();
         ptx::tc_fence_before();
         ebar();
-        if (te == 0) {
+        if (warp == 0) {
             ptx::tc_fence_after();
             const uint32_t idesc = ptx::umma_idesc_bf16(128, 128) | ptx::kIdescBMajorMN;
             const uint32_t m0 = ptx::smem_u32(smem + E_KI);
@@ -874,68 +793,56 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
                                ptx::umma_desc_sw128_mn(kg0 + k * 2048, E_KQ_HALF), idesc, k > 0);
             ptx::umma_commit(mma_bar);
         }
-        if (te == kMma2Thread) {   // the U half of the group is issued by a second thread at the same time
+        if (warp == kMma2Warp) {   // U^T = V^T Mm^T (the chain has its columns in the TMEM lanes), issued at the same time
             ptx::tc_fence_after();
-            const uint32_t idesc = ptx::umma_idesc_bf16(128, 128) | ptx::kIdescBMajorMN;
             const uint32_t m0 = ptx::smem_u32(smem + E_KI), v0 = ptx::smem_u32(smem + E_V);
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                ptx::umma_bf16(tmem_e + 128, ptx::umma_desc_sw128(m0 + k * 32),
-                               ptx::umma_desc_sw128_mn(v0 + k * 2048, E_V_BLOCK), idesc, k > 0);
+                ptx::umma_bf16(tmem_e + 128, ptx::umma_desc_sw128_mn(v0 + k * 2048, E_V_BLOCK), ptx::umma_desc_sw128(m0 + k * 32),
+                               ptx::umma_idesc_bf16(128, 64) | ptx::kIdescAMajorMN, k > 0);
             ptx::umma_commit(mma_bar);
         }
         if (!ptx::mbar_wait(mma_bar, 1, f.a.wait_limit_ns)) timed_out = true;
         KT_MARK(te == 0, 7);   // Mm + MMA B
-        if (has_next) {   // V and beta are free: the next tile's may land
-            if (te == kServiceThread) request_v(Dn);
-            request_beta(Dn);
-            pend_v = true;
-        }
+        if (has_next) request_beta(Dn);   // (beta is free)
         ptx::tc_fence_after();
-        {   // The A operand held every row twice, so TMEM lanes 0-63 and 64-127 both carry rows 0-63:
-            // each warp converts rows 32 (q4 & 1) + lane of one 64-column block of [W | U].
-            const int q4 = warp & 3, cbk = (warp >> 2) * 2 + (q4 >> 1);
-            const int col0 = cbk * 64;             // first column inside [W | U]
-            const int i = (q4 & 1) * 32 + lane;
-            const uint32_t ta = tmem_e + ((uint32_t)(q4 * 32) << 16) + col0;
+        {   // W' rows lie in TMEM lanes 0-63 and again in 64-127: 32 columns a warp; U^T has a lane per column of U
+            const int q4 = warp & 3, g = warp >> 2, i = (q4 & 1) * 32 + lane;
+            const uint32_t tq = tmem_e + ((uint32_t)(q4 * 32) << 16);
+            const int col0 = (g * 2 + (q4 >> 1)) * 32;
+            uint32_t r[32];
+            ptx::tmem_ld_32x32b_x32(tq + col0, r);
+            ptx::tmem_ld_wait();
 #pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                uint32_t r[32];
-                ptx::tmem_ld_32x32b_x32(ta + b * 32, r);
-                ptx::tmem_ld_wait();
-                if (col0 < 128) {   // W' = Mm Kg: K-half col0 / 64 of the [W' ; Q'] image
-                    uint8_t* dst = smem + E_KI + (col0 >> 6) * 8192;
-#pragma unroll
-                    for (int j8 = 0; j8 < 32; j8 += 8)
-                        *reinterpret_cast<uint4*>(dst + ptx::sw128_off(i, b * 32 + j8)) =
-                            make_uint4(pack_bf16(__uint_as_float(r[j8]), __uint_as_float(r[j8 + 1])),
-                                       pack_bf16(__uint_as_float(r[j8 + 2]), __uint_as_float(r[j8 + 3])),
-                                       pack_bf16(__uint_as_float(r[j8 + 4]), __uint_as_float(r[j8 + 5])),
-                                       pack_bf16(__uint_as_float(r[j8 + 6]), __uint_as_float(r[j8 + 7])));
-                } else {            // U: 32-column block (col0 - 128) / 32 + b
-                    uint8_t* dst = smem + E_A + (((col0 - 128) >> 5) + b) * tc::U_BLOCK;
-#pragma unroll
-                    for (int j8 = 0; j8 < 32; j8 += 8)
-                        *reinterpret_cast<uint4*>(dst + tc::u_off(i, j8 >> 3)) =
-                            make_uint4(pack_bf16(__uint_as_float(r[j8]), __uint_as_float(r[j8 + 1])),
-                                       pack_bf16(__uint_as_float(r[j8 + 2]), __uint_as_float(r[j8 + 3])),
-                                       pack_bf16(__uint_as_float(r[j8 + 4]), __uint_as_float(r[j8 + 5])),
-                                       pack_bf16(__uint_as_float(r[j8 + 6]), __uint_as_float(r[j8 + 7])));
-                }
+            for (int j8 = 0; j8 < 32; j8 += 8) {   // W = exp(G_m) . W'
+                const float4 e0 = *reinterpret_cast<const float4*>(smem + E_GV + 512 + (col0 + j8) * 4);
+                const float4 e1 = *reinterpret_cast<const float4*>(smem + E_GV + 512 + (col0 + j8) * 4 + 16);
+                *reinterpret_cast<uint4*>(smem + E_V + (col0 >> 6) * 8192 + ptx::sw128_off(i, (col0 & 63) + j8)) =
+                    make_uint4(pack_bf16(__uint_as_float(r[j8]) * e0.x, __uint_as_float(r[j8 + 1]) * e0.y),
+                               pack_bf16(__uint_as_float(r[j8 + 2]) * e0.z, __uint_as_float(r[j8 + 3]) * e0.w),
+                               pack_bf16(__uint_as_float(r[j8 + 4]) * e1.x, __uint_as_float(r[j8 + 5]) * e1.y),
+                               pack_bf16(__uint_as_float(r[j8 + 6]) * e1.z, __uint_as_float(r[j8 + 7]) * e1.w));
             }
+            ptx::tmem_ld_32x32b_x32(tq + 128 + g * 32, r);
+            ptx::tmem_ld_wait();
+#pragma unroll
+            for (int j8 = 0; j8 < 32; j8 += 8)
+                *reinterpret_cast<uint4*>(smem + E_A + tc::ut_off(q4 * 32 + lane, g * 4 + (j8 >> 3))) =
+                    make_uint4(pack_bf16(__uint_as_float(r[j8]), __uint_as_float(r[j8 + 1])),
+                               pack_bf16(__uint_as_float(r[j8 + 2]), __uint_as_float(r[j8 + 3])),
+                               pack_bf16(__uint_as_float(r[j8 + 4]), __uint_as_float(r[j8 + 5])),
+                               pack_bf16(__uint_as_float(r[j8 + 6]), __uint_as_float(r[j8 + 7])));
         }
         ptx::fence_async_smem();
         ptx::tc_fence_before();
         if (timed_out) *abort_word = 1;
         ebar();
         if (te == kServiceThread) {
-            ptx::bulk_s2g(tile + tc::OFF_QW, smem + E_KI, 8192);
-            ptx::bulk_s2g(tile + tc::OFF_QW + tc::QW_HALF, smem + E_KI + 8192, 8192);
-            ptx::bulk_s2g(tile + tc::OFF_U, smem + E_A, 16384);
+            ptx::bulk_s2g(D.tile + tc::OFF_QW, smem + E_V, 8192);
+            ptx::bulk_s2g(D.tile + tc::OFF_QW + tc::QW_HALF, smem + E_V + 8192, 8192);
+            ptx::bulk_s2g(D.tile + tc::OFF_U, smem + E_A, 16384);
             ptx::bulk_commit();
-            pending_ready = D.ready;
-            pending_val = D.ready_val;
-            stores_pending = true;
+            if (kFused) ++cursor.done;
         }
         KT_MARK(te == 0, 8);   // epilogue
 #ifdef KDA_FUSED_TIMING
@@ -948,11 +855,8 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
     if (timed_out) report_timeout(f, 10);
     if (out_of_range) atomicOr(&f.hdr->flags, 1);
     if (te == kServiceThread) {
+        if (kFused && !timed_out && !*abort_word) publish();
         ptx::bulk_wait_all0();   // shared memory must outlive the reads of every bulk store
-        if (kFused && pending_ready && !timed_out && !*abort_word) {
-            ptx::fence_proxy_async_all();
-            ptx::st_release_gpu(pending_ready, pending_val);
-        }
     }
     ptx::cp_async_wait_all();
     // an aborted engine may still have a TMA load in flight (requested for a tile it never started)
@@ -967,86 +871,44 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 }
 
 // ====================================================================================================
-// inter-chunk chain: a whole CTA (t = 0..511), 384 TMEM columns at tmem_c
-//   warps 0-7  compute: TMEM lane quadrant = warp & 3 (token row for V_new / O, dk row for the state),
-//              32-column half of the slice = warp >> 2
-//   warps 8-9  lane 0 of each issues MMAs;  warp 10 lane 0 requests the operand copies
+// inter-chunk chain: a whole CTA (t = 0..511), all 512 TMEM columns
 // ====================================================================================================
-__device__ __forceinline__ uint32_t pack2(float a, float b) {
-    __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&p);
+// Everything is transposed: TMEM lanes are the 128 columns of the state (dv), so that the state and V_new are A
+// operands in TMEM and nothing on the chain goes through shared memory:
+//   MMA1  D1[dv][0:64] = (W S)^T, D1[dv][64:128] = (Gamma.Q S)^T     A = bf16 state, B = [W ; Q]
+//   V_new^T = U^T - D1[:, 0:64]  -> bf16 -> TMEM
+//   MMA2  D3[dv][dk] = (K'^T V_new)^T,  D1[dv][64:128] += (Aqk V_new)^T            A = V_new, B = K', Aqk
+//   S <- gamma^C . S + exp(G_C - G_m) . D3  (fp32, in registers: thread = column, half of dk)  -> bf16 -> TMEM
+// A step is two dependent round trips tensor core -> registers -> tensor core (with the operands written to shared
+// memory with lanes = dk for all 128 columns: 32 + 16 KB a step, a proxy fence in each trip: 2.3 us a step).
+//   warps 0-7  compute: TMEM lane quadrant = warp & 3, half of dk / of the tokens = warp >> 2
+//   warp 8 issues the MMAs, warp 9 lane 0 loads the tiles, warps 12-15 write the output rows
+// kRing: tiles come from the engines of the cluster; otherwise from the plain array that the intra-chunk kernel
+// has written, and `cid` numbers the (sequence, head) pairs.
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
-// 32 fp32 values as bf16 into row `row` (four 16-byte chunks starting at chunk `c0`) of an MN-major
-// operand image with 128-byte rows and 128-byte swizzle
-__device__ __forceinline__ void store_row32(uint8_t* img, int row, int c0, const float (&x)[32]) {
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-        *reinterpret_cast<uint4*>(img + row * 128 + (((c0 + c) ^ (row & 7)) << 4)) =
-            make_uint4(pack2(x[8 * c], x[8 * c + 1]), pack2(x[8 * c + 2], x[8 * c + 3]),
-                       pack2(x[8 * c + 4], x[8 * c + 5]), pack2(x[8 * c + 6], x[8 * c + 7]));
-}
-// sum of the two partial accumulators (NS columns apart in TMEM) of one matrix, 32 columns
-__device__ __forceinline__ void tmem_ld_sum32(uint32_t taddr, float (&acc)[32]) {
-#pragma unroll
-    for (int hb = 0; hb < 2; ++hb) {
-        uint32_t r[16], r2[16];
-        ptx::tmem_ld_32x32b_x16(taddr + hb * 16, r);
-        ptx::tmem_ld_32x32b_x16(taddr + NS + hb * 16, r2);
-        ptx::tmem_ld_wait();
-#pragma unroll
-        for (int j = 0; j < 16; ++j) acc[hb * 16 + j] = __uint_as_float(r[j]) + __uint_as_float(r2[j]);
-    }
-}
+__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
-template <bool kHasQ>
-__device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_c, int t, int q, int slice)
+template <bool kHasQ, bool kLayer, bool kRing>
+__device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t, int cid, const CUtensorMap* tm_o)
 {
     const ChunkArgs& a = f.a;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C_BAR);
-    uint64_t* fullA = bars;                  // [2] [W';Q'] landed
-    uint64_t* fullB = fullA + 2;             // [2] K', Aqk, U landed
-    uint64_t* fullG = fullB + 2;             // [3] gate vectors landed
-    uint64_t* emptyA = fullG + 3;            // [2] MMA1 done with the stage
-    uint64_t* emptyB = emptyA + 2;           // [2] MMA2 / output product and the U readers done with the stage
-    uint64_t* emptyG = emptyB + 2;           // [3] gate vectors read
-    uint64_t* mma1_bar = emptyG + 3;         // MMA1 of a chunk complete
-    uint64_t* mma2_bar = mma1_bar + 1;       // MMA2 of a chunk complete
-    uint64_t* out_bar = mma2_bar + 1;        // [2] output accumulator of a chunk complete (alternating)
-    uint64_t* sbf_ready = out_bar + 2;       // 8 warp arrivals: bf16 state copy written
-    uint64_t* vn_ready = sbf_ready + 1;      // 4 warp arrivals: V_new written
+    uint64_t* ready = reinterpret_cast<uint64_t*>(smem + C_BAR);   // [engine][depth] a ring position holds a tile
+    uint64_t* full = ready + 6 * kMaxDepth;  // [kStages] a tile has landed
+    uint64_t* empty = full + kStages;        // [kStages] and is no longer needed: last commit, 8 compute warps, output store
+    uint64_t* m1 = empty + kStages;          // MMA1 of a chunk complete
+    uint64_t* m2 = m1 + 1;                   // MMA2
+    uint64_t* out_bar = m2 + 1;              // [2] output accumulator complete (alternating)
+    uint64_t* o_done = out_bar + 2;          // [2] and read (4 warps)
+    uint64_t* s_ready = o_done + 2;          // state operand written (8 warps)
+    uint64_t* vn_ready = s_ready + 1;        // V_new operand written (8 warps)
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(vn_ready + 1);
-    uint8_t* sbf = smem + C_SBF;
-    uint8_t* vn = smem + C_VN;
-
-    const int warp = t >> 5, lane = t & 31;
-    const int col0 = slice * NS;
+    const int warp = ptx::warp_uniform(t >> 5), lane = t & 31;
     __nv_bfloat16* op = kHasQ ? reinterpret_cast<__nv_bfloat16*>(a.o) : nullptr;
-
-    if (t == 0) {
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            ptx::mbar_init(&fullA[s], 1);
-            ptx::mbar_init(&fullB[s], 1);
-            ptx::mbar_init(&emptyA[s], 2);    // one commit from each MMA-issuing thread
-            ptx::mbar_init(&emptyB[s], 6);    // two commits + the four warps that read U
-            ptx::mbar_init(&out_bar[s], 1);
-        }
-#pragma unroll
-        for (int s = 0; s < 3; ++s) {
-            ptx::mbar_init(&fullG[s], 1);
-            ptx::mbar_init(&emptyG[s], 8);    // the eight compute warps
-        }
-        ptx::mbar_init(mma1_bar, 2);
-        ptx::mbar_init(mma2_bar, 2);
-        ptx::mbar_init(sbf_ready, 8);
-        ptx::mbar_init(vn_ready, 4);
-        abort_flag[0] = 0;
-        abort_flag[1] = 0;   // s_ready
-        abort_flag[2] = 0;   // s_done
-        abort_flag[3] = 0;   // s_exit
-        ptx::fence_mbar_init();
-    }
-    __syncthreads();
 
     auto wait = [&](uint64_t* bar, uint32_t parity, int where) {
         if (*abort_flag) return;
@@ -1057,7 +919,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_c, in
             if ((++spins & 15u) == 0) {
                 if (*abort_flag) return;
                 if (call_aborted(f)) { *abort_flag = 1; return; }
-                if (ptx::globaltimer_ns() - t0 > f.a.wait_limit_ns) {
+                if (ptx::globaltimer_ns() - t0 > a.wait_limit_ns) {
                     *abort_flag = 1;
                     report_timeout(f, where);
                     return;
@@ -1065,392 +927,380 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_c, in
             }
         }
     };
-    // TMEM columns: D1 {parity 0,1} x {part 0,1} (NS each), then the two D3 parts
-    const uint32_t d1c = tmem_c, d3c = tmem_c + 4 * NS;
+    auto warp_arrive = [&](uint64_t* bar) {
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(bar);
+    };
+    JobInfo J;
+    auto next_job = [&](int r) { return kRing ? job_info(f, cid, r, J) : pass_job(f, cid, r, J); };
 
-    // two words the loader and the flag thread talk through (shared memory, CTA-scope ordering)
-    volatile uint32_t* s_ready = abort_flag + 1;   // chunks (running number) whose tiles are complete in the ring
-    volatile uint32_t* s_done = abort_flag + 2;    // progress value to publish for the engines
-    volatile uint32_t* s_exit = abort_flag + 3;    // the loader has finished
-    if (warp == 11) {
-        // ================= flag thread: all traffic with the flag words in global memory =================
-        // An acquire load or a release store at GPU scope costs of the order of a microsecond; done by
-        // the loader they would sit on the chain's path once per chunk.  This thread confirms tiles
-        // ahead of the loader (up to the ring depth) and publishes the loader's progress behind it.
+    if (warp == 9) {
+        // ================= loader =================
         if (lane == 0) {
-            unsigned long long* cw = f.consumed + q * kSlices + slice;
-            uint32_t pr = 0, published = 0;
-            int r = 0, c = 0;
-            bool jobs_left = r * f.Q + q < f.J;
-            RoundInfo R = {0, 1};
-            JobInfo J = {};
-            auto load_job = [&]() {
-                while (jobs_left) {
-                    R = round_info(f, r);
-                    J = job_info(f, r * f.Q + q);
-                    if (J.nch > 0) break;
-                    ++r;
-                    jobs_left = r * f.Q + q < f.J;
-                }
-                c = 0;
+            if (!kRing) ptx::grid_dep_wait();   // the tiles come from the intra-chunk kernel launched just before
+            // (kRing) a position is given back this many tiles later, when its copy has landed for certain
+            const uint32_t lag = f.n_eng * f.depth >= 3 ? 2 : 0;   // (less than the number of positions)
+            uint32_t g = 0;
+            const uint32_t base = ptx::smem_u32(smem);
+            auto give_back = [&](uint32_t x) {
+                wait(&full[x % kStages], (x / kStages) & 1u, 31);
+                const uint32_t e = x % (uint32_t)f.n_eng, slot = (x / (uint32_t)f.n_eng) % (uint32_t)f.depth;
+                ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(base + (e & 1u) * E_BYTES + E_BAR + 48 + slot * 8, 1 + (e >> 1)));
             };
-            load_job();
-            uint64_t t0 = 0;
-            while (!*abort_flag) {
-                bool progressed = false;
-                if (jobs_left) {
-                    const int pos = q * f.R + c % f.R;
-                    const uint32_t idx = R.base + (uint32_t)c * (uint32_t)R.Qr + (uint32_t)q;
-                    if (ptx::ld_acquire_gpu(f.ready + pos) == tag(f.epoch, idx + 1u)) {
-                        ++pr;
-                        __threadfence_block();
-                        *s_ready = pr;
-                        progressed = true;
-                        if (++c == J.nch) {
-                            ++r;
-                            jobs_left = r * f.Q + q < f.J;
-                            load_job();
-                        }
-                    }
-                }
-                const uint32_t d = *s_done;
-                if (d != published) {
-                    __threadfence_block();
-                    ptx::st_release_gpu(cw, tag(f.epoch, d));
-                    published = d;
-                    progressed = true;
-                }
-                if (progressed) {
-                    t0 = 0;
-                } else {
-                    if (*s_exit && *s_done == published) break;
-                    if (t0 == 0) t0 = ptx::globaltimer_ns();
-                    if (call_aborted(f)) { *abort_flag = 1; break; }
-                    if (jobs_left && ptx::globaltimer_ns() - t0 > f.a.wait_limit_ns) {
-                        *abort_flag = 1;
-                        report_timeout(f, 30);
-                        break;
-                    }
-                    ptx::nanosleep(32);
-                }
-            }
-        }
-    } else if (warp == 10) {
-        // ================= loader: one thread requests every piece as early as its buffer frees up =======
-        if (lane == 0) {
-            uint32_t p = 0;                       // running chunk number of this chain role
-            uint32_t nG = 0, nA = 0, nB = 0;      // pieces requested so far
-            // production index + 1 of the last two chunks; a chunk counts as consumed (its ring
-            // position may be overwritten) once its copies have landed, which is certain when the
-            // stage it went to is free again, i.e. two chunks later.  A ring of fewer than four
-            // positions cannot afford that lag: there the landing is waited for.
-            uint32_t done1 = 0, done2 = 0;
-            const bool lazy = f.R >= 4;
-            KT_DECL(6);
-            auto landed = [&](uint32_t pp) {
-                wait(&fullG[pp % 3], (pp / 3) & 1u, 31);
-                wait(&fullA[pp & 1], (pp >> 1) & 1u, 32);
-                wait(&fullB[pp & 1], (pp >> 1) & 1u, 33);
-            };
-            for (int r = 0; r * f.Q + q < f.J && !*abort_flag; ++r) {
-                const RoundInfo R = round_info(f, r);
-                const JobInfo J = job_info(f, r * f.Q + q);
-                const uint32_t p0 = p;
-                for (int c = 0; c < J.nch && !*abort_flag; ++c, ++p) {
-                    const int pos = q * f.R + c % f.R;
-                    const char* tile = f.ring + (size_t)pos * tc::TILE_BYTES;
-                    const uint32_t idx = R.base + (uint32_t)c * (uint32_t)R.Qr + (uint32_t)q;
-                    KT_MARK(true, 0);
-                    {   // the engines have completed the tile (confirmed by the flag thread)
-                        uint64_t t0 = 0;
-                        while (*s_ready <= p) {
-                            if (t0 == 0) t0 = ptx::globaltimer_ns();
-                            if (*abort_flag) break;
-                            if (ptx::globaltimer_ns() - t0 > 2 * f.a.wait_limit_ns) {   // (the flag thread gives up first)
-                                *abort_flag = 1;
-                                report_timeout(f, 37);
-                                break;
-                            }
-                        }
-                        if (*abort_flag) break;
-                        __threadfence_block();
-                        ptx::fence_proxy_async_all();
-                    }
-                    KT_MARK(true, 1);   // tile ready
-                    const uint32_t s2 = p & 1, s3 = p % 3;
-                    uint8_t* sb = smem + s2 * C_STAGE;
-                    wait(&emptyG[s3], ((p / 3) & 1u) ^ 1u, 34);
-                    if (*abort_flag) break;
-                    ptx::mbar_expect_tx(&fullG[s3], tc::GV_BYTES);
-                    ptx::bulk_g2s(smem + C_GV + s3 * tc::GV_BYTES, tile + tc::OFF_GV, tc::GV_BYTES, &fullG[s3]);
-                    ++nG;
-                    wait(&emptyA[s2], ((p >> 1) & 1u) ^ 1u, 35);
-                    if (*abort_flag) break;
-                    if (kHasQ) {
-                        ptx::mbar_expect_tx(&fullA[s2], 32768);
-                        ptx::bulk_g2s(sb + C_QW, tile + tc::OFF_QW, 32768, &fullA[s2]);
-                    } else {   // state-only call: only the W' rows exist
-                        ptx::mbar_expect_tx(&fullA[s2], 16384);
-                        ptx::bulk_g2s(sb + C_QW, tile + tc::OFF_QW, 8192, &fullA[s2]);
-                        ptx::bulk_g2s(sb + C_QW + tc::QW_HALF, tile + tc::OFF_QW + tc::QW_HALF, 8192, &fullA[s2]);
-                    }
-                    ++nA;
-                    wait(&emptyB[s2], ((p >> 1) & 1u) ^ 1u, 36);
-                    if (*abort_flag) break;
-                    ptx::mbar_expect_tx(&fullB[s2], (kHasQ ? 24576u : 16384u) + C_UBYTES);
-                    ptx::bulk_g2s(sb + C_KT, tile + tc::OFF_KI, kHasQ ? 24576u : 16384u, &fullB[s2]);
-                    ptx::bulk_g2s(sb + C_U, tile + tc::OFF_U + (size_t)slice * C_UBYTES, C_UBYTES, &fullB[s2]);
-                    ++nB;
-                    KT_MARK(true, 2);   // buffers free + requests
-                    if (lazy) {
-                        // stage s2 was free: the chunk that used it two steps ago (if of this job) has landed
-                        if (p >= p0 + 2) *s_done = done2;
-                    } else if (p > p0) {
-                        landed(p - 1);
-                        if (!*abort_flag) *s_done = done1;
-                    }
-                    done2 = done1;
-                    done1 = idx + 1u;
-                    KT_MARK(true, 3);   // progress handed to the flag thread
-                }
-                if (*abort_flag) break;
-                // the job is over for this slice: once its last copies have landed, everything of this
-                // round counts as consumed
-                if (p > p0) landed(p - 1);
-                if (p > p0 + 1) landed(p - 2);
-                if (!*abort_flag) *s_done = (r + 1 < f.n_rounds) ? round_info(f, r + 1).base : f.n_prod;
-            }
-            __threadfence_block();
-            *s_exit = 1;
-            KT_FLUSH(true, f.hdr, 24, 4);
-            if (*abort_flag) {
-                // drain: the copies already requested must land before the shared memory goes away
-                // (bounded waits without the abort short-cut; a completed phase returns at once)
-                for (uint32_t pp = (nG > 3 ? nG - 3 : 0); pp < nG; ++pp)
-                    ptx::mbar_wait(&fullG[pp % 3], (pp / 3) & 1u, f.a.wait_limit_ns / 8);
-                for (uint32_t pp = (nA > 2 ? nA - 2 : 0); pp < nA; ++pp)
-                    ptx::mbar_wait(&fullA[pp & 1], (pp >> 1) & 1u, f.a.wait_limit_ns / 8);
-                for (uint32_t pp = (nB > 2 ? nB - 2 : 0); pp < nB; ++pp)
-                    ptx::mbar_wait(&fullB[pp & 1], (pp >> 1) & 1u, f.a.wait_limit_ns / 8);
-            }
-        }
-    } else if (warp == 8 || warp == 9) {
-        // ================= control warps: lane 0 of each issues MMAs =================
-        // Issuing one tcgen05.mma costs the issuing thread several tens of cycles whatever the tile
-        // size, and both products on the sequential chain are small, so each is split along its
-        // summation index between the two control threads, into one accumulator each; the
-        // accumulators are added when they are read back.  The first thread also issues the output
-        // product.
-        const int half = warp - 8;
-        if (lane == 0) {
-            const uint32_t idesc = ptx::umma_idesc_bf16(128, NS) | ptx::kIdescBMajorMN;
-            const uint32_t sbf_a = ptx::smem_u32(sbf), vn_a = ptx::smem_u32(vn);
-            uint32_t g = 0, last_out = 0;
-            bool any_out = false;
-            KT_DECL(8);
-            for (int r = 0; r * f.Q + q < f.J && !*abort_flag; ++r) {
-                const JobInfo J = job_info(f, r * f.Q + q);
+            KT_DECL(4);
+            for (int r = 0; next_job(r) && !*abort_flag; ++r)
                 for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
-                    const uint32_t s2 = g & 1;
-                    const uint32_t sb = ptx::smem_u32(smem + s2 * C_STAGE);
-                    const uint32_t d1 = d1c + (uint32_t)((g & 1) * 2 + half) * NS;
-                    // MMA1(g): D1 = [W' ; Q'] (exp(G_m) . S), this thread's half of the sum over dk
-                    KT_MARK(half == 0, 0);
-                    wait(&fullA[s2], (g >> 1) & 1u, 1);
-                    KT_MARK(half == 0, 1);   // operands A
-                    wait(sbf_ready, g & 1u, 4);
-                    KT_MARK(half == 0, 2);   // state copy
-                    ptx::tc_fence_after();
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int kk = half * 4 + k;   // 16-wide step of the sum over dk
-                        ptx::umma_bf16(d1, ptx::umma_desc_sw128(sb + C_QW + (kk >> 2) * tc::QW_HALF + (kk & 3) * 32),
-                                       ptx::umma_desc_sw128_mn(sbf_a + kk * 2048, 8192), idesc, k > 0);
+                    const uint32_t e = g % (uint32_t)f.n_eng, m = g / (uint32_t)f.n_eng;
+                    const uint32_t slot = m % (uint32_t)f.depth, s = g % kStages;
+                    const char* tile = kRing ? f.ring + (size_t)(((uint32_t)cid * f.n_eng + e) * f.depth + slot) * tc::TILE_BYTES
+                                             : f.ring + (size_t)(J.tile0 + (int64_t)c * a.H) * tc::TILE_BYTES;
+                    KT_MARK(true, 0);
+                    if (kRing) wait(&ready[e * (uint32_t)f.depth + slot], (m / (uint32_t)f.depth) & 1u, 30);
+                    KT_MARK(true, 1);
+                    if (g >= kStages) wait(&empty[s], (g / kStages - 1) & 1u, 32);
+                    if (*abort_flag) break;
+                    KT_MARK(true, 2);
+                    uint8_t* sb = smem + s * C_STAGE;
+                    if (kHasQ) {
+                        ptx::mbar_expect_tx(&full[s], tc::TILE_BYTES);
+                        ptx::bulk_g2s(sb, tile, tc::TILE_BYTES, &full[s]);
+                    } else {   // state-only call: only the W rows exist, and no Aqk
+                        ptx::mbar_expect_tx(&full[s], 8192 + 8192 + 16384 + tc::GV_BYTES + 16384);
+                        ptx::bulk_g2s(sb, tile, 8192, &full[s]);
+                        ptx::bulk_g2s(sb + tc::QW_HALF, tile + tc::QW_HALF, 8192, &full[s]);
+                        ptx::bulk_g2s(sb + tc::OFF_KI, tile + tc::OFF_KI, 16384, &full[s]);
+                        ptx::bulk_g2s(sb + tc::OFF_GV, tile + tc::OFF_GV, tc::GV_BYTES + 16384, &full[s]);
                     }
-                    ptx::umma_commit(mma1_bar);
-                    ptx::umma_commit(&emptyA[s2]);
-                    KT_MARK(half == 0, 3);   // MMA1 issue
-                    // MMA2(g): D3 = K'^T V_new (K' token-major = MN-major A operand), this thread's half of
-                    // the sum over the chunk's tokens; the state product sits on the sequential chain, so it
-                    // is issued and committed first
-                    wait(vn_ready, g & 1u, 5);
-                    KT_MARK(half == 0, 4);   // V_new
-                    wait(&fullB[s2], (g >> 1) & 1u, 6);
-                    KT_MARK(half == 0, 5);   // operands B
-                    ptx::tc_fence_after();
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        const int kk = half * 2 + k;   // 16-wide step of the sum over tokens
-                        ptx::umma_bf16(d3c + half * NS,
-                                       ptx::umma_desc_sw128_mn(sb + C_KT + kk * 2048, tc::KI_HALF),
-                                       ptx::umma_desc_sw128_mn(vn_a + kk * 2048, 8192), idesc | ptx::kIdescAMajorMN,
-                                       k > 0);
-                    }
-                    ptx::umma_commit(mma2_bar);
-                    if (half == 0 && op) {
-                        // D1[64:128] += Aqk V_new.  The 128-row A operand starts 64 rows before Aqk: those
-                        // rows (the tail of the K' image) only touch accumulator rows 0-63, which are dead
-                        // once V_new has been taken.
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            ptx::umma_bf16(d1, ptx::umma_desc_sw128(sb + C_AQ - 8192 + k * 32),
-                                           ptx::umma_desc_sw128_mn(vn_a + k * 2048, 8192), idesc, 1);
-                        ptx::umma_commit(&out_bar[g & 1]);
-                        last_out = g;
-                        any_out = true;
-                    }
-                    ptx::umma_commit(&emptyB[s2]);
-                    KT_MARK(half == 0, 6);   // MMA2 + output issue
-#ifdef KDA_FUSED_TIMING
-                    kt_acc_[7] += 16;
-#endif
+                    if (kRing && g >= lag) give_back(g - lag);
                 }
-            }
-            KT_FLUSH(half == 0, f.hdr, 16, 8);
-            // every MMA of this thread has completed before the TMEM goes away
-            if (half == 0 && any_out) wait(&out_bar[last_out & 1], (last_out >> 1) & 1u, 7);
-            else if (g > 0) wait(&emptyB[(g - 1) & 1], ((g - 1) >> 1) & 1u, 8);
+            KT_FLUSH(true, f.hdr, 24, 3);
+            if (*abort_flag)   // the copies already requested must land before the shared memory goes away
+                for (uint32_t x = g > kStages ? g - kStages : 0; x < g; ++x)
+                    ptx::mbar_wait(&full[x % kStages], (x / kStages) & 1u, a.wait_limit_ns / 8);
         }
+    } else if (warp == 8) {
+        // ================= MMA issue =================
+        const uint32_t id1 = ptx::umma_idesc_bf16(128, kHasQ ? 128 : 64), ido = ptx::umma_idesc_bf16(128, 64);
+        const uint32_t id2 = ptx::umma_idesc_bf16(128, 128) | ptx::kIdescBMajorMN;
+        const uint32_t base = (uint32_t)ptx::warp_uniform((int)ptx::smem_u32(smem));
+        uint32_t g = 0;
+        KT_DECL(8);
+        for (int r = 0; next_job(r) && !*abort_flag; ++r)
+            for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
+                const uint32_t s = g % kStages, sb = base + s * C_STAGE;
+                const uint32_t d1 = tm + T_D1 + (g & 1u) * 128u;
+                KT_MARK(lane == 0, 0);
+                wait(&full[s], (g / kStages) & 1u, 1);
+                KT_MARK(lane == 0, 1);   // operands
+                if (op && g >= 2) wait(&o_done[g & 1u], ((g >> 1) - 1) & 1u, 2);
+                wait(s_ready, g & 1u, 3);
+                __syncwarp();
+                KT_MARK(lane == 0, 2);   // state
+                ptx::tc_fence_after();
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    ptx::umma_bf16_ta(d1, tm + T_S + k * 8, ptx::umma_desc_sw128(sb + tc::OFF_QW + (k >> 2) * tc::QW_HALF + (k & 3) * 32),
+                                      id1, k > 0);
+                ptx::umma_commit(m1);
+                KT_MARK(lane == 0, 3);   // MMA1 issue
+                wait(vn_ready, g & 1u, 4);
+                __syncwarp();
+                KT_MARK(lane == 0, 4);   // V_new
+                ptx::tc_fence_after();
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    ptx::umma_bf16_ta(tm + T_D3, tm + T_VN + k * 8, ptx::umma_desc_sw128_mn(sb + tc::OFF_KI + k * 2048, tc::KI_HALF),
+                                      id2, k > 0);
+                ptx::umma_commit(m2);
+                if (op) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        ptx::umma_bf16_ta(d1 + 64, tm + T_VN + k * 8, ptx::umma_desc_sw128(sb + tc::OFF_AQ + k * 32), ido, 1);
+                    ptx::umma_commit(&out_bar[g & 1u]);
+                }
+                ptx::umma_commit(&empty[s]);
+                KT_MARK(lane == 0, 5);   // MMA2 + output issue
+            }
+        KT_FLUSH(lane == 0, f.hdr, 16, 6);
+        // every MMA has completed before the TMEM goes away
+        if (g > 0) wait(&empty[(g - 1) % kStages], ((g - 1) / kStages) & 1u, 5);
     } else if (warp < 8) {
         // ================= compute warps =================
-        const int quad = warp & 3, ch = warp >> 2;       // TMEM lane quadrant, 32-column half of the slice
-        const int tid = quad * 32 + lane;                // 0..127: token row for V_new / O, dk row for the state
-        const uint32_t tmem_lane = ((uint32_t)(quad * 32) << 16) + (uint32_t)ch * 32;
-        auto warp_arrive = [&](uint64_t* bar) {
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(bar);
-        };
-        float S[32];
+        const int quad = warp & 3, half = warp >> 2, dv = quad * 32 + lane, dk0 = half * 64;
+        const uint32_t tq = tm + ((uint32_t)(quad * 32) << 16);
+        float S[64];
+#pragma unroll
+        for (int i = 0; i < 64; ++i) S[i] = 0.f;
         uint32_t g = 0;
-        for (int r = 0; r * f.Q + q < f.J; ++r) {
-            const JobInfo J = job_info(f, r * f.Q + q);
-            const size_t sbase = ((size_t)J.n * a.H + J.h) * (size_t)(kD * kD) + (size_t)tid * kD + col0 + ch * 32;
+        KT_DECL(8);
+        for (int r = 0; next_job(r); ++r) {
+            const size_t sbase = ((size_t)J.n * a.H + J.h) * (size_t)(kD * kD) + (size_t)dk0 * kD + dv;
 #pragma unroll
-            for (int j = 0; j < 32; j += 4) {
-                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (a.S_in) x = *reinterpret_cast<const float4*>(a.S_in + sbase + j);
-                S[j] = x.x; S[j + 1] = x.y; S[j + 2] = x.z; S[j + 3] = x.w;
-            }
-            auto ref_scale_of = [&](uint32_t gg) {   // exp(G_m) of the chunk with running number gg
-                wait(&fullG[gg % 3], (gg / 3) & 1u, 8);
-                return reinterpret_cast<const float*>(smem + C_GV + (gg % 3) * tc::GV_BYTES + 512)[tid];
-            };
-            auto store_scaled = [&](float cgn) {
-                float z[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) z[j] = cgn * S[j];
-                store_row32(sbf, tid, ch * 4, z);
-            };
+            for (int i = 0; i < 64; ++i) S[i] = a.S_in ? a.S_in[sbase + (size_t)i * kD] : 0.f;
             if (J.nch > 0) {
-                store_scaled(ref_scale_of(g));
-                ptx::fence_async_smem();
-                warp_arrive(sbf_ready);
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    uint32_t z[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) z[i] = pack_bf16(S[b * 32 + 2 * i], S[b * 32 + 2 * i + 1]);
+                    ptx::tmem_st_32x32b_x16(tq + T_S + half * 32 + b * 16, z);
+                }
+                ptx::tmem_st_wait();
+                ptx::tc_fence_before();
+                warp_arrive(s_ready);
             }
             for (int c = 0; c < J.nch; ++c, ++g) {
-                const uint32_t s2 = g & 1, par = g & 1u;
-                const uint8_t* sb = smem + s2 * C_STAGE;
-                const uint32_t d1 = d1c + tmem_lane + (uint32_t)(g & 1) * 2 * NS;
-                if (quad < 2) {   // a6: V_new = U - W S  (token row = tid)
-                    wait(&fullB[s2], (g >> 1) & 1u, 1);
-                    uint4 uq[4];   // this token's 32 values of U
+                const uint32_t s = g % kStages;
+                const uint8_t* sb = smem + s * C_STAGE;
+                const bool more = c + 1 < J.nch;
+                // four values of a gate vector of the chunk (0: gamma^C, 1: exp(G_C - G_m))
+                auto vec = [&](int which, int i) {
+                    return *reinterpret_cast<const float4*>(sb + tc::OFF_GV + which * 512 + (dk0 + i) * 4);
+                };
+                KT_MARK(t == 0, 0);
+                wait(&full[s], (g / kStages) & 1u, 6);
+                KT_MARK(t == 0, 1);
+                {   // V_new^T = U^T - (W S)^T: column dv, tokens 32 half ..
+                    uint4 uq[4];
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc)
-                        uq[cc] = *reinterpret_cast<const uint4*>(sb + C_U + ch * tc::U_BLOCK + tc::u_off(tid, cc));
-                    warp_arrive(&emptyB[s2]);
-                    const __nv_bfloat16* U = reinterpret_cast<const __nv_bfloat16*>(uq);
-                    wait(mma1_bar, par, 2);
+                    for (int k = 0; k < 4; ++k)
+                        uq[k] = *reinterpret_cast<const uint4*>(sb + tc::OFF_U + tc::ut_off((uint32_t)dv, (uint32_t)(half * 4 + k)));
+                    const uint32_t* u = reinterpret_cast<const uint32_t*>(uq);
+                    wait(m1, g & 1u, 7);
+                    __syncwarp();
+                    KT_MARK(t == 0, 2);
                     ptx::tc_fence_after();
-                    float x[32];
-                    tmem_ld_sum32(d1, x);
+                    uint32_t y[32], z[16];
+                    ptx::tmem_ld_32x32b_x32(tq + T_D1 + (g & 1u) * 128u + half * 32, y);
+                    ptx::tmem_ld_wait();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) x[j] = __bfloat162float(U[j]) - x[j];
-                    store_row32(vn, tid, ch * 4, x);
-                    ptx::fence_async_smem();
+                    for (int i = 0; i < 16; ++i)
+                        z[i] = pack_bf16(bf16_lo(u[i]) - __uint_as_float(y[2 * i]), bf16_hi(u[i]) - __uint_as_float(y[2 * i + 1]));
+                    ptx::tmem_st_32x32b_x16(tq + T_VN + half * 16, z);
+                    ptx::tmem_st_wait();
                     ptx::tc_fence_before();
                     warp_arrive(vn_ready);
                 }
-                wait(&fullG[g % 3], (g / 3) & 1u, 9);
-                const float* gv = reinterpret_cast<const float*>(smem + C_GV + (g % 3) * tc::GV_BYTES);
-                const float gc = gv[tid];          // gamma^C
-                const float ct = gv[256 + tid];    // exp(G_C - G_m)
-                const bool more = c + 1 < J.nch;
-                const float cgn = more ? ref_scale_of(g + 1) : 0.f;   // fetched off the chain, before the wait below
-                warp_arrive(&emptyG[g % 3]);
-                // S_new = gc . S + ct . D3; the part that does not need D3 is formed before the wait.  (The
-                // scales are applied one after the other: ct . D3 is of ordinary size although ct can be
-                // e^-80 and D3 e^+80, whereas a pre-multiplied cgn * ct would underflow.)
+                KT_MARK(t == 0, 3);
+                // S_new = gamma^C . S + exp(G_C - G_m) . D3; the part that does not need D3 comes before the wait
 #pragma unroll
-                for (int j = 0; j < 32; ++j) S[j] *= gc;
-                wait(mma2_bar, par, 3);
+                for (int i = 0; i < 64; i += 4) {
+                    const float4 e = vec(0, i);
+                    S[i] *= e.x; S[i + 1] *= e.y; S[i + 2] *= e.z; S[i + 3] *= e.w;
+                }
+                KT_MARK(t == 0, 4);
+                wait(m2, g & 1u, 9);
+                __syncwarp();
+                KT_MARK(t == 0, 5);
                 ptx::tc_fence_after();
-                {   // a8: S <- gamma^C . S + exp(G_C - G_m) . (K'^T V_new) ; refresh the bf16 operand copy
-                    float ds[32];
-                    tmem_ld_sum32(d3c + tmem_lane, ds);
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) S[j] = fmaf(ct, ds[j], S[j]);
-                    if (more) {
-                        store_scaled(cgn);   // next chunk's operand copy: bf16(exp(G_m') . S_new)
-                        ptx::fence_async_smem();
-                    }
-                    ptx::tc_fence_before();
-                    if (more) warp_arrive(sbf_ready);
-                }
-                if (quad >= 2 && op) {   // a7: O = (Gamma.Q) S + Aqk V_new  (token row = tid - 64)
-                    const int i = tid - 64;
-                    const int64_t tok0 = J.tok_begin + (int64_t)c * kC;
-                    const int len = (J.tok_end - tok0) < kC ? (int)(J.tok_end - tok0) : kC;
-                    __nv_bfloat16* orow = op + ((tok0 + i) * a.H + J.h) * kD + col0 + ch * 32;
-                    wait(&out_bar[g & 1], (g >> 1) & 1u, 6);
-                    ptx::tc_fence_after();
-                    float ov[32];
-                    tmem_ld_sum32(d1, ov);
-                    if (i < len && !*abort_flag) {
+                for (int b = 0; b < 4; ++b) {
+                    uint32_t y[16], z[8];
+                    ptx::tmem_ld_32x32b_x16(tq + T_D3 + dk0 + b * 16, y);
+                    float4 ct[4];      // (fetched while the accumulator is)
 #pragma unroll
-                        for (int j = 0; j < 32; j += 8)
-                            *reinterpret_cast<uint4*>(orow + j) =
-                                make_uint4(pack2(ov[j], ov[j + 1]), pack2(ov[j + 2], ov[j + 3]),
-                                           pack2(ov[j + 4], ov[j + 5]), pack2(ov[j + 6], ov[j + 7]));
+                    for (int i = 0; i < 4; ++i) ct[i] = vec(1, b * 16 + 4 * i);
+                    ptx::tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 16; i += 4) {
+                        float* s4 = &S[b * 16 + i];
+                        const float4 e = ct[i / 4];
+                        const float2 lo = __ffma2_rn(make_float2(e.x, e.y), make_float2(__uint_as_float(y[i]), __uint_as_float(y[i + 1])),
+                                                     make_float2(s4[0], s4[1]));
+                        const float2 hi = __ffma2_rn(make_float2(e.z, e.w), make_float2(__uint_as_float(y[i + 2]), __uint_as_float(y[i + 3])),
+                                                     make_float2(s4[2], s4[3]));
+                        s4[0] = lo.x; s4[1] = lo.y; s4[2] = hi.x; s4[3] = hi.y;
+                        z[i / 2] = pack_bf16(lo.x, lo.y);
+                        z[i / 2 + 1] = pack_bf16(hi.x, hi.y);
                     }
-                    ptx::tc_fence_before();
+                    if (more) ptx::tmem_st_32x32b_x8(tq + T_S + half * 32 + b * 8, z);
                 }
+                if (more) ptx::tmem_st_wait();
+                ptx::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if (more) ptx::mbar_arrive(s_ready);
+                    ptx::mbar_arrive(&empty[s]);
+                }
+                KT_MARK(t == 0, 6);
             }
             if (*abort_flag) break;
-            if (a.S_out) {
-                float* so = a.S_out + sbase;
+            if (a.S_out)
 #pragma unroll
-                for (int j = 0; j < 32; j += 4)
-                    *reinterpret_cast<float4*>(so + j) = make_float4(S[j], S[j + 1], S[j + 2], S[j + 3]);
-            }
+                for (int i = 0; i < 64; ++i) a.S_out[sbase + (size_t)i * kD] = S[i];
         }
+        KT_FLUSH(t == 0, f.hdr, 28, 7);
+    } else if (warp >= 12 && op) {
+        // ================= output rows =================
+        // The accumulator has a lane per column and a TMEM column per token; read as 8 x 8 fragments and stored with
+        // stmatrix.trans it becomes rows of the output, over the stage's [W ; Q] image (no longer needed), and
+        // leaves by two tiled TMA stores.  (Straight from the lanes, 64 two-byte stores a thread, the stores
+        // crowded out the loads of the compute warps: 2.6 instead of 1.6 us a step.)
+        const int quad = warp & 3, ot = t - 384;
+        const uint32_t tq = tm + ((uint32_t)(quad * 32) << 16);
+        float* ssq = reinterpret_cast<float*>(smem + C_SSQ);              // [2][64][4]
+        const bool epi = kLayer && a.out_gate != nullptr;
+        // this lane's row of the four 8 x 8 matrices of token block 0, in the swizzled [2][64 tokens][64] image
+        const uint32_t mrow = (uint32_t)(lane & 7), mcol = (uint32_t)((quad & 1) * 32 + (lane >> 3) * 8);
+        const uint32_t moff = (uint32_t)(quad >> 1) * 8192u + ptx::sw128_off(mrow, mcol);
+        float wgt[4] = {0.f, 0.f, 0.f, 0.f};     // RMSNorm weights of this lane's four columns
+        if (epi)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) wgt[b] = a.rms_weight[quad * 32 + b * 8 + (lane >> 2)];
+        uint32_t g = 0;
+        for (int r = 0; next_job(r) && !*abort_flag; ++r)
+            for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
+                const int64_t tok0 = J.tok_begin + (int64_t)c * kC;
+                const int len = (J.tok_end - tok0) < kC ? (int)(J.tok_end - tok0) : kC;
+                const uint32_t s = g % kStages;
+                uint8_t* sb = smem + s * C_STAGE;
+                uint4 gq[kLayer ? 8 : 1];        // gate pre-activations, 16-byte piece ot + 128 k of the [64][256 B] block
+                if (kLayer && epi)
+#pragma unroll
+                    for (int k = 0; k < (kLayer ? 8 : 0); ++k) {
+                        const int idx = ot + 128 * k, row = idx >> 4;
+                        gq[k] = make_uint4(0u, 0u, 0u, 0u);
+                        if (row < len)
+                            gq[k] = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(a.out_gate) +
+                                                                    ((size_t)(tok0 + row) * a.H + J.h) * kD + (idx & 15) * 8);
+                    }
+                wait(&out_bar[g & 1u], (g >> 1) & 1u, 10);
+                __syncwarp();
+                ptx::tc_fence_after();
+                // y[b >> 1][4 j + 2 (b & 1) + e]: column 8 b + lane / 4 of the quadrant, token 8 j + 2 (lane % 4) + e
+                uint32_t y[2][32];
+                ptx::tmem_ld_16x256b_x8(tq + T_D1 + (g & 1u) * 128u + 64, y[0]);
+                ptx::tmem_ld_16x256b_x8(tq + (16u << 16) + T_D1 + (g & 1u) * 128u + 64, y[1]);
+                ptx::tmem_ld_wait();
+                ptx::tc_fence_before();
+                warp_arrive(&o_done[g & 1u]);
+                if (kLayer && epi) {
+                    // the gate block next to the output block, the row sums of squares of this quadrant beside them
+#pragma unroll
+                    for (int k = 0; k < (kLayer ? 8 : 0); ++k) {
+                        const int idx = ot + 128 * k, ch = idx & 15;
+                        *reinterpret_cast<uint4*>(sb + 16384 + (ch >> 3) * 8192 + ptx::sw128_off((uint32_t)(idx >> 4), (uint32_t)(ch & 7) * 8)) = gq[k];
+                    }
+                    float q[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        q[i] = 0.f;
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) {
+                            const float v = __uint_as_float(y[b >> 1][4 * (i >> 1) + 2 * (b & 1) + (i & 1)]);
+                            q[i] = fmaf(v, v, q[i]);
+                        }
+                    }
+#pragma unroll
+                    for (int n = 8, x = 16; n >= 2; n >>= 1, x >>= 1) {   // over the eight lanes that share a token: two tokens each
+                        const bool up = (lane & x) != 0;
+#pragma unroll
+                        for (int i = 0; i < n; ++i) {
+                            const float send = up ? q[i] : q[i + n], keep = up ? q[i + n] : q[i];
+                            q[i] = keep + __shfl_xor_sync(0xffffffffu, send, x);
+                        }
+                    }
+                    // lane bits 4, 3, 2 have chosen the token block's bits 2, 1, 0
+                    const int jb = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+                    float* sq = ssq + (g & 1u) * 256;
+                    sq[(8 * jb + 2 * (lane & 3)) * 4 + quad] = q[0];
+                    sq[(8 * jb + 2 * (lane & 3) + 1) * 4 + quad] = q[1];
+                    ptx::named_bar_sync(5, 128);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        uint32_t gt[4];
+                        ptx::ldmatrix_x4_trans(sb + 16384 + moff + j * 1024, gt);
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const float4 p = *reinterpret_cast<const float4*>(sq + (8 * j + 2 * (lane & 3) + e) * 4);
+                            const float rstd = rsqrtf(((p.x + p.y) + (p.z + p.w)) * (1.f / kD) + a.rms_eps);
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) {
+                                uint32_t& v = y[b >> 1][4 * j + 2 * (b & 1) + e];
+                                const float gv = e ? bf16_hi(gt[b]) : bf16_lo(gt[b]);
+                                v = __float_as_uint(__uint_as_float(v) * (rstd * wgt[b]) * rcp_approx(1.f + __expf(-gv)));
+                            }
+                        }
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    uint32_t z[4];
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)
+                        z[b] = pack_bf16(__uint_as_float(y[b >> 1][4 * j + 2 * (b & 1)]), __uint_as_float(y[b >> 1][4 * j + 2 * (b & 1) + 1]));
+                    ptx::stmatrix_x4_trans(sb + moff + j * 1024, z);
+                }
+                ptx::fence_async_smem();
+                ptx::named_bar_sync(6, 128);
+                if (len == kC) {
+                    if (ot == 0 && !*abort_flag) {
+                        ptx::tma_store_2d(tm_o, sb, J.h * kD, (int)tok0);
+                        ptx::tma_store_2d(tm_o, sb + 8192, J.h * kD + 64, (int)tok0);
+                        ptx::bulk_commit();
+                        ptx::bulk_wait_read0();
+                    }
+                } else {       // the rows past the end of the sequence belong to the next one
+                    if (!*abort_flag)
+                        for (int idx = ot; idx < len * 16; idx += 128) {
+                            const int row = idx >> 4, ch = idx & 15;
+                            *reinterpret_cast<uint4*>(op + ((size_t)(tok0 + row) * a.H + J.h) * kD + ch * 8) =
+                                *reinterpret_cast<const uint4*>(sb + (ch >> 3) * 8192 + ptx::sw128_off((uint32_t)row, (uint32_t)(ch & 7) * 8));
+                        }
+                    ptx::named_bar_sync(6, 128);
+                }
+                if (ot == 0) ptx::mbar_arrive(&empty[s]);
+            }
+        if (ot == 0) ptx::bulk_wait_all0();
     }
     ptx::tc_fence_before();
     __syncthreads();
 }
 
-template <bool kHasQ>
+// barriers of a chain CTA; ONE thread
+__device__ void chain_init(uint8_t* smem, bool has_out)
+{
+    uint64_t* b = reinterpret_cast<uint64_t*>(smem + C_BAR);
+    for (int i = 0; i < 6 * kMaxDepth; ++i) ptx::mbar_init(b++, 1);   // ready
+    for (int i = 0; i < kStages; ++i) ptx::mbar_init(b++, 1);         // full
+    for (int i = 0; i < kStages; ++i) ptx::mbar_init(b++, has_out ? 10 : 9);   // empty
+    ptx::mbar_init(b++, 1);                                           // m1
+    ptx::mbar_init(b++, 1);                                           // m2
+    for (int i = 0; i < 2; ++i) ptx::mbar_init(b++, 1);               // out_bar
+    for (int i = 0; i < 2; ++i) ptx::mbar_init(b++, 4);               // o_done
+    ptx::mbar_init(b++, 8);                                           // s_ready
+    ptx::mbar_init(b++, 8);                                           // vn_ready
+    *reinterpret_cast<volatile uint32_t*>(b) = 0;                     // abort flag
+    ptx::fence_mbar_init();
+}
+
+// One cluster = a chain CTA (rank 0) and CTAs of two engines each; ring positions are handed over by
+// mbarriers in each other's shared memory.  The ring is written and read by bulk copies alone: an engine
+// announces a tile once its copies have completed (performed at L2, where the chain's copies read), the chain
+// gives a position back once its copy has landed.  Neither arrival has anything of its own thread to order, so
+// both are relaxed (release arrivals and proxy fences in their place cost about a microsecond each).
+template <bool kHasQ, bool kLayer>
 __global__ void __launch_bounds__(kThreads, 1)
 kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtensorMap tm_k,
              const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_v,
-             int clear_status)
+             const __grid_constant__ CUtensorMap tm_o)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     const int t = threadIdx.x, warp = t >> 5;
-    const bool chain_cta = (int)blockIdx.x < f.n_chain_cta;
+    // (from blockIdx and not from %cluster_ctarank: a branch that the compiler does not know to be uniform costs the
+    // MMA-issuing warps their uniform registers, 381 instead of 85 ns for the first product of a step)
+    const int cid = (int)blockIdx.x / f.cluster_size, rank = (int)blockIdx.x - cid * f.cluster_size;
+    const bool chain_cta = rank == 0;
     // (the TMEM slot sits in a spare word of the barrier block of either layout)
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + (chain_cta ? C_BAR + 248 : E_BAR + 32));
-
-    if (clear_status && blockIdx.x == 0 && t == 0) {
-        f.hdr->status = 0;      // (an equal-length call has no prologue kernel to do this)
-        f.hdr->where = 0;
-        f.hdr->flags = 0;
-    }
-    // barriers of the engines
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + (chain_cta ? C_BAR + 500 : E_BAR + 32));
+    if (chain_cta && t == 0) chain_init(smem, kHasQ && f.a.o != nullptr);
     if (!chain_cta && (t == 0 || t == kEngThreads)) {
         uint64_t* mb = reinterpret_cast<uint64_t*>(smem + (t ? E_BYTES : 0) + E_BAR);
-        ptx::mbar_init(mb, 2);       // MMA group complete (two issuing threads)
+        ptx::mbar_init(mb, 2);       // MMA group complete (two issuing warps)
         ptx::mbar_init(mb + 1, 1);   // k landed
         ptx::mbar_init(mb + 3, 1);   // q landed
         ptx::mbar_init(mb + 5, 1);   // v landed
+        for (int i = 0; i < kMaxDepth; ++i) ptx::mbar_init(mb + 6 + i, 1);   // ring positions free
         *reinterpret_cast<volatile uint32_t*>(mb + 2) = 0;
         ptx::fence_mbar_init();
         if (t == 0) {
@@ -1465,19 +1315,57 @@ kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     }
     ptx::tc_fence_before();
     __syncthreads();
+    ptx::cluster_sync_all();      // every CTA's barriers exist before anybody arrives on them
     ptx::tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
-    const bool aligned = (ptx::smem_u32(smem) & 1023u) == 0;   // the operand images need 1024-byte alignment
-    if (!aligned) {
+    ptx::grid_dep_wait();         // (launched before the preceding kernel has ended)
+    ptx::grid_dep_launch();
+    if (blockIdx.x == 0 && t == 0) {
+        f.hdr->status = 0;
+        f.hdr->where = 0;
+        f.hdr->flags = 0;
+    }
+    const uint32_t tmem_base = (uint32_t)ptx::warp_uniform((int)*tmem_slot);
+    if ((ptx::smem_u32(smem) & 1023u) != 0) {   // the operand images need 1024-byte alignment
         if (t == 0) report_timeout(f, 90);
     } else if (chain_cta) {
-        chain_run<kHasQ>(f, smem, tmem_base, t, (int)blockIdx.x / kSlices, (int)blockIdx.x % kSlices);
+        chain_run<kHasQ, kLayer, true>(f, smem, tmem_base, t, cid, &tm_o);
     } else {
-        // two engines per CTA
-        if (t < kEngThreads)
-            engine_run<kHasQ, true>(f, smem, tmem_base, 1, t, 0, 0, &tm_k, &tm_q, &tm_v);
-        else
-            engine_run<kHasQ, true>(f, smem + E_BYTES, tmem_base + 256, 2, t - kEngThreads, 0, 0, &tm_k, &tm_q, &tm_v);
+        const int sub = ptx::warp_uniform(t / kEngThreads), e = (rank - 1) * 2 + sub;
+        if (e < f.n_eng) {
+            uint8_t* es = smem + sub * E_BYTES;
+            if (t - sub * kEngThreads == kServiceThread)
+                *reinterpret_cast<EngineCursor*>(es + E_CUR) = {
+                    cid, e, 0, e, 0, ptx::map_to_cta(ptx::smem_u32(smem) + C_BAR + (uint32_t)(e * f.depth) * 8u, 0), 0, 0};
+            engine_run<kHasQ, true, kLayer>(f, es, tmem_base + sub * 256, 1 + sub, t - sub * kEngThreads, 0, 0, &tm_k, &tm_q, &tm_v);
+        }
+    }
+    ptx::tc_fence_before();
+    __syncthreads();
+    if (warp == 0) ptx::tmem_dealloc(tmem_base, kTmemCols);
+    ptx::cluster_sync_all();      // no CTA leaves while another may still arrive on its barriers
+}
+
+// ---- the chains alone (second kernel of the two-kernel schedule): a CTA per (sequence, head) -------------------
+template <bool kHasQ, bool kLayer>
+__global__ void __launch_bounds__(kThreads, 1)
+kda_chain_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtensorMap tm_o)
+{
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const int t = threadIdx.x, warp = t >> 5;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C_BAR + 500);
+    if (t == 0) chain_init(smem, kHasQ && f.a.o != nullptr);
+    if (warp == 0) {
+        ptx::tmem_alloc(tmem_slot, kTmemCols);
+        ptx::tmem_relinquish();
+    }
+    ptx::tc_fence_before();
+    __syncthreads();
+    ptx::tc_fence_after();
+    const uint32_t tmem_base = (uint32_t)ptx::warp_uniform((int)*tmem_slot);
+    if ((ptx::smem_u32(smem) & 1023u) != 0) {
+        if (t == 0) report_timeout(f, 90);
+    } else {
+        chain_run<kHasQ, kLayer, false>(f, smem, tmem_base, t, (int)blockIdx.x, &tm_o);
     }
     ptx::tc_fence_before();
     __syncthreads();
@@ -1520,7 +1408,7 @@ kda_intra_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = (uint32_t)ptx::warp_uniform((int)*tmem_slot);
     if ((ptx::smem_u32(smem) & 1023u) != 0) {
         if (t == 0) report_timeout(f, 90);   // the operand images need 1024-byte alignment
     } else {
@@ -1529,52 +1417,6 @@ kda_intra_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     ptx::tc_fence_before();
     __syncthreads();
     if (warp == 0) ptx::tmem_dealloc(tmem_base, 256);
-}
-
-// ---- prologue of a packed batch: status word + production-index base of every round ----------------------
-__global__ void kda_fused_prep_kernel(WsHeader* hdr, const int32_t* __restrict__ cu, uint32_t* __restrict__ round_base,
-                                      int n_seqs, int H, int Q, int n_rounds)
-{
-    // one CTA; thread i handles rounds i, i + blockDim.x, ...; a running offset chains the passes
-    __shared__ uint32_t s_part[1024];
-    __shared__ uint32_t s_carry;
-    const int t = threadIdx.x;
-    if (t == 0) {
-        hdr->status = 0;
-        hdr->where = 0;
-        hdr->flags = 0;
-        s_carry = 0;
-    }
-    __syncthreads();
-    const int J = n_seqs * H;
-    for (int r0 = 0; r0 < n_rounds; r0 += (int)blockDim.x) {
-        const int r = r0 + t;
-        uint32_t cnt = 0;
-        if (r < n_rounds) {
-            const int j0 = r * Q, j1 = (j0 + Q < J ? j0 + Q : J) - 1;
-            int maxlen = 0;
-            for (int n = j0 / H; n <= j1 / H; ++n) {
-                const int len = (cu[n + 1] - cu[n] + kC - 1) / kC;
-                maxlen = len > maxlen ? len : maxlen;
-            }
-            cnt = (uint32_t)maxlen * (uint32_t)(j1 - j0 + 1);
-        }
-        s_part[t] = cnt;
-        __syncthreads();
-        // inclusive scan (Hillis-Steele)
-        for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-            uint32_t v = 0;
-            if (t >= off) v = s_part[t - off];
-            __syncthreads();
-            s_part[t] += v;
-            __syncthreads();
-        }
-        if (r < n_rounds) round_base[r] = s_carry + s_part[t] - cnt;
-        __syncthreads();
-        if (t == (int)blockDim.x - 1) s_carry += s_part[t];
-        __syncthreads();
-    }
-    if (t == 0) round_base[n_rounds] = s_carry;
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry-point query (no link dependency on
@@ -1613,36 +1455,6 @@ kda_status_t make_tmap(CUtensorMap* tm, const void* base, int64_t total_tokens, 
 
 }  // namespace
 
-// [total_tokens, H*128] bf16 matrix, boxes of `rows` tokens x `cols` channels, no swizzle (rows of the
-// box land back to back); used for the output-gate blocks of the layer wrap
-kda_status_t make_plain_tmap(CUtensorMap* tm, const void* base, int64_t total_tokens, int H, int cols, int rows)
-{
-    EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return fail(KDA_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    const cuuint64_t dims[2] = {(cuuint64_t)H * kD, (cuuint64_t)total_tokens};
-    const cuuint64_t strides[1] = {(cuuint64_t)H * kD * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)cols, (cuuint32_t)rows};
-    const cuuint32_t estr[2] = {1, 1};
-    CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
-                    estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(KDA_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
-    return KDA_OK;
-}
-
-// (tc_tile_bytes is defined beside the two-kernel path)
-
-kda_status_t launch_fused_prep(WsHeader* hdr, const int32_t* cu_seqlens, uint32_t* round_base, int n_seqs,
-                               int H, int Q, int n_rounds, cudaStream_t st)
-{
-    ProfScope ps(PROF_PREP, st);
-    kda_fused_prep_kernel<<<1, 1024, 0, st>>>(hdr, cu_seqlens, round_base, n_seqs, H, Q, n_rounds);
-    count_launch();
-    KDA_CUDA_TRY(cudaGetLastError());
-    return KDA_OK;
-}
-
-// chain CTAs: kSlices per running (sequence, head); at least half of the SMs stay with the engines
 kda_status_t launch_intra_tc(const ChunkArgs& a, void* tiles, WsHeader* hdr, bool clear_status,
                              cudaStream_t st)
 {
@@ -1700,48 +1512,142 @@ kda_status_t launch_intra_tc(const ChunkArgs& a, void* tiles, WsHeader* hdr, boo
     return KDA_OK;
 }
 
-int fused_max_slots(int n_sm) { return n_sm / (2 * kSlices); }
-int fused_slices() { return kSlices; }
-
-kda_status_t launch_fused_tc(FusedArgs f, bool has_q, bool clear_status, cudaStream_t st)
+namespace {
+using FusedFn = void (*)(FusedArgs, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap);
+using ChainFn = void (*)(FusedArgs, CUtensorMap);
+FusedFn fused_fn(bool has_q, bool layer)
 {
-    int n_sm = 0;
-    {
-        DeviceLock lk;
-        if (!lk.st) return lk.rc;
-        if (lk.st->n_sm == 0) {
-            int dev = 0, coop = 0;
-            KDA_CUDA_TRY(cudaGetDevice(&dev));
-            KDA_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-            if (!coop) return fail(KDA_ERR_UNSUPPORTED, "the device does not support cooperative launches");
-            KDA_CUDA_TRY(cudaDeviceGetAttribute(&lk.st->n_sm, cudaDevAttrMultiProcessorCount, dev));
-        }
-        if (!lk.st->attr_done[0]) {
-            KDA_CUDA_TRY(cudaFuncSetAttribute(kda_fused_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (layer) return has_q ? kda_fused_tc<true, true> : kda_fused_tc<false, true>;
+    return has_q ? kda_fused_tc<true, false> : kda_fused_tc<false, false>;
+}
+ChainFn chain_fn(bool has_q, bool layer)
+{
+    if (layer) return has_q ? kda_chain_tc<true, true> : kda_chain_tc<false, true>;
+    return has_q ? kda_chain_tc<true, false> : kda_chain_tc<false, false>;
+}
+void fused_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[2], int cluster, int n_clusters, cudaStream_t st)
+{
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3((unsigned)(cluster * n_clusters));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+}
+}  // namespace
+
+// Resident clusters of 3 and of 4 CTAs on the current device (asked once per device).
+kda_status_t fused_max_clusters(int (&n)[2])
+{
+    DeviceLock lk;
+    if (!lk.st) return lk.rc;
+    if (!lk.st->attr_done[0]) {
+        for (int i = 0; i < 4; ++i)
+            KDA_CUDA_TRY(cudaFuncSetAttribute((const void*)fused_fn(i & 1, i & 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)kSmemBytes));
-            KDA_CUDA_TRY(cudaFuncSetAttribute(kda_fused_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)kSmemBytes));
-            lk.st->attr_done[0] = true;
+        for (int i = 0; i < 2; ++i) {
+            cudaLaunchConfig_t cfg;
+            cudaLaunchAttribute at[2];
+            fused_config(cfg, at, 3 + i, 1, nullptr);
+            cfg.numAttrs = 1;
+            int c = 0;
+            KDA_CUDA_TRY(cudaOccupancyMaxActiveClusters(&c, (const void*)fused_fn(true, false), &cfg));
+            lk.st->fused_clusters[i] = c;
         }
-        n_sm = lk.st->n_sm;
+        lk.st->attr_done[0] = true;
     }
+    n[0] = lk.st->fused_clusters[0];
+    n[1] = lk.st->fused_clusters[1];
+    return KDA_OK;
+}
+
+kda_status_t launch_fused_tc(const FusedArgs& f, bool has_q, cudaStream_t st)
+{
     if (f.a.total_tokens > 0x7fffffff)
         return fail(KDA_ERR_UNSUPPORTED, "kda_chunk_fwd: more than 2^31 tokens in one call");
-    CUtensorMap tm_k, tm_q, tm_v;
-    kda_status_t rc = make_tmap(&tm_k, f.a.k, f.a.total_tokens, f.a.H);
-    if (rc == KDA_OK) rc = make_tmap(&tm_v, f.a.v, f.a.total_tokens, f.a.H);
-    if (rc == KDA_OK) rc = make_tmap(&tm_q, has_q ? f.a.q : f.a.k, f.a.total_tokens, f.a.H);
+    const int64_t T = f.a.total_tokens > 0 ? f.a.total_tokens : 1;   // (a call of empty sequences loads nothing)
+    const void* any = f.a.k ? f.a.k : f.hdr;
+    CUtensorMap tm_k, tm_q, tm_v, tm_o;
+    kda_status_t rc = make_tmap(&tm_k, any, T, f.a.H);
+    if (rc == KDA_OK) rc = make_tmap(&tm_v, f.a.v ? f.a.v : any, T, f.a.H);
+    if (rc == KDA_OK) rc = make_tmap(&tm_q, has_q ? f.a.q : any, T, f.a.H);
+    if (rc == KDA_OK) rc = make_tmap(&tm_o, has_q ? f.a.o : any, T, f.a.H);
     if (rc != KDA_OK) return rc;
-    if (f.n_chain_cta >= n_sm)
-        return fail(KDA_ERR_UNSUPPORTED, "kda_chunk_fwd: %d chain CTAs leave no SM of %d for the engines",
-                    f.n_chain_cta, n_sm);
-    int cs = clear_status ? 1 : 0;
-    void* args[] = {(void*)&f, (void*)&tm_k, (void*)&tm_q, (void*)&tm_v, (void*)&cs};
-    const void* fn = has_q ? (const void*)kda_fused_tc<true> : (const void*)kda_fused_tc<false>;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[2];
+    fused_config(cfg, at, f.cluster_size, f.n_clusters, st);
     ProfScope ps(PROF_FUSED, st);
-    KDA_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3((unsigned)n_sm), dim3(kThreads), args, kSmemBytes, st));
+    KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, fused_fn(has_q, f.a.gate_rate != nullptr), f, tm_k, tm_q, tm_v, tm_o));
     count_launch();
     return KDA_OK;
 }
+
+// second kernel of the two-kernel schedule, for n_count sequences (f.n_begin .., or by f.order)
+kda_status_t launch_chain_tc(const FusedArgs& f, int n_count, cudaStream_t st)
+{
+    const ChunkArgs& a = f.a;
+    const bool has_q = a.q != nullptr && a.o != nullptr, layer = a.gate_rate != nullptr;
+    {
+        DeviceLock lk;
+        if (!lk.st) return lk.rc;
+        if (!lk.st->attr_done[2]) {
+            for (int i = 0; i < 4; ++i)
+                KDA_CUDA_TRY(cudaFuncSetAttribute((const void*)chain_fn(i & 1, i & 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)kSmemBytes));
+            lk.st->attr_done[2] = true;
+        }
+    }
+    CUtensorMap tm_o;
+    const kda_status_t rc = make_tmap(&tm_o, has_q ? a.o : f.hdr, a.total_tokens > 0 ? a.total_tokens : 1, a.H);
+    if (rc != KDA_OK) return rc;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)n_count * (unsigned)a.H);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    // only overlap with this library's own intra-chunk kernel, never with a caller's kernel that may still be
+    // producing S0
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = a.g1 > a.g0 ? 1 : 0;
+    ProfScope ps(PROF_INTER, st);
+    KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, chain_fn(has_q, layer), f, tm_o));
+    count_launch();
+    return KDA_OK;
+}
+
+namespace {
+// Self-test of the bounded-wait path: one CTA waits on an mbarrier that nothing ever arrives on,
+// with a short limit, and must come back with KDA_ERR_TIMEOUT in the status word.
+__global__ void kda_wait_selftest_kernel(WsHeader* hdr, uint64_t limit_ns)
+{
+    __shared__ uint64_t bar;
+    if (threadIdx.x == 0) {
+        ptx::mbar_init(&bar, 1);
+        ptx::fence_mbar_init();
+    }
+    __syncthreads();
+    if (!ptx::mbar_wait(&bar, 0, limit_ns)) {
+        if (atomicCAS(&hdr->status, 0, (int)KDA_ERR_TIMEOUT) == 0) hdr->where = 99;
+    }
+}
+}  // namespace
+
+kda_status_t launch_wait_selftest(WsHeader* hdr, uint64_t limit_ns, cudaStream_t st)
+{
+    kda_wait_selftest_kernel<<<1, 32, 0, st>>>(hdr, limit_ns);
+    count_launch();
+    KDA_CUDA_TRY(cudaGetLastError());
+    return KDA_OK;
+}
+
+size_t tc_tile_bytes() { return tc::TILE_BYTES; }
 
 }  // namespace kda

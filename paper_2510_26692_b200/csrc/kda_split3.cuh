@@ -62,7 +62,7 @@ __device__ __forceinline__ Operand mn_major(const uint8_t* img, int row0 = 0, bo
     return {ptx::umma_desc_sw128_mn(ptx::smem_u32(img) + row0 * 128, dup ? 0u : R * 128u), NB * R * 8u, 128u, 512u};
 }
 
-// d (+)= A B over KS steps of 16 in K; ONE thread.  idesc carries M, N and the majors.
+// d (+)= A B over KS steps of 16 in K; a whole converged warp.  idesc carries M, N and the majors.
 template <int KS>
 __device__ __forceinline__ void mma6(uint32_t d_tmem, const Operand& A, const Operand& B, uint32_t idesc, bool accumulate) {
     // (sa, sb): (2,0) (0,2) (1,1) (1,0) (0,1) (0,0)
