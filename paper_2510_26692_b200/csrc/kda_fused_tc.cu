@@ -90,11 +90,20 @@ constexpr uint32_t E_BYTES = (E_GV + tc::GV_BYTES + 1023) / 1024 * 1024;
 static_assert(E_TD_BYTES >= 8 * 128 * 4 && E_TD_BYTES >= 4 * 16 * LDD * 4, "scan exchange and diagonal blocks fit");
 
 // ---- shared-memory map of a chain CTA (bytes from the 1024-aligned base) -----------------------------
-constexpr int kStages = 3;                         // tiles on their way or in work
-constexpr uint32_t C_STAGE = (tc::TILE_BYTES + 1023) / 1024 * 1024;
-constexpr uint32_t C_SSQ = kStages * C_STAGE;      // output stage: [2][64][4] fp32 row sums of squares
+// Two rings: [W ; Q] is free again once the first product of its chunk is complete, the rest of the tile half a step
+// later; the output block has a buffer of its own (kept over the [W ; Q] image of a three-stage ring of whole
+// tiles, it held the stage back: 1.73 instead of 1.5 us a step).
+constexpr int kStagesA = 2, kStagesB = 3;
+constexpr uint32_t kABytes = 32768, kBBytes = tc::TILE_BYTES - tc::OFF_KI;   // B: K', Aqk, gate vectors, U^T
+constexpr uint32_t C_STAGEB = (kBBytes + 1023) / 1024 * 1024;
+constexpr uint32_t C_A = 0, C_B = kStagesA * kABytes;
+constexpr uint32_t C_OUT = C_B + kStagesB * C_STAGEB;   // output block [2][64 tokens][64] bf16
+constexpr uint32_t C_GATE = C_OUT + 16384;              // layer mode: output gates of the same rows
+constexpr uint32_t C_SSQ = C_GATE + 16384;              // layer mode: [2][64][4] fp32 row sums of squares
 constexpr uint32_t C_BAR = C_SSQ + 2048;
 constexpr uint32_t C_BYTES = C_BAR + 512;
+// offsets inside a B stage
+constexpr uint32_t B_KI = 0, B_AQ = tc::OFF_AQ - tc::OFF_KI, B_GV = tc::OFF_GV - tc::OFF_KI, B_U = tc::OFF_U - tc::OFF_KI;
 constexpr uint32_t kSmemBytes = 2 * E_BYTES > C_BYTES ? 2 * E_BYTES : C_BYTES;
 static_assert(E_BYTES % 1024 == 0, "operand images stay 1024-byte aligned");
 static_assert(kSmemBytes <= 232448, "fits the shared memory of one SM");
@@ -383,6 +392,14 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         ptx::mbar_arrive_cluster_relaxed(cursor.ready + (uint32_t)(cursor.published % f.depth) * 8u);
         ++cursor.published;
     };
+    bool staged = false;             // W and U^T of the tile before this one lie in their staging buffers
+    auto store_staged = [&](char* to) {   // (service thread)
+        ptx::bulk_s2g(to + tc::OFF_QW, smem + E_V, 8192);
+        ptx::bulk_s2g(to + tc::OFF_QW + tc::QW_HALF, smem + E_V + 8192, 8192);
+        ptx::bulk_s2g(to + tc::OFF_U, smem + E_A, 16384);
+        ptx::bulk_commit();
+        if (kFused) ++cursor.done;
+    };
     auto find_tile = [&](TileDesc* d) {   // (service thread)
         if (kFused) {
             cluster_tile(f, cursor, d);
@@ -412,7 +429,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         // (the descriptors are read where they are used: registers are short)
         const TileDesc& D = desc[cur];
         const int d_len = D.len;
-        if (d_len == 0 || *abort_word) break;
+        if (d_len == 0) break;       // (an abort is looked at behind a barrier only)
         KT_MARK(te == 0, 0);   // loop overhead
 
         if (kLayer) {
@@ -440,7 +457,9 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         if (kLayer && te < kC)                // (each of these threads copied its own element)
             sBeta[te] = te < d_len ? 1.f / (1.f + __expf(-sBeta[te])) : 0.f;
         ebar();
-        KT_MARK(te == 0, 1);   // scan + publish + slot wait
+        KT_MARK(te == 0, 1);   // scan
+        if (te == kServiceThread && staged) store_staged(desc[cur == 0 ? 2 : cur - 1].tile);
+        staged = false;
         if (*abort_word) break;
         float base[4] = {0.f, 0.f, 0.f, 0.f}, gref[4], glast[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -571,6 +590,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             if (__any_sync(0xffffffffu, may_clamp)) gate_rows(std::true_type{});
             else gate_rows(std::false_type{});
         }
+        if (te == kServiceThread) ptx::bulk_wait_read0();   // the previous tile's W and U^T have been read out
         ptx::fence_async_smem();
         ptx::tc_fence_before();
         ebar();
@@ -597,7 +617,9 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             ptx::bulk_s2g(D.tile + tc::OFF_KI, smem + E_KI, 16384);
             ptx::bulk_s2g(D.tile + tc::OFF_GV, smem + E_GV, tc::GV_BYTES);
             ptx::bulk_commit();
+            request_v(D);            // over W
         }
+        pend_v = true;
         if (warp == 0) {
             const uint32_t idesc = ptx::umma_idesc_bf16(128, 64);
             const uint32_t a0 = ptx::smem_u32(smem + E_KQ), b0 = ptx::smem_u32(smem + E_KI);
@@ -616,15 +638,6 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             pend_k = true;
         }
         if (!ptx::mbar_wait(mma_bar, 0, f.a.wait_limit_ns)) timed_out = true;
-        // everything staged for bulk stores has been read out of shared memory (this tile's Q and K', the previous
-        // tile's W and U^T): the next k goes over Q, v over W, L over U^T
-        if (te == kServiceThread) {
-            ptx::bulk_wait_read0();
-            request_v(D);
-            if (has_next) request_k(Dn);
-        }
-        pend_v = true;
-        ebar();
         ptx::tc_fence_after();
         KT_MARK(te == 0, 4);   // MMA A
         {
@@ -670,9 +683,10 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
                 ptx::bulk_s2g(D.tile + tc::OFF_AQ, smem + E_AQ, 8192);
                 ptx::bulk_commit();
             }
-            if (has_q) {   // the Aqk staging has been read out: the next tile's q may land over it
-                ptx::bulk_wait_read0();
-                if (has_next) request_q(Dn);
+            ptx::bulk_wait_read0();   // Q, K' and Aqk have been read out: the next q and k may land over them
+            if (has_next) {
+                request_k(Dn);
+                if (has_q) request_q(Dn);
             }
             if (has_next) find_tile(&desc[nxt2]);
             else desc[nxt2].len = 0;
@@ -836,14 +850,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         ptx::fence_async_smem();
         ptx::tc_fence_before();
         if (timed_out) *abort_word = 1;
-        ebar();
-        if (te == kServiceThread) {
-            ptx::bulk_s2g(D.tile + tc::OFF_QW, smem + E_V, 8192);
-            ptx::bulk_s2g(D.tile + tc::OFF_QW + tc::QW_HALF, smem + E_V + 8192, 8192);
-            ptx::bulk_s2g(D.tile + tc::OFF_U, smem + E_A, 16384);
-            ptx::bulk_commit();
-            if (kFused) ++cursor.done;
-        }
+        staged = true;               // stored after the next barrier
         KT_MARK(te == 0, 8);   // epilogue
 #ifdef KDA_FUSED_TIMING
         if (te == 0) kt_acc_[9] += 16;   // tiles
@@ -852,6 +859,11 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
     }   // tile loop
     KT_FLUSH(te == 0, f.hdr, 0, 10);
 
+    ebar();
+    if (te == kServiceThread && staged && !*abort_word) {
+        const int last = cur == 0 ? 2 : cur - 1;
+        store_staged(desc[last].tile);
+    }
     if (timed_out) report_timeout(f, 10);
     if (out_of_range) atomicOr(&f.hdr->flags, 1);
     if (te == kServiceThread) {
@@ -898,9 +910,11 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
 {
     const ChunkArgs& a = f.a;
     uint64_t* ready = reinterpret_cast<uint64_t*>(smem + C_BAR);   // [engine][depth] a ring position holds a tile
-    uint64_t* full = ready + 6 * kMaxDepth;  // [kStages] a tile has landed
-    uint64_t* empty = full + kStages;        // [kStages] and is no longer needed: last commit, 8 compute warps, output store
-    uint64_t* m1 = empty + kStages;          // MMA1 of a chunk complete
+    uint64_t* fullA = ready + 6 * kMaxDepth; // [kStagesA] landed
+    uint64_t* fullB = fullA + kStagesA;      // [kStagesB]
+    uint64_t* emptyA = fullB + kStagesB;     // [kStagesA] MMA1 done with it
+    uint64_t* emptyB = emptyA + kStagesA;    // [kStagesB] last product and the 8 compute warps done with it
+    uint64_t* m1 = emptyB + kStagesB;        // MMA1 of a chunk complete
     uint64_t* m2 = m1 + 1;                   // MMA2
     uint64_t* out_bar = m2 + 1;              // [2] output accumulator complete (alternating)
     uint64_t* o_done = out_bar + 2;          // [2] and read (4 warps)
@@ -940,10 +954,13 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
             if (!kRing) ptx::grid_dep_wait();   // the tiles come from the intra-chunk kernel launched just before
             // (kRing) a position is given back this many tiles later, when its copy has landed for certain
             const uint32_t lag = f.n_eng * f.depth >= 3 ? 2 : 0;   // (less than the number of positions)
+            static_assert(kStagesA == 2 && kStagesB == 3, "give_back relies on them");
             uint32_t g = 0;
             const uint32_t base = ptx::smem_u32(smem);
             auto give_back = [&](uint32_t x) {
-                wait(&full[x % kStages], (x / kStages) & 1u, 31);
+                wait(&fullB[x % kStagesB], (x / kStagesB) & 1u, 31);
+                // (with a lag of two the stage of its [W ; Q] has been reused already: landed, and its barrier moved on)
+                if (lag == 0) wait(&fullA[x % kStagesA], (x / kStagesA) & 1u, 33);
                 const uint32_t e = x % (uint32_t)f.n_eng, slot = (x / (uint32_t)f.n_eng) % (uint32_t)f.depth;
                 ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(base + (e & 1u) * E_BYTES + E_BAR + 48 + slot * 8, 1 + (e >> 1)));
             };
@@ -951,32 +968,43 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
             for (int r = 0; next_job(r) && !*abort_flag; ++r)
                 for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
                     const uint32_t e = g % (uint32_t)f.n_eng, m = g / (uint32_t)f.n_eng;
-                    const uint32_t slot = m % (uint32_t)f.depth, s = g % kStages;
+                    const uint32_t slot = m % (uint32_t)f.depth, sa = g % kStagesA, s = g % kStagesB;
                     const char* tile = kRing ? f.ring + (size_t)(((uint32_t)cid * f.n_eng + e) * f.depth + slot) * tc::TILE_BYTES
                                              : f.ring + (size_t)(J.tile0 + (int64_t)c * a.H) * tc::TILE_BYTES;
                     KT_MARK(true, 0);
                     if (kRing) wait(&ready[e * (uint32_t)f.depth + slot], (m / (uint32_t)f.depth) & 1u, 30);
                     KT_MARK(true, 1);
-                    if (g >= kStages) wait(&empty[s], (g / kStages - 1) & 1u, 32);
+                    if (g >= kStagesB) wait(&emptyB[s], (g / kStagesB - 1) & 1u, 32);
                     if (*abort_flag) break;
                     KT_MARK(true, 2);
-                    uint8_t* sb = smem + s * C_STAGE;
+                    uint8_t* sB = smem + C_B + s * C_STAGEB;
                     if (kHasQ) {
-                        ptx::mbar_expect_tx(&full[s], tc::TILE_BYTES);
-                        ptx::bulk_g2s(sb, tile, tc::TILE_BYTES, &full[s]);
+                        ptx::mbar_expect_tx(&fullB[s], kBBytes);
+                        ptx::bulk_g2s(sB, tile + tc::OFF_KI, kBBytes, &fullB[s]);
                     } else {   // state-only call: only the W rows exist, and no Aqk
-                        ptx::mbar_expect_tx(&full[s], 8192 + 8192 + 16384 + tc::GV_BYTES + 16384);
-                        ptx::bulk_g2s(sb, tile, 8192, &full[s]);
-                        ptx::bulk_g2s(sb + tc::QW_HALF, tile + tc::QW_HALF, 8192, &full[s]);
-                        ptx::bulk_g2s(sb + tc::OFF_KI, tile + tc::OFF_KI, 16384, &full[s]);
-                        ptx::bulk_g2s(sb + tc::OFF_GV, tile + tc::OFF_GV, tc::GV_BYTES + 16384, &full[s]);
+                        ptx::mbar_expect_tx(&fullB[s], kBBytes - 8192);
+                        ptx::bulk_g2s(sB, tile + tc::OFF_KI, 16384, &fullB[s]);
+                        ptx::bulk_g2s(sB + B_GV, tile + tc::OFF_GV, tc::GV_BYTES + 16384, &fullB[s]);
+                    }
+                    if (g >= kStagesA) wait(&emptyA[sa], (g / kStagesA - 1) & 1u, 34);
+                    uint8_t* sA = smem + C_A + sa * kABytes;
+                    if (kHasQ) {
+                        ptx::mbar_expect_tx(&fullA[sa], kABytes);
+                        ptx::bulk_g2s(sA, tile, kABytes, &fullA[sa]);
+                    } else {
+                        ptx::mbar_expect_tx(&fullA[sa], 16384);
+                        ptx::bulk_g2s(sA, tile, 8192, &fullA[sa]);
+                        ptx::bulk_g2s(sA + tc::QW_HALF, tile + tc::QW_HALF, 8192, &fullA[sa]);
                     }
                     if (kRing && g >= lag) give_back(g - lag);
                 }
             KT_FLUSH(true, f.hdr, 24, 3);
-            if (*abort_flag)   // the copies already requested must land before the shared memory goes away
-                for (uint32_t x = g > kStages ? g - kStages : 0; x < g; ++x)
-                    ptx::mbar_wait(&full[x % kStages], (x / kStages) & 1u, a.wait_limit_ns / 8);
+            if (*abort_flag) {   // the copies already requested must land before the shared memory goes away
+                for (uint32_t x = g > kStagesB ? g - kStagesB : 0; x < g; ++x)
+                    ptx::mbar_wait(&fullB[x % kStagesB], (x / kStagesB) & 1u, a.wait_limit_ns / 8);
+                for (uint32_t x = g > kStagesA ? g - kStagesA : 0; x < g; ++x)
+                    ptx::mbar_wait(&fullA[x % kStagesA], (x / kStagesA) & 1u, a.wait_limit_ns / 8);
+            }
         }
     } else if (warp == 8) {
         // ================= MMA issue =================
@@ -987,10 +1015,11 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
         KT_DECL(8);
         for (int r = 0; next_job(r) && !*abort_flag; ++r)
             for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
-                const uint32_t s = g % kStages, sb = base + s * C_STAGE;
+                const uint32_t sa = g % kStagesA, s = g % kStagesB;
+                const uint32_t pA = base + C_A + sa * kABytes, pB = base + C_B + s * C_STAGEB;
                 const uint32_t d1 = tm + T_D1 + (g & 1u) * 128u;
                 KT_MARK(lane == 0, 0);
-                wait(&full[s], (g / kStages) & 1u, 1);
+                wait(&fullA[sa], (g / kStagesA) & 1u, 1);
                 KT_MARK(lane == 0, 1);   // operands
                 if (op && g >= 2) wait(&o_done[g & 1u], ((g >> 1) - 1) & 1u, 2);
                 wait(s_ready, g & 1u, 3);
@@ -999,31 +1028,31 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                 ptx::tc_fence_after();
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
-                    ptx::umma_bf16_ta(d1, tm + T_S + k * 8, ptx::umma_desc_sw128(sb + tc::OFF_QW + (k >> 2) * tc::QW_HALF + (k & 3) * 32),
-                                      id1, k > 0);
+                    ptx::umma_bf16_ta(d1, tm + T_S + k * 8, ptx::umma_desc_sw128(pA + (k >> 2) * tc::QW_HALF + (k & 3) * 32), id1, k > 0);
                 ptx::umma_commit(m1);
+                ptx::umma_commit(&emptyA[sa]);
                 KT_MARK(lane == 0, 3);   // MMA1 issue
+                wait(&fullB[s], (g / kStagesB) & 1u, 11);
                 wait(vn_ready, g & 1u, 4);
                 __syncwarp();
                 KT_MARK(lane == 0, 4);   // V_new
                 ptx::tc_fence_after();
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    ptx::umma_bf16_ta(tm + T_D3, tm + T_VN + k * 8, ptx::umma_desc_sw128_mn(sb + tc::OFF_KI + k * 2048, tc::KI_HALF),
-                                      id2, k > 0);
+                    ptx::umma_bf16_ta(tm + T_D3, tm + T_VN + k * 8, ptx::umma_desc_sw128_mn(pB + B_KI + k * 2048, tc::KI_HALF), id2, k > 0);
                 ptx::umma_commit(m2);
                 if (op) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        ptx::umma_bf16_ta(d1 + 64, tm + T_VN + k * 8, ptx::umma_desc_sw128(sb + tc::OFF_AQ + k * 32), ido, 1);
+                        ptx::umma_bf16_ta(d1 + 64, tm + T_VN + k * 8, ptx::umma_desc_sw128(pB + B_AQ + k * 32), ido, 1);
                     ptx::umma_commit(&out_bar[g & 1u]);
                 }
-                ptx::umma_commit(&empty[s]);
+                ptx::umma_commit(&emptyB[s]);
                 KT_MARK(lane == 0, 5);   // MMA2 + output issue
             }
         KT_FLUSH(lane == 0, f.hdr, 16, 6);
         // every MMA has completed before the TMEM goes away
-        if (g > 0) wait(&empty[(g - 1) % kStages], ((g - 1) / kStages) & 1u, 5);
+        if (g > 0) wait(&emptyB[(g - 1) % kStagesB], ((g - 1) / kStagesB) & 1u, 5);
     } else if (warp < 8) {
         // ================= compute warps =================
         const int quad = warp & 3, half = warp >> 2, dv = quad * 32 + lane, dk0 = half * 64;
@@ -1050,21 +1079,21 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                 warp_arrive(s_ready);
             }
             for (int c = 0; c < J.nch; ++c, ++g) {
-                const uint32_t s = g % kStages;
-                const uint8_t* sb = smem + s * C_STAGE;
+                const uint32_t s = g % kStagesB;
+                const uint8_t* sb = smem + C_B + s * C_STAGEB;
                 const bool more = c + 1 < J.nch;
                 // four values of a gate vector of the chunk (0: gamma^C, 1: exp(G_C - G_m))
                 auto vec = [&](int which, int i) {
-                    return *reinterpret_cast<const float4*>(sb + tc::OFF_GV + which * 512 + (dk0 + i) * 4);
+                    return *reinterpret_cast<const float4*>(sb + B_GV + which * 512 + (dk0 + i) * 4);
                 };
                 KT_MARK(t == 0, 0);
-                wait(&full[s], (g / kStages) & 1u, 6);
+                wait(&fullB[s], (g / kStagesB) & 1u, 6);
                 KT_MARK(t == 0, 1);
                 {   // V_new^T = U^T - (W S)^T: column dv, tokens 32 half ..
                     uint4 uq[4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        uq[k] = *reinterpret_cast<const uint4*>(sb + tc::OFF_U + tc::ut_off((uint32_t)dv, (uint32_t)(half * 4 + k)));
+                        uq[k] = *reinterpret_cast<const uint4*>(sb + B_U + tc::ut_off((uint32_t)dv, (uint32_t)(half * 4 + k)));
                     const uint32_t* u = reinterpret_cast<const uint32_t*>(uq);
                     wait(m1, g & 1u, 7);
                     __syncwarp();
@@ -1120,7 +1149,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                 __syncwarp();
                 if (lane == 0) {
                     if (more) ptx::mbar_arrive(s_ready);
-                    ptx::mbar_arrive(&empty[s]);
+                    ptx::mbar_arrive(&emptyB[s]);
                 }
                 KT_MARK(t == 0, 6);
             }
@@ -1133,8 +1162,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
     } else if (warp >= 12 && op) {
         // ================= output rows =================
         // The accumulator has a lane per column and a TMEM column per token; read as 8 x 8 fragments and stored with
-        // stmatrix.trans it becomes rows of the output, over the stage's [W ; Q] image (no longer needed), and
-        // leaves by two tiled TMA stores.  (Straight from the lanes, 64 two-byte stores a thread, the stores
+        // stmatrix.trans it becomes rows of the output, which leave by two tiled TMA stores.  (Straight from the lanes, 64 two-byte stores a thread, the stores
         // crowded out the loads of the compute warps: 2.6 instead of 1.6 us a step.)
         const int quad = warp & 3, ot = t - 384;
         const uint32_t tq = tm + ((uint32_t)(quad * 32) << 16);
@@ -1147,23 +1175,26 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
         if (epi)
 #pragma unroll
             for (int b = 0; b < 4; ++b) wgt[b] = a.rms_weight[quad * 32 + b * 8 + (lane >> 2)];
+        uint8_t* sb = smem + C_OUT;
+        uint8_t* sg = smem + C_GATE;
+        uint4 gq[kLayer ? 8 : 1];        // gate pre-activations, 16-byte piece ot + 128 k of a [64][256 B] block
+        auto load_gates = [&](int64_t tok0, int len) {
+#pragma unroll
+            for (int k = 0; k < (kLayer ? 8 : 0); ++k) {
+                const int idx = ot + 128 * k, row = idx >> 4;
+                gq[k] = make_uint4(0u, 0u, 0u, 0u);
+                if (row < len)
+                    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+                                 : "=r"(gq[k].x), "=r"(gq[k].y), "=r"(gq[k].z), "=r"(gq[k].w)
+                                 : "l"(reinterpret_cast<const __nv_bfloat16*>(a.out_gate) + ((size_t)(tok0 + row) * a.H + J.h) * kD + (idx & 15) * 8));
+            }
+        };
         uint32_t g = 0;
         for (int r = 0; next_job(r) && !*abort_flag; ++r)
             for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
                 const int64_t tok0 = J.tok_begin + (int64_t)c * kC;
                 const int len = (J.tok_end - tok0) < kC ? (int)(J.tok_end - tok0) : kC;
-                const uint32_t s = g % kStages;
-                uint8_t* sb = smem + s * C_STAGE;
-                uint4 gq[kLayer ? 8 : 1];        // gate pre-activations, 16-byte piece ot + 128 k of the [64][256 B] block
-                if (kLayer && epi)
-#pragma unroll
-                    for (int k = 0; k < (kLayer ? 8 : 0); ++k) {
-                        const int idx = ot + 128 * k, row = idx >> 4;
-                        gq[k] = make_uint4(0u, 0u, 0u, 0u);
-                        if (row < len)
-                            gq[k] = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(a.out_gate) +
-                                                                    ((size_t)(tok0 + row) * a.H + J.h) * kD + (idx & 15) * 8);
-                    }
+                if (kLayer && epi && c == 0) load_gates(tok0, len);
                 wait(&out_bar[g & 1u], (g >> 1) & 1u, 10);
                 __syncwarp();
                 ptx::tc_fence_after();
@@ -1179,7 +1210,11 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
 #pragma unroll
                     for (int k = 0; k < (kLayer ? 8 : 0); ++k) {
                         const int idx = ot + 128 * k, ch = idx & 15;
-                        *reinterpret_cast<uint4*>(sb + 16384 + (ch >> 3) * 8192 + ptx::sw128_off((uint32_t)(idx >> 4), (uint32_t)(ch & 7) * 8)) = gq[k];
+                        *reinterpret_cast<uint4*>(sg + (ch >> 3) * 8192 + ptx::sw128_off((uint32_t)(idx >> 4), (uint32_t)(ch & 7) * 8)) = gq[k];
+                    }
+                    if (c + 1 < J.nch) {     // the next chunk's gates are on their way while this one's are used
+                        const int64_t left = J.tok_end - tok0 - kC;
+                        load_gates(tok0 + kC, left < kC ? (int)left : kC);
                     }
                     float q[16];
 #pragma unroll
@@ -1209,7 +1244,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         uint32_t gt[4];
-                        ptx::ldmatrix_x4_trans(sb + 16384 + moff + j * 1024, gt);
+                        ptx::ldmatrix_x4_trans(sg + moff + j * 1024, gt);
 #pragma unroll
                         for (int e = 0; e < 2; ++e) {
                             const float4 p = *reinterpret_cast<const float4*>(sq + (8 * j + 2 * (lane & 3) + e) * 4);
@@ -1223,6 +1258,9 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                         }
                     }
                 }
+                // the previous block has been read out of its buffer
+                if (ot == 0) ptx::bulk_wait_read0();
+                ptx::named_bar_sync(6, 128);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     uint32_t z[4];
@@ -1238,7 +1276,6 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                         ptx::tma_store_2d(tm_o, sb, J.h * kD, (int)tok0);
                         ptx::tma_store_2d(tm_o, sb + 8192, J.h * kD + 64, (int)tok0);
                         ptx::bulk_commit();
-                        ptx::bulk_wait_read0();
                     }
                 } else {       // the rows past the end of the sequence belong to the next one
                     if (!*abort_flag)
@@ -1247,9 +1284,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                             *reinterpret_cast<uint4*>(op + ((size_t)(tok0 + row) * a.H + J.h) * kD + ch * 8) =
                                 *reinterpret_cast<const uint4*>(sb + (ch >> 3) * 8192 + ptx::sw128_off((uint32_t)row, (uint32_t)(ch & 7) * 8));
                         }
-                    ptx::named_bar_sync(6, 128);
                 }
-                if (ot == 0) ptx::mbar_arrive(&empty[s]);
             }
         if (ot == 0) ptx::bulk_wait_all0();
     }
@@ -1258,12 +1293,13 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
 }
 
 // barriers of a chain CTA; ONE thread
-__device__ void chain_init(uint8_t* smem, bool has_out)
+__device__ void chain_init(uint8_t* smem)
 {
     uint64_t* b = reinterpret_cast<uint64_t*>(smem + C_BAR);
     for (int i = 0; i < 6 * kMaxDepth; ++i) ptx::mbar_init(b++, 1);   // ready
-    for (int i = 0; i < kStages; ++i) ptx::mbar_init(b++, 1);         // full
-    for (int i = 0; i < kStages; ++i) ptx::mbar_init(b++, has_out ? 10 : 9);   // empty
+    for (int i = 0; i < kStagesA + kStagesB; ++i) ptx::mbar_init(b++, 1);   // fullA, fullB
+    for (int i = 0; i < kStagesA; ++i) ptx::mbar_init(b++, 1);        // emptyA
+    for (int i = 0; i < kStagesB; ++i) ptx::mbar_init(b++, 9);        // emptyB
     ptx::mbar_init(b++, 1);                                           // m1
     ptx::mbar_init(b++, 1);                                           // m2
     for (int i = 0; i < 2; ++i) ptx::mbar_init(b++, 1);               // out_bar
@@ -1293,7 +1329,7 @@ kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     const bool chain_cta = rank == 0;
     // (the TMEM slot sits in a spare word of the barrier block of either layout)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + (chain_cta ? C_BAR + 500 : E_BAR + 32));
-    if (chain_cta && t == 0) chain_init(smem, kHasQ && f.a.o != nullptr);
+    if (chain_cta && t == 0) chain_init(smem);
     if (!chain_cta && (t == 0 || t == kEngThreads)) {
         uint64_t* mb = reinterpret_cast<uint64_t*>(smem + (t ? E_BYTES : 0) + E_BAR);
         ptx::mbar_init(mb, 2);       // MMA group complete (two issuing warps)
@@ -1353,7 +1389,7 @@ kda_chain_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     extern __shared__ __align__(1024) uint8_t smem[];
     const int t = threadIdx.x, warp = t >> 5;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C_BAR + 500);
-    if (t == 0) chain_init(smem, kHasQ && f.a.o != nullptr);
+    if (t == 0) chain_init(smem);
     if (warp == 0) {
         ptx::tmem_alloc(tmem_slot, kTmemCols);
         ptx::tmem_relinquish();
