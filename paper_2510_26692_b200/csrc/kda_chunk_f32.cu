@@ -311,7 +311,8 @@ __global__ void __launch_bounds__(kT2, 1) kda_inter_f32(ChunkArgs a, const float
 __global__ void kda_prep_kernel(WsHeader* hdr, const int32_t* __restrict__ cu,
                                 int32_t* __restrict__ chunk_cu, int n_seqs)
 {
-    ptx::grid_dep_launch();      // (its dependents wait for its end before they read anything)
+    ptx::grid_dep_wait();        // (launched before the preceding kernel has ended)
+    ptx::grid_dep_launch();
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         hdr->status = 0;
         hdr->where = 0;
@@ -381,9 +382,8 @@ kda_status_t launch_prep(WsHeader* hdr, const int32_t* cu_seqlens, int32_t* chun
                          cudaStream_t st)
 {
     ProfScope ps(PROF_PREP, st);
-    kda_prep_kernel<<<1, 32, 0, st>>>(hdr, cu_seqlens, chunk_cu, n_seqs);
+    KDA_CUDA_TRY(launch_dependent(kda_prep_kernel, dim3(1), 32, 0, st, hdr, cu_seqlens, chunk_cu, n_seqs));
     count_launch();
-    KDA_CUDA_TRY(cudaGetLastError());
     return KDA_OK;
 }
 

@@ -503,7 +503,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         if (kLayer) {
             // L2Norm of k and q: the warp owns its eight rows whole (32 lanes x 4 channels)
             const int hf = c4 >> 4;
-            float ssk[kRPT], ssq[kRPT];
+            float ss[2 * kRPT];   // k rows, q rows
 #pragma unroll
             for (int r = 0; r < kRPT; ++r) {
                 const int i = i0 + r;
@@ -515,23 +515,24 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
                 const float k2f = __uint_as_float(k2.y << 16), k3 = __uint_as_float(k2.y & 0xffff0000u);
                 const float q0 = __uint_as_float(q2.x << 16), q1 = __uint_as_float(q2.x & 0xffff0000u);
                 const float q2f = __uint_as_float(q2.y << 16), q3 = __uint_as_float(q2.y & 0xffff0000u);
-                ssk[r] = k0 * k0 + k1 * k1 + k2f * k2f + k3 * k3;
-                ssq[r] = q0 * q0 + q1 * q1 + q2f * q2f + q3 * q3;
+                ss[r] = k0 * k0 + k1 * k1 + k2f * k2f + k3 * k3;
+                ss[kRPT + r] = q0 * q0 + q1 * q1 + q2f * q2f + q3 * q3;
             }
+            // sums over the 32 lanes: each exchange halves the values a lane still carries (16 shuffles, not 80)
 #pragma unroll
-            for (int s = 16; s >= 1; s >>= 1)
+            for (int n = kRPT, x = 16; n >= 1; n >>= 1, x >>= 1) {
+                const bool up = (lane & x) != 0;
 #pragma unroll
-                for (int r = 0; r < kRPT; ++r) {
-                    ssk[r] += __shfl_xor_sync(0xffffffffu, ssk[r], s);
-                    ssq[r] += __shfl_xor_sync(0xffffffffu, ssq[r], s);
+                for (int i = 0; i < n; ++i) {
+                    const float send = up ? ss[i] : ss[i + n], keep = up ? ss[i + n] : ss[i];
+                    ss[i] = keep + __shfl_xor_sync(0xffffffffu, send, x);
                 }
-#pragma unroll
-            for (int r = 0; r < kRPT; ++r)
-                if (lane == r) {   // (rows past the end of the sequence are zeroed below: keep their factor finite)
-                    const bool in = i0 + r < d_len;
-                    sNorm[i0 + r] = in ? rsqrtf(ssk[r] + a.l2_eps) : 0.f;
-                    sNorm[kC + i0 + r] = in ? rsqrtf(ssq[r] + a.l2_eps) : 0.f;
-                }
+            }
+            ss[0] += __shfl_xor_sync(0xffffffffu, ss[0], 1);
+            if ((lane & 1) == 0) {   // (rows past the end of the sequence are zeroed below: finite factor)
+                const int v = lane >> 1, r = v & (kRPT - 1);
+                sNorm[(v >= kRPT ? kC : 0) + i0 + r] = i0 + r < d_len ? rsqrtf(ss[0] + a.l2_eps) : 0.f;
+            }
             __syncwarp();
         }
         auto gate_rows = [&](auto clamp_tag) {
@@ -887,7 +888,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 // ====================================================================================================
 // Everything is transposed: TMEM lanes are the 128 columns of the state (dv), so that the state and V_new are A
 // operands in TMEM and nothing on the chain goes through shared memory:
-//   MMA1  D1[dv][0:64] = (W S)^T, D1[dv][64:128] = (Gamma.Q S)^T     A = bf16 state, B = [W ; Q]
+//   MMA1  D1[dv][0:64] = (W S)^T, then D1[dv][64:128] = (Gamma.Q S)^T     A = bf16 state, B = W, Q
 //   V_new^T = U^T - D1[:, 0:64]  -> bf16 -> TMEM
 //   MMA2  D3[dv][dk] = (K'^T V_new)^T,  D1[dv][64:128] += (Aqk V_new)^T            A = V_new, B = K', Aqk
 //   S <- gamma^C . S + exp(G_C - G_m) . D3  (fp32, in registers: thread = column, half of dk)  -> bf16 -> TMEM
@@ -1008,7 +1009,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
         }
     } else if (warp == 8) {
         // ================= MMA issue =================
-        const uint32_t id1 = ptx::umma_idesc_bf16(128, kHasQ ? 128 : 64), ido = ptx::umma_idesc_bf16(128, 64);
+        const uint32_t id1 = ptx::umma_idesc_bf16(128, 64);
         const uint32_t id2 = ptx::umma_idesc_bf16(128, 128) | ptx::kIdescBMajorMN;
         const uint32_t base = (uint32_t)ptx::warp_uniform((int)ptx::smem_u32(smem));
         uint32_t g = 0;
@@ -1026,10 +1027,17 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                 __syncwarp();
                 KT_MARK(lane == 0, 2);   // state
                 ptx::tc_fence_after();
+                // W S first: V_new waits for it alone, Q S runs beside V_new's arithmetic
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
                     ptx::umma_bf16_ta(d1, tm + T_S + k * 8, ptx::umma_desc_sw128(pA + (k >> 2) * tc::QW_HALF + (k & 3) * 32), id1, k > 0);
                 ptx::umma_commit(m1);
+                if (kHasQ) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        ptx::umma_bf16_ta(d1 + 64, tm + T_S + k * 8,
+                                          ptx::umma_desc_sw128(pA + 8192 + (k >> 2) * tc::QW_HALF + (k & 3) * 32), id1, k > 0);
+                }
                 ptx::umma_commit(&emptyA[sa]);
                 KT_MARK(lane == 0, 3);   // MMA1 issue
                 wait(&fullB[s], (g / kStagesB) & 1u, 11);
@@ -1044,7 +1052,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                 if (op) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        ptx::umma_bf16_ta(d1 + 64, tm + T_VN + k * 8, ptx::umma_desc_sw128(pB + B_AQ + k * 32), ido, 1);
+                        ptx::umma_bf16_ta(d1 + 64, tm + T_VN + k * 8, ptx::umma_desc_sw128(pB + B_AQ + k * 32), id1, 1);
                     ptx::umma_commit(&out_bar[g & 1u]);
                 }
                 ptx::umma_commit(&emptyB[s]);
@@ -1123,26 +1131,31 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                 KT_MARK(t == 0, 5);
                 ptx::tc_fence_after();
 #pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    uint32_t y[16], z[8];
-                    ptx::tmem_ld_32x32b_x16(tq + T_D3 + dk0 + b * 16, y);
-                    float4 ct[4];      // (fetched while the accumulator is)
+                for (int b = 0; b < 2; ++b) {
+                    uint32_t y[32];
+                    ptx::tmem_ld_32x32b_x32(tq + T_D3 + dk0 + b * 32, y);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) ct[i] = vec(1, b * 16 + 4 * i);
-                    ptx::tmem_ld_wait();
+                    for (int hb = 0; hb < 2; ++hb) {
+                        float4 ct[4];      // (the first fetched while the accumulator is)
 #pragma unroll
-                    for (int i = 0; i < 16; i += 4) {
-                        float* s4 = &S[b * 16 + i];
-                        const float4 e = ct[i / 4];
-                        const float2 lo = __ffma2_rn(make_float2(e.x, e.y), make_float2(__uint_as_float(y[i]), __uint_as_float(y[i + 1])),
-                                                     make_float2(s4[0], s4[1]));
-                        const float2 hi = __ffma2_rn(make_float2(e.z, e.w), make_float2(__uint_as_float(y[i + 2]), __uint_as_float(y[i + 3])),
-                                                     make_float2(s4[2], s4[3]));
-                        s4[0] = lo.x; s4[1] = lo.y; s4[2] = hi.x; s4[3] = hi.y;
-                        z[i / 2] = pack_bf16(lo.x, lo.y);
-                        z[i / 2 + 1] = pack_bf16(hi.x, hi.y);
+                        for (int i = 0; i < 4; ++i) ct[i] = vec(1, b * 32 + hb * 16 + 4 * i);
+                        if (hb == 0) ptx::tmem_ld_wait();
+                        uint32_t z[8];
+#pragma unroll
+                        for (int i = 0; i < 16; i += 4) {
+                            float* s4 = &S[b * 32 + hb * 16 + i];
+                            const uint32_t* d = y + hb * 16 + i;
+                            const float4 e = ct[i / 4];
+                            const float2 lo = __ffma2_rn(make_float2(e.x, e.y), make_float2(__uint_as_float(d[0]), __uint_as_float(d[1])),
+                                                         make_float2(s4[0], s4[1]));
+                            const float2 hi = __ffma2_rn(make_float2(e.z, e.w), make_float2(__uint_as_float(d[2]), __uint_as_float(d[3])),
+                                                         make_float2(s4[2], s4[3]));
+                            s4[0] = lo.x; s4[1] = lo.y; s4[2] = hi.x; s4[3] = hi.y;
+                            z[i / 2] = pack_bf16(lo.x, lo.y);
+                            z[i / 2 + 1] = pack_bf16(hi.x, hi.y);
+                        }
+                        if (more) ptx::tmem_st_32x32b_x8(tq + T_S + half * 32 + b * 16 + hb * 8, z);
                     }
-                    if (more) ptx::tmem_st_32x32b_x8(tq + T_S + half * 32 + b * 8, z);
                 }
                 if (more) ptx::tmem_st_wait();
                 ptx::tc_fence_before();
@@ -1175,7 +1188,6 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
         if (epi)
 #pragma unroll
             for (int b = 0; b < 4; ++b) wgt[b] = a.rms_weight[quad * 32 + b * 8 + (lane >> 2)];
-        uint8_t* sb = smem + C_OUT;
         uint8_t* sg = smem + C_GATE;
         uint4 gq[kLayer ? 8 : 1];        // gate pre-activations, 16-byte piece ot + 128 k of a [64][256 B] block
         auto load_gates = [&](int64_t tok0, int len) {
@@ -1259,6 +1271,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                     }
                 }
                 // the previous block has been read out of its buffer
+                uint8_t* sb = smem + C_OUT;
                 if (ot == 0) ptx::bulk_wait_read0();
                 ptx::named_bar_sync(6, 128);
 #pragma unroll
@@ -1419,12 +1432,6 @@ kda_intra_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     extern __shared__ __align__(1024) uint8_t smem[];
     const int t = threadIdx.x, warp = t >> 5;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + E_BAR + 32);
-    ptx::grid_dep_launch();   // the inter-chunk kernel may set itself up while this one drains
-    if (clear_status && blockIdx.x == 0 && t == 0) {
-        f.hdr->status = 0;      // (an equal-length call has no prologue kernel to do this)
-        f.hdr->where = 0;
-        f.hdr->flags = 0;
-    }
     if (t == 0) {
         uint64_t* mb = reinterpret_cast<uint64_t*>(smem + E_BAR);
         ptx::mbar_init(mb, 2);       // MMA group complete (two issuing threads)
@@ -1448,6 +1455,13 @@ kda_intra_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     if ((ptx::smem_u32(smem) & 1023u) != 0) {
         if (t == 0) report_timeout(f, 90);   // the operand images need 1024-byte alignment
     } else {
+        ptx::grid_dep_wait();     // (launched before the preceding kernel has ended)
+        ptx::grid_dep_launch();   // the chains may set themselves up while this one drains (not before: they read S0)
+        if (clear_status && blockIdx.x == 0 && t == 0) {
+            f.hdr->status = 0;      // (an equal-length call has no prologue kernel to do this)
+            f.hdr->where = 0;
+            f.hdr->flags = 0;
+        }
         engine_run<kHasQ, false, kLayer>(f, smem, tmem_base, 1, t, blockIdx.x, gridDim.x, &tm_k, &tm_q, &tm_v);
     }
     ptx::tc_fence_before();
@@ -1535,14 +1549,19 @@ kda_status_t launch_intra_tc(const ChunkArgs& a, void* tiles, WsHeader* hdr, boo
     const unsigned grid = (unsigned)(n_tiles < resident ? n_tiles : resident);
     ProfScope ps(PROF_INTRA, st);
     const bool layer = a.gate_rate != nullptr;
-    if (layer && has_q)
-        kda_intra_tc<true, true><<<grid, kEngThreads, E_BYTES, st>>>(f, tm_k, tm_q, tm_v, clear_status ? 1 : 0);
-    else if (layer)
-        kda_intra_tc<false, true><<<grid, kEngThreads, E_BYTES, st>>>(f, tm_k, tm_q, tm_v, clear_status ? 1 : 0);
-    else if (has_q)
-        kda_intra_tc<true, false><<<grid, kEngThreads, E_BYTES, st>>>(f, tm_k, tm_q, tm_v, clear_status ? 1 : 0);
-    else
-        kda_intra_tc<false, false><<<grid, kEngThreads, E_BYTES, st>>>(f, tm_k, tm_q, tm_v, clear_status ? 1 : 0);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kEngThreads);
+    cfg.dynamicSmemBytes = E_BYTES;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    auto fn = layer ? (has_q ? kda_intra_tc<true, true> : kda_intra_tc<false, true>)
+                    : (has_q ? kda_intra_tc<true, false> : kda_intra_tc<false, false>);
+    KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, f, tm_k, tm_q, tm_v, clear_status ? 1 : 0));
     count_launch();
     KDA_CUDA_TRY(cudaGetLastError());
     return KDA_OK;
