@@ -7,7 +7,7 @@
 //          StrictTril((Gamma.K)(K/Gamma)^T) (a2) and Aqk = Tril((Gamma.Q)(K/Gamma)^T) (a5),
 //          T = (I + . Diag(beta))^-1 (a3; Diag(beta) T = (I + Akk)^-1 Diag(beta)), W = Diag(beta) T (Gamma.K),
 //          U = Diag(beta) T V (a4).  Writes W, U, Gamma.Q, (gamma^C/Gamma).K, Aqk, gamma^C to a scratch tile.
-//   inter  one CTA per (sequence, head, 16-column slice of dv), sequential over the chunks:
+//   inter  one CTA per (sequence, head, 8- or 16-column slice of dv), sequential over the chunks:
 //          V_new = U - W S (a6), O = (Gamma.Q) S + Aqk V_new (a7),
 //          S <- Diag(gamma^C) S + ((gamma^C/Gamma).K)^T V_new (a8).  State columns are independent,
 //          which is what lets dv be sliced across CTAs.
@@ -18,8 +18,12 @@
 //
 // A call of this path is small (256 tokens x 2 heads: eight tiles), so what bounds it is the length of a tile's
 // chain of phases and of a chain step, not any throughput: 512 threads per tile, the substitution as
-// blocks, the operands of a chain phase fetched during the other.  Measured at 256 tokens x 2 heads: 41 us a call
-// (intra 23, inter 20, overlapping), 104 us with FMA products and a substitution of one thread per column.
+// blocks, the operands of a chain phase fetched during the other; a tile in three CTAs and a chain of 8 columns
+// where SMs would be idle.  Measured at 256 tokens x 2 heads: 29.7 us a call (intra 17, inter 16, overlapping),
+// 39.5 with one CTA per tile and 16 columns per chain, 104 us with FMA products and a substitution of one
+// thread per column; 2048 tokens x 8 heads: 155 us, 185 before.
+#include <type_traits>
+
 #include "kda_common.cuh"
 #include "kda_mma3.cuh"
 #include "kda_ptx.cuh"
@@ -60,12 +64,16 @@ constexpr int kFloats = VEC + 128 + 64 + 512;
 constexpr size_t kSmem1 = (size_t)s1::kFloats * 4;
 static_assert(kSmem1 <= 232448, "fits the shared memory of one SM");
 
+template <bool whole>
 __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __restrict__ tiles, WsHeader* hdr)
 {
     extern __shared__ __align__(16) float sm[];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int h = blockIdx.y;
     const int64_t gc_idx = a.g0 + blockIdx.x;
+    // a tile whole, or in three parts
+    const bool part_w = whole || blockIdx.z == 0, part_u = whole || blockIdx.z == 1,
+               part_q = whole || blockIdx.z == 2;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
     const ChunkLoc loc = locate_chunk(a, gc_idx);
@@ -87,9 +95,9 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
         const bool in = r < loc.len;
         G[i] = in ? a.log_alpha[off] : 0.f;
         kk[i] = in ? kp[off] : 0.f;
-        qq[i] = in && qp ? qp[off] : 0.f;
+        qq[i] = in && qp && part_q ? qp[off] : 0.f;
     }
-    for (int idx = t; idx < 64 * 32; idx += kT1) {
+    for (int idx = part_u ? t : 64 * 32; idx < 64 * 32; idx += kT1) {
         const int r = idx >> 5, x = (idx & 31) * 4;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (r < loc.len) v = *reinterpret_cast<const float4*>(vp + ((size_t)(loc.tok0 + r) * a.H + h) * kD + x);
@@ -120,31 +128,34 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
         const float e1 = expf(clampf(g - gm)), e2 = expf(clampf(gm - g));
         sKG[r * LR + c] = kk[i] * e1;
         sKI[r * LR + c] = kk[i] * e2;
-        const float x = a.scale * qq[i] * e1;
-        sQG[r * LR + c] = x;
-        tile[T_QG + r * kD + c] = x * em;
-        tile[T_KT + r * kD + c] = kk[i] * expf(total - g);
+        if (part_q) {
+            const float x = a.scale * qq[i] * e1;
+            sQG[r * LR + c] = x;
+            tile[T_QG + r * kD + c] = x * em;
+            tile[T_KT + r * kD + c] = kk[i] * expf(total - g);
+        }
     }
     if (seg == 0) {
         sEm[c] = em;
-        tile[T_GC + c] = expf(total);
+        if (part_q) tile[T_GC + c] = expf(total);
     }
     const int far = __syncthreads_or(total < kSplitRange);
 
-    // a2 + a5: [K^ ; Q] K_^T: warps 4 x 4, 32 x 16 entries each; only blocks that reach the triangle
-    {
-        const int mi = w >> 2, ni = w & 3, r0 = (mi & 1) * 32, c0 = ni * 16;
-        const float* A = (mi < 2 ? sKG : sQG) + r0 * LR;
-        float acc[2][2][4];
+    // a2 + a5: [K^ ; Q] K_^T: warps 4 x 4, 32 x 16 entries each of 128 rows, or 16 x 16 of 64; only blocks that
+    // reach the triangle
+    auto gram = [&](auto tag, bool is_q, int r0, int c0) {
+        constexpr int MT = decltype(tag)::value;
+        const float* A = (is_q ? sQG : sKG) + r0 * LR;
+        float acc[MT][2][4];
         zero(acc);
-        if (c0 < r0 + 32 && (mi < 2 || qp)) {
+        if (c0 < r0 + 16 * MT && (!is_q || qp)) {
             if (!far) {
                 gemm<0, 2, false, true, false, false>(acc, A, LR, sKI + c0 * LR, LR, 0, kD, lane);
             } else {
                 const int g = lane >> 2, c2 = 2 * (lane & 3);
                 for (int k = 0; k < kD; ++k)
 #pragma unroll
-                    for (int m = 0; m < 2; ++m)
+                    for (int m = 0; m < MT; ++m)
 #pragma unroll
                         for (int n = 0; n < 2; ++n)
 #pragma unroll
@@ -155,13 +166,16 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
         }
         each_pair(acc, lane, [&](int i, int j, float x, float y) {
             i += r0; j += c0;
-            if (mi < 2) {
+            if (!is_q) {
                 st2(sB + i * LM + j, j < i ? x * sBeta[j] : 0.f, j + 1 < i ? y * sBeta[j + 1] : 0.f);
             } else {
                 st2(tile + T_AQK + i * kC + j, j <= i ? x : 0.f, j + 1 <= i ? y : 0.f);
             }
         });
-    }
+    };
+    if (whole) gram(std::integral_constant<int, 2>{}, w >= 8, ((w >> 2) & 1) * 32, (w & 3) * 16);
+    else gram(std::integral_constant<int, 1>{}, part_q, (w >> 2) * 16, (w & 3) * 16);
+    if (!part_w && !part_u) return;
     __syncthreads();
     invert_unit_lower<LM>(sB, sT, t);      // a3
 
@@ -170,11 +184,12 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
         const int r0 = (w >> 3) * 32, c0 = (w & 7) * 16;
         float acc[2][2][4];
         zero(acc);
-        gemm<0, 2, false, false, false, false>(acc, sT + r0 * LM, LM, sKG + c0, LR, 0, r0 + 32, lane);
-        each_pair(acc, lane, [&](int i, int j, float x, float y) {
+        if (part_w) gemm<0, 2, false, false, false, false>(acc, sT + r0 * LM, LM, sKG + c0, LR, 0, r0 + 32, lane);
+        if (part_w) each_pair(acc, lane, [&](int i, int j, float x, float y) {
             const float b = sBeta[r0 + i];
             st2(tile + T_W + (r0 + i) * kD + c0 + j, b * x * sEm[c0 + j], b * y * sEm[c0 + j + 1]);
         });
+        if (!part_u) return;
         zero(acc);
         gemm<0, 2, false, false, false, false>(acc, sT + r0 * LM, LM, sV + c0, LC, 0, r0 + 32, lane);
         each_pair(acc, lane, [&](int i, int j, float x, float y) {
@@ -184,26 +199,27 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
     }
 }
 
-constexpr int NS = 16;               // dv columns per inter-chunk CTA
 constexpr int kT2 = 256;
-constexpr int LS = NS + 8;
-namespace s2 {
-constexpr int W = 0;                 // [64][LR]   operands of the first phase: W, Gamma.Q, U
-constexpr int Q = W + 64 * LR;       // [64][LR]
-constexpr int U = Q + 64 * LR;       // [64][LS]
-constexpr int KT = U + 64 * LS;      // [64][LC]   operands of the second: (gamma^C/Gamma).K, Aqk
-constexpr int A = KT + 64 * LC;      // [64][LM]
-constexpr int S = A + 64 * LM;       // [128][LS]  state
-constexpr int VN = S + 128 * LS;     // [64][LS]   V_new
-constexpr int kFloats = VN + 64 * LS;
-}  // namespace s2
-constexpr size_t kSmem2 = (size_t)s2::kFloats * 4;
+template <int NS> struct s2 {                           // NS = dv columns per inter-chunk CTA
+    static constexpr int LS = NS == 8 ? 8 : NS + 8;
+    static constexpr int W = 0;                 // [64][LR]   operands of the first phase: W, Gamma.Q, U
+    static constexpr int Q = W + 64 * LR;       // [64][LR]
+    static constexpr int U = Q + 64 * LR;       // [64][LS]
+    static constexpr int KT = U + 64 * LS;      // [64][LC]   operands of the second: (gamma^C/Gamma).K, Aqk
+    static constexpr int A = KT + 64 * LC;      // [64][LM]
+    static constexpr int S = A + 64 * LM;       // [128][LS]  state
+    static constexpr int VN = S + 128 * LS;     // [64][LS]   V_new
+    static constexpr size_t kBytes = (size_t)(VN + 64 * LS) * 4;
+};
 
 // Eight warps of 16 rows each.  First phase: [W ; Gamma.Q] S (128 rows); second: Aqk V_new into the output rows
 // of warps 4-7, and the state's 128 rows, which stay in the accumulator fragments of all warps (copy in
 // shared memory as B operand).  The operands of each phase arrive by cp.async during the other.
+template <int NS>
 __global__ void __launch_bounds__(kT2, 1) kda_inter_f32(ChunkArgs a, const float* __restrict__ tiles, int n_begin)
 {
+    using L = s2<NS>;
+    constexpr int LS = L::LS, NT = NS / 8;
     extern __shared__ __align__(16) float sm[];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5, g = lane >> 2;
     const int h = blockIdx.y, n = n_begin + blockIdx.z;
@@ -229,12 +245,12 @@ __global__ void __launch_bounds__(kT2, 1) kda_inter_f32(ChunkArgs a, const float
         const float* tile = tile_of(ch);
         for (int idx = t; idx < 64 * 32; idx += kT2) {
             const int r = idx >> 5, x = (idx & 31) * 4;
-            cp16(sm + s2::W + r * LR + x, tile + T_W + r * kD + x);
-            if (op) cp16(sm + s2::Q + r * LR + x, tile + T_QG + r * kD + x);
+            cp16(sm + L::W + r * LR + x, tile + T_W + r * kD + x);
+            if (op) cp16(sm + L::Q + r * LR + x, tile + T_QG + r * kD + x);
         }
         for (int idx = t; idx < 64 * (NS / 4); idx += kT2) {
             const int r = idx / (NS / 4), x = idx % (NS / 4) * 4;
-            cp16(sm + s2::U + r * LS + x, tile + T_U + r * kD + col0 + x);
+            cp16(sm + L::U + r * LS + x, tile + T_U + r * kD + col0 + x);
         }
         cp_commit();
     };
@@ -242,23 +258,23 @@ __global__ void __launch_bounds__(kT2, 1) kda_inter_f32(ChunkArgs a, const float
         const float* tile = tile_of(ch);
         for (int idx = t; idx < 64 * 32; idx += kT2) {
             const int r = idx >> 5, x = (idx & 31) * 4;
-            cp16(sm + s2::KT + r * LC + x, tile + T_KT + r * kD + x);
+            cp16(sm + L::KT + r * LC + x, tile + T_KT + r * kD + x);
         }
         if (op)
             for (int idx = t; idx < 64 * 16; idx += kT2) {
                 const int r = idx >> 4, x = (idx & 15) * 4;
-                cp16(sm + s2::A + r * LM + x, tile + T_AQK + r * kC + x);
+                cp16(sm + L::A + r * LM + x, tile + T_AQK + r * kC + x);
             }
         cp_commit();
     };
 
     if (cb < ce) { fetch1(cb); fetch2(cb); }
     const size_t sbase = ((size_t)n * a.H + h) * (size_t)(kD * kD) + col0;
-    float* sS = sm + s2::S;
-    float* sVn = sm + s2::VN;
-    float S[1][2][4];
+    float* sS = sm + L::S;
+    float* sVn = sm + L::VN;
+    float S[1][NT][4];
 #pragma unroll
-    for (int nt = 0; nt < 2; ++nt)
+    for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
             const int r = 16 * w + 8 * hf + g, x = 8 * nt + 2 * (lane & 3);
@@ -272,29 +288,29 @@ __global__ void __launch_bounds__(kT2, 1) kda_inter_f32(ChunkArgs a, const float
     for (int64_t ch = cb; ch < ce; ++ch) {
         const float* tile = tile_of(ch);
         const float gam0 = tile[T_GC + 16 * w + g], gam1 = tile[T_GC + 16 * w + 8 + g];
-        float acc[1][2][4];
+        float acc[1][NT][4];
         zero(acc);
         if (w < 4 || op)
-            gemm<0, 2, false, false, false, false>(acc, sm + (w < 4 ? s2::W + 16 * w * LR : s2::Q + 16 * (w - 4) * LR), LR, sS,
+            gemm<0, NT, false, false, false, false>(acc, sm + (w < 4 ? L::W + 16 * w * LR : L::Q + 16 * (w - 4) * LR), LR, sS,
                                                    LS, 0, kD, lane);
         if (w < 4)
             each_pair(acc, lane, [&](int i, int j, float x, float y) {
-                const float2 u = *reinterpret_cast<const float2*>(sm + s2::U + (16 * w + i) * LS + j);
+                const float2 u = *reinterpret_cast<const float2*>(sm + L::U + (16 * w + i) * LS + j);
                 st2(sVn + (16 * w + i) * LS + j, u.x - x, u.y - y);
             });
         cp_wait0();
         __syncthreads();
         if (ch + 1 < ce) fetch1(ch + 1);
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
+        for (int nt = 0; nt < NT; ++nt) {
             S[0][nt][0] *= gam0; S[0][nt][1] *= gam0;
             S[0][nt][2] *= gam1; S[0][nt][3] *= gam1;
         }
-        gemm<0, 2, true, false, false, false>(S, sm + s2::KT + 16 * w, LC, sVn, LS, 0, kC, lane);
+        gemm<0, NT, true, false, false, false>(S, sm + L::KT + 16 * w, LC, sVn, LS, 0, kC, lane);
         each_pair(S, lane, [&](int i, int j, float x, float y) { st2(sS + (16 * w + i) * LS + j, x, y); });
         if (w >= 4 && op) {
             const int r0 = 16 * (w - 4);
-            gemm<0, 2, false, false, false, false>(acc, sm + s2::A + r0 * LM, LM, sVn, LS, 0, r0 + 16, lane);
+            gemm<0, NT, false, false, false, false>(acc, sm + L::A + r0 * LM, LM, sVn, LS, 0, r0 + 16, lane);
             const int64_t tok0 = tok_begin + (ch - seq_c0) * kC;
             each_pair(acc, lane, [&](int i, int j, float x, float y) {
                 const int64_t tok = tok0 + r0 + i;
@@ -351,14 +367,23 @@ size_t f32_tile_bytes() { return (size_t)T_FLOATS * sizeof(float); }
 
 kda_status_t launch_chunk_f32(const ChunkArgs& a, void* tiles, int n_begin, int n_count, WsHeader* hdr, cudaStream_t st)
 {
+    int n_sm = 0;
     {
         DeviceLock lk;
         if (!lk.st) return lk.rc;
         if (!lk.st->attr_done[4]) {
-            KDA_CUDA_TRY(cudaFuncSetAttribute(kda_intra_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem1));
-            KDA_CUDA_TRY(cudaFuncSetAttribute(kda_inter_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem2));
+            KDA_CUDA_TRY(cudaFuncSetAttribute(kda_intra_f32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem1));
+            KDA_CUDA_TRY(cudaFuncSetAttribute(kda_intra_f32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem1));
+            KDA_CUDA_TRY(cudaFuncSetAttribute(kda_inter_f32<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s2<8>::kBytes));
+            KDA_CUDA_TRY(cudaFuncSetAttribute(kda_inter_f32<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s2<16>::kBytes));
             lk.st->attr_done[4] = true;
         }
+        if (lk.st->n_sm == 0) {
+            int dev = 0;
+            KDA_CUDA_TRY(cudaGetDevice(&dev));
+            KDA_CUDA_TRY(cudaDeviceGetAttribute(&lk.st->n_sm, cudaDevAttrMultiProcessorCount, dev));
+        }
+        n_sm = lk.st->n_sm;
     }
     if (n_count > 65535)
         return fail(KDA_ERR_UNSUPPORTED, "kda_chunk_fwd: more than 65535 sequences in one fp32 call");
@@ -366,13 +391,21 @@ kda_status_t launch_chunk_f32(const ChunkArgs& a, void* tiles, int n_begin, int 
     float* tp = static_cast<float*>(tiles);
     if (n_chunks > 0) {
         ProfScope ps(PROF_INTRA, st);
-        KDA_CUDA_TRY(launch_dependent(kda_intra_f32, dim3((unsigned)n_chunks, (unsigned)a.H), kT1, kSmem1, st, a, tp, hdr));
+        // three CTAs per tile (W; U; Aqk and what is only gated) while there are SMs for all: each repeats the
+        // gating, and W and U the Gram matrix and its inverse, so more of them cost work but no time
+        const bool parts = n_chunks * a.H * 3 <= n_sm;
+        KDA_CUDA_TRY(launch_dependent(parts ? kda_intra_f32<false> : kda_intra_f32<true>,
+                                      dim3((unsigned)n_chunks, (unsigned)a.H, parts ? 3 : 1), kT1, kSmem1, st, a, tp, hdr));
         count_launch();
     }
     if (n_count > 0) {
         ProfScope ps(PROF_INTER, st);
-        KDA_CUDA_TRY(launch_dependent(kda_inter_f32, dim3(kD / NS, (unsigned)a.H, (unsigned)n_count), kT2, kSmem2, st, a,
-                                      (const float*)tp, n_begin));
+        const dim3 grid16(kD / 16, (unsigned)a.H, (unsigned)n_count), grid8(kD / 8, (unsigned)a.H, (unsigned)n_count);
+        // a chain step is a latency, shorter for fewer columns: 8 as long as those CTAs have an SM each
+        if ((int64_t)(kD / 8) * a.H * n_count <= n_sm)
+            KDA_CUDA_TRY(launch_dependent(kda_inter_f32<8>, grid8, kT2, s2<8>::kBytes, st, a, (const float*)tp, n_begin));
+        else
+            KDA_CUDA_TRY(launch_dependent(kda_inter_f32<16>, grid16, kT2, s2<16>::kBytes, st, a, (const float*)tp, n_begin));
         count_launch();
     }
     return KDA_OK;

@@ -41,7 +41,9 @@ __device__ __forceinline__ void gemm(float (&acc)[MT][NT][4], const float* __res
     const int sbn = BT ? ldb : 1, sbk = BT ? 1 : ldb;
     const float* pa = A + g * sam + (k0 + c) * sak;
     const float* pb = B + g * sbn + (k0 + c) * sbk;
-#pragma unroll 2
+    // (steps depend on each other through the additions to acc alone: small blocks overlap more of them)
+    constexpr int kUnroll = MT * NU == 1 ? 4 : 2;
+#pragma unroll kUnroll
     for (int k = k0; k < k1; k += 8, pa += 8 * sak, pb += 8 * sbk) {
         uint32_t ah[MT][4], al[MT][4], bh[NU][2], bl[NU][2];
 #pragma unroll
