@@ -272,20 +272,24 @@ struct LayerMode {
     const float* rate = nullptr;
     const float* bias = nullptr;
     float l2_eps = 0.f;
-    const void* out_gate = nullptr;     // non-null: the output stage runs inside the inter-chunk kernel
+    const void* out_gate = nullptr;     // non-null: output stage from fp32 rows, pass by pass
     const float* rms_weight = nullptr;
     float rms_eps = 0.f;
 };
 
-// Whether a bf16 call runs as the fused kernel (kda_set_chunk_path).
-bool use_fused(int n_seqs, int H, int64_t total_chunks, size_t workspace_bytes, bool layer, bool has_q)
+// Whether a bf16 call without the layer's functions runs as the fused kernel (kda_set_chunk_path).  It does where
+// the tiles of all chunks do not fit the workspace, and where the chains fit one wave of clusters (37 of four CTAs)
+// with enough tiles to make up for the first ones of each chain, which nothing overlaps: 8 heads x 4096 tokens 101
+// (fused) / 100 us (two kernels), 32 x 1000 42.5 / 43.8, 32 x 4096 113 / 143, 16 x 131072 2720 / 3360; below,
+// 32 x 400 25.5 / 24.1, 8 x 1000 37.7 / 31.5; above, 64 chains 105 / 105, 128 chains 202 / 178, 512 chains 3200 / 2900.
+// Layer calls: never faster (96 chains 294 / 237 us, 8 heads x 4096 145 / 113).
+bool use_fused(int n_seqs, int H, int64_t total_chunks, size_t workspace_bytes)
 {
     const int mode = g_chunk_path.load(std::memory_order_relaxed);
-    if (mode != 0) return mode == 2 && (!layer || workspace_bytes >= kFusedRing + 2 * tc_tile_bytes());
+    if (mode != 0) return mode == 2;
     const size_t fixed = ws_layout(n_seqs, H).fixed, row = (size_t)H * tc_tile_bytes();
     const bool one_pass = workspace_bytes >= fixed && (int64_t)((workspace_bytes - fixed) / row) >= total_chunks;
-    if (layer && workspace_bytes < kFusedRing + 2 * tc_tile_bytes()) return false;
-    return !one_pass || (int64_t)n_seqs * H <= (layer ? 37 : 148);
+    return !one_pass || ((int64_t)n_seqs * H <= 37 && total_chunks * H >= 512);
 }
 
 // Cluster shape, number of clusters and ring depth of a call of the fused kernel.
@@ -299,7 +303,7 @@ kda_status_t fused_schedule(FusedArgs& f, const std::vector<int64_t>& chunk_cu, 
     if (most[0] < 1 && most[1] < 1) return fail(KDA_ERR_UNSUPPORTED, "kda_chunk_fwd: the device holds no cluster of the fused kernel");
     // Two or three engine CTAs per chain: microseconds a tile costs the chain and an engine (measured), times the
     // tiles of the most loaded cluster.
-    const double chain = has_q ? 1.5 : 1.3, engine = f.a.gate_rate ? 9.5 : has_q ? 8.0 : 7.5;
+    const double chain = has_q ? 1.5 : 1.3, engine = has_q ? 8.0 : 7.5;
     double best = 0.;
     for (int i = 0; i < 2; ++i) {
         if (most[i] < 1) continue;
@@ -402,7 +406,7 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
         }
         f.epoch = next_epoch();
     }
-    if (dt == KDA_BF16 && use_fused(n_seqs, H, total_chunks, workspace_bytes, lm.rate != nullptr, q && o)) {
+    if (dt == KDA_BF16 && !lm.rate && use_fused(n_seqs, H, total_chunks, workspace_bytes)) {
         const size_t tbf = tc_tile_bytes();
         if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) || workspace_bytes < kFusedRing + 2 * tbf)
             return fail(KDA_ERR_WORKSPACE, "kda_chunk_fwd: workspace must be 256-byte aligned and at "
@@ -419,8 +423,6 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
         f.a.total_tokens = total_tokens; f.a.seq_len = seq_len; f.a.chunks_per_seq = chunks_per_seq;
         f.a.g0 = 0; f.a.g1 = total_chunks; f.a.scale = scale;
         f.a.wait_limit_ns = wait_limit_ns();
-        f.a.gate_rate = lm.rate; f.a.gate_bias = lm.bias; f.a.l2_eps = lm.l2_eps;
-        f.a.out_gate = lm.out_gate; f.a.rms_weight = lm.rms_weight; f.a.rms_eps = lm.rms_eps;
         f.ring = wsb + kFusedRing;
         const kda_status_t rcf = fused_schedule(f, chunk_cu, (int64_t)((workspace_bytes - kFusedRing) / tbf), q && o);
         if (rcf != KDA_OK) return rcf;
@@ -456,7 +458,7 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
     a.S_out = state;
     a.gate_rate = lm.rate; a.gate_bias = lm.bias; a.l2_eps = lm.l2_eps;
     a.wait_limit_ns = wait_limit_ns();
-    a.out_gate = lm.out_gate; a.rms_weight = lm.rms_weight; a.rms_eps = lm.rms_eps;
+    a.rows32 = lm.out_gate != nullptr;
 
     int64_t g0 = 0;
     bool first = true;
@@ -480,6 +482,7 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
             f.n_begin = n_begin;
             f.ordered = f.ordered && n_count == n_seqs;
             if (rc == KDA_OK && n_count > 0) rc = launch_chain_tc(f, n_count, st);
+            if (rc == KDA_OK && a.rows32) rc = launch_layer_rows(a, ws + L.off_tiles, o, lm.out_gate, lm.rms_weight, lm.rms_eps, st);
         } else
             rc = launch_chunk_f32(a, ws + L.off_tiles, n_begin, n_count, hdr, st);
         if (rc != KDA_OK) return rc;
@@ -541,7 +544,8 @@ kda_status_t kda_layer_fwd(const void* q_c, const void* k_c, const void* v, cons
                                        "aligned", p);
     LayerMode lm;
     lm.rate = A_log; lm.bias = dt_bias; lm.l2_eps = l2_eps;
-    // The output stage runs where the output rows are formed, unless a pass of its own is asked for.
+    // The output stage starts from fp32 rows where the chains are few (their tiles are still in L2 when it runs),
+    // unless bf16 rows are asked for, and from the bf16 output in place otherwise.
     const bool fuse_out = y && total_tokens > 0 && n_seqs > 0 && g_fuse_output.load(std::memory_order_relaxed) &&
                           (int64_t)n_seqs * H <= 37;
     if (fuse_out) {

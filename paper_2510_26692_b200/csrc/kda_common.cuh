@@ -71,14 +71,10 @@ struct ChunkArgs {
     const float* gate_rate = nullptr;   // [H]
     const float* gate_bias = nullptr;   // [H, dk]
     float l2_eps = 0.f;
-    // Output stage of the layer wrap inside the inter-chunk kernel (off when out_gate is nullptr):
-    // o is replaced by sigmoid(out_gate) . RMSNorm(o) . rms_weight before it is stored.
     // Upper bound of every device-side wait of the tensor-core kernels (ns); set from the environment
     // variable KDA_WAIT_LIMIT_MS by the host entry points (default 1 s).
     unsigned long long wait_limit_ns = 1000000000ull;
-    const void* out_gate = nullptr;     // bf16 [T_total, H, dv]
-    const float* rms_weight = nullptr;  // [dv]
-    float rms_eps = 0.f;
+    bool rows32 = false;                // bf16 layer calls: output rows in fp32, left in the scratch tiles
 };
 
 // Work description of the fused bf16 chunk-forward kernel and of the two kernels of the two-kernel schedule.
@@ -208,6 +204,8 @@ struct DeviceLock {
 DeviceState* device_slot(int ordinal);
 
 // output stage of the layer wrap: y = sigmoid(g_o) . RMSNorm(y) . w in place, rows of kD bf16 values
+kda_status_t launch_layer_rows(const ChunkArgs& a, const void* tiles, void* y, const void* g_o, const float* w, float eps,
+                               cudaStream_t st);
 kda_status_t launch_layer_epilogue(void* y, const void* g_o, const float* w, float eps, int64_t n_rows,
                                    cudaStream_t st);
 

@@ -97,10 +97,8 @@ constexpr int kStagesA = 2, kStagesB = 3;
 constexpr uint32_t kABytes = 32768, kBBytes = tc::TILE_BYTES - tc::OFF_KI;   // B: K', Aqk, gate vectors, U^T
 constexpr uint32_t C_STAGEB = (kBBytes + 1023) / 1024 * 1024;
 constexpr uint32_t C_A = 0, C_B = kStagesA * kABytes;
-constexpr uint32_t C_OUT = C_B + kStagesB * C_STAGEB;   // output block [2][64 tokens][64] bf16
-constexpr uint32_t C_GATE = C_OUT + 16384;              // layer mode: output gates of the same rows
-constexpr uint32_t C_SSQ = C_GATE + 16384;              // layer mode: [2][64][4] fp32 row sums of squares
-constexpr uint32_t C_BAR = C_SSQ + 2048;
+constexpr uint32_t C_OUT = C_B + kStagesB * C_STAGEB;   // output block: [2][64 tokens][64] bf16, or 64 rows in fp32
+constexpr uint32_t C_BAR = C_OUT + 32768;
 constexpr uint32_t C_BYTES = C_BAR + 512;
 // offsets inside a B stage
 constexpr uint32_t B_KI = 0, B_AQ = tc::OFF_AQ - tc::OFF_KI, B_GV = tc::OFF_GV - tc::OFF_KI, B_U = tc::OFF_U - tc::OFF_KI;
@@ -167,6 +165,11 @@ __device__ __forceinline__ void block16_store(float* pc, const float (&acc)[2][4
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float lg2(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
@@ -330,8 +333,8 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
                     asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];"
                                  : "=r"(lo), "=r"(hi)
                                  : "l"(gp + (size_t)i * a.H * kD));
-                G[r][0] = __uint_as_float(lo << 16); G[r][1] = __uint_as_float(lo & 0xffff0000u);
-                G[r][2] = __uint_as_float(hi << 16); G[r][3] = __uint_as_float(hi & 0xffff0000u);
+                G[r][0] = __uint_as_float(lo);    // (unpacked when they are used: nothing here waits for the loads)
+                G[r][1] = __uint_as_float(hi);
             }
             rate = a.gate_rate[D.h];
             const float4 b4 = *reinterpret_cast<const float4*>(a.gate_bias + (size_t)D.h * kD + d0);
@@ -433,24 +436,33 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         KT_MARK(te == 0, 0);   // loop overhead
 
         if (kLayer) {
-            // log alpha = -exp(rate) * softplus(x + bias); rows past the end of the sequence do not decay
+            // log2 alpha = -exp(rate) * log2(1 + e^(x + bias)); rows past the end of the sequence do not decay
             const float nr = -__expf(rate);
+            float b2[4];
 #pragma unroll
-            for (int r = 0; r < kRPT; ++r)
+            for (int e = 0; e < 4; ++e) b2[e] = bias[e] * kLog2e;
+#pragma unroll
+            for (int r = 0; r < kRPT; ++r) {
+                const uint32_t lo = __float_as_uint(G[r][0]), hi = __float_as_uint(G[r][1]);
+                const float x[4] = {__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u), __uint_as_float(hi << 16),
+                                    __uint_as_float(hi & 0xffff0000u)};
+                const float nrr = i0 + r < d_len ? nr : 0.f;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const float x = G[r][e] + bias[e];
-                    const float sp = fmaxf(x, 0.f) + __logf(1.f + __expf(-fabsf(x)));
-                    G[r][e] = (i0 + r < d_len) ? nr * sp : 0.f;
+                    const float x2 = fmaf(x[e], kLog2e, b2[e]);
+                    G[r][e] = fmaf(nrr, fmaxf(x2, 0.f) + lg2(1.f + ex2(-fabsf(x2))), r > 0 ? G[r - 1][e] : 0.f);
                 }
+            }
         }
         // ---- a1: cumulative log-decay, in the log2 domain (exponentials below are bare ex2) ---------
+        if (!kLayer) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) G[0][e] *= kLog2e;
+            for (int e = 0; e < 4; ++e) G[0][e] *= kLog2e;
 #pragma unroll
-        for (int r = 1; r < kRPT; ++r)
+            for (int r = 1; r < kRPT; ++r)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) G[r][e] = fmaf(G[r][e], kLog2e, G[r - 1][e]);
+                for (int e = 0; e < 4; ++e) G[r][e] = fmaf(G[r][e], kLog2e, G[r - 1][e]);
+        }
         *reinterpret_cast<float4*>(sTot + warp * kD + d0) =
             make_float4(G[kRPT - 1][0], G[kRPT - 1][1], G[kRPT - 1][2], G[kRPT - 1][3]);
         ptx::cp_async_wait_all();             // beta
@@ -897,16 +909,12 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 //   warps 0-7  compute: TMEM lane quadrant = warp & 3, half of dk / of the tokens = warp >> 2
 //   warp 8 issues the MMAs, warp 9 lane 0 loads the tiles, warps 12-15 write the output rows
 // kRing: tiles come from the engines of the cluster; otherwise from the plain array that the intra-chunk kernel
-// has written, and `cid` numbers the (sequence, head) pairs.
-__device__ __forceinline__ float rcp_approx(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
+// has written, and `cid` numbers the (sequence, head) pairs.  kRows32 (layer calls): the output rows stay in fp32,
+// in the place of the tile's [W ; Q], for the output stage (kda_layer.cu).
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
-template <bool kHasQ, bool kLayer, bool kRing>
+template <bool kHasQ, bool kRows32, bool kRing>
 __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t, int cid, const CUtensorMap* tm_o)
 {
     const ChunkArgs& a = f.a;
@@ -1179,37 +1187,39 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
         // crowded out the loads of the compute warps: 2.6 instead of 1.6 us a step.)
         const int quad = warp & 3, ot = t - 384;
         const uint32_t tq = tm + ((uint32_t)(quad * 32) << 16);
-        float* ssq = reinterpret_cast<float*>(smem + C_SSQ);              // [2][64][4]
-        const bool epi = kLayer && a.out_gate != nullptr;
         // this lane's row of the four 8 x 8 matrices of token block 0, in the swizzled [2][64 tokens][64] image
         const uint32_t mrow = (uint32_t)(lane & 7), mcol = (uint32_t)((quad & 1) * 32 + (lane >> 3) * 8);
         const uint32_t moff = (uint32_t)(quad >> 1) * 8192u + ptx::sw128_off(mrow, mcol);
-        float wgt[4] = {0.f, 0.f, 0.f, 0.f};     // RMSNorm weights of this lane's four columns
-        if (epi)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) wgt[b] = a.rms_weight[quad * 32 + b * 8 + (lane >> 2)];
-        uint8_t* sg = smem + C_GATE;
-        uint4 gq[kLayer ? 8 : 1];        // gate pre-activations, 16-byte piece ot + 128 k of a [64][256 B] block
-        auto load_gates = [&](int64_t tok0, int len) {
-#pragma unroll
-            for (int k = 0; k < (kLayer ? 8 : 0); ++k) {
-                const int idx = ot + 128 * k, row = idx >> 4;
-                gq[k] = make_uint4(0u, 0u, 0u, 0u);
-                if (row < len)
-                    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                                 : "=r"(gq[k].x), "=r"(gq[k].y), "=r"(gq[k].z), "=r"(gq[k].w)
-                                 : "l"(reinterpret_cast<const __nv_bfloat16*>(a.out_gate) + ((size_t)(tok0 + row) * a.H + J.h) * kD + (idx & 15) * 8));
-            }
-        };
         uint32_t g = 0;
         for (int r = 0; next_job(r) && !*abort_flag; ++r)
             for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
                 const int64_t tok0 = J.tok_begin + (int64_t)c * kC;
                 const int len = (J.tok_end - tok0) < kC ? (int)(J.tok_end - tok0) : kC;
-                if (kLayer && epi && c == 0) load_gates(tok0, len);
                 wait(&out_bar[g & 1u], (g >> 1) & 1u, 10);
                 __syncwarp();
                 ptx::tc_fence_after();
+                if (kRows32) {     // lane = column, four tokens a piece
+                    uint32_t y[2][32];
+                    ptx::tmem_ld_32x32b_x32(tq + T_D1 + (g & 1u) * 128u + 64, y[0]);
+                    ptx::tmem_ld_32x32b_x32(tq + T_D1 + (g & 1u) * 128u + 96, y[1]);
+                    ptx::tmem_ld_wait();
+                    ptx::tc_fence_before();
+                    warp_arrive(&o_done[g & 1u]);
+                    if (ot == 0) ptx::bulk_wait_read0();      // the previous block has been read out of its buffer
+                    ptx::named_bar_sync(6, 128);
+                    uint4* rows = reinterpret_cast<uint4*>(smem + C_OUT) + ot;
+#pragma unroll
+                    for (int q = 0; q < 16; ++q)
+                        rows[q * 128] = make_uint4(y[q >> 3][4 * (q & 7)], y[q >> 3][4 * (q & 7) + 1], y[q >> 3][4 * (q & 7) + 2],
+                                                   y[q >> 3][4 * (q & 7) + 3]);
+                    ptx::fence_async_smem();
+                    ptx::named_bar_sync(6, 128);
+                    if (ot == 0 && !*abort_flag) {
+                        ptx::bulk_s2g(f.ring + (size_t)(J.tile0 + (int64_t)c * a.H) * tc::TILE_BYTES + tc::OFF_O32, smem + C_OUT, 32768);
+                        ptx::bulk_commit();
+                    }
+                    continue;
+                }
                 // y[b >> 1][4 j + 2 (b & 1) + e]: column 8 b + lane / 4 of the quadrant, token 8 j + 2 (lane % 4) + e
                 uint32_t y[2][32];
                 ptx::tmem_ld_16x256b_x8(tq + T_D1 + (g & 1u) * 128u + 64, y[0]);
@@ -1217,59 +1227,6 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                 ptx::tmem_ld_wait();
                 ptx::tc_fence_before();
                 warp_arrive(&o_done[g & 1u]);
-                if (kLayer && epi) {
-                    // the gate block next to the output block, the row sums of squares of this quadrant beside them
-#pragma unroll
-                    for (int k = 0; k < (kLayer ? 8 : 0); ++k) {
-                        const int idx = ot + 128 * k, ch = idx & 15;
-                        *reinterpret_cast<uint4*>(sg + (ch >> 3) * 8192 + ptx::sw128_off((uint32_t)(idx >> 4), (uint32_t)(ch & 7) * 8)) = gq[k];
-                    }
-                    if (c + 1 < J.nch) {     // the next chunk's gates are on their way while this one's are used
-                        const int64_t left = J.tok_end - tok0 - kC;
-                        load_gates(tok0 + kC, left < kC ? (int)left : kC);
-                    }
-                    float q[16];
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        q[i] = 0.f;
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) {
-                            const float v = __uint_as_float(y[b >> 1][4 * (i >> 1) + 2 * (b & 1) + (i & 1)]);
-                            q[i] = fmaf(v, v, q[i]);
-                        }
-                    }
-#pragma unroll
-                    for (int n = 8, x = 16; n >= 2; n >>= 1, x >>= 1) {   // over the eight lanes that share a token: two tokens each
-                        const bool up = (lane & x) != 0;
-#pragma unroll
-                        for (int i = 0; i < n; ++i) {
-                            const float send = up ? q[i] : q[i + n], keep = up ? q[i + n] : q[i];
-                            q[i] = keep + __shfl_xor_sync(0xffffffffu, send, x);
-                        }
-                    }
-                    // lane bits 4, 3, 2 have chosen the token block's bits 2, 1, 0
-                    const int jb = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
-                    float* sq = ssq + (g & 1u) * 256;
-                    sq[(8 * jb + 2 * (lane & 3)) * 4 + quad] = q[0];
-                    sq[(8 * jb + 2 * (lane & 3) + 1) * 4 + quad] = q[1];
-                    ptx::named_bar_sync(5, 128);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        uint32_t gt[4];
-                        ptx::ldmatrix_x4_trans(sg + moff + j * 1024, gt);
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const float4 p = *reinterpret_cast<const float4*>(sq + (8 * j + 2 * (lane & 3) + e) * 4);
-                            const float rstd = rsqrtf(((p.x + p.y) + (p.z + p.w)) * (1.f / kD) + a.rms_eps);
-#pragma unroll
-                            for (int b = 0; b < 4; ++b) {
-                                uint32_t& v = y[b >> 1][4 * j + 2 * (b & 1) + e];
-                                const float gv = e ? bf16_hi(gt[b]) : bf16_lo(gt[b]);
-                                v = __float_as_uint(__uint_as_float(v) * (rstd * wgt[b]) * rcp_approx(1.f + __expf(-gv)));
-                            }
-                        }
-                    }
-                }
                 // the previous block has been read out of its buffer
                 uint8_t* sb = smem + C_OUT;
                 if (ot == 0) ptx::bulk_wait_read0();
@@ -1328,7 +1285,7 @@ __device__ void chain_init(uint8_t* smem)
 // announces a tile once its copies have completed (performed at L2, where the chain's copies read), the chain
 // gives a position back once its copy has landed.  Neither arrival has anything of its own thread to order, so
 // both are relaxed (release arrivals and proxy fences in their place cost about a microsecond each).
-template <bool kHasQ, bool kLayer>
+template <bool kHasQ>
 __global__ void __launch_bounds__(kThreads, 1)
 kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtensorMap tm_k,
              const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_v,
@@ -1377,7 +1334,7 @@ kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     if ((ptx::smem_u32(smem) & 1023u) != 0) {   // the operand images need 1024-byte alignment
         if (t == 0) report_timeout(f, 90);
     } else if (chain_cta) {
-        chain_run<kHasQ, kLayer, true>(f, smem, tmem_base, t, cid, &tm_o);
+        chain_run<kHasQ, false, true>(f, smem, tmem_base, t, cid, &tm_o);
     } else {
         const int sub = ptx::warp_uniform(t / kEngThreads), e = (rank - 1) * 2 + sub;
         if (e < f.n_eng) {
@@ -1385,7 +1342,7 @@ kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
             if (t - sub * kEngThreads == kServiceThread)
                 *reinterpret_cast<EngineCursor*>(es + E_CUR) = {
                     cid, e, 0, e, 0, ptx::map_to_cta(ptx::smem_u32(smem) + C_BAR + (uint32_t)(e * f.depth) * 8u, 0), 0, 0};
-            engine_run<kHasQ, true, kLayer>(f, es, tmem_base + sub * 256, 1 + sub, t - sub * kEngThreads, 0, 0, &tm_k, &tm_q, &tm_v);
+            engine_run<kHasQ, true>(f, es, tmem_base + sub * 256, 1 + sub, t - sub * kEngThreads, 0, 0, &tm_k, &tm_q, &tm_v);
         }
     }
     ptx::tc_fence_before();
@@ -1395,13 +1352,14 @@ kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
 }
 
 // ---- the chains alone (second kernel of the two-kernel schedule): a CTA per (sequence, head) -------------------
-template <bool kHasQ, bool kLayer>
+template <bool kHasQ, bool kRows32>
 __global__ void __launch_bounds__(kThreads, 1)
 kda_chain_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtensorMap tm_o)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     const int t = threadIdx.x, warp = t >> 5;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C_BAR + 500);
+    ptx::grid_dep_launch();   // (what follows waits for this kernel's end before it reads anything)
     if (t == 0) chain_init(smem);
     if (warp == 0) {
         ptx::tmem_alloc(tmem_slot, kTmemCols);
@@ -1414,7 +1372,7 @@ kda_chain_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     if ((ptx::smem_u32(smem) & 1023u) != 0) {
         if (t == 0) report_timeout(f, 90);
     } else {
-        chain_run<kHasQ, kLayer, false>(f, smem, tmem_base, t, (int)blockIdx.x, &tm_o);
+        chain_run<kHasQ, kRows32, false>(f, smem, tmem_base, t, (int)blockIdx.x, &tm_o);
     }
     ptx::tc_fence_before();
     __syncthreads();
@@ -1570,15 +1528,11 @@ kda_status_t launch_intra_tc(const ChunkArgs& a, void* tiles, WsHeader* hdr, boo
 namespace {
 using FusedFn = void (*)(FusedArgs, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap);
 using ChainFn = void (*)(FusedArgs, CUtensorMap);
-FusedFn fused_fn(bool has_q, bool layer)
+FusedFn fused_fn(bool has_q) { return has_q ? kda_fused_tc<true> : kda_fused_tc<false>; }
+ChainFn chain_fn(bool has_q, bool rows32)
 {
-    if (layer) return has_q ? kda_fused_tc<true, true> : kda_fused_tc<false, true>;
-    return has_q ? kda_fused_tc<true, false> : kda_fused_tc<false, false>;
-}
-ChainFn chain_fn(bool has_q, bool layer)
-{
-    if (layer) return has_q ? kda_chain_tc<true, true> : kda_chain_tc<false, true>;
-    return has_q ? kda_chain_tc<true, false> : kda_chain_tc<false, false>;
+    if (!has_q) return kda_chain_tc<false, false>;
+    return rows32 ? kda_chain_tc<true, true> : kda_chain_tc<true, false>;
 }
 void fused_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[2], int cluster, int n_clusters, cudaStream_t st)
 {
@@ -1602,8 +1556,8 @@ kda_status_t fused_max_clusters(int (&n)[2])
     DeviceLock lk;
     if (!lk.st) return lk.rc;
     if (!lk.st->attr_done[0]) {
-        for (int i = 0; i < 4; ++i)
-            KDA_CUDA_TRY(cudaFuncSetAttribute((const void*)fused_fn(i & 1, i & 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
+        for (int i = 0; i < 2; ++i)
+            KDA_CUDA_TRY(cudaFuncSetAttribute((const void*)fused_fn(i), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)kSmemBytes));
         for (int i = 0; i < 2; ++i) {
             cudaLaunchConfig_t cfg;
@@ -1611,7 +1565,7 @@ kda_status_t fused_max_clusters(int (&n)[2])
             fused_config(cfg, at, 3 + i, 1, nullptr);
             cfg.numAttrs = 1;
             int c = 0;
-            KDA_CUDA_TRY(cudaOccupancyMaxActiveClusters(&c, (const void*)fused_fn(true, false), &cfg));
+            KDA_CUDA_TRY(cudaOccupancyMaxActiveClusters(&c, (const void*)fused_fn(true), &cfg));
             lk.st->fused_clusters[i] = c;
         }
         lk.st->attr_done[0] = true;
@@ -1637,7 +1591,7 @@ kda_status_t launch_fused_tc(const FusedArgs& f, bool has_q, cudaStream_t st)
     cudaLaunchAttribute at[2];
     fused_config(cfg, at, f.cluster_size, f.n_clusters, st);
     ProfScope ps(PROF_FUSED, st);
-    KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, fused_fn(has_q, f.a.gate_rate != nullptr), f, tm_k, tm_q, tm_v, tm_o));
+    KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, fused_fn(has_q), f, tm_k, tm_q, tm_v, tm_o));
     count_launch();
     return KDA_OK;
 }
@@ -1646,7 +1600,7 @@ kda_status_t launch_fused_tc(const FusedArgs& f, bool has_q, cudaStream_t st)
 kda_status_t launch_chain_tc(const FusedArgs& f, int n_count, cudaStream_t st)
 {
     const ChunkArgs& a = f.a;
-    const bool has_q = a.q != nullptr && a.o != nullptr, layer = a.gate_rate != nullptr;
+    const bool has_q = a.q != nullptr && a.o != nullptr;
     {
         DeviceLock lk;
         if (!lk.st) return lk.rc;
@@ -1673,7 +1627,7 @@ kda_status_t launch_chain_tc(const FusedArgs& f, int n_count, cudaStream_t st)
     cfg.attrs = at;
     cfg.numAttrs = a.g1 > a.g0 ? 1 : 0;
     ProfScope ps(PROF_INTER, st);
-    KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, chain_fn(has_q, layer), f, tm_o));
+    KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, chain_fn(has_q, a.rows32), f, tm_o));
     count_launch();
     return KDA_OK;
 }

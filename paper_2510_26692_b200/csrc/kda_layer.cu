@@ -4,6 +4,8 @@
 // output of the chunk kernels.  Rows are spread over a grid sized to the device; HBM-bound: 256 B
 // read + 256 B gate + 256 B written per row.
 #include "kda_common.cuh"
+#include "kda_ptx.cuh"
+#include "kda_tiles.cuh"
 
 namespace kda {
 namespace {
@@ -28,6 +30,8 @@ __global__ void __launch_bounds__(256) kda_layer_epilogue_kernel(__nv_bfloat16* 
                                                                  const float* __restrict__ w, float eps,
                                                                  int64_t n_rows)
 {
+    ptx::grid_dep_wait();      // (launched while the chains end)
+    ptx::grid_dep_launch();
     const int lane = threadIdx.x & 31, sub = lane & 15, half = lane >> 4;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const float4 wa = *reinterpret_cast<const float4*>(w + sub * 8);
@@ -67,7 +71,84 @@ __global__ void __launch_bounds__(256) kda_layer_epilogue_kernel(__nv_bfloat16* 
     }
 }
 
+// The same from the fp32 rows that the chains left in the scratch tiles: one CTA per (chunk, head), a warp per
+// four tokens at a time, four columns a lane.
+__global__ void __launch_bounds__(256) kda_layer_rows_kernel(ChunkArgs a, const char* __restrict__ tiles,
+                                                             __nv_bfloat16* __restrict__ y,
+                                                             const __nv_bfloat16* __restrict__ g_o,
+                                                             const float* __restrict__ w, float eps)
+{
+    ptx::grid_dep_wait();      // (launched while the chains end)
+    ptx::grid_dep_launch();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t gl = blockIdx.x / (unsigned)a.H;
+    const int h = (int)(blockIdx.x - gl * a.H);
+    const ChunkLoc loc = locate_chunk(a, a.g0 + gl);
+    const float4* rows = reinterpret_cast<const float4*>(tiles + (size_t)blockIdx.x * tc::TILE_BYTES + tc::OFF_O32);
+    const float4 w4 = *reinterpret_cast<const float4*>(w + lane * 4);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int quad = u * 8 + warp;
+        if (4 * quad >= loc.len) break;
+        float o[4][4];                   // [column][token]
+        uint2 rg[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float4 v = rows[quad * 128 + lane * 4 + c];
+            o[c][0] = v.x; o[c][1] = v.y; o[c][2] = v.z; o[c][3] = v.w;
+        }
+        auto off = [&](int k) { return ((size_t)(loc.tok0 + 4 * quad + k) * a.H + h) * kD + lane * 4; };
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            rg[k] = make_uint2(0u, 0u);
+            if (4 * quad + k < loc.len) rg[k] = *reinterpret_cast<const uint2*>(g_o + off(k));
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            float ss = fmaf(o[0][k], o[0][k], fmaf(o[1][k], o[1][k], fmaf(o[2][k], o[2][k], o[3][k] * o[3][k])));
+#pragma unroll
+            for (int s = 16; s >= 1; s >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, s);
+            const float rstd = rsqrtf(ss * (1.f / kD) + eps);
+            const float g[4] = {__uint_as_float(rg[k].x << 16), __uint_as_float(rg[k].x & 0xffff0000u),
+                                __uint_as_float(rg[k].y << 16), __uint_as_float(rg[k].y & 0xffff0000u)};
+            const float ww[4] = {w4.x, w4.y, w4.z, w4.w};
+            float r[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) r[c] = o[c][k] * rstd * ww[c] / (1.f + __expf(-g[c]));
+            if (4 * quad + k < loc.len) *reinterpret_cast<uint2*>(y + off(k)) = make_uint2(pack2(r[0], r[1]), pack2(r[2], r[3]));
+        }
+    }
+}
+
+// as the programmatic dependent of the kernel before it: the launch overlaps its end
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kern)(P...), unsigned grid, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 }  // namespace
+
+kda_status_t launch_layer_rows(const ChunkArgs& a, const void* tiles, void* y, const void* g_o, const float* w, float eps,
+                               cudaStream_t st)
+{
+    const int64_t n_tiles = (a.g1 - a.g0) * a.H;
+    if (n_tiles <= 0) return KDA_OK;
+    ProfScope ps(PROF_DECODE, st);
+    KDA_CUDA_TRY(launch_after(kda_layer_rows_kernel, (unsigned)n_tiles, st, a, static_cast<const char*>(tiles),
+                              static_cast<__nv_bfloat16*>(y), static_cast<const __nv_bfloat16*>(g_o), w, eps));
+    count_launch();
+    return KDA_OK;
+}
 
 kda_status_t launch_layer_epilogue(void* y, const void* g_o, const float* w, float eps, int64_t n_rows,
                                    cudaStream_t st)
@@ -87,11 +168,9 @@ kda_status_t launch_layer_epilogue(void* y, const void* g_o, const float* w, flo
     int64_t blocks = (n_rows + 8 * 2 * kRows - 1) / (8 * 2 * kRows);   // 8 warps per block, 2 kRows rows per warp step
     if (blocks > (int64_t)n_sm * 64) blocks = (int64_t)n_sm * 64;
     ProfScope ps(PROF_DECODE, st);
-    kda_layer_epilogue_kernel<<<(unsigned)blocks, 256, 0, st>>>(static_cast<__nv_bfloat16*>(y),
-                                                                 static_cast<const __nv_bfloat16*>(g_o), w, eps,
-                                                                 n_rows);
+    KDA_CUDA_TRY(launch_after(kda_layer_epilogue_kernel, (unsigned)blocks, st, static_cast<__nv_bfloat16*>(y),
+                              static_cast<const __nv_bfloat16*>(g_o), w, eps, n_rows));
     count_launch();
-    KDA_CUDA_TRY(cudaGetLastError());
     return KDA_OK;
 }
 

@@ -10,6 +10,9 @@ namespace tc {
 // [ W ; Q ] = [ T Diag(beta) (Gamma.K) ; scale Gamma.Q ]: two K-halves of [128 rows][64], rows 0-63 = W, 64-127 = Q
 constexpr uint32_t OFF_QW = 0;
 constexpr uint32_t QW_HALF = 128 * 128;
+// layer calls of few chains: the chunk's output rows in fp32, over [ W ; Q ] once the chain has read them; element
+// (token, column) at float ((token / 4) 128 + column) 4 + token % 4
+constexpr uint32_t OFF_O32 = OFF_QW;
 // K' = K exp(G_m - G), relative to the middle G_m = G_C / 2 of the chunk's log-decay range (the reference of the decay
 // factorisation), as two dk-halves of [64 tokens][64 channels]; the consumer restores exp(G_C - G_m) in fp32
 constexpr uint32_t OFF_KI = 32768;
