@@ -101,6 +101,9 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr size_t kWorkspaceCap = (size_t)8 << 30;
+constexpr int kMaxRuns = 148;                                          // runs of a stage of kda_segments.cu
+constexpr int64_t kMinCut = 48;                                        // chunks of a chain worth cutting
+constexpr size_t kSegScratch = (size_t)kMaxRuns * kD * kD * 4;
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline size_t esize(kda_dtype_t dt) { return dt == KDA_BF16 ? 2 : 4; }
@@ -260,6 +263,7 @@ size_t kda_chunk_fwd_workspace_bytes(int64_t total_tokens, int n_seqs, int H, in
         const size_t ring = kFusedRing + (size_t)(J < kSlotCap ? J : kSlotCap) * kRingMax * tc_tile_bytes();
         if (want < ring) want = ring;
     }
+    if (dt == KDA_BF16 && (int64_t)n_seqs * H <= kMaxRuns / 3) want += kSegScratch;   // (segments of long chains)
     return want < lo ? lo : want;
 }
 
@@ -290,6 +294,28 @@ bool use_fused(int n_seqs, int H, int64_t total_chunks, size_t workspace_bytes)
     const size_t fixed = ws_layout(n_seqs, H).fixed, row = (size_t)H * tc_tile_bytes();
     const bool one_pass = workspace_bytes >= fixed && (int64_t)((workspace_bytes - fixed) / row) >= total_chunks;
     return !one_pass || ((int64_t)n_seqs * H <= 37 && total_chunks * H >= 512);
+}
+
+// Into how many segments the chains of a bf16 call are cut (kda_segments.cu), 1 = none.  All runs of a stage must
+// be resident at once.  Times in us, measured: a chain step 1.33 without, 1.4 (maps) and 1.5 (outputs) with all SMs
+// at it, a tile of the intra-chunk kernel 8 over two CTAs per SM, launches 22 and a border 1.5.
+// Prefill, 8 heads x 4096 tokens 101 -> 72 us, 8 x 30000: 627 -> 256, 16 x 131072: 2720 -> 1830; 16 x 65536 for the
+// final state 1246 -> 656.  Modes 1 and 2 of kda_set_chunk_path never cut.
+// Below 48 chunks it gains at most a tenth, and a short sequence keeps the same bits however it is handed over.
+int segments(int64_t J, int64_t longest, int64_t tiles, bool out, int n_sm)
+{
+    if (g_chunk_path.load(std::memory_order_relaxed) != 0) return 1;
+    const int64_t runs = (n_sm < kMaxRuns ? n_sm : kMaxRuns) / J;
+    const int64_t most = out ? (runs + 3) / 2 : (runs + 1) / 2;     // maps of P - 1 and P - 2 segments, or of P and P - 1
+    const double intra = 8. * tiles / (2 * n_sm), two = intra + 1.4 * longest + 4.;
+    const double fused = std::max(1.33 * longest, 8. * tiles / (6. * J)) + 17.;
+    double best = 0.95 * std::min(two, fused);
+    int P = 1;
+    for (int64_t p = 3; p <= most && 4 * p <= longest; ++p) {
+        const double us = intra + (double)((longest + p - 1) / p) * (out ? 1.4 + 1.5 : 1.4) + 1.5 * p + 22.;
+        if (us < best) { best = us; P = (int)p; }
+    }
+    return P;
 }
 
 // Cluster shape, number of clusters and ring depth of a call of the fused kernel.
@@ -406,7 +432,21 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
         }
         f.epoch = next_epoch();
     }
-    if (dt == KDA_BF16 && !lm.rate && use_fused(n_seqs, H, total_chunks, workspace_bytes)) {
+    int P = 1;
+    int64_t longest = 0;
+    for (int n = 0; n < n_seqs; ++n) longest = std::max(longest, chunk_cu[n + 1] - chunk_cu[n]);
+    if (dt == KDA_BF16 && (o || S_T) && workspace && longest >= kMinCut && (int64_t)n_seqs * H <= kMaxRuns / 3) {
+        int n_sm = 0;
+        if (const kda_status_t rc = sm_count(&n_sm)) return rc;
+        P = segments((int64_t)n_seqs * H, longest, total_chunks * H, q && o, n_sm);
+        // Their scratch lies behind the tiles, which should all fit; one sequence without outputs may also go in passes.
+        // With outputs the last segment writes the final state while the first may not have read S0 yet.
+        const bool out = q && o, passes = n_seqs == 1 && !out;
+        const size_t need = ws_layout(n_seqs, H).fixed + kSegScratch + kAlign +
+                            (size_t)H * tc_tile_bytes() * (size_t)(passes ? std::min<int64_t>(64 * P, total_chunks) : total_chunks);
+        if (P > 1 && (workspace_bytes < need || (out && S0 && S0 == S_T))) P = 1;
+    }
+    if (dt == KDA_BF16 && P == 1 && !lm.rate && use_fused(n_seqs, H, total_chunks, workspace_bytes)) {
         const size_t tbf = tc_tile_bytes();
         if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) || workspace_bytes < kFusedRing + 2 * tbf)
             return fail(KDA_ERR_WORKSPACE, "kda_chunk_fwd: workspace must be 256-byte aligned and at "
@@ -436,6 +476,11 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
         return fail(KDA_ERR_WORKSPACE, "kda_chunk_fwd: workspace must be 256-byte aligned and at "
                     "least %zu bytes (got %zu)", L.fixed + (size_t)H * tb, workspace_bytes);
     char* ws = static_cast<char*>(workspace);
+    if (P > 1) {
+        const size_t at = (workspace_bytes - kSegScratch) & ~(size_t)(kAlign - 1);
+        f.seg_scratch = reinterpret_cast<float*>(ws + at);
+        workspace_bytes = at;
+    }
     int64_t cap = (int64_t)((workspace_bytes - L.fixed) / ((size_t)H * tb));
     if (cap > 0x7fffffff) cap = 0x7fffffff;
 
@@ -481,7 +526,17 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
             f.hdr = hdr;
             f.n_begin = n_begin;
             f.ordered = f.ordered && n_count == n_seqs;
-            if (rc == KDA_OK && n_count > 0) rc = launch_chain_tc(f, n_count, st);
+            if (P > 1 && rc == KDA_OK) {
+                const bool out = q && o;
+                f.seg_P = P;
+                f.seg_val = out ? P - 1 : P;
+                f.seg_runs = 2 * f.seg_val - 1;
+                f.seg_mode = 1;
+                rc = launch_chain_tc(f, n_count, st);
+                if (rc == KDA_OK) rc = launch_segment_states(f, n_count, !out, st);
+                f.seg_mode = 2;
+                if (rc == KDA_OK && out) rc = launch_chain_tc(f, n_count, st);
+            } else if (rc == KDA_OK && n_count > 0) rc = launch_chain_tc(f, n_count, st);
             if (rc == KDA_OK && a.rows32) rc = launch_layer_rows(a, ws + L.off_tiles, o, lm.out_gate, lm.rms_weight, lm.rms_eps, st);
         } else
             rc = launch_chunk_f32(a, ws + L.off_tiles, n_begin, n_count, hdr, st);

@@ -93,6 +93,10 @@ struct FusedArgs {
     int ordered;                     // order[] holds the sequences, longest first
     static constexpr int kMaxDepth = 4, kMaxOrder = 256;
     uint16_t order[kMaxOrder];
+    // chains cut into segments (kda_segments.cu): 1 = find the segments' maps, 2 = run from the states found; a chain
+    // has seg_P segments and, for 1, seg_runs runs: of seg_val segments from a zero state, then from the identity
+    int seg_mode, seg_P, seg_val, seg_runs;
+    float* seg_scratch;              // [chain][seg_runs][128][128]
 };
 
 // ---- dtype helpers ------------------------------------------------------------------------------
@@ -204,6 +208,8 @@ struct DeviceLock {
 DeviceState* device_slot(int ordinal);
 
 // output stage of the layer wrap: y = sigmoid(g_o) . RMSNorm(y) . w in place, rows of kD bf16 values
+kda_status_t sm_count(int* n_sm);      // multiprocessors of the current device (kda_decode.cu)
+kda_status_t launch_segment_states(const FusedArgs& f, int n_count, bool final_state, cudaStream_t st);
 kda_status_t launch_layer_rows(const ChunkArgs& a, const void* tiles, void* y, const void* g_o, const float* w, float eps,
                                cudaStream_t st);
 kda_status_t launch_layer_epilogue(void* y, const void* g_o, const float* w, float eps, int64_t n_rows,

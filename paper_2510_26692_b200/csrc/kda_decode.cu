@@ -427,7 +427,6 @@ kda_decode_multi_kernel(const T* __restrict__ q, const T* __restrict__ k, const 
 
 }  // namespace
 
-namespace {
 kda_status_t sm_count(int* n_sm)
 {
     DeviceLock lk;
@@ -440,6 +439,7 @@ kda_status_t sm_count(int* n_sm)
     *n_sm = lk.st->n_sm;
     return KDA_OK;
 }
+namespace {
 template <typename T, bool kLayer>
 kda_status_t launch_decode_t(const void* q, const void* k, const void* v, const float* log_alpha, const float* beta,
                              float* S, const int32_t* slot, void* o, int n_seqs, int H, float scale,

@@ -183,6 +183,34 @@ struct JobInfo {
     int64_t tok_begin, tok_end;
     int64_t tile0;                // two-kernel schedule: index of the first tile (then every H-th)
 };
+// A run of a call cut into segments (kda_segments.cu).  kSeg: 0 = not cut, 1 = runs that find the segments' maps,
+// 2 = runs from the states found.  Compiled apart: decided at run time it cost the whole chains 1 to 2 per cent.
+struct SegInfo {
+    int chain, p;                 // segment p of this chain
+    bool unit;                    // its linear part: from the identity, without U
+};
+template <int kSeg>
+__device__ __forceinline__ SegInfo seg_info(const FusedArgs& f, int id) {
+    if (kSeg == 0) return {id, 0, false};
+    const int runs = kSeg == 1 ? f.seg_runs : f.seg_P;
+    const int s = id % runs;
+    const bool unit = kSeg == 1 && s >= f.seg_val;
+    return {id / runs, unit ? s - f.seg_val + 1 : s, unit};
+}
+// The state that a job starts from (nullptr = zero, or the identity) and the place of its final state (nullptr = not
+// wanted).
+template <int kSeg>
+__device__ __forceinline__ const float* state_in(const FusedArgs& f, size_t off, int id) {
+    const SegInfo s = seg_info<kSeg>(f, id);
+    if (kSeg && s.p > 0) return kSeg == 1 ? nullptr : f.seg_scratch + ((size_t)s.chain * f.seg_runs + s.p - 1) * (kD * kD);
+    return f.a.S_in ? f.a.S_in + off : nullptr;
+}
+template <int kSeg>
+__device__ __forceinline__ float* state_out(const FusedArgs& f, size_t off, int id) {
+    if (kSeg == 1) return f.seg_scratch + (size_t)id * (kD * kD);
+    if (kSeg == 2 && seg_info<2>(f, id).p + 1 < f.seg_P) return nullptr;
+    return f.a.S_out ? f.a.S_out + off : nullptr;
+}
 // Job number r of cluster cid; false past its last.  Sequences come longest first (f.order) and the
 // clusters take turns back and forth, so that their loads stay close to each other.
 __device__ __forceinline__ bool job_info(const FusedArgs& f, int cid, int r, JobInfo& I) {
@@ -201,10 +229,14 @@ __device__ __forceinline__ bool job_info(const FusedArgs& f, int cid, int r, Job
     I.nch = (int)((I.tok_end - I.tok_begin + kC - 1) / kC);
     return true;
 }
-// The one job of a chain CTA of the two-kernel schedule: the chunks that the pass has of its (sequence, head).
+// The one job of a chain CTA of the two-kernel schedule: the chunks that the pass has of its (sequence, head), or a
+// segment of them.
+template <int kSeg>
 __device__ __forceinline__ bool pass_job(const FusedArgs& f, int id, int r, JobInfo& I) {
     if (r > 0) return false;
     const ChunkArgs& a = f.a;
+    const SegInfo s = seg_info<kSeg>(f, id);
+    id = s.chain;
     const int rank = id / a.H;
     I.n = f.ordered ? (int)f.order[rank] : f.n_begin + rank;
     I.h = id - rank * a.H;
@@ -221,6 +253,13 @@ __device__ __forceinline__ bool pass_job(const FusedArgs& f, int id, int r, JobI
     I.nch = ce > first ? (int)(ce - first) : 0;
     I.tok_begin = tok0 + (first - cb) * kC;
     I.tile0 = (first - a.g0) * a.H + I.h;
+    if (kSeg) {
+        const int len = (I.nch + f.seg_P - 1) / f.seg_P;
+        const int c0 = s.p * len < I.nch ? s.p * len : I.nch, c1 = c0 + len < I.nch ? c0 + len : I.nch;
+        I.nch = c1 - c0;
+        I.tok_begin += (int64_t)c0 * kC;
+        I.tile0 += (int64_t)c0 * a.H;
+    }
     return true;
 }
 __device__ __forceinline__ bool call_aborted(const FusedArgs& f) {
@@ -910,11 +949,12 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 //   warp 8 issues the MMAs, warp 9 lane 0 loads the tiles, warps 12-15 write the output rows
 // kRing: tiles come from the engines of the cluster; otherwise from the plain array that the intra-chunk kernel
 // has written, and `cid` numbers the (sequence, head) pairs.  kRows32 (layer calls): the output rows stay in fp32,
-// in the place of the tile's [W ; Q], for the output stage (kda_layer.cu).
+// in the place of the tile's [W ; Q], for the output stage (kda_layer.cu).  kSeg: see
+// SegInfo.
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
-template <bool kHasQ, bool kRows32, bool kRing>
+template <bool kHasQ, bool kRows32, bool kRing, int kSeg = 0>
 __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t, int cid, const CUtensorMap* tm_o)
 {
     const ChunkArgs& a = f.a;
@@ -955,7 +995,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
         if (lane == 0) ptx::mbar_arrive(bar);
     };
     JobInfo J;
-    auto next_job = [&](int r) { return kRing ? job_info(f, cid, r, J) : pass_job(f, cid, r, J); };
+    auto next_job = [&](int r) { return kRing ? job_info(f, cid, r, J) : pass_job<kSeg>(f, cid, r, J); };
 
     if (warp == 9) {
         // ================= loader =================
@@ -1079,9 +1119,13 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
         uint32_t g = 0;
         KT_DECL(8);
         for (int r = 0; next_job(r); ++r) {
-            const size_t sbase = ((size_t)J.n * a.H + J.h) * (size_t)(kD * kD) + (size_t)dk0 * kD + dv;
+            const size_t s_off = ((size_t)J.n * a.H + J.h) * (size_t)(kD * kD);
+            const int s_at = dk0 * kD + dv;
+            const float* s_in = state_in<kSeg>(f, s_off, cid);
+            const bool unit = seg_info<kSeg>(f, cid).unit;
 #pragma unroll
-            for (int i = 0; i < 64; ++i) S[i] = a.S_in ? a.S_in[sbase + (size_t)i * kD] : 0.f;
+            for (int i = 0; i < 64; ++i) S[i] = s_in ? s_in[s_at + i * kD] : unit && dk0 + i == dv ? 1.f : 0.f;
+            const float um = unit ? 0.f : 1.f;
             if (J.nch > 0) {
 #pragma unroll
                 for (int b = 0; b < 2; ++b) {
@@ -1120,7 +1164,8 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                     ptx::tmem_ld_wait();
 #pragma unroll
                     for (int i = 0; i < 16; ++i)
-                        z[i] = pack_bf16(bf16_lo(u[i]) - __uint_as_float(y[2 * i]), bf16_hi(u[i]) - __uint_as_float(y[2 * i + 1]));
+                        z[i] = kSeg == 1 ? pack_bf16(fmaf(um, bf16_lo(u[i]), -__uint_as_float(y[2 * i])), fmaf(um, bf16_hi(u[i]), -__uint_as_float(y[2 * i + 1])))
+                                         : pack_bf16(bf16_lo(u[i]) - __uint_as_float(y[2 * i]), bf16_hi(u[i]) - __uint_as_float(y[2 * i + 1]));
                     ptx::tmem_st_32x32b_x16(tq + T_VN + half * 16, z);
                     ptx::tmem_st_wait();
                     ptx::tc_fence_before();
@@ -1175,9 +1220,9 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                 KT_MARK(t == 0, 6);
             }
             if (*abort_flag) break;
-            if (a.S_out)
+            if (float* s_out = state_out<kSeg>(f, s_off, cid))
 #pragma unroll
-                for (int i = 0; i < 64; ++i) a.S_out[sbase + (size_t)i * kD] = S[i];
+                for (int i = 0; i < 64; ++i) s_out[s_at + i * kD] = S[i];
         }
         KT_FLUSH(t == 0, f.hdr, 28, 7);
     } else if (warp >= 12 && op) {
@@ -1352,7 +1397,7 @@ kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
 }
 
 // ---- the chains alone (second kernel of the two-kernel schedule): a CTA per (sequence, head) -------------------
-template <bool kHasQ, bool kRows32>
+template <bool kHasQ, bool kRows32, int kSeg>
 __global__ void __launch_bounds__(kThreads, 1)
 kda_chain_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtensorMap tm_o)
 {
@@ -1372,7 +1417,7 @@ kda_chain_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     if ((ptx::smem_u32(smem) & 1023u) != 0) {
         if (t == 0) report_timeout(f, 90);
     } else {
-        chain_run<kHasQ, kRows32, false>(f, smem, tmem_base, t, (int)blockIdx.x, &tm_o);
+        chain_run<kHasQ, kRows32, false, kSeg>(f, smem, tmem_base, t, (int)blockIdx.x, &tm_o);
     }
     ptx::tc_fence_before();
     __syncthreads();
@@ -1529,10 +1574,12 @@ namespace {
 using FusedFn = void (*)(FusedArgs, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap);
 using ChainFn = void (*)(FusedArgs, CUtensorMap);
 FusedFn fused_fn(bool has_q) { return has_q ? kda_fused_tc<true> : kda_fused_tc<false>; }
-ChainFn chain_fn(bool has_q, bool rows32)
+ChainFn chain_fn(bool has_q, bool rows32, int seg)
 {
-    if (!has_q) return kda_chain_tc<false, false>;
-    return rows32 ? kda_chain_tc<true, true> : kda_chain_tc<true, false>;
+    if (seg == 1) return kda_chain_tc<false, false, 1>;
+    if (!has_q) return kda_chain_tc<false, false, 0>;
+    if (seg == 2) return rows32 ? kda_chain_tc<true, true, 2> : kda_chain_tc<true, false, 2>;
+    return rows32 ? kda_chain_tc<true, true, 0> : kda_chain_tc<true, false, 0>;
 }
 void fused_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[2], int cluster, int n_clusters, cudaStream_t st)
 {
@@ -1600,13 +1647,13 @@ kda_status_t launch_fused_tc(const FusedArgs& f, bool has_q, cudaStream_t st)
 kda_status_t launch_chain_tc(const FusedArgs& f, int n_count, cudaStream_t st)
 {
     const ChunkArgs& a = f.a;
-    const bool has_q = a.q != nullptr && a.o != nullptr;
+    const bool maps = f.seg_mode == 1, has_q = a.q != nullptr && a.o != nullptr && !maps;
     {
         DeviceLock lk;
         if (!lk.st) return lk.rc;
         if (!lk.st->attr_done[2]) {
-            for (int i = 0; i < 4; ++i)
-                KDA_CUDA_TRY(cudaFuncSetAttribute((const void*)chain_fn(i & 1, i & 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
+            for (int i = 0; i < 12; ++i)
+                KDA_CUDA_TRY(cudaFuncSetAttribute((const void*)chain_fn(i & 1, i & 2, i / 4), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   (int)kSmemBytes));
             lk.st->attr_done[2] = true;
         }
@@ -1615,7 +1662,7 @@ kda_status_t launch_chain_tc(const FusedArgs& f, int n_count, cudaStream_t st)
     const kda_status_t rc = make_tmap(&tm_o, has_q ? a.o : f.hdr, a.total_tokens > 0 ? a.total_tokens : 1, a.H);
     if (rc != KDA_OK) return rc;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)n_count * (unsigned)a.H);
+    cfg.gridDim = dim3((unsigned)n_count * (unsigned)a.H * (unsigned)(maps ? f.seg_runs : f.seg_mode ? f.seg_P : 1));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = st;
@@ -1625,9 +1672,9 @@ kda_status_t launch_chain_tc(const FusedArgs& f, int n_count, cudaStream_t st)
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = a.g1 > a.g0 ? 1 : 0;
+    cfg.numAttrs = a.g1 > a.g0 && f.seg_mode != 2 ? 1 : 0;     // (nor with the kernel that finds the segments' states)
     ProfScope ps(PROF_INTER, st);
-    KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, chain_fn(has_q, a.rows32), f, tm_o));
+    KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, chain_fn(has_q, a.rows32, f.seg_mode), f, tm_o));
     count_launch();
     return KDA_OK;
 }

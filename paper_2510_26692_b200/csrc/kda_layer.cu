@@ -72,61 +72,65 @@ __global__ void __launch_bounds__(256) kda_layer_epilogue_kernel(__nv_bfloat16* 
 }
 
 // The same from the fp32 rows that the chains left in the scratch tiles: one CTA per (chunk, head), a warp per
-// four tokens at a time, four columns a lane.
-__global__ void __launch_bounds__(256) kda_layer_rows_kernel(ChunkArgs a, const char* __restrict__ tiles,
+// four tokens, four columns a lane.  The caller's tensors are fetched before the chains have ended.
+__global__ void __launch_bounds__(512) kda_layer_rows_kernel(ChunkArgs a, const char* __restrict__ tiles,
                                                              __nv_bfloat16* __restrict__ y,
                                                              const __nv_bfloat16* __restrict__ g_o,
                                                              const float* __restrict__ w, float eps)
 {
-    ptx::grid_dep_wait();      // (launched while the chains end)
-    ptx::grid_dep_launch();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, quad = threadIdx.x >> 5;
     const int64_t gl = blockIdx.x / (unsigned)a.H;
     const int h = (int)(blockIdx.x - gl * a.H);
     const ChunkLoc loc = locate_chunk(a, a.g0 + gl);
     const float4* rows = reinterpret_cast<const float4*>(tiles + (size_t)blockIdx.x * tc::TILE_BYTES + tc::OFF_O32);
     const float4 w4 = *reinterpret_cast<const float4*>(w + lane * 4);
+    auto off = [&](int k) { return ((size_t)(loc.tok0 + 4 * quad + k) * a.H + h) * kD + lane * 4; };
+    uint2 rg[4];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const int quad = u * 8 + warp;
-        if (4 * quad >= loc.len) break;
-        float o[4][4];                   // [column][token]
-        uint2 rg[4];
+    for (int k = 0; k < 4; ++k) {
+        rg[k] = make_uint2(0u, 0u);
+        if (4 * quad + k < loc.len) rg[k] = *reinterpret_cast<const uint2*>(g_o + off(k));
+    }
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    if (4 * quad >= loc.len) return;
+    float4 o[4];                         // column 4 lane + c, four tokens
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const float4 v = rows[quad * 128 + lane * 4 + c];
-            o[c][0] = v.x; o[c][1] = v.y; o[c][2] = v.z; o[c][3] = v.w;
-        }
-        auto off = [&](int k) { return ((size_t)(loc.tok0 + 4 * quad + k) * a.H + h) * kD + lane * 4; };
+    for (int c = 0; c < 4; ++c)
+        asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(o[c].x), "=f"(o[c].y), "=f"(o[c].z), "=f"(o[c].w)
+                     : "l"(rows + quad * 128 + lane * 4 + c) : "memory");
+    auto token = [&](const float4& v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; };
+    float ss[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            rg[k] = make_uint2(0u, 0u);
-            if (4 * quad + k < loc.len) rg[k] = *reinterpret_cast<const uint2*>(g_o + off(k));
-        }
+    for (int k = 0; k < 4; ++k) {
+        ss[k] = 0.f;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            float ss = fmaf(o[0][k], o[0][k], fmaf(o[1][k], o[1][k], fmaf(o[2][k], o[2][k], o[3][k] * o[3][k])));
+        for (int c = 0; c < 4; ++c) ss[k] = fmaf(token(o[c], k), token(o[c], k), ss[k]);
+    }
 #pragma unroll
-            for (int s = 16; s >= 1; s >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, s);
-            const float rstd = rsqrtf(ss * (1.f / kD) + eps);
-            const float g[4] = {__uint_as_float(rg[k].x << 16), __uint_as_float(rg[k].x & 0xffff0000u),
-                                __uint_as_float(rg[k].y << 16), __uint_as_float(rg[k].y & 0xffff0000u)};
-            const float ww[4] = {w4.x, w4.y, w4.z, w4.w};
-            float r[4];
+    for (int s = 16; s >= 1; s >>= 1)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) r[c] = o[c][k] * rstd * ww[c] / (1.f + __expf(-g[c]));
-            if (4 * quad + k < loc.len) *reinterpret_cast<uint2*>(y + off(k)) = make_uint2(pack2(r[0], r[1]), pack2(r[2], r[3]));
-        }
+        for (int k = 0; k < 4; ++k) ss[k] += __shfl_xor_sync(0xffffffffu, ss[k], s);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float rstd = rsqrtf(ss[k] * (1.f / kD) + eps);
+        const float g[4] = {__uint_as_float(rg[k].x << 16), __uint_as_float(rg[k].x & 0xffff0000u),
+                            __uint_as_float(rg[k].y << 16), __uint_as_float(rg[k].y & 0xffff0000u)};
+        const float ww[4] = {w4.x, w4.y, w4.z, w4.w};
+        float r[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) r[c] = token(o[c], k) * rstd * ww[c] / (1.f + __expf(-g[c]));
+        if (4 * quad + k < loc.len) *reinterpret_cast<uint2*>(y + off(k)) = make_uint2(pack2(r[0], r[1]), pack2(r[2], r[3]));
     }
 }
 
 // as the programmatic dependent of the kernel before it: the launch overlaps its end
 template <typename... P, typename... A>
-cudaError_t launch_after(void (*kern)(P...), unsigned grid, cudaStream_t st, A... args)
+cudaError_t launch_after(void (*kern)(P...), unsigned grid, unsigned threads, cudaStream_t st, A... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(256);
+    cfg.blockDim = dim3(threads);
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -144,7 +148,7 @@ kda_status_t launch_layer_rows(const ChunkArgs& a, const void* tiles, void* y, c
     const int64_t n_tiles = (a.g1 - a.g0) * a.H;
     if (n_tiles <= 0) return KDA_OK;
     ProfScope ps(PROF_DECODE, st);
-    KDA_CUDA_TRY(launch_after(kda_layer_rows_kernel, (unsigned)n_tiles, st, a, static_cast<const char*>(tiles),
+    KDA_CUDA_TRY(launch_after(kda_layer_rows_kernel, (unsigned)n_tiles, 512, st, a, static_cast<const char*>(tiles),
                               static_cast<__nv_bfloat16*>(y), static_cast<const __nv_bfloat16*>(g_o), w, eps));
     count_launch();
     return KDA_OK;
@@ -168,7 +172,7 @@ kda_status_t launch_layer_epilogue(void* y, const void* g_o, const float* w, flo
     int64_t blocks = (n_rows + 8 * 2 * kRows - 1) / (8 * 2 * kRows);   // 8 warps per block, 2 kRows rows per warp step
     if (blocks > (int64_t)n_sm * 64) blocks = (int64_t)n_sm * 64;
     ProfScope ps(PROF_DECODE, st);
-    KDA_CUDA_TRY(launch_after(kda_layer_epilogue_kernel, (unsigned)blocks, st, static_cast<__nv_bfloat16*>(y),
+    KDA_CUDA_TRY(launch_after(kda_layer_epilogue_kernel, (unsigned)blocks, 256, st, static_cast<__nv_bfloat16*>(y),
                               static_cast<const __nv_bfloat16*>(g_o), w, eps, n_rows));
     count_launch();
     return KDA_OK;

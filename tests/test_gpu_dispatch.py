@@ -4,7 +4,8 @@ import torch
 
 import paper_2510_26692_b200 as K
 from paper_2510_26692_b200 import inputs
-from kda_testlib import rel_l2, to_np32
+from kda_testlib import TOL, oracle_chunk, rel_l2, run_chunk, to_np32
+from test_gpu_layer import oracle_layer, run_layer
 
 pytestmark = pytest.mark.gpu
 
@@ -51,3 +52,55 @@ def test_binding_takes_what_it_took():
     with pytest.raises(K.KdaError) as ei:
         K.kda_decode_step(*a, d["S"], None, None, 3, 2, 128, 128, 1.0, K.KDA_BF16)
     assert ei.value.code == 1
+
+
+@pytest.mark.parametrize("lens,H", [([448], 7), ([320], 10), ([70, 1, 64], 3), ([65, 130], 5)])
+def test_fp32_prefill_splits(oracle_mod, lens, H):
+    """Last and first sizes of tiles in three parts (49 and 50 tiles) and of 8-column chains (9 and 10
+    chains).  22-bit operands with fp32 sums: 1e-5."""
+    d = inputs.chunk_inputs(lens, H=H, dtype=torch.float32, seed=53, s0_std=0.02)
+    o, S = run_chunk(d)
+    o_ref, S_ref = oracle_chunk(oracle_mod, d)
+    assert rel_l2(to_np32(o), o_ref) <= 1e-5 and rel_l2(to_np32(S), S_ref) <= 1e-5
+
+
+@pytest.mark.parametrize("lens,H", [([960], 37), ([832], 37), ([896], 38), ([70, 130], 37), ([1] * 256 + [90], 1)])
+def test_bf16_schedules(oracle_mod, lens, H):
+    """Around the lines between the fused kernel and two kernels (512 tiles, 37 chains), and more
+    sequences than the table of lengths holds.  Operands rounded to bf16: TOL."""
+    d = inputs.chunk_inputs(lens, H=H, dtype=torch.bfloat16, seed=54, s0_std=0.02)
+    o, S = run_chunk(d)
+    o_ref, S_ref = oracle_chunk(oracle_mod, d)
+    assert rel_l2(to_np32(o), o_ref) <= TOL[K.KDA_BF16] and rel_l2(to_np32(S), S_ref) <= TOL[K.KDA_BF16]
+
+
+@pytest.mark.parametrize("lens,H,out", [([4100], 3, True), ([4033], 3, False), ([5000, 70, 0, 2000], 1, True),
+                                        ([6000, 64, 3000], 2, False)])
+def test_bf16_segments(oracle_mod, lens, H, out):
+    """Chains cut into segments, the last ones short or empty: within TOL of the oracle and no further
+    from it than the uncut chains but for the rounding of other operands (a tenth)."""
+    d = inputs.chunk_inputs(lens, H=H, dtype=torch.bfloat16, seed=55, s0_std=0.02)
+    o_ref, S_ref = oracle_chunk(oracle_mod, d)
+    err = []
+    for mode in (0, 1):
+        K.kda_set_chunk_path(mode)
+        try:
+            before = K.kda_launch_count()
+            o, S = run_chunk(d, want_o=out)
+            launches = K.kda_launch_count() - before
+        finally:
+            K.kda_set_chunk_path(0)
+        err.append((launches, rel_l2(to_np32(o), o_ref) if out else 0.0, rel_l2(to_np32(S), S_ref)))
+    (n0, eo0, es0), (n1, eo1, es1) = err
+    assert n0 == n1 + (2 if out else 1)       # it was cut
+    assert eo0 <= min(TOL[K.KDA_BF16], 1.1 * eo1) and es0 <= min(TOL[K.KDA_BF16], 1.1 * es1)
+
+
+@pytest.mark.parametrize("lens,H", [([300, 70], 18), ([300, 70], 19), ([4100], 3)])
+def test_layer_output_rows(oracle_mod, lens, H):
+    """Output stage from fp32 rows (up to 37 chains) and from bf16 rows, chains whole and in segments:
+    bf16 operands and output, TOL."""
+    d = inputs.layer_inputs(lens, H=H, seed=56, s0_std=0.02)
+    y, S = run_layer(d, 128 ** -0.5)
+    y_ref, S_ref, _ = oracle_layer(oracle_mod, d, 128 ** -0.5)
+    assert rel_l2(to_np32(y), y_ref) <= TOL[K.KDA_BF16] and rel_l2(to_np32(S), S_ref) <= TOL[K.KDA_BF16]
