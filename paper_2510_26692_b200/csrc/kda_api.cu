@@ -263,7 +263,7 @@ size_t kda_chunk_fwd_workspace_bytes(int64_t total_tokens, int n_seqs, int H, in
         const size_t ring = kFusedRing + (size_t)(J < kSlotCap ? J : kSlotCap) * kRingMax * tc_tile_bytes();
         if (want < ring) want = ring;
     }
-    if (dt == KDA_BF16 && (int64_t)n_seqs * H <= kMaxRuns / 3) want += kSegScratch;   // (segments of long chains)
+    if (dt == KDA_BF16 && (int64_t)n_seqs * H <= kMaxRuns / 3) want = std::min(want + kSegScratch, kWorkspaceCap);   // (segments of long chains)
     return want < lo ? lo : want;
 }
 
