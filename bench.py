@@ -37,11 +37,11 @@ STATE_BYTES = 2 * D * D * 4
 DEC_BYTES_PER_STATE = 2 * D * D * 4 + 4 * D * 2 + D * 4 + 4
 FLOPS_PER_TOKEN_HEAD = 6 * D * D + 3 * CHUNK * D + CHUNK * CHUNK   # the paper's FLOPs model
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised under
-# profiles/ (prefill: intra 168.4 + 98.7 MB, inter 156.3 + 20.0 MB, fused kernel 170.8 + 33.6 MB;
+# profiles/ (prefill, which runs as the fused kernel: 171.8 + 106.7 MB;
 # decode: 547.4 + 484.7 MB)
-PREFILL_DRAM_TRAFFIC = {"intra_chunk": 267.1e6, "inter_chunk": 176.3e6}
+PREFILL_DRAM_TRAFFIC = {"fused": 278.6e6}
 DECODE_DRAM_TRAFFIC = 1032.1e6
-FUSED_DRAM_TRAFFIC = 204.4e6
+FUSED_DRAM_TRAFFIC = 278.6e6
 TRAFFIC_SOURCE = "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch, copied from the summaries under profiles/ (not measured in this run)"
 MIN_TIMED_S = 0.5      # the timed region is extended (whole blocks of `steps` calls) to at least this
 MAX_BLOCKS = 2000
@@ -325,8 +325,8 @@ def backward_figure(K, inputs, torch, dev, peaks):
     return {"workload": "gradients of the prefill workload (B=1 T=4096 H=32, bf16 q/k/v/d_o, fp32 gradients)",
             "ms": ms, "tokens_per_s": T / (ms * 1e-3), "algorithmic_bytes": nbytes,
             "achieved_gbs": nbytes / (ms * 1e-3) / 1e9, "frac": nbytes / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
-            "note": "token-sequential adjoint in fp32 FMA (one CTA per sequence, head and 32-column slice): "
-                    "bound by the 4096 dependent steps, not by memory"}
+            "note": "chunkwise adjoint, fp32 accuracy (six bf16 MMAs per product): bound by the operand splitting "
+                    "between its products and by the chains, not by memory"}
 
 
 def layer_figure(K, inputs, torch, dev, peaks):
@@ -360,7 +360,7 @@ def layer_figure(K, inputs, torch, dev, peaks):
     return {"workload": "B=1 T=4096 H=32, bf16 pre-activations (q_c, k_c, v, g_a, g_o), fp32 b_pre; inputs rotate over 3 copies",
             "ms": ms, "tokens_per_s": T / (ms * 1e-3), "algorithmic_bytes": nbytes,
             "achieved_gbs": nbytes / (ms * 1e-3) / 1e9, "frac": nbytes / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
-            "note": "two kernels per call: intra-chunk with the prologue inside, inter-chunk with the output stage inside (clusters of the four slice CTAs)"}
+            "note": "three kernels per call: intra-chunk with the prologue inside, the chains, the output stage"}
 
 
 def decode_only(args, K, inputs, torch, dev, peaks):
@@ -510,7 +510,7 @@ def main():
     for i in range(nprof):
         prefill_step(i)
     kern = {}
-    for kind, name in ((0, "prologue"), (1, "intra_chunk"), (2, "inter_chunk")):
+    for kind, name in ((0, "prologue"), (1, "intra_chunk"), (2, "inter_chunk"), (4, "fused")):
         ms, n = K.kda_profile_read(kind)
         if n:
             kern[name] = {"launches_per_step": n / nprof, "ms_per_step": ms / nprof}
@@ -627,7 +627,7 @@ def main():
                      "algorithmic_bytes_per_step": dec_bytes, "traffic": DECODE_DRAM_TRAFFIC},
     }
 
-    # ---- the same prefill through the fused cooperative kernel (the path of small workspaces) --------
+    # ---- the same prefill through the fused kernel whatever the workspace --------
     fused = None
     if world == 1:
         K.kda_set_chunk_path(2)
@@ -641,7 +641,7 @@ def main():
             e1.record(stream)
             barrier()
             fms = e0.elapsed_time(e1) / 20
-            fused = {"kernel": "kda_fused_tc (one cooperative launch: intra-chunk engines and inter-chunk "
+            fused = {"kernel": "kda_fused_tc (one launch of clusters: intra-chunk engines and inter-chunk "
                                "chains, tiles through a ring in L2)", "ms_per_step": fms,
                      "tokens_per_s": T_PREFILL / (fms * 1e-3),
                      "frac": step_bytes / (fms * 1e-3) / 1e9 / peaks["hbm_gbs"],

@@ -273,11 +273,12 @@ kda_status_t kda_dplr_chunk_fwd(const float *q, const float *k, const float *v, 
 
 /*
  * Chooses how kda_chunk_fwd schedules a bf16 call (process-wide; no counterpart in the paper).
- *   0  automatic (default): when the workspace has room for every (chunk, head) tile of the call,
- *      the intra-chunk stage (Section 3.1: gates, UT transform) runs as one kernel and the
- *      inter-chunk stage (state and output equations) as a second one; with a smaller workspace
- *      one fused cooperative kernel runs both stages at once and hands the tiles over through a
- *      ring of a few tiles per (sequence, head) that stays in the L2 cache.
+ *   0  automatic (default), by the number and length of the chains and the size of the workspace:
+ *      the intra-chunk stage (Section 3.1: gates, UT transform) as one kernel and the inter-chunk
+ *      stage (state and output equations) as a second one, the latter with few long chains cut
+ *      into segments that run side by side; or one fused kernel that runs both stages at once and
+ *      hands the tiles over through a ring of a few tiles that stays in the L2 cache (always,
+ *      where the workspace does not hold every (chunk, head) tile of the call).
  *   1  always the two kernels (a small workspace then makes the call walk the chunks in passes)
  *   2  always the fused kernel
  * All three give the same results up to the rounding of the chunk states' bf16 operand copies

@@ -4,8 +4,8 @@
 //     S_t = (Diag(exp(g_t)) + b_t a_t^T) S_{t-1} + k_t v_t^T ,      o_t = scale * S_t^T q_t .
 //
 // It is the comparison workload for the KDA kernels: same chunk length, same two-kernel structure
-// and the same arithmetic style as the fp32 KDA path (kda_chunk_simt.cu), so that the ratio of the
-// two run times shows what binding a and b to k saves (Section 6.1 counts four second-level Gram
+// as the fp32 KDA path (kda_chunk_f32.cu; that one has since moved to split tf32 products).  What
+// binding a and b to k saves is in the counts (Section 6.1 counts four second-level Gram
 // matrices against two, and three more matrix products in the inter-chunk and output stage).
 //
 //   intra  one CTA per (chunk, head): cumulative log-decay G; the four gated Gram matrices

@@ -1,9 +1,9 @@
-// bf16 tensor-core path of the chunkwise KDA forward (paper Section 3.1; Appendix C), as ONE
-// persistent cooperative kernel with one CTA of 512 threads per SM.  Every CTA runs warp-specialised
-// roles that meet only on mbarriers, named barriers and a few flag words in global memory:
+// bf16 tensor-core path of the chunkwise KDA forward (paper Section 3.1; Appendix C): two stages, either as two
+// kernels (kda_intra_tc over all tiles, then kda_chain_tc, a CTA per chain) or as one (kda_fused_tc: thread-block
+// clusters of one chain CTA and two or three engine CTAs).  CTAs of 512 threads run warp-specialised roles that meet
+// only on mbarriers and named barriers, those of a cluster on mbarriers in distributed shared memory:
 //
-//   intra-chunk engine (8 warps; every CTA has one in warps 0-7, CTAs without a chain role a second
-//   one in warps 8-15): everything of a (chunk, head) tile that does not depend on the state --
+//   intra-chunk engine (8 warps, two to a CTA): everything of a (chunk, head) tile that does not depend on the state --
 //     a1   G = cumulative sum of log alpha over the chunk's tokens (fp32, log2 domain)
 //          gated operands, bf16:  Kg = K exp(G - G_m),  Qg = scale Q exp(G - G_m),  Ki = K exp(G_m - G)
 //          with G_m = G_C / 2 per channel (the middle of the chunk's log-decay range), so that
@@ -13,19 +13,15 @@
 //     a3   T = (I + L)^-1 by blocked forward substitution: 16x16 diagonal blocks column by column in
 //          fp32 registers, sub-diagonal blocks as warp-level 16x16 products (mma.sync, tf32 inputs)
 //     a4   Mm = T Diag(beta) (bf16);  second MMA group  [Mm ; Mm] x [Kg | V]  ->  W' = Mm Kg, U = Mm V
-//   The tile (operand images of kda_tiles.cuh) goes to a small ring in global memory that stays in
-//   L2: R tiles per running (sequence, head).
+//   The tile (operand images of kda_tiles.cuh) goes to global memory; in the fused kernel to a ring of a few tiles per
+//   engine that stays in L2.
+//   Two kernels: 8.1 us a tile with two in flight per SM, where reading its inputs and writing it takes 7.2 at the copy
+//   bandwidth.  Fused (3.8 without the write): the chain of its phases, of which shared memory lets no third one overlap.
 //
-//   inter-chunk chain (CTAs 0 .. 4 Q - 1; warps 8-11 compute, 12-13 issue MMAs, 14 loads): one
-//   32-column slice of the state of one (sequence, head), walked over the chunks in order --
-//     MMA1  D1 = [W' ; Q'] x bf16(exp(G_m) . S)         rows 0-63 = W S, rows 64-127 = (Gamma.Q) S
-//     a6    V_new = U - W S                              TMEM -> registers -> bf16 -> shared memory
-//     MMA2  D3 = K'^T V_new ;  D1[64:128] += Aqk V_new   (a8, a7)
-//     a8    S <- gamma^C . S + exp(G_C - G_m) . D3       fp32 master copy in registers
-//     a7    O = D1[64:128] -> bf16 -> global
-//   Tiles arrive by 1-D bulk copies (TMA engine) in three pieces with their own rings (gate vectors
-//   3 deep, [W';Q'] 2 deep, K'/Aqk/U 2 deep) so that each piece is requested as early as its buffer
-//   frees up.
+//   inter-chunk chain (a CTA; roles and products: see chain_run): all 128 columns of the state of one (sequence,
+//   head), walked over the chunks in order -- a6 V_new = U - W S, a8 the state, a7 the outputs.  1.23 us a step for
+//   the final state alone, 1.33 with outputs: two dependent round trips tensor core - registers - tensor core.
+//   Tiles arrive by 1-D bulk copies (TMA engine).
 //
 // Every wait (mbarrier, flag word) is bounded by a wall-clock limit; when one runs out the role
 // records KDA_ERR_TIMEOUT in the workspace header, marks the call as aborted so that every other
@@ -949,8 +945,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 //   warp 8 issues the MMAs, warp 9 lane 0 loads the tiles, warps 12-15 write the output rows
 // kRing: tiles come from the engines of the cluster; otherwise from the plain array that the intra-chunk kernel
 // has written, and `cid` numbers the (sequence, head) pairs.  kRows32 (layer calls): the output rows stay in fp32,
-// in the place of the tile's [W ; Q], for the output stage (kda_layer.cu).  kSeg: see
-// SegInfo.
+// in the place of the tile's [W ; Q], for the output stage (kda_layer.cu).  kSeg: see SegInfo.
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
