@@ -302,14 +302,14 @@ bool use_fused(int n_seqs, int H, int64_t total_chunks, size_t workspace_bytes)
 // Prefill, 8 heads x 4096 tokens 101 -> 72 us, 8 x 30000: 627 -> 256, 16 x 131072: 2720 -> 1830; 16 x 65536 for the
 // final state 1246 -> 656.  Modes 1 and 2 of kda_set_chunk_path never cut.
 // Below 48 chunks it gains at most a tenth, and a short sequence keeps the same bits however it is handed over.
-int segments(int64_t J, int64_t longest, int64_t tiles, bool out, int n_sm)
+int segments(int64_t J, int64_t longest, int64_t tiles, bool out, bool layer, int n_sm)
 {
     if (g_chunk_path.load(std::memory_order_relaxed) != 0) return 1;
     const int64_t runs = (n_sm < kMaxRuns ? n_sm : kMaxRuns) / J;
     const int64_t most = out ? (runs + 3) / 2 : (runs + 1) / 2;     // maps of P - 1 and P - 2 segments, or of P and P - 1
     const double intra = 8. * tiles / (2 * n_sm), two = intra + 1.4 * longest + 4.;
     const double fused = std::max(1.33 * longest, 8. * tiles / (6. * J)) + 17.;
-    double best = 0.95 * std::min(two, fused);
+    double best = 0.95 * (layer ? two : std::min(two, fused));      // (layer calls never run fused)
     int P = 1;
     for (int64_t p = 3; p <= most && 4 * p <= longest; ++p) {
         const double us = intra + (double)((longest + p - 1) / p) * (out ? 1.4 + 1.5 : 1.4) + 1.5 * p + 22.;
@@ -438,7 +438,7 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
     if (dt == KDA_BF16 && (o || S_T) && workspace && longest >= kMinCut && (int64_t)n_seqs * H <= kMaxRuns / 3) {
         int n_sm = 0;
         if (const kda_status_t rc = sm_count(&n_sm)) return rc;
-        P = segments((int64_t)n_seqs * H, longest, total_chunks * H, q && o, n_sm);
+        P = segments((int64_t)n_seqs * H, longest, total_chunks * H, q && o, lm.rate != nullptr, n_sm);
         // Their scratch lies behind the tiles, which should all fit; one sequence without outputs may also go in passes.
         // With outputs the last segment writes the final state while the first may not have read S0 yet.
         const bool out = q && o, passes = n_seqs == 1 && !out;
