@@ -48,7 +48,8 @@ constexpr int T_AQK = T_KT + kC * kD;
 constexpr int T_GC = T_AQK + kC * kC;
 constexpr int T_FLOATS = T_GC + kD;
 
-__device__ __forceinline__ float clampf(float x) { return fminf(fmaxf(x, -kClamp), kClamp); }
+// (a NaN stays one: fminf and fmaxf would turn it into a bound)
+__device__ __forceinline__ float clampf(float x) { return x == x ? fminf(fmaxf(x, -kClamp), kClamp) : x; }
 
 constexpr int kT1 = 512;
 namespace s1 {

@@ -1,0 +1,47 @@
+"""What a NaN or an infinity in one token does: everything that Eq. 1 makes non-finite (the fp64 oracle on the
+same inputs) is not finite in the outputs either, and the other head is untouched."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2510_26692_b200 as K
+from paper_2510_26692_b200 import inputs
+from kda_testlib import oracle_chunk, run_chunk, to_np32
+
+pytestmark = pytest.mark.gpu
+NAN, INF = float("nan"), float("inf")
+
+
+def spoiled(d, what, token, value):
+    """The inputs with one element of head 0 replaced."""
+    d = dict(d)
+    d[what] = d[what].clone()
+    if what == "beta":
+        d[what][token, 0] = value
+    else:
+        d[what][token, 0, 5] = value
+    return d
+
+
+@pytest.mark.parametrize("what,value", [("q", NAN), ("k", NAN), ("v", NAN), ("beta", NAN), ("log_alpha", NAN),
+                                        ("q", INF), ("k", INF), ("v", INF), ("beta", INF)])
+def test_fp32_prefill_keeps_non_finite(oracle_mod, what, value):
+    d = spoiled(inputs.chunk_inputs([200], H=2, dtype=torch.float32, seed=61, s0_std=0.02), what, 100, value)
+    o, S = run_chunk(d)
+    o_ref, S_ref = oracle_chunk(oracle_mod, d)
+    bad_o, bad_S = ~np.isfinite(to_np32(o)), ~np.isfinite(to_np32(S))
+    assert bad_o[~np.isfinite(o_ref)].all() and bad_S[~np.isfinite(S_ref)].all()
+    assert not bad_o[:64].any() and not bad_o[:, 1].any() and not bad_S[:, 1].any()
+
+
+@pytest.mark.parametrize("what,value", [("k", NAN), ("v", NAN), ("log_alpha", NAN), ("v", INF)])
+def test_segments_keep_non_finite(oracle_mod, what, value):
+    """Chains that are cut into segments: the state over a border is as non-finite as the one before it."""
+    d = spoiled(inputs.chunk_inputs([4100], H=2, dtype=torch.bfloat16, seed=62), what, 700, value)
+    o, S = run_chunk(d)
+    o_ref, S_ref = oracle_chunk(oracle_mod, d)
+    bad_o, bad_S = ~np.isfinite(to_np32(o)), ~np.isfinite(to_np32(S))
+    assert bad_o[~np.isfinite(o_ref)].all() and bad_S[~np.isfinite(S_ref)].all()
+    assert not bad_o[:640].any() and not bad_o[:, 1].any() and not bad_S[:, 1].any()
+    _, S = run_chunk(d, want_o=False)
+    assert (~np.isfinite(to_np32(S)))[~np.isfinite(S_ref)].all()
