@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
     // a1: thread = channel c of 16 consecutive tokens (identity padding past the sequence end)
     const int c = t & 127, seg = t >> 7;
     float G[16], kk[16], qq[16];
+    float z = 0.f;       // becomes a NaN with the first value that is not finite
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         const int r = seg * 16 + i;
@@ -98,11 +99,14 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
         kk[i] = in ? kp[off] : 0.f;
         qq[i] = in && qp && part_q ? qp[off] : 0.f;
     }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) z = fmaf(0.f, G[i], fmaf(0.f, kk[i], fmaf(0.f, qq[i], z)));
     for (int idx = part_u ? t : 64 * 32; idx < 64 * 32; idx += kT1) {
         const int r = idx >> 5, x = (idx & 31) * 4;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (r < loc.len) v = *reinterpret_cast<const float4*>(vp + ((size_t)(loc.tok0 + r) * a.H + h) * kD + x);
         *reinterpret_cast<float4*>(sV + r * LC + x) = v;
+        z = fmaf(0.f, v.x, fmaf(0.f, v.y, fmaf(0.f, v.z, fmaf(0.f, v.w, z))));
     }
     if (t < 64) sBeta[t] = t < loc.len ? a.beta[(size_t)(loc.tok0 + t) * a.H + h] : 0.f;
     float run = 0.f;
@@ -110,7 +114,10 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
     for (int i = 0; i < 16; ++i) { run += G[i]; G[i] = run; }
     sSeg[seg * 128 + c] = run;
     for (int idx = t; idx < 64 * LM; idx += kT1) sT[idx] = 0.f;
-    __syncthreads();
+    if (t < 64) z = fmaf(0.f, sBeta[t], z);
+    // A token that is not finite may spoil later tokens but no earlier ones: such a tile forms its products entry by
+    // entry over the triangle, where a matrix instruction would multiply the zeros beside it.
+    const int odd = __syncthreads_or(z != 0.f);
     float base = 0.f, total = 0.f;
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
@@ -121,7 +128,7 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
     // a channel that decays by more than e^-160 inside the chunk leaves the range of the
     // two-factor form (the clamp keeps everything finite): flag the call
     if (total < -2.f * kClamp) atomicOr(&hdr->flags, 1);
-    const float gm = 0.5f * total, em = expf(gm);
+    const float gm = total == total ? 0.5f * total : 0.f, em = expf(gm);
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         const int r = seg * 16 + i;
@@ -140,7 +147,7 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
         sEm[c] = em;
         if (part_q) tile[T_GC + c] = expf(total);
     }
-    const int far = __syncthreads_or(total < kSplitRange);
+    const int far = __syncthreads_or(total < kSplitRange) | odd;
 
     // a2 + a5: [K^ ; Q] K_^T: warps 4 x 4, 32 x 16 entries each of 128 rows, or 16 x 16 of 64; only blocks that
     // reach the triangle
@@ -178,6 +185,26 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
     else gram(std::integral_constant<int, 1>{}, part_q, (w >> 2) * 16, (w & 3) * 16);
     if (!part_w && !part_u) return;
     __syncthreads();
+    if (odd) {
+        if (t < 64)
+            for (int i = t; i < 64; ++i) {       // column t
+                float x = i == t ? 1.f : 0.f;
+                for (int m = t; m < i; ++m) x = fmaf(-sB[i * LM + m], sT[m * LM + t], x);
+                sT[i * LM + t] = x;
+            }
+        __syncthreads();
+        for (int idx = t; idx < 64 * kD; idx += kT1) {
+            const int i = idx >> 7, x = idx & 127;
+            float wi = 0.f, ui = 0.f;
+            for (int j = 0; j <= i; ++j) {
+                wi = fmaf(sT[i * LM + j], sKG[j * LR + x], wi);
+                if (part_u) ui = fmaf(sT[i * LM + j], sV[j * LC + x], ui);
+            }
+            if (part_w) tile[T_W + idx] = sBeta[i] * wi * sEm[x];
+            if (part_u) tile[T_U + idx] = sBeta[i] * ui;
+        }
+        return;
+    }
     invert_unit_lower<LM>(sB, sT, t);      // a3
 
     // a4: warps 2 x 8, 32 x 16 entries each; the triangle bounds the sums
@@ -294,13 +321,15 @@ __global__ void __launch_bounds__(kT2, 1) kda_inter_f32(ChunkArgs a, const float
         if (w < 4 || op)
             gemm<0, NT, false, false, false, false>(acc, sm + (w < 4 ? L::W + 16 * w * LR : L::Q + 16 * (w - 4) * LR), LR, sS,
                                                    LS, 0, kD, lane);
+        float z = 0.f;
         if (w < 4)
             each_pair(acc, lane, [&](int i, int j, float x, float y) {
                 const float2 u = *reinterpret_cast<const float2*>(sm + L::U + (16 * w + i) * LS + j);
                 st2(sVn + (16 * w + i) * LS + j, u.x - x, u.y - y);
+                z = fmaf(0.f, u.x - x, fmaf(0.f, u.y - y, z));
             });
         cp_wait0();
-        __syncthreads();
+        const int odd = __syncthreads_or(z != 0.f);     // (V_new not finite: see kda_intra_f32)
         if (ch + 1 < ce) fetch1(ch + 1);
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
@@ -311,7 +340,16 @@ __global__ void __launch_bounds__(kT2, 1) kda_inter_f32(ChunkArgs a, const float
         each_pair(S, lane, [&](int i, int j, float x, float y) { st2(sS + (16 * w + i) * LS + j, x, y); });
         if (w >= 4 && op) {
             const int r0 = 16 * (w - 4);
-            gemm<0, NT, false, false, false, false>(acc, sm + L::A + r0 * LM, LM, sVn, LS, 0, r0 + 16, lane);
+            if (!odd)
+                gemm<0, NT, false, false, false, false>(acc, sm + L::A + r0 * LM, LM, sVn, LS, 0, r0 + 16, lane);
+            else
+                for (int nt = 0; nt < NT; ++nt)
+                    for (int e = 0; e < 4; ++e) {
+                        const int row = r0 + g + 8 * (e >> 1), x = 8 * nt + 2 * (lane & 3) + (e & 1);
+                        float s = acc[0][nt][e];
+                        for (int j = 0; j <= row; ++j) s = fmaf(sm[L::A + row * LM + j], sVn[j * LS + x], s);
+                        acc[0][nt][e] = s;
+                    }
             const int64_t tok0 = tok_begin + (ch - seq_c0) * kC;
             each_pair(acc, lane, [&](int i, int j, float x, float y) {
                 const int64_t tok = tok0 + r0 + i;

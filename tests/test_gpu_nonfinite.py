@@ -34,6 +34,22 @@ def test_fp32_prefill_keeps_non_finite(oracle_mod, what, value):
     assert not bad_o[:64].any() and not bad_o[:, 1].any() and not bad_S[:, 1].any()
 
 
+@pytest.mark.parametrize("token", [0, 100, 127])
+@pytest.mark.parametrize("H", [2, 37])
+@pytest.mark.parametrize("what,value", [("q", NAN), ("k", NAN), ("v", NAN), ("beta", NAN), ("log_alpha", NAN),
+                                        ("k", INF), ("v", INF)])
+def test_fp32_prefill_non_finite_is_causal(oracle_mod, what, value, H, token):
+    """A tile in three CTAs (2 heads) and in one (37): what the recurrence leaves finite, the earlier tokens of
+    the same chunk among it, is finite and right (22-bit operands, fp32 sums: 1e-5)."""
+    d = spoiled(inputs.chunk_inputs([200], H=H, dtype=torch.float32, seed=63, s0_std=0.02), what, token, value)
+    o, S = (to_np32(x) for x in run_chunk(d))
+    o_ref, S_ref = oracle_chunk(oracle_mod, d)
+    for x, ref in ((o, o_ref), (S, S_ref)):
+        assert (np.isfinite(x) == np.isfinite(ref)).all()
+        ok = np.isfinite(ref)
+        assert np.linalg.norm(x[ok] - ref[ok]) <= 1e-5 * np.linalg.norm(ref[ok])
+
+
 @pytest.mark.parametrize("what,value", [("k", NAN), ("v", NAN), ("log_alpha", NAN), ("v", INF)])
 def test_segments_keep_non_finite(oracle_mod, what, value):
     """Chains that are cut into segments: the state over a border is as non-finite as the one before it."""
