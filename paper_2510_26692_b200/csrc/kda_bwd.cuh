@@ -13,7 +13,7 @@ struct BwdChunkArgs {
     float* dq; float* dk; float* dv; float* dg; float* db; float* dS0;   // dS0 may be nullptr
     const int32_t* cu_seqlens; const int32_t* chunk_cu;              // nullptr = equal lengths
     float* tiles;                                                    // [chunks][H][kBwdTile]
-    int* seq_heads;   // [H]: 1 = a chunk of this head decays too fast for the chunkwise form
+    int* seq_heads;   // [H]: 1 = a chunk of this head decays too fast for the chunkwise form, or a token is not finite
     int n_seqs, H;
     WsHeader* hdr;
     int64_t seq_len, chunks_per_seq, n_chunks;
@@ -126,6 +126,20 @@ __device__ __forceinline__ void to_f(const Raw8<float>& r, float (&x)[8]) {
 __device__ __forceinline__ void to_f(const Raw8<__nv_bfloat16>& r, float (&x)[8]) {
 #pragma unroll
     for (int e = 0; e < 4; ++e) { x[2 * e] = __uint_as_float(r.w[e] << 16); x[2 * e + 1] = __uint_as_float(r.w[e] & 0xffff0000u); }
+}
+
+// Whether a value that the split images (kda_split3.cuh) cannot hold is among those looked at: not finite, or
+// rounded to an infinity as a bf16 number.
+__device__ __forceinline__ void look(uint32_t& seen, const Raw8<float>& r) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) seen |= (r.w[e] & 0x7fffffffu) + 0x00808000u;
+}
+__device__ __forceinline__ void look(uint32_t& seen, const Raw8<__nv_bfloat16>& r) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) seen |= (r.w[e] & 0x7f807f80u) + 0x00800080u;
+}
+template <typename T> __device__ __forceinline__ bool seen_odd(uint32_t seen) {
+    return (seen & (sizeof(T) == 4 ? 0x80000000u : 0x80008000u)) != 0u;
 }
 
 kda_status_t launch_bwd_intra(const BwdChunkArgs& a, kda_dtype_t dt, cudaStream_t st);

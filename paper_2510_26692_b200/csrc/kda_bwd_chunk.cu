@@ -15,7 +15,8 @@
 // Three kernels: what is local to a chunk (kda_bwd_intra.cu, all chunks at once), the two state recurrences
 // (kda_bwd_chain.cu, forward and backward chains side by side) and the gradients (kda_bwd_out.cu, all chunks
 // at once).  e^G and e^-G are taken relative to the middle of the chunk's decay range.  A head with a chunk
-// whose log decay leaves [-kBwdRange, 1] is left to the token-sequential kernels (kda_bwd.cu).
+// whose log decay leaves [-kBwdRange, 1], or with a token that is not finite, is left to the token-sequential kernels
+// (kda_bwd.cu).
 #include "kda_bwd.cuh"
 
 namespace kda {

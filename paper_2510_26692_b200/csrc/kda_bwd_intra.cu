@@ -123,7 +123,12 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
             tile[bt::G + r * kD + c] = G[i];
             sG[r * 132 + c] = G[i] - 0.5f * total;
         }
-        if (!(lo >= -kBwdRange && hi <= 1.f && total - total == 0.f)) a.seq_heads[h] = 1;
+        // (a token that is not finite would spoil the earlier ones of its chunk: zeros of a triangle times an infinity)
+        uint32_t seen = 0u;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) { look(seen, kr[j]); look(seen, qr[j]); look(seen, dr[j]); look(seen, vr[j]); }
+        const float b = sBeta[t & 63];
+        if (!(lo >= -kBwdRange && hi <= 1.f && total - total == 0.f && b - b == 0.f) || seen_odd<T>(seen)) a.seq_heads[h] = 1;
         if (seg == 0) {
             sGm[c] = 0.5f * total;
             tile[bt::GC + c] = expf(total);

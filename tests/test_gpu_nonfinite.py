@@ -7,6 +7,7 @@ import torch
 import paper_2510_26692_b200 as K
 from paper_2510_26692_b200 import inputs
 from kda_testlib import oracle_chunk, run_chunk, to_np32
+from test_gpu_backward import cotangents, oracle_bwd, run_bwd
 
 pytestmark = pytest.mark.gpu
 NAN, INF = float("nan"), float("inf")
@@ -61,3 +62,19 @@ def test_segments_keep_non_finite(oracle_mod, what, value):
     assert not bad_o[:640].any() and not bad_o[:, 1].any() and not bad_S[:, 1].any()
     _, S = run_chunk(d, want_o=False)
     assert (~np.isfinite(to_np32(S)))[~np.isfinite(S_ref)].all()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("what,value", [("q", NAN), ("k", NAN), ("v", NAN), ("beta", NAN), ("d_o", NAN), ("k", INF),
+                                        ("v", INF), ("d_o", INF)])
+def test_backward_non_finite(oracle_mod, what, value, dtype):
+    """Gradients are finite where the adjoint of the recurrence is, tokens of the same chunk among them, and right
+    there (fp32 arithmetic: 1e-5)."""
+    d = inputs.chunk_inputs([200], H=2, dtype=dtype, seed=64, s0_std=0.02)
+    d["d_o"], dS_T = cotangents(d, 65, dtype)
+    d = spoiled(d, what, 100, value)
+    got, ref = run_bwd(d, d["d_o"], dS_T), oracle_bwd(oracle_mod, d, d["d_o"], dS_T)
+    for n, x in got.items():
+        x, ok = to_np32(x), np.isfinite(ref[n])
+        assert (np.isfinite(x) == ok).all(), n
+        assert np.linalg.norm(x[ok] - ref[n][ok]) <= 1e-5 * np.linalg.norm(ref[n][ok]), n
