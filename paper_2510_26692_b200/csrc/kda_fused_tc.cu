@@ -7,7 +7,10 @@
 //     a1   G = cumulative sum of log alpha over the chunk's tokens (fp32, log2 domain)
 //          gated operands, bf16:  Kg = K exp(G - G_m),  Qg = scale Q exp(G - G_m),  Ki = K exp(G_m - G)
 //          with G_m = G_C / 2 per channel (the middle of the chunk's log-decay range), so that
-//          exp(G_i - G_j) = exp(G_i - G_m) exp(G_m - G_j) is formed from two factors of bounded range
+//          exp(G_i - G_j) = exp(G_i - G_m) exp(G_m - G_j) is formed from two factors of bounded range.  G_m is taken
+//          as a whole number of halvings: W and Q get their true scale exp(G_m) without another rounding, and the
+//          rounding of Qg is the same in Aqk and in Q S.  (Rounded a second time: error of o 0.2 per cent larger at
+//          a decay of sigmoid(4) a token, 1 per cent at sigmoid(6).)
 //     a2/a5  one tcgen05 MMA group  [Kg ; Qg] (128 x 128)  x  Ki^T (128 x 64)  ->  TMEM:
 //          L = Diag(beta) StrictTril(rows 0-63) (fp32),  Aqk = Tril(rows 64-127) (bf16)
 //     a3   T = (I + L)^-1 by blocked forward substitution: 16x16 diagonal blocks column by column in
@@ -48,6 +51,7 @@ constexpr int LDT = 68;                                   // padded fp32 row of 
 constexpr int LDD = 16;                                   // padded fp32 row of a 16x16 diagonal block
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kClamp2 = 80.f * 1.4426950408889634f;     // the +-80 clamp in the log2 domain
+constexpr float kClampX = kClamp2 + 0.5f;                 // (G_m is rounded to a whole number)
 
 // Optional role timing (compile with -DKDA_FUSED_TIMING): one thread per role accumulates the
 // nanoseconds spent between marks and adds them to the header's spare words at the end.
@@ -81,8 +85,9 @@ constexpr uint32_t E_BAR = E_CUR + 64;          // 8-byte words: mma barrier, K 
                                                   // (first engine) TMEM slot, V barrier
 constexpr uint32_t E_KS = (E_BAR + 96 + 1023) / 1024 * 1024;   // raw k of the NEXT tile [2 K-halves][64][64] bf16
 constexpr uint32_t E_NORM = E_KS + 16384;         // layer mode: 1 / |k_i|, 1 / |q_i| (64 fp32 each)
-constexpr uint32_t E_GV = E_NORM + 512;           // gamma^C and exp(G_m) on their way to the tile
-constexpr uint32_t E_BYTES = (E_GV + tc::GV_BYTES + 1023) / 1024 * 1024;
+constexpr uint32_t E_GV = E_NORM + 512;           // gamma^C and exp(G_C - G_m) on their way to the tile
+constexpr uint32_t E_EM = E_GV + tc::GV_BYTES;    // exp(G_m)
+constexpr uint32_t E_BYTES = (E_EM + 512 + 1023) / 1024 * 1024;
 static_assert(E_TD_BYTES >= 8 * 128 * 4 && E_TD_BYTES >= 4 * 16 * LDD * 4, "scan exchange and diagonal blocks fit");
 
 // ---- shared-memory map of a chain CTA (bytes from the 1024-aligned base) -----------------------------
@@ -520,16 +525,20 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             }
         }
         // reference of the decay factorisation: half the chunk's total log-decay, per channel, so that
-        // |G_i - G_ref| <= |G_C| / 2 for every row whatever the distribution of the decay over the chunk
+        // |G_i - G_ref| <= |G_C| / 2 (+ 1/2) for every row whatever the distribution of the decay over the chunk
 #pragma unroll
-        for (int e = 0; e < 4; ++e) gref[e] = 0.5f * glast[e];
-        float em[4];   // exp(G_m) = exp(G_C - G_m)
+        for (int e = 0; e < 4; ++e) gref[e] = (0.5f * glast[e] + 12582912.f) - 12582912.f;   // to a whole number
+        float em[4];   // exp(G_m), a power of two
 #pragma unroll
         for (int e = 0; e < 4; ++e) em[e] = ex2(gref[e]);
         if (warp == 0) {
+            float ec[4];   // exp(G_C - G_m)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) ec[e] = ex2(glast[e] - gref[e]);
             *reinterpret_cast<float4*>(smem + E_GV + d0 * 4) =
-                make_float4(ex2(glast[0]), ex2(glast[1]), ex2(glast[2]), ex2(glast[3]));
-            *reinterpret_cast<float4*>(smem + E_GV + 512 + d0 * 4) = make_float4(em[0], em[1], em[2], em[3]);
+                make_float4(ec[0] * em[0], ec[1] * em[1], ec[2] * em[2], ec[3] * em[3]);
+            *reinterpret_cast<float4*>(smem + E_GV + 512 + d0 * 4) = make_float4(ec[0], ec[1], ec[2], ec[3]);
+            *reinterpret_cast<float4*>(smem + E_EM + d0 * 4) = make_float4(em[0], em[1], em[2], em[3]);
             // a channel that decays by more than e^-160 inside this chunk leaves the range of the
             // two-factor form: flag it (the clamp below keeps everything finite)
             if (fminf(fminf(glast[0], glast[1]), fminf(glast[2], glast[3])) < -2.f * kClamp2) out_of_range = true;
@@ -610,7 +619,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     float x = G[r][e] + off[e];
-                    if (kClamp) x = fminf(fmaxf(x, -kClamp2), kClamp2);
+                    if (kClamp) x = fminf(fmaxf(x, -kClampX), kClampX);
                     const float e1 = ex2(x);                     // exp(G - G_m)
                     const float e2 = ex2(-x);                    // exp(G_m - G)
                     if (kLayer) {
@@ -634,7 +643,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             }
         };
         {
-            const bool may_clamp = fminf(fminf(gref[0], gref[1]), fminf(gref[2], gref[3])) < -kClamp2;
+            const bool may_clamp = fminf(fminf(gref[0], gref[1]), fminf(gref[2], gref[3])) < -kClamp2 + 0.5f;
             if (__any_sync(0xffffffffu, may_clamp)) gate_rows(std::true_type{});
             else gate_rows(std::false_type{});
         }
@@ -877,8 +886,8 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             ptx::tmem_ld_wait();
 #pragma unroll
             for (int j8 = 0; j8 < 32; j8 += 8) {   // W = exp(G_m) . W'
-                const float4 e0 = *reinterpret_cast<const float4*>(smem + E_GV + 512 + (col0 + j8) * 4);
-                const float4 e1 = *reinterpret_cast<const float4*>(smem + E_GV + 512 + (col0 + j8) * 4 + 16);
+                const float4 e0 = *reinterpret_cast<const float4*>(smem + E_EM + (col0 + j8) * 4);
+                const float4 e1 = *reinterpret_cast<const float4*>(smem + E_EM + (col0 + j8) * 4 + 16);
                 *reinterpret_cast<uint4*>(smem + E_V + (col0 >> 6) * 8192 + ptx::sw128_off(i, (col0 & 63) + j8)) =
                     make_uint4(pack_bf16(__uint_as_float(r[j8]) * e0.x, __uint_as_float(r[j8 + 1]) * e0.y),
                                pack_bf16(__uint_as_float(r[j8 + 2]) * e0.z, __uint_as_float(r[j8 + 3]) * e0.w),

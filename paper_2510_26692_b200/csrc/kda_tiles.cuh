@@ -13,13 +13,13 @@ constexpr uint32_t QW_HALF = 128 * 128;
 // layer calls of few chains: the chunk's output rows in fp32, over [ W ; Q ] once the chain has read them; element
 // (token, column) at float ((token / 4) 128 + column) 4 + token % 4
 constexpr uint32_t OFF_O32 = OFF_QW;
-// K' = K exp(G_m - G), relative to the middle G_m = G_C / 2 of the chunk's log-decay range (the reference of the decay
-// factorisation), as two dk-halves of [64 tokens][64 channels]; the consumer restores exp(G_C - G_m) in fp32
+// K' = K exp(G_m - G), relative to the middle G_m of the chunk's log-decay range (the reference of the decay
+// factorisation: G_C / 2 as a whole number of halvings), as two dk-halves of [64 tokens][64 channels]; the consumer restores exp(G_C - G_m) in fp32
 constexpr uint32_t OFF_KI = 32768;
 constexpr uint32_t KI_HALF = 64 * 128;
 // Aqk [64][64] (lower triangular incl. diagonal)
 constexpr uint32_t OFF_AQ = 49152;
-// gamma^C = exp(G_C) and exp(G_C - G_m) = exp(G_m), 128 fp32 each
+// gamma^C = exp(G_C) and exp(G_C - G_m), 128 fp32 each
 constexpr uint32_t OFF_GV = 57344;
 constexpr uint32_t GV_BYTES = 1024;
 // U^T: 16-byte chunk c holds tokens 8 c .. 8 c + 7 of column `col`; read with plain loads, a thread per column
