@@ -48,6 +48,19 @@ constexpr int T_AQK = T_KT + kC * kD;
 constexpr int T_GC = T_AQK + kC * kC;
 constexpr int T_FLOATS = T_GC + kD;
 
+// The log decay as a sum of two fp32 numbers, lo the rounding errors of hi (Knuth's two-sum); an exponential takes lo
+// as a factor.  With hi alone every decay ratio carries 2^-24 of the chunk's log decay: error of o 2.1e-7 at a decay
+// of sigmoid(4) a token but 7.2e-7 at sigmoid(-1), with lo 2.0e-7 and 2.5e-7.
+struct LogSum { float hi, lo; };
+__device__ __forceinline__ LogSum operator+(LogSum a, float b) {
+    const float s = a.hi + b, z = s - a.hi;
+    return {s, a.lo + ((a.hi - (s - z)) + (b - z))};
+}
+__device__ __forceinline__ LogSum operator-(LogSum a, LogSum b) {
+    const LogSum d = a + -b.hi;
+    return {d.hi, d.lo - b.lo};
+}
+__device__ __forceinline__ float exp_of(LogSum x) { const float e = expf(x.hi); return fmaf(e, x.lo, e); }
 // (a NaN stays one: fminf and fmaxf would turn it into a bound)
 __device__ __forceinline__ float clampf(float x) { return x == x ? fminf(fmaxf(x, -kClamp), kClamp) : x; }
 
@@ -59,8 +72,8 @@ constexpr int QG = KI + 64 * LR;                 // scale Q exp(G - G_m)    [64]
 constexpr int V = QG + 64 * LR;                  // [64][LC]
 constexpr int B = V + 64 * LC;                   // [64][LM]
 constexpr int T = B + 64 * LM;                   // [64][LM]
-constexpr int VEC = T + 64 * LM;                 // exp(G_m) [128], beta [64], segment sums [4][128]
-constexpr int kFloats = VEC + 128 + 64 + 512;
+constexpr int VEC = T + 64 * LM;                 // exp(G_m) [128], beta [64], segment sums [4][128] twice
+constexpr int kFloats = VEC + 128 + 64 + 1024;
 }  // namespace s1
 constexpr size_t kSmem1 = (size_t)s1::kFloats * 4;
 static_assert(kSmem1 <= 232448, "fits the shared memory of one SM");
@@ -109,45 +122,51 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
         z = fmaf(0.f, v.x, fmaf(0.f, v.y, fmaf(0.f, v.z, fmaf(0.f, v.w, z))));
     }
     if (t < 64) sBeta[t] = t < loc.len ? a.beta[(size_t)(loc.tok0 + t) * a.H + h] : 0.f;
-    float run = 0.f;
+    LogSum run = {0.f, 0.f};
 #pragma unroll
-    for (int i = 0; i < 16; ++i) { run += G[i]; G[i] = run; }
-    sSeg[seg * 128 + c] = run;
+    for (int i = 0; i < 16; ++i) run = run + G[i];
+    sSeg[seg * 128 + c] = run.hi;
+    sSeg[512 + seg * 128 + c] = run.lo;
     for (int idx = t; idx < 64 * LM; idx += kT1) sT[idx] = 0.f;
     if (t < 64) z = fmaf(0.f, sBeta[t], z);
     // A token that is not finite may spoil later tokens but no earlier ones: such a tile forms its products entry by
     // entry over the triangle, where a matrix instruction would multiply the zeros beside it.
     const int odd = __syncthreads_or(z != 0.f);
-    float base = 0.f, total = 0.f;
+    LogSum g = {0.f, 0.f}, total = {0.f, 0.f};
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
-        const float x = sSeg[s * 128 + c];
-        if (s < seg) base += x;
-        total += x;
+        if (s == seg) g = total;
+        total = total + sSeg[s * 128 + c];
+        total.lo += sSeg[512 + s * 128 + c];
     }
     // a channel that decays by more than e^-160 inside the chunk leaves the range of the
     // two-factor form (the clamp keeps everything finite): flag the call
-    if (total < -2.f * kClamp) atomicOr(&hdr->flags, 1);
-    const float gm = total == total ? 0.5f * total : 0.f, em = expf(gm);
+    if (total.hi < -2.f * kClamp) atomicOr(&hdr->flags, 1);
+    const bool nan = total.hi != total.hi;
+    const LogSum gm = {nan ? 0.f : 0.5f * total.hi, nan ? 0.f : 0.5f * total.lo};
+    const float em = exp_of(gm);
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         const int r = seg * 16 + i;
-        const float g = G[i] + base;
-        const float e1 = expf(clampf(g - gm)), e2 = expf(clampf(gm - g));
+        g = g + G[i];
+        LogSum x = g - gm;
+        const float cut = clampf(x.hi);
+        x = {cut, cut == x.hi ? x.lo : 0.f};
+        const float e1 = exp_of(x), e2 = exp_of({-x.hi, -x.lo});
         sKG[r * LR + c] = kk[i] * e1;
         sKI[r * LR + c] = kk[i] * e2;
         if (part_q) {
-            const float x = a.scale * qq[i] * e1;
-            sQG[r * LR + c] = x;
-            tile[T_QG + r * kD + c] = x * em;
-            tile[T_KT + r * kD + c] = kk[i] * expf(total - g);
+            const float q1 = a.scale * qq[i] * e1;
+            sQG[r * LR + c] = q1;
+            tile[T_QG + r * kD + c] = q1 * em;
+            tile[T_KT + r * kD + c] = kk[i] * exp_of(total - g);
         }
     }
     if (seg == 0) {
         sEm[c] = em;
-        if (part_q) tile[T_GC + c] = expf(total);
+        if (part_q) tile[T_GC + c] = exp_of(total);
     }
-    const int far = __syncthreads_or(total < kSplitRange) | odd;
+    const int far = __syncthreads_or(total.hi < kSplitRange) | odd;
 
     // a2 + a5: [K^ ; Q] K_^T: warps 4 x 4, 32 x 16 entries each of 128 rows, or 16 x 16 of 64; only blocks that
     // reach the triangle

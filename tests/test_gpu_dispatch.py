@@ -115,3 +115,13 @@ def test_bf16_one_rounding_of_q(oracle_mod, lens, H):
     o, _ = run_chunk(d)
     o_ref, _ = oracle_chunk(oracle_mod, d)
     assert rel_l2(to_np32(o), o_ref) <= 4.85e-3
+
+
+@pytest.mark.parametrize("H", [2, 37])
+def test_fp32_prefill_fast_decay(oracle_mod, H):
+    """Decay of about e^-84 a chunk: the exponents are exact, so the error stays that of the products and sums (2.0e-7
+    at slow decay, plus that of entries far below the largest); 7.2e-7 and 9.8e-7 with the log decay summed in fp32."""
+    d = inputs.chunk_inputs([300], H=H, dtype=torch.float32, seed=58, gate_mean=-1.0, s0_std=0.02)
+    o, S = run_chunk(d)
+    o_ref, S_ref = oracle_chunk(oracle_mod, d)
+    assert rel_l2(to_np32(o), o_ref) <= 4e-7 and rel_l2(to_np32(S), S_ref) <= 3e-7
