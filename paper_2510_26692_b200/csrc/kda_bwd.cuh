@@ -35,8 +35,8 @@ constexpr int X = R + 64 * 128;      // [64][128] rf: P^T dO, replaced by dX = P
 constexpr int N = X + 64 * 128;      // [128][128] rf: Q^T dO
 constexpr int S = N + 128 * 128;     // [128][128] rf: state entering the chunk (forward chain)
 constexpr int L = S + 128 * 128;     // [128][128] rf: adjoint of the state leaving the chunk (backward chain)
-constexpr int G = L + 128 * 128;     // [64][128] cumulative log decay
-constexpr int T = G + 64 * 128;      // [64][64] T'
+constexpr int F = L + 128 * 128;     // [64][128] e^(G - G_m)
+constexpr int T = F + 64 * 128;      // [64][64] T'
 constexpr int B = T + 64 * 64;       // [64][64] B = StrictTril(K^ K_^T)
 constexpr int GC = B + 64 * 64;      // [128] e^(G_C)
 constexpr int EM = GC + 128;         // [128] e^(G_m), also e^(G_C - G_m)
@@ -44,8 +44,7 @@ constexpr int kFloats = EM + 128;
 }  // namespace bt
 __device__ __forceinline__ int rf(int rows, int row, int c) { return ((c >> 2) * rows + row) * 4 + (c & 3); }
 
-// Largest decay of a chunk taken in chunk form.  The cumulative sum is rounded to 2^-24 of its size, so
-// every decay ratio carries a relative error of up to kBwdRange 2^-24 = 2.4e-6.
+// Largest decay of a chunk taken in chunk form.
 constexpr float kBwdRange = 40.f;
 
 // first token, valid tokens (1..64) and sequence of global chunk g
@@ -94,6 +93,12 @@ __device__ __forceinline__ bool bwd_next(const BwdChunkArgs& a, int64_t& g, int&
     return true;
 }
 
+// 1 / x of a factor e^(+-20), one instruction (at most one unit in the last place off)
+__device__ __forceinline__ float reciprocal(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 // Eight consecutive elements as they are stored.  The loads are volatile so that they stay where they are
 // written, ahead of the stores and waits that they overlap; `in` = false gives zeros.
 template <typename T> struct Raw8 { uint32_t w[2 * sizeof(T)]; };

@@ -19,10 +19,10 @@ using namespace split3;
 constexpr int kT = 512;
 constexpr int LM = 68;
 constexpr uint32_t O_RQ = 0, O_RK = 98304, O_RP = O_RK + 49152, O_L = O_RP + 24576, O_T = O_L + 64 * LM * 4,
-                   O_G = O_RP,                       // G [64][132] fp32 before P, L and T' exist
+                   O_G = O_RP,                       // e^(G - G_m) [64][132] fp32 before P, L and T' exist
                    O_VEC = O_T + 64 * LM * 4;
 static_assert(O_G + 64 * 132 * 4 <= O_VEC, "G fits where P, L and T' come to lie");
-constexpr int V_BETA = 0, V_GM = 64, V_SEG = 192, V_BAR = 704;     // floats: beta, G_m, segment sums [4][128], barriers
+constexpr int V_BETA = 0, V_SEG = 64, V_BAR = 1088;     // floats: beta, segment sums [2][4][128], barriers
 constexpr uint32_t kSmem = O_VEC + V_BAR * 4 + 64 + 1024;
 static_assert(kSmem <= 232448, "fits the shared memory of one SM");
 constexpr uint32_t C_N = 0, C_X = 128, C_A = 256, C_W = 256, C_U = 384;   // TMEM columns (A is read before W' is formed)
@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
     bwd_tile(a, blockIdx.x, chunk, h);
     uint8_t* sm = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
     float* vec = reinterpret_cast<float*>(sm + O_VEC);
-    float* sBeta = vec + V_BETA; float* sGm = vec + V_GM; float* sSeg = vec + V_SEG;
+    float* sBeta = vec + V_BETA; float* sSeg = vec + V_SEG;
     uint64_t* bar = reinterpret_cast<uint64_t*>(vec + V_BAR);   // one per group of MMAs, each used once
     uint32_t* slot = reinterpret_cast<uint32_t*>(bar + 4);
     const BwdLoc loc = bwd_locate(a, chunk);
@@ -102,37 +102,40 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
         }
     }
     {
-        float run = 0.f, lo = 0.f, hi = 0.f;
+        LogSum run = {0.f, 0.f};
+        float lo = 0.f, hi = 0.f;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) { run += G[i]; G[i] = run; }
-        sSeg[seg * 128 + c] = run;
+        for (int i = 0; i < 16; ++i) run = run + G[i];
+        sSeg[seg * 128 + c] = run.hi;
+        sSeg[512 + seg * 128 + c] = run.lo;
         __syncthreads();
-        float base = 0.f, total = 0.f;
+        LogSum g = {0.f, 0.f}, total = {0.f, 0.f};
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-            const float x = sSeg[s * 128 + c];
-            if (s < seg) base += x;
-            total += x;
+            if (s == seg) g = total;
+            total = total + sSeg[s * 128 + c];
+            total.lo += sSeg[512 + s * 128 + c];
         }
+        const LogSum gm = {0.5f * total.hi, 0.5f * total.lo};
         float* sG = reinterpret_cast<float*>(sm + O_G);
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const int r = seg * 16 + i;
-            G[i] += base;
-            lo = fminf(lo, G[i]); hi = fmaxf(hi, G[i]);
-            tile[bt::G + r * kD + c] = G[i];
-            sG[r * 132 + c] = G[i] - 0.5f * total;
+            g = g + G[i];
+            lo = fminf(lo, g.hi); hi = fmaxf(hi, g.hi);
+            const float f1 = exp_of(g - gm);
+            tile[bt::F + r * kD + c] = f1;
+            sG[r * 132 + c] = f1;
         }
         // (a token that is not finite would spoil the earlier ones of its chunk: zeros of a triangle times an infinity)
         uint32_t seen = 0u;
 #pragma unroll
         for (int j = 0; j < 2; ++j) { look(seen, kr[j]); look(seen, qr[j]); look(seen, dr[j]); look(seen, vr[j]); }
         const float b = sBeta[t & 63];
-        if (!(lo >= -kBwdRange && hi <= 1.f && total - total == 0.f && b - b == 0.f) || seen_odd<T>(seen)) a.seq_heads[h] = 1;
+        if (!(lo >= -kBwdRange && hi <= 1.f && total.hi - total.hi == 0.f && b - b == 0.f) || seen_odd<T>(seen)) a.seq_heads[h] = 1;
         if (seg == 0) {
-            sGm[c] = 0.5f * total;
-            tile[bt::GC + c] = expf(total);
-            tile[bt::EM + c] = expf(0.5f * total);
+            tile[bt::GC + c] = exp_of(total);
+            tile[bt::EM + c] = exp_of(gm);
         }
     }
     __syncthreads();
@@ -146,8 +149,8 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
             to_f(qr[j], qq);
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                const float x = sG[r * 132 + c8 + e], f1 = expf(x);
-                ki[e] = kk[e] * expf(-x);
+                const float f1 = sG[r * 132 + c8 + e];
+                ki[e] = kk[e] * reciprocal(f1);
                 kk[e] *= f1;
                 qq[e] *= a.scale * f1;
             }

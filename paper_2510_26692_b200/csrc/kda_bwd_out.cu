@@ -25,8 +25,8 @@ constexpr uint32_t O_DX = O_RA + 3 * 8192;                    // dX beside T'
 constexpr uint32_t O_LAM0 = O_RB + 3 * 16384;                 // Lam, v columns 0-63, beside r
 constexpr uint32_t O_LAM1 = O_RA;                             // Lam, v columns 64-127; then K_
 constexpr uint32_t O_DPB = O_RA + 3 * 16384;                  // [dP ; dB]
-// fp32 vectors (floats from O_VEC): beta[64] gm[128] dbeta[8][64] sGC[4][128] colsum[2][64] seg[4][128], then barriers
-constexpr int V_BETA = 0, V_GM = 64, V_DB = 192, V_GC = 704, V_CS = 1216, V_SEG = 1344, V_BAR = 1856;
+// fp32 vectors (floats from O_VEC): beta[64] em[128] dbeta[8][64] sGC[4][128] colsum[2][64] seg[4][128], then barriers
+constexpr int V_BETA = 0, V_EM = 64, V_DB = 192, V_GC = 704, V_CS = 1216, V_SEG = 1344, V_BAR = 1856;
 constexpr uint32_t kSmem = O_VEC + V_BAR * 4 + 64 + 1024;     // + alignment slack
 static_assert(4 * 64 * LR * 4 <= O_VEC, "the staged accumulators fit over the images");
 static_assert(kSmem <= 232448, "fits the shared memory of one SM");
@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     if (a.seq_heads[h]) return;
     uint8_t* sm = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
     float* vec = reinterpret_cast<float*>(sm + O_VEC);
-    float* sBeta = vec + V_BETA; float* sDb = vec + V_DB; float* sGm = vec + V_GM; float* sGC = vec + V_GC;
+    float* sBeta = vec + V_BETA; float* sDb = vec + V_DB; float* sEm = vec + V_EM; float* sGC = vec + V_GC;
     float* sCs = vec + V_CS; float* sSeg = vec + V_SEG;
     uint64_t* bar = reinterpret_cast<uint64_t*>(vec + V_BAR);   // one per group of MMAs, each used once
     uint32_t* slot = reinterpret_cast<uint32_t*>(bar + 6);
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
 #pragma unroll
         for (int j = 0; j < 2; ++j) ldraw_rf(rr[j], tile + bt::R, 64, ra, ca + 64 * j);
         const float b = r < loc.len ? a.beta[(size_t)(loc.tok0 + r) * a.H + h] : 0.f;
-        const float gl = tile[bt::G + 63 * kD + (t & 127)];
+        const float em = tile[bt::EM + (t & 127)];
 #pragma unroll
         for (int j = 0; j < 4; ++j) ldraw_rf(xs[j], tile + bt::S, 128, rs, cs + 32 * j);
         float v[8], u[8];
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         for (int e = 0; e < 8; ++e) v[e] *= b;
         put8<64, 1>(sm + O_RA, r, x, v);
         if (x == 0) sBeta[r] = b;
-        if (t < 128) sGm[t] = 0.5f * gl;
+        if (t < 128) sEm[t] = em;
         float s = 0.f;      // share of r_j . dX_j
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     }
     // meanwhile: e^(G_m) S, and its dot products with Lam
     {
-        const float em = expf(sGm[rs]);
+        const float em = sEm[rs];
         float s = 0.f;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         const int r = row0 + 32 * j;
         ldraw(kr[j], static_cast<const T*>(a.k) + tok_off(r) + c8, r < loc.len);
         ldraw(qr[j], static_cast<const T*>(a.q) + tok_off(r) + c8, r < loc.len);
-        ldraw(gr[j], tile + bt::G + r * kD + c8);
+        ldraw(gr[j], tile + bt::F + r * kD + c8);
     }
     wait(1);
 #pragma unroll
@@ -299,8 +299,8 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         to_f(gr[j], gg[j]);
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const float x = gg[j][e] - sGm[c8 + e], f1 = expf(x);
-            gg[j][e] = kk[j][e] * expf(-x);          // K_
+            const float f1 = gg[j][e];
+            gg[j][e] = kk[j][e] * reciprocal(f1);     // K_
             kk[j][e] *= f1;                          // K^
             qq[j][e] *= a.scale * f1;                // Q
         }
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     }
     // the column pass's inputs: thread = channel c of 16 consecutive tokens
     const int c = t & 127, seg = t >> 7;
-    const float gm = sGm[c];
+    const float ec = sEm[c];          // e^(G_C - G_m): G_m = G_C / 2
     const T* kp = static_cast<const T*>(a.k);
     const T* qp = static_cast<const T*>(a.q);
     float kv[16], qv[16], gv[16];
@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         const bool in = r < loc.len;
         kv[i] = ldv(kp + tok_off(r) + c, in);
         qv[i] = ldv(qp + tok_off(r) + c, in);
-        gv[i] = ldv(tile + bt::G + r * kD + c, true);
+        gv[i] = ldv(tile + bt::F + r * kD + c, true);
     }
     wait(4);
     {
@@ -368,15 +368,13 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     }
     ptx::tc_fence_before();
     __syncthreads();
-    const float ec = expf(gm);        // e^(G_C - G_m): G_m = G_C / 2
     float dG[16], run = 0.f, gsum = 0.f;
 #pragma unroll
     for (int i = 15; i >= 0; --i) {
         const int r = seg * 16 + i;
         const size_t off = tok_off(r) + c;
         const bool in = r < loc.len;
-        const float x = gv[i] - gm;
-        const float f1 = expf(x), f2 = expf(-x);
+        const float f1 = gv[i], f2 = reciprocal(f1);
         const float dq = a.scale * f1 * stage[r * LR + c];
         const float p3 = ec * f2 * stage[(192 + r) * LR + c];       // e^(G_C - G) (beta r Lam^T)
         const float dk1 = f1 * stage[(64 + r) * LR + c], dk2 = fmaf(f2, stage[(128 + r) * LR + c], p3);

@@ -48,19 +48,8 @@ constexpr int T_AQK = T_KT + kC * kD;
 constexpr int T_GC = T_AQK + kC * kC;
 constexpr int T_FLOATS = T_GC + kD;
 
-// The log decay as a sum of two fp32 numbers, lo the rounding errors of hi (Knuth's two-sum); an exponential takes lo
-// as a factor.  With hi alone every decay ratio carries 2^-24 of the chunk's log decay: error of o 2.1e-7 at a decay
-// of sigmoid(4) a token but 7.2e-7 at sigmoid(-1), with lo 2.0e-7 and 2.5e-7.
-struct LogSum { float hi, lo; };
-__device__ __forceinline__ LogSum operator+(LogSum a, float b) {
-    const float s = a.hi + b, z = s - a.hi;
-    return {s, a.lo + ((a.hi - (s - z)) + (b - z))};
-}
-__device__ __forceinline__ LogSum operator-(LogSum a, LogSum b) {
-    const LogSum d = a + -b.hi;
-    return {d.hi, d.lo - b.lo};
-}
-__device__ __forceinline__ float exp_of(LogSum x) { const float e = expf(x.hi); return fmaf(e, x.lo, e); }
+// The log decay as a LogSum.  With its high part alone: error of o 2.1e-7 at a decay of sigmoid(4) a token but 7.2e-7 at
+// sigmoid(-1); with both 2.0e-7 and 2.5e-7.
 // (a NaN stays one: fminf and fmaxf would turn it into a bound)
 __device__ __forceinline__ float clampf(float x) { return x == x ? fminf(fmaxf(x, -kClamp), kClamp) : x; }
 

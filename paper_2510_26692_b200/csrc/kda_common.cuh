@@ -158,6 +158,19 @@ __device__ __forceinline__ ChunkLoc locate_chunk(const ChunkArgs& a, int64_t g) 
     return L;
 }
 
+// A sum of two fp32 numbers, lo the rounding errors of hi (Knuth's two-sum); the exponential takes lo as a factor.  The
+// cumulative log decay in hi alone would give every decay ratio an error of 2^-24 of the chunk's log decay.
+struct LogSum { float hi, lo; };
+__device__ __forceinline__ LogSum operator+(LogSum a, float b) {
+    const float s = a.hi + b, z = s - a.hi;
+    return {s, a.lo + ((a.hi - (s - z)) + (b - z))};
+}
+__device__ __forceinline__ LogSum operator-(LogSum a, LogSum b) {
+    const LogSum d = a + -b.hi;
+    return {d.hi, d.lo - b.lo};
+}
+__device__ __forceinline__ float exp_of(LogSum x) { const float e = expf(x.hi); return fmaf(e, x.lo, e); }
+
 // ---- launchers implemented by the kernel translation units --------------------------------------
 kda_status_t launch_decode(const void* q, const void* k, const void* v, const float* log_alpha,
                            const float* beta, float* S, const int32_t* slot, void* o, int n_seqs,

@@ -123,3 +123,13 @@ def test_backward_fast_decay_heads(oracle_mod, lens, dtype):
         x, y = to_np32(out[n]), ref[n]
         for h in range(4):      # (a decay ratio of head 3 carries up to 38 * 2^-24 = 2.3e-6)
             assert rel_l2(x[:, h], y[:, h]) <= TOL, (n, h)
+
+
+def test_backward_fast_decay_error(oracle_mod):
+    """A chunk decays by about e^-37 (the chunk form goes to e^-40): exact exponents leave the products' and sums'
+    error, 1.9e-7 on dq; 4.1e-7 with the log decay summed in fp32."""
+    d = inputs.chunk_inputs([512], H=4, dtype=torch.float32, seed=33, gate_mean=1.0, s0_std=0.02)
+    d_o, dS_T = cotangents(d, 33, torch.float32)
+    out, ref = run_bwd(d, d_o, dS_T), oracle_bwd(oracle_mod, d, d_o, dS_T)
+    assert rel_l2(to_np32(out["dq"]), ref["dq"]) <= 2.8e-7
+    assert rel_l2(to_np32(out["dS0"]), ref["dS0"]) <= 2.2e-7
