@@ -79,7 +79,8 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
             int64_t i = 0;
             for (; i < nc; ++i) {
                 const float* tile = tile_of(i);
-                if (i >= 2 && !wait(m1, i - 2)) break;
+                // (i >= 2: the second product of chunk i - 2 has been waited for below, and with it the first, which
+                // read this buffer.  The barrier of the first may be a phase further on by now.)
                 ptx::mbar_expect_tx(&fullA[i & 1], kImg);
                 ptx::bulk_g2s(sm + O_A + (i & 1) * kImg, tile + (kFwd ? bt::WI : bt::KI), kImg, &fullA[i & 1]);
                 if (i >= 1 && !wait(m2, i - 1)) { ++i; break; }

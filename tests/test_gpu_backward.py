@@ -133,3 +133,18 @@ def test_backward_fast_decay_error(oracle_mod):
     out, ref = run_bwd(d, d_o, dS_T), oracle_bwd(oracle_mod, d, d_o, dS_T)
     assert rel_l2(to_np32(out["dq"]), ref["dq"]) <= 2.8e-7
     assert rel_l2(to_np32(out["dS0"]), ref["dS0"]) <= 2.2e-7
+
+
+def test_backward_chains_of_every_length(oracle_mod):
+    """Chains of one to six chunks side by side, again and again: the loader's and the products' buffers at every
+    phase of their barriers, the same bits each time."""
+    lens = [64, 128, 130, 256, 5, 320, 384, 200]
+    d = inputs.chunk_inputs(lens, H=5, dtype=torch.bfloat16, seed=34, s0_std=0.02)
+    d_o, dS_T = cotangents(d, 34, torch.bfloat16)
+    first = run_bwd(d, d_o, dS_T)
+    ref = oracle_bwd(oracle_mod, d, d_o, dS_T)
+    for n in NAMES:
+        assert rel_l2(to_np32(first[n]), ref[n]) <= 1e-5
+    for _ in range(10):
+        out = run_bwd(d, d_o, dS_T)
+        assert all(torch.equal(out[n], first[n]) for n in NAMES)
