@@ -1004,7 +1004,6 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
     if (warp == 9) {
         // ================= loader =================
         if (lane == 0) {
-            if (!kRing) ptx::grid_dep_wait();   // the tiles come from the intra-chunk kernel launched just before
             // (kRing) a position is given back this many tiles later, when its copy has landed for certain
             const uint32_t lag = f.n_eng * f.depth >= 3 ? 2 : 0;   // (less than the number of positions)
             static_assert(kStagesA == 2 && kStagesB == 3, "give_back relies on them");
@@ -1408,7 +1407,6 @@ kda_chain_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     extern __shared__ __align__(1024) uint8_t smem[];
     const int t = threadIdx.x, warp = t >> 5;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C_BAR + 500);
-    ptx::grid_dep_launch();   // (what follows waits for this kernel's end before it reads anything)
     if (t == 0) chain_init(smem);
     if (warp == 0) {
         ptx::tmem_alloc(tmem_slot, kTmemCols);
@@ -1421,6 +1419,10 @@ kda_chain_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     if ((ptx::smem_u32(smem) & 1023u) != 0) {
         if (t == 0) report_timeout(f, 90);
     } else {
+        // The tiles, the chunk table and S0 come from kernels before this one.  Only then the next may start: what
+        // that reads before its own wait (the gates of kda_layer_rows_kernel) is older than this kernel's inputs.
+        ptx::grid_dep_wait();
+        ptx::grid_dep_launch();
         chain_run<kHasQ, kRows32, false, kSeg>(f, smem, tmem_base, t, (int)blockIdx.x, &tm_o);
     }
     ptx::tc_fence_before();
@@ -1463,7 +1465,7 @@ kda_intra_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
         if (t == 0) report_timeout(f, 90);   // the operand images need 1024-byte alignment
     } else {
         ptx::grid_dep_wait();     // (launched before the preceding kernel has ended)
-        ptx::grid_dep_launch();   // the chains may set themselves up while this one drains (not before: they read S0)
+        ptx::grid_dep_launch();   // the chains may set themselves up while this one drains
         if (clear_status && blockIdx.x == 0 && t == 0) {
             f.hdr->status = 0;      // (an equal-length call has no prologue kernel to do this)
             f.hdr->where = 0;
@@ -1671,12 +1673,11 @@ kda_status_t launch_chain_tc(const FusedArgs& f, int n_count, cudaStream_t st)
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
-    // only overlap with this library's own intra-chunk kernel, never with a caller's kernel that may still be
-    // producing S0
+    // set up beside this library's own intra-chunk kernel
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = a.g1 > a.g0 && f.seg_mode != 2 ? 1 : 0;     // (nor with the kernel that finds the segments' states)
+    cfg.numAttrs = a.g1 > a.g0 && f.seg_mode != 2 ? 1 : 0;
     ProfScope ps(PROF_INTER, st);
     KDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, chain_fn(has_q, a.rows32, f.seg_mode), f, tm_o));
     count_launch();

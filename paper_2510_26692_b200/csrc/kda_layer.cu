@@ -72,7 +72,8 @@ __global__ void __launch_bounds__(256) kda_layer_epilogue_kernel(__nv_bfloat16* 
 }
 
 // The same from the fp32 rows that the chains left in the scratch tiles: one CTA per (chunk, head), a warp per
-// four tokens, four columns a lane.  The caller's tensors are fetched before the chains have ended.
+// four tokens, four columns a lane.  The caller's tensors are fetched before the chains have ended
+// (kda_chain_tc allows this launch only once everything before it is complete).
 __global__ void __launch_bounds__(512) kda_layer_rows_kernel(ChunkArgs a, const char* __restrict__ tiles,
                                                              __nv_bfloat16* __restrict__ y,
                                                              const __nv_bfloat16* __restrict__ g_o,
