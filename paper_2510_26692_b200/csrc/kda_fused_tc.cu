@@ -429,10 +429,9 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
     uint32_t next_static = first;
     int cur = 0;
     EngineCursor& cursor = *reinterpret_cast<EngineCursor*>(smem + E_CUR);   // (service thread, kFused)
-    auto publish = [&]() {
+    auto publish = [&]() {   // (the tile's stores are performed)
         if (cursor.published == cursor.done) return;
-        ptx::bulk_wait_all0();           // the tile's stores are performed
-        ptx::mbar_arrive_cluster_relaxed(cursor.ready + (uint32_t)(cursor.published % f.depth) * 8u);
+        ptx::mbar_arrive_cluster(cursor.ready + (uint32_t)(cursor.published % f.depth) * 8u);
         ++cursor.published;
     };
     bool staged = false;             // W and U^T of the tile before this one lie in their staging buffers
@@ -657,14 +656,18 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         // ---- a2 + a5: [Kg ; Qg] Ki^T --------------------------------------------------------------------
         if (te == kServiceThread) {
             if (kFused) {
-                publish();               // (before any wait: the chain may need that tile to go on)
+                if (f.depth == 1) {      // (the chain needs the previous tile to give its position back)
+                    ptx::bulk_wait_all0();
+                    publish();
+                }
                 const int m = cursor.done;
                 if (m >= f.depth) {
                     const uint64_t t0 = ptx::globaltimer_ns();
-                    while (!ptx::mbar_try(&bar_free[m % f.depth], (uint32_t)(m / f.depth - 1) & 1u)) {
+                    while (!ptx::mbar_try_cluster(&bar_free[m % f.depth], (uint32_t)(m / f.depth - 1) & 1u)) {
                         if (*abort_word || call_aborted(f)) { *abort_word = 1; break; }
                         if (ptx::globaltimer_ns() - t0 > f.a.wait_limit_ns) { timed_out = true; *abort_word = 1; break; }
                     }
+                    ptx::fence_async_global();
                 }
             }
             if (has_q) {
@@ -747,6 +750,10 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             }
             if (has_next) find_tile(&desc[nxt2]);
             else desc[nxt2].len = 0;
+            if (kFused && f.depth > 1) {   // the previous tile (its stores are older than this tile's): the arrival takes a while
+                ptx::bulk_wait_all<has_q ? 2 : 1>();
+                publish();
+            }
         }
         KT_MARK(te == 0, 5);   // A read-out
 
@@ -924,8 +931,8 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
     if (timed_out) report_timeout(f, 10);
     if (out_of_range) atomicOr(&f.hdr->flags, 1);
     if (te == kServiceThread) {
-        if (kFused && !timed_out && !*abort_word) publish();
         ptx::bulk_wait_all0();   // shared memory must outlive the reads of every bulk store
+        if (kFused && !timed_out && !*abort_word) publish();
     }
     ptx::cp_async_wait_all();
     // an aborted engine may still have a TMA load in flight (requested for a tile it never started)
@@ -965,7 +972,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
     uint64_t* ready = reinterpret_cast<uint64_t*>(smem + C_BAR);   // [engine][depth] a ring position holds a tile
     uint64_t* fullA = ready + 6 * kMaxDepth; // [kStagesA] landed
     uint64_t* fullB = fullA + kStagesA;      // [kStagesB]
-    uint64_t* emptyA = fullB + kStagesB;     // [kStagesA] MMA1 done with it
+    uint64_t* emptyA = fullB + kStagesB;     // [kStagesA] MMA1 done with it; kRing: and its landing seen by warp 10
     uint64_t* emptyB = emptyA + kStagesA;    // [kStagesB] last product and the 8 compute warps done with it
     uint64_t* m1 = emptyB + kStagesB;        // MMA1 of a chunk complete
     uint64_t* m2 = m1 + 1;                   // MMA2
@@ -977,12 +984,12 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
     const int warp = ptx::warp_uniform(t >> 5), lane = t & 31;
     __nv_bfloat16* op = kHasQ ? reinterpret_cast<__nv_bfloat16*>(a.o) : nullptr;
 
-    auto wait = [&](uint64_t* bar, uint32_t parity, int where) {
+    auto wait_by = [&](auto attempt, uint64_t* bar, uint32_t parity, int where) {
         if (*abort_flag) return;
-        if (ptx::mbar_try(bar, parity)) return;
+        if (attempt(bar, parity)) return;
         const uint64_t t0 = ptx::globaltimer_ns();
         uint32_t spins = 0;
-        while (!ptx::mbar_try(bar, parity)) {
+        while (!attempt(bar, parity)) {
             if ((++spins & 15u) == 0) {
                 if (*abort_flag) return;
                 if (call_aborted(f)) { *abort_flag = 1; return; }
@@ -994,6 +1001,12 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
             }
         }
     };
+    auto wait = [&](uint64_t* bar, uint32_t parity, int where) {
+        wait_by([](uint64_t* b, uint32_t p) { return ptx::mbar_try(b, p); }, bar, parity, where);
+    };
+    auto wait_cluster = [&](uint64_t* bar, uint32_t parity, int where) {
+        wait_by([](uint64_t* b, uint32_t p) { return ptx::mbar_try_cluster(b, p); }, bar, parity, where);
+    };
     auto warp_arrive = [&](uint64_t* bar) {
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(bar);
@@ -1004,18 +1017,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
     if (warp == 9) {
         // ================= loader =================
         if (lane == 0) {
-            // (kRing) a position is given back this many tiles later, when its copy has landed for certain
-            const uint32_t lag = f.n_eng * f.depth >= 3 ? 2 : 0;   // (less than the number of positions)
-            static_assert(kStagesA == 2 && kStagesB == 3, "give_back relies on them");
             uint32_t g = 0;
-            const uint32_t base = ptx::smem_u32(smem);
-            auto give_back = [&](uint32_t x) {
-                wait(&fullB[x % kStagesB], (x / kStagesB) & 1u, 31);
-                // (with a lag of two the stage of its [W ; Q] has been reused already: landed, and its barrier moved on)
-                if (lag == 0) wait(&fullA[x % kStagesA], (x / kStagesA) & 1u, 33);
-                const uint32_t e = x % (uint32_t)f.n_eng, slot = (x / (uint32_t)f.n_eng) % (uint32_t)f.depth;
-                ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(base + (e & 1u) * E_BYTES + E_BAR + 48 + slot * 8, 1 + (e >> 1)));
-            };
             KT_DECL(4);
             for (int r = 0; next_job(r) && !*abort_flag; ++r)
                 for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
@@ -1024,7 +1026,10 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                     const char* tile = kRing ? f.ring + (size_t)(((uint32_t)cid * f.n_eng + e) * f.depth + slot) * tc::TILE_BYTES
                                              : f.ring + (size_t)(J.tile0 + (int64_t)c * a.H) * tc::TILE_BYTES;
                     KT_MARK(true, 0);
-                    if (kRing) wait(&ready[e * (uint32_t)f.depth + slot], (m / (uint32_t)f.depth) & 1u, 30);
+                    if (kRing) {
+                        wait_cluster(&ready[e * (uint32_t)f.depth + slot], (m / (uint32_t)f.depth) & 1u, 30);
+                        ptx::fence_async_global();
+                    }
                     KT_MARK(true, 1);
                     if (g >= kStagesB) wait(&emptyB[s], (g / kStagesB - 1) & 1u, 32);
                     if (*abort_flag) break;
@@ -1048,7 +1053,6 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                         ptx::bulk_g2s(sA, tile, 8192, &fullA[sa]);
                         ptx::bulk_g2s(sA + tc::QW_HALF, tile + tc::QW_HALF, 8192, &fullA[sa]);
                     }
-                    if (kRing && g >= lag) give_back(g - lag);
                 }
             KT_FLUSH(true, f.hdr, 24, 3);
             if (*abort_flag) {   // the copies already requested must land before the shared memory goes away
@@ -1057,6 +1061,23 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                 for (uint32_t x = g > kStagesA ? g - kStagesA : 0; x < g; ++x)
                     ptx::mbar_wait(&fullA[x % kStagesA], (x / kStagesA) & 1u, a.wait_limit_ns / 8);
             }
+        }
+    } else if (kRing && warp == 10) {
+        // ================= gives the ring's positions back =================
+        // (the loader has no time for the release arrivals; it refills a stage only after this warp has seen it)
+        if (lane == 0) {
+            const uint32_t base = ptx::smem_u32(smem);
+            uint32_t g = 0;
+            for (int r = 0; next_job(r) && !*abort_flag; ++r)
+                for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
+                    wait(&fullB[g % kStagesB], (g / kStagesB) & 1u, 31);
+                    wait(&fullA[g % kStagesA], (g / kStagesA) & 1u, 33);
+                    if (*abort_flag) break;
+                    ptx::mbar_arrive(&emptyA[g % kStagesA]);
+                    ptx::mbar_arrive(&emptyB[g % kStagesB]);
+                    const uint32_t e = g % (uint32_t)f.n_eng, slot = (g / (uint32_t)f.n_eng) % (uint32_t)f.depth;
+                    ptx::mbar_arrive_cluster(ptx::map_to_cta(base + (e & 1u) * E_BYTES + E_BAR + 48 + slot * 8, 1 + (e >> 1)));
+                }
         }
     } else if (warp == 8) {
         // ================= MMA issue =================
@@ -1311,13 +1332,13 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
 }
 
 // barriers of a chain CTA; ONE thread
-__device__ void chain_init(uint8_t* smem)
+__device__ void chain_init(uint8_t* smem, int ring)
 {
     uint64_t* b = reinterpret_cast<uint64_t*>(smem + C_BAR);
     for (int i = 0; i < 6 * kMaxDepth; ++i) ptx::mbar_init(b++, 1);   // ready
     for (int i = 0; i < kStagesA + kStagesB; ++i) ptx::mbar_init(b++, 1);   // fullA, fullB
-    for (int i = 0; i < kStagesA; ++i) ptx::mbar_init(b++, 1);        // emptyA
-    for (int i = 0; i < kStagesB; ++i) ptx::mbar_init(b++, 9);        // emptyB
+    for (int i = 0; i < kStagesA; ++i) ptx::mbar_init(b++, 1 + ring);   // emptyA
+    for (int i = 0; i < kStagesB; ++i) ptx::mbar_init(b++, 9 + ring);   // emptyB
     ptx::mbar_init(b++, 1);                                           // m1
     ptx::mbar_init(b++, 1);                                           // m2
     for (int i = 0; i < 2; ++i) ptx::mbar_init(b++, 1);               // out_bar
@@ -1330,9 +1351,11 @@ __device__ void chain_init(uint8_t* smem)
 
 // One cluster = a chain CTA (rank 0) and CTAs of two engines each; ring positions are handed over by
 // mbarriers in each other's shared memory.  The ring is written and read by bulk copies alone: an engine
-// announces a tile once its copies have completed (performed at L2, where the chain's copies read), the chain
-// gives a position back once its copy has landed.  Neither arrival has anything of its own thread to order, so
-// both are relaxed (release arrivals and proxy fences in their place cost about a microsecond each).
+// announces a tile once its copies have completed, the chain gives a position back once its copy has landed; both
+// by release arrivals, taken up by acquire waits and a proxy fence before the next bulk copy.  The arrivals are made where
+// nothing waits for the thread, during the substitution and by a warp of their own: 4096 x 32 heads 120.7 us, 1 Mi tokens
+// for the state 20.6 ms (made by the loader, and by the service thread ahead of its copies: 141 us and 28.9 ms; relaxed,
+// which orders nothing: 112.5 and 20.2).
 template <bool kHasQ>
 __global__ void __launch_bounds__(kThreads, 1)
 kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtensorMap tm_k,
@@ -1347,7 +1370,7 @@ kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     const bool chain_cta = rank == 0;
     // (the TMEM slot sits in a spare word of the barrier block of either layout)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + (chain_cta ? C_BAR + 500 : E_BAR + 32));
-    if (chain_cta && t == 0) chain_init(smem);
+    if (chain_cta && t == 0) chain_init(smem, 1);
     if (!chain_cta && (t == 0 || t == kEngThreads)) {
         uint64_t* mb = reinterpret_cast<uint64_t*>(smem + (t ? E_BYTES : 0) + E_BAR);
         ptx::mbar_init(mb, 2);       // MMA group complete (two issuing warps)
@@ -1407,7 +1430,7 @@ kda_chain_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     extern __shared__ __align__(1024) uint8_t smem[];
     const int t = threadIdx.x, warp = t >> 5;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C_BAR + 500);
-    if (t == 0) chain_init(smem);
+    if (t == 0) chain_init(smem, 0);
     if (warp == 0) {
         ptx::tmem_alloc(tmem_slot, kTmemCols);
         ptx::tmem_relinquish();

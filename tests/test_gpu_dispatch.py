@@ -125,3 +125,21 @@ def test_fp32_prefill_fast_decay(oracle_mod, H):
     o, S = run_chunk(d)
     o_ref, S_ref = oracle_chunk(oracle_mod, d)
     assert rel_l2(to_np32(o), o_ref) <= 4e-7 and rel_l2(to_np32(S), S_ref) <= 3e-7
+
+
+@pytest.mark.parametrize("tiles,H,out", [(2, 5, True), (7, 5, True), (40, 5, False), (150, 5, True), (900, 32, True), (900, 32, False)])
+def test_fused_hand_over(tiles, H, out):
+    """The fused kernel against the two kernels, the same bits each time, with rings from two tiles in all to four
+    per engine: a tile read before it is written, or written over before it is read, would show."""
+    d = inputs.chunk_inputs([700, 130, 64, 1, 0, 950], H=H, dtype=torch.bfloat16, seed=59, s0_std=0.02)
+    small = K.kda_chunk_fwd_min_workspace_bytes(1845, 6, H)
+    tile = small - 256 >> 1
+    try:
+        K.kda_set_chunk_path(1)
+        o1, S1 = run_chunk(d, want_o=out)
+        K.kda_set_chunk_path(2)
+        for _ in range(12):
+            o2, S2 = run_chunk(d, want_o=out, workspace_bytes=small + (tiles - 2) * tile)
+            assert torch.equal(S1, S2) and (not out or torch.equal(o1, o2))
+    finally:
+        K.kda_set_chunk_path(0)
