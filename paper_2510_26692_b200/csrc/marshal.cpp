@@ -80,13 +80,19 @@ struct Args {
     void* stream() {
         if (*a++ != Py_None) ok = false;
         if (!ok) return nullptr;
-        return c10::cuda::getCurrentCUDAStream().stream();
+        try {   // (a machine without a GPU throws)
+            return c10::cuda::getCurrentCUDAStream().stream();
+        } catch (...) {
+            ok = false;
+            return nullptr;
+        }
     }
 };
 
 // the element type that an argument `dt` further on names
 at::ScalarType elem(PyObject* dt, bool& ok) {
-    const long v = PyLong_CheckExact(dt) ? PyLong_AsLong(dt) : -1;
+    int over = 0;
+    const long v = PyLong_CheckExact(dt) ? PyLong_AsLongAndOverflow(dt, &over) : -1;
     if (v != KDA_BF16 && v != KDA_F32) ok = false;
     return v == KDA_BF16 ? at::kBFloat16 : at::kFloat;
 }

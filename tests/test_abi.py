@@ -221,3 +221,50 @@ def test_wait_limit_from_environment(lib):
         out = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=env, capture_output=True, text=True)
         assert out.returncode == 0, out.stderr
         assert int(out.stdout.strip().splitlines()[-1]) == want, (val, out.stdout)
+
+
+def _calls():
+    """The entry points with a native marshalling, and their arguments with None and a host tensor for every pointer."""
+    import torch
+    import paper_2510_26692_b200 as K
+    def of(x, ws):
+        return {
+            "kda_decode_step": [x] * 8 + [0, 2, 128, 128, 1.0, K.KDA_BF16],
+            "kda_decode_multi": [x] * 8 + [0, 1, 2, 128, 128, 1.0, K.KDA_BF16],
+            "kda_layer_decode_step": [x] * 9 + [1e-6, 1e-5, x, x, x, 0, 2, 128, 128, 1.0],
+            "kda_chunk_fwd": [x] * 10 + [0, 0, 2, 128, 128, 64, 1.0, K.KDA_BF16, ws],
+            "kda_layer_fwd": [x] * 9 + [1e-6, 1e-5] + [x] * 5 + [0, 0, 2, 128, 128, 64, 1.0, ws],
+            "kda_chunk_bwd": [x] * 16 + [0, 0, 2, 128, 128, 64, 1.0, K.KDA_BF16, ws]}
+    return of(None, torch.zeros(1024, dtype=torch.uint8)), of(torch.zeros(4, dtype=torch.bfloat16), None)
+
+
+def test_binding_raises_and_never_ends_the_process(lib):
+    """Without a GPU, with host tensors, and with element types out of range: a Python exception each time (in a child
+    process: a C++ exception behind the interpreter's back would end it)."""
+    import subprocess
+    import sys
+    code = ("import sys; sys.path.insert(0, 'tests'); import torch, test_abi, paper_2510_26692_b200 as K\n"
+            "none, host = test_abi._calls()\n"
+            "at = dict(kda_decode_step=13, kda_decode_multi=14, kda_chunk_fwd=17, kda_chunk_bwd=23)   # element types\n"
+            "for n in none:\n"
+            "    for args, want in ((none[n], (RuntimeError, AssertionError, ValueError)), (host[n], (ValueError, TypeError, AttributeError))):\n"
+            "        for dt in (1, 2 ** 40, 2 ** 70, -2 ** 70):\n"
+            "            a = list(args)\n"
+            "            if n in at: a[at[n]] = dt\n"
+            "            if torch.cuda.is_available() and args is none[n]: continue\n"
+            "            try: getattr(K, n)(*a)\n"
+            "            except want: continue\n"
+            "            raise SystemExit('%s returned' % n)\n"
+            "print('done')\n")
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.strip().endswith("done"), (r.returncode, r.stdout[-500:], r.stderr[-500:])
+
+
+def test_binding_host_tensors_are_refused(lib):
+    """All six entry points name the first tensor that is not on the GPU."""
+    import paper_2510_26692_b200 as K
+    import torch
+    for n, args in _calls()[1].items():
+        a = [torch.zeros(4, dtype=torch.uint8) if x is None else x for x in args]
+        with pytest.raises(ValueError, match="live on"):
+            getattr(K, n)(*a)
