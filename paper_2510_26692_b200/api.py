@@ -111,6 +111,10 @@ def load():
     lib.kda_version.restype = ctypes.c_char_p
     lib.kda_set_chunk_path.restype = i32
     lib.kda_set_chunk_path.argtypes = [i32]
+    from .build import marshal_fits
+    if not marshal_fits():
+        raise ImportError("_marshal.so is missing or was built for another Python or torch: run `python -m "
+                          "paper_2510_26692_b200.build`; there is no fallback path")
     from . import _marshal
     _marshal.bind(*(ctypes.cast(f, vp).value for f in (
         lib.kda_decode_step, lib.kda_decode_multi, lib.kda_layer_decode_step, lib.kda_chunk_fwd, lib.kda_layer_fwd,

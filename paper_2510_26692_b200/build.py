@@ -39,6 +39,20 @@ def needs_build() -> bool:
     return _older(LIB, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + _headers())
 
 
+def marshal_fits() -> bool:
+    """Whether ``_marshal.so`` was built for this Python and this torch, by the text it carries."""
+    try:
+        with open(MARSHAL, "rb") as f:
+            return _built_for().encode() in f.read()
+    except OSError:
+        return False
+
+
+def _built_for() -> str:
+    import torch
+    return "kda marshalling for python %d.%d, torch %s;" % (sys.version_info[:2] + (torch.__version__,))
+
+
 def _build_marshal() -> None:
     import sysconfig
 
@@ -47,7 +61,8 @@ def _build_marshal() -> None:
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
     tmp = MARSHAL + ".tmp.%d" % os.getpid()
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
-           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)]
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+           "-DKDA_BUILT_FOR=\"%s\"" % _built_for()]
     for d in (os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
               os.path.join(cuda, "include"), sysconfig.get_paths()["include"], os.path.join(ROOT, "include")):
         cmd += ["-I", d]
@@ -57,7 +72,7 @@ def _build_marshal() -> None:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if force or _older(MARSHAL, [MARSHAL_SRC] + _headers()):
+    if force or _older(MARSHAL, [MARSHAL_SRC] + _headers()) or not marshal_fits():
         _build_marshal()
     if not force and not needs_build():
         return LIB

@@ -248,7 +248,8 @@ PyObject* bind(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
 #define FN(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {FN(bind), FN(decode_step), FN(decode_multi), FN(layer_decode_step), FN(chunk_fwd), FN(layer_fwd),
                          FN(chunk_bwd), {nullptr, nullptr, 0, nullptr}};
-PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+// (build.py and api.py look for this text in the file: torch's C++ interface changes from version to version)
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", KDA_BUILT_FOR, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
 

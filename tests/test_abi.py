@@ -268,3 +268,20 @@ def test_binding_host_tensors_are_refused(lib):
         a = [torch.zeros(4, dtype=torch.uint8) if x is None else x for x in args]
         with pytest.raises(ValueError, match="live on"):
             getattr(K, n)(*a)
+
+
+def test_marshalling_of_another_torch_is_refused(lib, monkeypatch, tmp_path):
+    """The native marshalling is compiled against torch's C++ headers: after an upgrade of torch it is built anew, and
+    not called before that."""
+    import torch
+    from paper_2510_26692_b200 import api, build
+    assert build.marshal_fits()
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    assert not build.marshal_fits()
+    monkeypatch.setattr(api, "_lib", None)
+    with pytest.raises(ImportError, match="another Python or torch"):
+        api.kda_version()
+    built = []
+    monkeypatch.setattr(build, "_build_marshal", lambda: built.append(1))
+    build.build()
+    assert built
