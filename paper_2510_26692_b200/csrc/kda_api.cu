@@ -281,21 +281,6 @@ struct LayerMode {
     float rms_eps = 0.f;
 };
 
-// Whether a bf16 call without the layer's functions runs as the fused kernel (kda_set_chunk_path).  It does where
-// the tiles of all chunks do not fit the workspace, and where the chains fit one wave of clusters (37 of four CTAs)
-// with enough tiles to make up for the first ones of each chain, which nothing overlaps: 8 heads x 4096 tokens 101
-// (fused) / 100 us (two kernels), 32 x 1000 42.5 / 43.8, 32 x 4096 113 / 143, 16 x 131072 2720 / 3360; below,
-// 32 x 400 25.5 / 24.1, 8 x 1000 37.7 / 31.5; above, 64 chains 105 / 105, 128 chains 202 / 178, 512 chains 3200 / 2900.
-// Layer calls: never faster (96 chains 294 / 237 us, 8 heads x 4096 145 / 113).
-bool use_fused(int n_seqs, int H, int64_t total_chunks, size_t workspace_bytes)
-{
-    const int mode = g_chunk_path.load(std::memory_order_relaxed);
-    if (mode != 0) return mode == 2;
-    const size_t fixed = ws_layout(n_seqs, H).fixed, row = (size_t)H * tc_tile_bytes();
-    const bool one_pass = workspace_bytes >= fixed && (int64_t)((workspace_bytes - fixed) / row) >= total_chunks;
-    return !one_pass || ((int64_t)n_seqs * H <= 37 && total_chunks * H >= 512);
-}
-
 // Into how many segments the chains of a bf16 call are cut (kda_segments.cu), 1 = none.  All runs of a stage must
 // be resident at once.  Times in us, measured: a chain step 1.33 without, 1.4 (maps) and 1.5 (outputs) with all SMs
 // at it, a tile of the intra-chunk kernel 8 over two CTAs per SM, launches 22 and a border 1.5.
@@ -308,7 +293,7 @@ int segments(int64_t J, int64_t longest, int64_t tiles, bool out, bool layer, in
     const int64_t runs = (n_sm < kMaxRuns ? n_sm : kMaxRuns) / J;
     const int64_t most = out ? (runs + 3) / 2 : (runs + 1) / 2;     // maps of P - 1 and P - 2 segments, or of P and P - 1
     const double intra = 8. * tiles / (2 * n_sm), two = intra + 1.4 * longest + 4.;
-    const double fused = std::max(1.33 * longest, 8. * tiles / (6. * J)) + 17.;
+    const double fused = 1.62 * longest + 17.;
     double best = 0.95 * (layer ? two : std::min(two, fused));      // (layer calls never run fused)
     int P = 1;
     for (int64_t p = 3; p <= most && 4 * p <= longest; ++p) {
@@ -318,8 +303,9 @@ int segments(int64_t J, int64_t longest, int64_t tiles, bool out, bool layer, in
     return P;
 }
 
-// Cluster shape, number of clusters and ring depth of a call of the fused kernel.
-kda_status_t fused_schedule(FusedArgs& f, const std::vector<int64_t>& chunk_cu, int64_t avail, bool has_q)
+// Cluster shape, number of clusters and ring depth of a call of the fused kernel, and the tiles of its most loaded
+// cluster.
+kda_status_t fused_schedule(FusedArgs& f, const std::vector<int64_t>& chunk_cu, int64_t avail, bool has_q, int64_t* load)
 {
     const int H = f.a.H, n_seqs = f.a.n_seqs;
     auto len = [&](int n) { return chunk_cu[n + 1] - chunk_cu[n]; };
@@ -331,17 +317,18 @@ kda_status_t fused_schedule(FusedArgs& f, const std::vector<int64_t>& chunk_cu, 
     // tiles of the most loaded cluster.
     const double chain = has_q ? 1.5 : 1.3, engine = has_q ? 8.0 : 7.5;
     double best = 0.;
+    f.n_clusters = 0;
     for (int i = 0; i < 2; ++i) {
         if (most[i] < 1) continue;
         const int nc = f.J < most[i] ? f.J : most[i];
         int64_t tiles = 0;
         if (f.J <= 4096) {
-            std::vector<int64_t> load((size_t)nc, 0);
+            std::vector<int64_t> at((size_t)nc, 0);
             for (int j = 0; j < f.J; ++j) {
                 const int r = j / nc, c = j - r * nc, n = f.ordered ? f.order[j / H] : j / H;
-                load[(size_t)((r & 1) ? nc - 1 - c : c)] += len(n);
+                at[(size_t)((r & 1) ? nc - 1 - c : c)] += len(n);
             }
-            tiles = *std::max_element(load.begin(), load.end());
+            tiles = *std::max_element(at.begin(), at.end());
         } else {
             tiles = (chunk_cu[n_seqs] * H + nc - 1) / nc;
         }
@@ -351,6 +338,7 @@ kda_status_t fused_schedule(FusedArgs& f, const std::vector<int64_t>& chunk_cu, 
             best = t;
             f.n_clusters = nc;
             f.cluster_size = 3 + i;
+            *load = tiles;
         }
     }
     f.n_eng = 2 * (f.cluster_size - 1);
@@ -358,6 +346,34 @@ kda_status_t fused_schedule(FusedArgs& f, const std::vector<int64_t>& chunk_cu, 
     if ((int64_t)f.n_clusters * f.n_eng > avail) f.n_clusters = (int)(avail / f.n_eng);
     const int64_t per = avail / ((int64_t)f.n_clusters * f.n_eng);
     f.depth = (int)(per < FusedArgs::kMaxDepth ? per : FusedArgs::kMaxDepth);
+    return KDA_OK;
+}
+
+// Whether a bf16 call without the layer's functions runs as the fused kernel (kda_set_chunk_path): always where the
+// tiles of all chunks do not fit the workspace, else by the time of both in us.  Fused: 17, and per tile of the most
+// loaded cluster 1.62 with one chain to a cluster; with several 1.5 where the others idle beside a few long chains, up
+// to 1.9 where all are loaded alike.  Two kernels: a tile 8 with two per SM, a chain step 1.4, 8 for the launches.
+// Measured, fused / two: 32 heads x 1000 tokens 44 / 44, x 1500 58 / 64, x 4096 121 / 148; 16 x 2000 64 / 62;
+// 37 x 900 48 / 43; 8 heads, 7 sequences of 813 .. 5057 tokens 144 / 184, one of 4000 and six of 600 111 / 121, of
+// 100 .. 12000 296 / 345; 32 heads, 2 x 2048 124 / 113; 16 heads, 7 of 500 .. 10000 481 / 432.  Layer calls: never faster.
+kda_status_t use_fused(FusedArgs& f, const std::vector<int64_t>& chunk_cu, const void* workspace, size_t bytes, bool has_q, bool* fused)
+{
+    const int mode = g_chunk_path.load(std::memory_order_relaxed);
+    const size_t fixed = ws_layout(f.a.n_seqs, f.a.H).fixed, row = (size_t)f.a.H * tc_tile_bytes();
+    const int64_t chunks = chunk_cu[f.a.n_seqs];
+    *fused = mode == 2 || (mode == 0 && (bytes < fixed || (int64_t)((bytes - fixed) / row) < chunks));
+    if (mode != 0 || *fused || f.J > kMaxRuns || chunks == 0 || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1))) return KDA_OK;
+    int n_sm = 0;
+    int64_t load = 0, longest = 0;
+    kda_status_t rc = sm_count(&n_sm);
+    if (rc == KDA_OK) rc = fused_schedule(f, chunk_cu, (int64_t)((bytes - kFusedRing) / tc_tile_bytes()), has_q, &load);
+    if (rc != KDA_OK) return rc;
+    if (load == 0) return KDA_OK;
+    for (int n = 0; n < f.a.n_seqs; ++n) longest = std::max(longest, chunk_cu[n + 1] - chunk_cu[n]);
+    const double tiles = (double)chunks * f.a.H, busy = tiles / ((double)f.n_clusters * load);
+    const double per = (f.J <= f.n_clusters ? 1.62 : 1.5 + std::max(0., busy - 0.5)) * (has_q ? 1. : 0.8);
+    const double two = (has_q ? 8. : 7.5) * tiles / (2 * n_sm) + (has_q ? 1.4 : 1.3) * std::max((double)longest, tiles / n_sm) + 8.;
+    *fused = per * load + 17. < 0.93 * two;
     return KDA_OK;
 }
 
@@ -446,7 +462,10 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
                             (size_t)H * tc_tile_bytes() * (size_t)(passes ? std::min<int64_t>(64 * P, total_chunks) : total_chunks);
         if (P > 1 && (workspace_bytes < need || (out && S0 && S0 == S_T))) P = 1;
     }
-    if (dt == KDA_BF16 && P == 1 && !lm.rate && use_fused(n_seqs, H, total_chunks, workspace_bytes)) {
+    bool fused = false;
+    if (dt == KDA_BF16 && P == 1 && !lm.rate)
+        if (const kda_status_t rc = use_fused(f, chunk_cu, workspace, workspace_bytes, q && o, &fused)) return rc;
+    if (fused) {
         const size_t tbf = tc_tile_bytes();
         if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) || workspace_bytes < kFusedRing + 2 * tbf)
             return fail(KDA_ERR_WORKSPACE, "kda_chunk_fwd: workspace must be 256-byte aligned and at "
@@ -464,7 +483,8 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
         f.a.g0 = 0; f.a.g1 = total_chunks; f.a.scale = scale;
         f.a.wait_limit_ns = wait_limit_ns();
         f.ring = wsb + kFusedRing;
-        const kda_status_t rcf = fused_schedule(f, chunk_cu, (int64_t)((workspace_bytes - kFusedRing) / tbf), q && o);
+        int64_t load = 0;
+        const kda_status_t rcf = fused_schedule(f, chunk_cu, (int64_t)((workspace_bytes - kFusedRing) / tbf), q && o, &load);
         if (rcf != KDA_OK) return rcf;
         return launch_fused_tc(f, q != nullptr && o != nullptr, st);
     }

@@ -143,3 +143,15 @@ def test_fused_hand_over(tiles, H, out):
             assert torch.equal(S1, S2) and (not out or torch.equal(o1, o2))
     finally:
         K.kda_set_chunk_path(0)
+
+
+@pytest.mark.parametrize("lens,fused", [([4000] + [600] * 6, True), ([1100] * 7, False)])
+def test_uneven_batches_take_the_faster_schedule(oracle_mod, lens, fused):
+    """More chains (56) than clusters: one launch where a few long chains set the time, three kernels (chunk table, tiles,
+    chains) where all are alike.  Operands rounded to bf16: TOL."""
+    d = inputs.chunk_inputs(lens, H=8, dtype=torch.bfloat16, seed=60, s0_std=0.02)
+    before = K.kda_launch_count()
+    o, S = run_chunk(d)
+    assert K.kda_launch_count() - before == (1 if fused else 3)
+    o_ref, S_ref = oracle_chunk(oracle_mod, d)
+    assert rel_l2(to_np32(o), o_ref) <= TOL[K.KDA_BF16] and rel_l2(to_np32(S), S_ref) <= TOL[K.KDA_BF16]
