@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
     uint64_t* bar = reinterpret_cast<uint64_t*>(vec + V_BAR);   // one per group of MMAs, each used once
     uint32_t* slot = reinterpret_cast<uint32_t*>(bar + 4);
     const BwdLoc loc = bwd_locate(a, chunk);
+    const int marked = *reinterpret_cast<volatile int*>(a.seq_heads + h);    // (by a tile before this one)
     float* tile = a.tiles + (size_t)blockIdx.x * bt::kFloats;
     auto tok_off = [&](int r) { return ((size_t)(loc.tok0 + r) * a.H + h) * kD; };
 
@@ -101,6 +102,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
             }
         }
     }
+    bool out_of_form;
     {
         LogSum run = {0.f, 0.f};
         float lo = 0.f, hi = 0.f;
@@ -132,13 +134,21 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
 #pragma unroll
         for (int j = 0; j < 2; ++j) { look(seen, kr[j]); look(seen, qr[j]); look(seen, dr[j]); look(seen, vr[j]); }
         const float b = sBeta[t & 63];
-        if (!(lo >= -kBwdRange && hi <= 1.f && total.hi - total.hi == 0.f && b - b == 0.f) || seen_odd<T>(seen)) a.seq_heads[h] = 1;
+        out_of_form = !(lo >= -kBwdRange && hi <= 1.f && total.hi - total.hi == 0.f && b - b == 0.f) || seen_odd<T>(seen);
+        if (out_of_form) a.seq_heads[h] = 1;
         if (seg == 0) {
             tile[bt::GC + c] = exp_of(total);
             tile[bt::EM + c] = exp_of(gm);
         }
     }
-    __syncthreads();
+    // A head that the sequential kernels do needs no tiles: its CTAs leave here (4096 x 32 heads, all of them out of
+    // range: the stage 326 us when they went on).
+    if (__syncthreads_or(out_of_form || marked)) {
+        ptx::tc_fence_before();
+        __syncthreads();
+        if (w == 0) ptx::tmem_dealloc((uint32_t)ptx::warp_uniform((int)*slot), 512);
+        return;
+    }
     {
         const float* sG = reinterpret_cast<const float*>(sm + O_G);
 #pragma unroll
