@@ -377,17 +377,18 @@ kda_status_t kda_profile_read(int kind, double *total_ms, int *launches);
 int kda_selftest_device_table(void);
 
 /*
- * The schedule that the fused bf16 prefill kernel of kda_chunk_fwd would use for a batch whose
- * sequence n has chunks_per_seq[n] chunks (HOST array of n_seqs entries), with H heads, room for
- * avail_tiles tiles in the workspace and n_sm multiprocessors: out[0] = Q, the (sequence, head)
- * chains that run side by side in one round; out[1] = R, the tiles per chain that the intra-chunk
- * stage (Section 3.1, the WY / UT part) may run ahead of the state recurrence; out[2] = rounds;
- * out[3] = production indices handed out in total (a round takes its longest chain times its number
- * of chains).  Host arithmetic only: no CUDA call, runs without a GPU.  Returns 0, or 1 on a bad
- * argument; Q = 0 in out[] means that no schedule exists (fewer than two tiles, or too few SMs).
+ * The schedule that the fused bf16 prefill kernel of kda_chunk_fwd would use for a packed batch whose sequence n
+ * has chunks_per_seq[n] chunks (HOST array of n_seqs entries), with H heads, outputs wanted, room for avail_tiles
+ * (>= 2) tiles in the workspace and n_sm / 3 resident clusters of three CTAs or n_sm / 4 of four: out[0] = clusters,
+ * each of which works through a share of the (sequence, head) pairs; out[1] = CTAs of a cluster; out[2] = its engines
+ * in use; out[3] = tiles in flight per engine.  Host arithmetic only: no CUDA call, runs without a GPU.  Returns
+ * 0, or 1 on a bad argument; out[0] = 0 means that no cluster fits the device.
+ * kda_selftest_fused_job is the pair, in the order longest sequence first, that a cluster takes in a round; one past
+ * the last pair is none (no counterparts in the paper).
  */
 int kda_selftest_fused_plan(const int32_t *chunks_per_seq, int n_seqs, int H, int64_t avail_tiles,
                             int n_sm, int64_t out[4]);
+int64_t kda_selftest_fused_job(int n_clusters, int cluster, int round);
 
 /*
  * Upper bound, in nanoseconds, of every wait inside the tensor-core kernels (on a barrier, a flag or

@@ -137,7 +137,7 @@ int64_t max_chunks(int64_t total_tokens, int n_seqs)
 
 // ---- fused bf16 path: workspace = header | ring of tiles ------------------------------------------------
 constexpr size_t kFusedRing = sizeof(WsHeader);
-constexpr int kSlotCap = 64, kRingMax = 16;   // bounds of fused_plan
+constexpr int kRingChains = 64, kRingTiles = 16;   // room for a ring: 1024 tiles (37 clusters of six engines use 4 each: 888)
 // Call counter of the tensor-core kernels, by which a call that gave up marks itself in the header.  It starts at a
 // value drawn per process: device memory handed from one process to the next may still hold the mark of an
 // earlier one.
@@ -154,37 +154,61 @@ uint32_t next_epoch()
     return e ? e : g_epoch.fetch_add(1, std::memory_order_relaxed) + 1;   // never 0
 }
 
-// Schedule of the fused kernel: Q chains run side by side (one round), each with a ring of R tiles;
-// n_prod counts the production indices, a round taking (longest chain) x (chains of the round).
-struct FusedPlan {
-    int64_t Q, R, n_rounds;
-    uint64_t n_prod;
-};
-FusedPlan fused_plan(const std::vector<int64_t>& chunk_cu, int n_seqs, int H, int64_t avail_tiles, int n_sm)
+// Sequences of a packed batch, longest first (f.ordered: the table holds them)
+void order_sequences(FusedArgs& f, const std::vector<int64_t>& chunk_cu, bool packed)
 {
-    FusedPlan P{0, 0, 0, 0};
-    const int64_t J = (int64_t)n_seqs * H;
-    int Qmax = n_sm / 4;
-    if (Qmax > kSlotCap) Qmax = kSlotCap;
-    if (Qmax < 1 || avail_tiles < 2 || J < 1) return P;
-    // whole sequences per round when the heads of one fit, so that the chains of a round have
-    // equal lengths
-    int64_t Q = (H <= Qmax) ? (int64_t)H * (Qmax / H) : Qmax;
-    if (Q > J) Q = J;
-    if (Q * 2 > avail_tiles) Q = avail_tiles / 2;
-    int64_t R = avail_tiles / Q;
-    if (R > kRingMax) R = kRingMax;
-    P.Q = Q; P.R = R; P.n_rounds = (J + Q - 1) / Q;
-    for (int64_t r = 0; r < P.n_rounds; ++r) {
-        const int64_t j0 = r * Q, j1 = (j0 + Q < J ? j0 + Q : J) - 1;
-        int64_t maxlen = 0;
-        for (int64_t n = j0 / H; n <= j1 / H; ++n) {
-            const int64_t len = chunk_cu[n + 1] - chunk_cu[n];
-            maxlen = len > maxlen ? len : maxlen;
+    const int n_seqs = f.a.n_seqs;
+    f.ordered = packed && n_seqs > 1 && n_seqs <= FusedArgs::kMaxOrder;
+    if (!f.ordered) return;
+    for (int n = 0; n < n_seqs; ++n) f.order[n] = (uint16_t)n;
+    std::stable_sort(f.order, f.order + n_seqs, [&](uint16_t x, uint16_t y) {
+        return chunk_cu[x + 1] - chunk_cu[x] > chunk_cu[y + 1] - chunk_cu[y];
+    });
+}
+
+// Cluster shape, number of clusters and ring depth of a call of the fused kernel, for most[i] resident clusters of
+// 3 + i CTAs and room for `avail` (>= 2) tiles; `load`: tiles of the fullest cluster.  false: no cluster is resident.
+bool fused_shape(FusedArgs& f, const std::vector<int64_t>& chunk_cu, int64_t avail, bool has_q, const int (&most)[2], int64_t* load)
+{
+    const int H = f.a.H, n_seqs = f.a.n_seqs;
+    // Two or three engine CTAs per chain: microseconds a tile costs the chain and an engine (measured), times the
+    // tiles of the most loaded cluster.
+    const double chain = has_q ? 1.5 : 1.3, engine = has_q ? 8.0 : 7.5;
+    double best = 0.;
+    f.n_clusters = 0;
+    for (int i = 0; i < 2; ++i) {
+        if (most[i] < 1) continue;
+        const int nc = f.J < most[i] ? f.J : most[i];
+        int64_t tiles = 0;
+        if (f.J <= 4096) {
+            std::vector<int64_t> at((size_t)nc, 0);
+            for (int r = 0; (int64_t)r * nc < f.J; ++r)
+                for (int c = 0; c < nc; ++c) {
+                    const int64_t j = fused_job(nc, c, r);
+                    if (j >= f.J) continue;
+                    const int n = f.ordered ? f.order[j / H] : (int)(j / H);
+                    at[(size_t)c] += chunk_cu[n + 1] - chunk_cu[n];
+                }
+            tiles = *std::max_element(at.begin(), at.end());
+        } else {
+            tiles = (chunk_cu[n_seqs] * H + nc - 1) / nc;
         }
-        P.n_prod += (uint64_t)maxlen * (uint64_t)(j1 - j0 + 1);
+        const double per = engine / (2 * (2 + i)) > chain ? engine / (2 * (2 + i)) : chain;
+        const double t = per * (double)tiles + engine;
+        if (f.n_clusters == 0 || t < best) {
+            best = t;
+            f.n_clusters = nc;
+            f.cluster_size = 3 + i;
+            *load = tiles;
+        }
     }
-    return P;
+    if (f.n_clusters == 0) return false;
+    f.n_eng = 2 * (f.cluster_size - 1);
+    if (avail < f.n_eng) f.n_eng = (int)avail;
+    if ((int64_t)f.n_clusters * f.n_eng > avail) f.n_clusters = (int)(avail / f.n_eng);
+    const int64_t per = avail / ((int64_t)f.n_clusters * f.n_eng);
+    f.depth = (int)(per < FusedArgs::kMaxDepth ? per : FusedArgs::kMaxDepth);
+    return true;
 }
 std::atomic<int> g_chunk_path{0};
 std::atomic<int> g_fuse_output{1};  // kda_layer_fwd: 1 = output stage inside the chains, 0 = a pass of its own
@@ -225,10 +249,19 @@ int kda_selftest_fused_plan(const int32_t* chunks_per_seq, int n_seqs, int H, in
     if (!chunks_per_seq || !out || n_seqs < 1 || H < 1) return 1;
     std::vector<int64_t> chunk_cu((size_t)n_seqs + 1, 0);
     for (int n = 0; n < n_seqs; ++n) chunk_cu[n + 1] = chunk_cu[n] + chunks_per_seq[n];
-    const FusedPlan P = fused_plan(chunk_cu, n_seqs, H, avail_tiles, n_sm);
-    out[0] = P.Q; out[1] = P.R; out[2] = P.n_rounds; out[3] = (int64_t)P.n_prod;
+    if (avail_tiles < 2) return 1;
+    FusedArgs f = {};
+    f.a.n_seqs = n_seqs; f.a.H = H; f.J = n_seqs * H;
+    order_sequences(f, chunk_cu, true);
+    const int most[2] = {n_sm / 3, n_sm / 4};
+    int64_t load = 0;
+    out[0] = out[1] = out[2] = out[3] = 0;
+    if (!fused_shape(f, chunk_cu, avail_tiles, true, most, &load)) return 0;
+    out[0] = f.n_clusters; out[1] = f.cluster_size; out[2] = f.n_eng; out[3] = f.depth;
     return 0;
 }
+
+int64_t kda_selftest_fused_job(int n_clusters, int cluster, int round) { return fused_job(n_clusters, cluster, round); }
 
 uint64_t kda_wait_limit_ns(void) { return wait_limit_ns(); }
 
@@ -244,7 +277,7 @@ size_t kda_chunk_fwd_min_workspace_bytes(int64_t total_tokens, int n_seqs, int H
 {
     if (!shape_ok(dk, dv, chunk, dt) || total_tokens < 0 || n_seqs < 0 || H <= 0) return 0;
     // fp32: state scratch + one tile per head (the call then walks the chunks one at a time).
-    // bf16: what the fused kernel needs -- header, flag words, round table and a ring of two tiles.
+    // bf16: what the fused kernel needs -- header and a ring of two tiles.
     if (dt != KDA_BF16) return ws_layout(n_seqs, H).fixed + align_up((size_t)H * tile_bytes(dt));
     return kFusedRing + 2 * tc_tile_bytes();
 }
@@ -258,9 +291,9 @@ size_t kda_chunk_fwd_workspace_bytes(int64_t total_tokens, int n_seqs, int H, in
     size_t want = fixed + align_up((size_t)max_chunks(total_tokens, n_seqs) * H * tile_bytes(dt));
     if (want > kWorkspaceCap) want = kWorkspaceCap;
     if (dt == KDA_BF16) {
-        // never below a full ring for the fused kernel (the path of a capped workspace)
+        // never below a ring of some depth for the fused kernel
         const int64_t J = (int64_t)n_seqs * H;
-        const size_t ring = kFusedRing + (size_t)(J < kSlotCap ? J : kSlotCap) * kRingMax * tc_tile_bytes();
+        const size_t ring = kFusedRing + (size_t)(J < kRingChains ? J : kRingChains) * kRingTiles * tc_tile_bytes();
         if (want < ring) want = ring;
     }
     if (dt == KDA_BF16 && (int64_t)n_seqs * H <= kMaxRuns / 3) want = std::min(want + kSegScratch, kWorkspaceCap);   // (segments of long chains)
@@ -303,49 +336,14 @@ int segments(int64_t J, int64_t longest, int64_t tiles, bool out, bool layer, in
     return P;
 }
 
-// Cluster shape, number of clusters and ring depth of a call of the fused kernel, and the tiles of its most loaded
-// cluster.
+// fused_shape for the current device
 kda_status_t fused_schedule(FusedArgs& f, const std::vector<int64_t>& chunk_cu, int64_t avail, bool has_q, int64_t* load)
 {
-    const int H = f.a.H, n_seqs = f.a.n_seqs;
-    auto len = [&](int n) { return chunk_cu[n + 1] - chunk_cu[n]; };
     int most[2];
     const kda_status_t rc = fused_max_clusters(most);
     if (rc != KDA_OK) return rc;
-    if (most[0] < 1 && most[1] < 1) return fail(KDA_ERR_UNSUPPORTED, "kda_chunk_fwd: the device holds no cluster of the fused kernel");
-    // Two or three engine CTAs per chain: microseconds a tile costs the chain and an engine (measured), times the
-    // tiles of the most loaded cluster.
-    const double chain = has_q ? 1.5 : 1.3, engine = has_q ? 8.0 : 7.5;
-    double best = 0.;
-    f.n_clusters = 0;
-    for (int i = 0; i < 2; ++i) {
-        if (most[i] < 1) continue;
-        const int nc = f.J < most[i] ? f.J : most[i];
-        int64_t tiles = 0;
-        if (f.J <= 4096) {
-            std::vector<int64_t> at((size_t)nc, 0);
-            for (int j = 0; j < f.J; ++j) {
-                const int r = j / nc, c = j - r * nc, n = f.ordered ? f.order[j / H] : j / H;
-                at[(size_t)((r & 1) ? nc - 1 - c : c)] += len(n);
-            }
-            tiles = *std::max_element(at.begin(), at.end());
-        } else {
-            tiles = (chunk_cu[n_seqs] * H + nc - 1) / nc;
-        }
-        const double per = engine / (2 * (2 + i)) > chain ? engine / (2 * (2 + i)) : chain;
-        const double t = per * (double)tiles + engine;
-        if (f.n_clusters == 0 || t < best) {
-            best = t;
-            f.n_clusters = nc;
-            f.cluster_size = 3 + i;
-            *load = tiles;
-        }
-    }
-    f.n_eng = 2 * (f.cluster_size - 1);
-    if (avail < f.n_eng) f.n_eng = (int)avail;          // (avail >= 2)
-    if ((int64_t)f.n_clusters * f.n_eng > avail) f.n_clusters = (int)(avail / f.n_eng);
-    const int64_t per = avail / ((int64_t)f.n_clusters * f.n_eng);
-    f.depth = (int)(per < FusedArgs::kMaxDepth ? per : FusedArgs::kMaxDepth);
+    if (!fused_shape(f, chunk_cu, avail, has_q, most, load))
+        return fail(KDA_ERR_UNSUPPORTED, "kda_chunk_fwd: the device holds no cluster of the fused kernel");
     return KDA_OK;
 }
 
@@ -439,13 +437,7 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
     if (dt == KDA_BF16) {
         f.a.n_seqs = n_seqs; f.a.H = H; f.a.cu_seqlens = cu_seqlens_dev;
         f.J = n_seqs * H;
-        f.ordered = cu_seqlens_dev != nullptr && n_seqs > 1 && n_seqs <= FusedArgs::kMaxOrder;
-        if (f.ordered) {
-            for (int n = 0; n < n_seqs; ++n) f.order[n] = (uint16_t)n;
-            std::stable_sort(f.order, f.order + n_seqs, [&](uint16_t x, uint16_t y) {
-                return chunk_cu[x + 1] - chunk_cu[x] > chunk_cu[y + 1] - chunk_cu[y];
-            });
-        }
+        order_sequences(f, chunk_cu, cu_seqlens_dev != nullptr);
         f.epoch = next_epoch();
     }
     int P = 1;

@@ -99,6 +99,12 @@ struct FusedArgs {
     float* seg_scratch;              // [chain][seg_runs][128][128]
 };
 
+// Job number r of cluster cid of the fused kernel: the clusters take turns back and forth, so that with the longest
+// sequences first their loads stay close to each other.
+__host__ __device__ __forceinline__ int64_t fused_job(int n_clusters, int cid, int r) {
+    return (int64_t)r * n_clusters + ((r & 1) ? n_clusters - 1 - cid : cid);
+}
+
 // ---- dtype helpers ------------------------------------------------------------------------------
 template <typename T> struct IO;
 template <> struct IO<float> {

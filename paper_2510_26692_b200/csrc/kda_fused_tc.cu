@@ -212,10 +212,9 @@ __device__ __forceinline__ float* state_out(const FusedArgs& f, size_t off, int 
     if (kSeg == 2 && seg_info<2>(f, id).p + 1 < f.seg_P) return nullptr;
     return f.a.S_out ? f.a.S_out + off : nullptr;
 }
-// Job number r of cluster cid; false past its last.  Sequences come longest first (f.order) and the
-// clusters take turns back and forth, so that their loads stay close to each other.
+// Job number r of cluster cid (fused_job; sequences by f.order); false past its last.
 __device__ __forceinline__ bool job_info(const FusedArgs& f, int cid, int r, JobInfo& I) {
-    const int64_t jr = (int64_t)r * f.n_clusters + ((r & 1) ? f.n_clusters - 1 - cid : cid);
+    const int64_t jr = fused_job(f.n_clusters, cid, r);
     if (jr >= f.J) return false;
     const int rank = (int)jr / f.a.H;
     I.h = (int)jr - rank * f.a.H;

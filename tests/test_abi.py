@@ -130,40 +130,36 @@ def _plan(lib, chunks, H, avail, n_sm):
 
 
 def test_fused_schedule_plan(lib):
-    """Host side of the fused prefill kernel: how many (sequence, head) chains run side by side, how
-    deep their tile rings are, and how many production indices the call hands out.  Checked against
-    the constraints the kernel relies on and against a count by enumeration."""
+    """Host side of the fused prefill kernel: clusters, engines and ring depth of a call within the constraints that the
+    kernel relies on, and every (sequence, head) pair dealt out exactly once."""
     import random
     rng = random.Random(7)
+    lib.kda_selftest_fused_job.restype = ctypes.c_int64
     cases = [([64], 32, 1024, 148), ([3, 11, 1, 5, 0, 14, 4, 3, 2, 0, 7], 5, 40, 148),
-             ([5, 4], 40, 1024, 148), ([1], 1, 2, 148), ([9] * 7, 3, 7, 148), ([2, 2], 2, 1000, 8)]
+             ([5, 4], 40, 1024, 148), ([1], 1, 2, 148), ([9] * 7, 3, 7, 148), ([2, 2], 2, 1000, 8),
+             ([4000, 20], 32, 5, 148), ([1] * 300, 32, 888, 148), ([3], 2, 3, 3)]
     for _ in range(200):
         n = rng.randint(1, 12)
         cases.append(([rng.randint(0, 20) for _ in range(n)], rng.randint(1, 70),
-                      rng.randint(2, 1200), rng.choice([4, 16, 132, 148, 160, 400])))
+                      rng.randint(2, 1200), rng.choice([3, 4, 16, 132, 148, 160, 400])))
     for chunks, H, avail, n_sm in cases:
-        Q, R, n_rounds, n_prod = _plan(lib, chunks, H, avail, n_sm)
+        n_clusters, size, n_eng, depth = _plan(lib, chunks, H, avail, n_sm)
+        what = (chunks, H, avail, n_sm, n_clusters, size, n_eng, depth)
         J = len(chunks) * H
-        q_max = min(n_sm // 4, 64)          # two CTAs per chain, as many CTAs again for the tiles
-        assert 1 <= Q <= min(J, q_max), (chunks, H, avail, n_sm, Q)
-        assert 2 <= R <= 16 and Q * R <= avail          # the rings fit the workspace
-        assert n_rounds == -(-J // Q)
-        if H <= q_max and Q * 2 <= avail and Q < J and (H * (q_max // H)) * 2 <= avail:
-            assert Q % H == 0                           # whole sequences per round
-        # enumeration: every round takes (its longest chain) x (its chains) indices, and each
-        # (chain, chunk) pair of the batch gets exactly one of them
-        total, tiles = 0, 0
-        for r in range(n_rounds):
-            js = range(r * Q, min((r + 1) * Q, J))
-            longest = max(chunks[j // H] for j in js)
-            for c in range(longest):
-                for j in js:
-                    total += 1
-                    tiles += c < chunks[j // H]
-        assert total == n_prod and tiles == sum(chunks) * H
-    # no schedule: fewer than two tiles of room, or a device with fewer than four SMs
-    assert _plan(lib, [4], 2, 1, 148)[0] == 0
-    assert _plan(lib, [4], 2, 64, 3)[0] == 0
+        assert size in (3, 4) and 1 <= n_clusters <= min(J, n_sm // size), what
+        assert 2 <= n_eng <= 2 * (size - 1) and 1 <= depth <= 4, what
+        assert n_clusters * n_eng * depth <= avail, what                        # the rings fit the workspace
+        assert depth == 4 or n_clusters * n_eng * (depth + 1) > avail, what     # and no room is left unused
+        jobs = []
+        for c in range(n_clusters):
+            r = 0
+            while lib.kda_selftest_fused_job(n_clusters, c, r) < J:
+                jobs.append(lib.kda_selftest_fused_job(n_clusters, c, r))
+                r += 1
+            # (a cluster stops at its first round without a job: there is none after it)
+            assert lib.kda_selftest_fused_job(n_clusters, c, r + 1) >= J, what
+        assert sorted(jobs) == list(range(J)), what
+    assert _plan(lib, [4], 2, 64, 2)[0] == 0      # no cluster of three CTAs
 
 
 def test_side_entry_points_reject_bad_arguments(lib):
