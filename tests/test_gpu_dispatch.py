@@ -66,8 +66,8 @@ def test_fp32_prefill_splits(oracle_mod, lens, H):
 
 @pytest.mark.parametrize("lens,H", [([960], 37), ([832], 37), ([896], 38), ([70, 130], 37), ([1] * 256 + [90], 1)])
 def test_bf16_schedules(oracle_mod, lens, H):
-    """Around the lines between the fused kernel and two kernels (512 tiles, 37 chains), and more
-    sequences than the table of lengths holds.  Operands rounded to bf16: TOL."""
+    """Fused kernel and two kernels near the line between them, and more sequences than the table of
+    lengths holds.  Operands rounded to bf16: TOL."""
     d = inputs.chunk_inputs(lens, H=H, dtype=torch.bfloat16, seed=54, s0_std=0.02)
     o, S = run_chunk(d)
     o_ref, S_ref = oracle_chunk(oracle_mod, d)
@@ -155,3 +155,51 @@ def test_uneven_batches_take_the_faster_schedule(oracle_mod, lens, fused):
     assert K.kda_launch_count() - before == (1 if fused else 3)
     o_ref, S_ref = oracle_chunk(oracle_mod, d)
     assert rel_l2(to_np32(o), o_ref) <= TOL[K.KDA_BF16] and rel_l2(to_np32(S), S_ref) <= TOL[K.KDA_BF16]
+
+
+def test_bf16_segments_in_passes(oracle_mod):
+    """The final state of one sequence with a workspace for 320 chunks of 323: cut into segments twice, the state of the
+    first pass entering the second, whose 3 chunks are fewer than the segments.  No further from the oracle than the
+    uncut chains but for other roundings (a tenth)."""
+    H, T = 16, 323 * 64 - 30
+    d = inputs.chunk_inputs([T], H=H, dtype=torch.bfloat16, seed=66, s0_std=0.02)
+    tile = (K.kda_chunk_fwd_min_workspace_bytes(T, 1, H) - 256) // 2
+    row = H * tile
+    fixed = K.kda_layer_fwd_min_workspace_bytes(T, 1, H) - row
+    nbytes = fixed + 320 * row + 148 * 65536 + 256
+    assert nbytes < K.kda_chunk_fwd_workspace_bytes(T, 1, H)
+    _, S_ref = oracle_chunk(oracle_mod, d, want_o=False)
+    before = K.kda_launch_count()
+    _, S = run_chunk(d, want_o=False, workspace_bytes=nbytes)
+    assert K.kda_launch_count() - before == 6          # tiles, maps, states: twice
+    K.kda_set_chunk_path(1)
+    try:
+        _, S1 = run_chunk(d, want_o=False)
+    finally:
+        K.kda_set_chunk_path(0)
+    err = rel_l2(to_np32(S), S_ref)
+    assert err <= TOL[K.KDA_BF16] and err <= 1.1 * rel_l2(to_np32(S1), S_ref)
+
+
+@pytest.mark.parametrize("out", [True, False])
+@pytest.mark.parametrize("lens,H", [([4100], 3), ([5000, 4000], 8)])
+def test_bf16_long_chains_in_place(oracle_mod, lens, H, out):
+    """S_T over S0 where chains are cut for the state alone, and may not be with outputs: the last segment would write
+    the state that the first may still have to read."""
+    d = inputs.chunk_inputs(lens, H=H, dtype=torch.bfloat16, seed=67, s0_std=0.3, device="cuda:0")
+    T, N, cu = sum(lens), len(lens), d["cu_seqlens"]
+    S = d["S0"].clone()
+    o = torch.full_like(d["v"], float("nan")) if out else None
+    ws = torch.empty(K.kda_chunk_fwd_workspace_bytes(T, N, H), dtype=torch.uint8, device="cuda:0")
+    before = K.kda_launch_count()
+    K.kda_chunk_fwd(d["q"] if out else None, d["k"], d["v"], d["log_alpha"], d["beta"], S, o, S, cu.cuda() if N > 1 else None,
+                    cu.cpu() if N > 1 else None, N, T, H, 128, 128, 64, 1.0, K.KDA_BF16, ws)
+    torch.cuda.synchronize()
+    launches = K.kda_launch_count() - before
+    if out:
+        assert launches <= 2 + (N > 1)                  # not cut
+    else:
+        assert launches == 3 + (N > 1)                  # (chunk table,) tiles, maps, states
+    o_ref, S_ref = oracle_chunk(oracle_mod, d, want_o=out)
+    assert rel_l2(to_np32(S), S_ref) <= TOL[K.KDA_BF16]
+    assert not out or rel_l2(to_np32(o), o_ref) <= TOL[K.KDA_BF16]

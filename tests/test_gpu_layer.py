@@ -90,11 +90,11 @@ def test_layer_equals_plain_call_on_precomputed_inputs(oracle_mod):
 
 
 def test_layer_output_stage_fused_and_separate_agree(oracle_mod):
-    """The output stage inside the inter-chunk kernel (clusters exchanging the rows' sums of squares)
-    against the same stage as a separate pass: both within tolerance of the oracle, and close to each
-    other (the separate pass normalises the bf16-rounded output)."""
+    """The output stage from the fp32 rows that the chains leave (up to 37 chains) against the same stage on the bf16
+    output: both within tolerance of the oracle, and close to each other but not the same (the second normalises
+    rounded rows)."""
     scale = 128 ** -0.5
-    for lens, H in (([700, 130, 64], 4), ([2048], 40)):      # 40 heads: more chains than 32-column slices fit
+    for lens, H in (([700, 130, 64], 4), ([1024], 37)):
         d = inputs.layer_inputs(lens, H=H, seed=44, s0_std=0.02)
         try:
             K.kda_layer_set_fused_output(False)
@@ -107,7 +107,7 @@ def test_layer_output_stage_fused_and_separate_agree(oracle_mod):
         e_sep, e_fus = rel_l2(to_np32(y_sep), y_ref), rel_l2(to_np32(y_fus), y_ref)
         print("output stage", lens, H, "separate", e_sep, "fused", e_fus)
         assert e_sep <= TOL and e_fus <= TOL
-        assert rel_l2(to_np32(y_fus), to_np32(y_sep)) <= 1e-2
+        assert rel_l2(to_np32(y_fus), to_np32(y_sep)) <= 1e-2 and not torch.equal(y_fus, y_sep)
 
 
 def test_layer_decode_step_matches_oracle(oracle_mod):

@@ -537,10 +537,9 @@ def test_fused_kernel_matches_two_kernel_path(oracle_mod, lens, H):
         K.kda_set_chunk_path(0)
 
 
-def test_many_chains_wide_inter_kernel(oracle_mod):
-    """More (sequence, head) chains than the device has SMs: the inter-chunk stage then runs in its
-    128-columns-per-CTA form.  Against the oracle, with several passes (bit-identical: the form is
-    chosen per call, not per pass), state-only, and without an initial state."""
+def test_many_chains(oracle_mod):
+    """More (sequence, head) chains than the device has SMs: two kernels, the chains in two waves.  Against the
+    oracle, with several passes (bit-identical), state-only, and without an initial state."""
     lens = [100, 64, 1, 200, 0, 333]
     H = 40                                              # 240 chains
     d = inputs.chunk_inputs(lens, H=H, dtype=torch.bfloat16, seed=51, s0_std=0.02)
