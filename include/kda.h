@@ -68,7 +68,7 @@ typedef enum { KDA_F32 = 0, KDA_BF16 = 1 } kda_dtype_t;
  * Workspace size that lets kda_chunk_fwd keep every (chunk, head) tile of the call at once (the
  * fastest schedule on this device: one kernel per stage), capped at 8 GiB.  Any workspace of at
  * least kda_chunk_fwd_min_workspace_bytes() works: with less than the full size a bf16 call runs
- * as one fused kernel whose stages exchange tiles through a ring (of up to 16 tiles per running
+ * as one fused kernel whose stages exchange tiles through a ring (of up to 24 tiles per running
  * head) inside the workspace, and an fp32 call proceeds in several passes over ranges of chunks
  * with the state carried between them.  Both return 0 for an unsupported shape.
  */
@@ -120,9 +120,9 @@ kda_status_t kda_chunk_fwd(const void *q, const void *k, const void *v, const fl
  * Same arguments, results and error codes as kda_chunk_fwd, with these differences:
  *   - A call whose minimum scratch (kda_chunk_fwd_min_workspace_bytes) exceeds the 16 MiB is
  *     rejected with KDA_ERR_WORKSPACE and a message naming both sizes; nothing is launched.  For
- *     bf16 the minimum is a few hundred KiB plus 4 bytes per (sequence, head), so practically every
- *     batch fits: the call runs as the fused kernel with a ring of about 220 tiles (e.g. 6 tiles
- *     ahead for each of 32 concurrently running heads).  For fp32 the minimum holds 64 KiB of state
+ *     bf16 the minimum is 150 KiB whatever the batch: the call runs as the fused kernel with a ring of
+ *     224 tiles (6 tiles ahead for each of 32 concurrently running heads), or as two kernels where
+ *     all tiles fit.  For fp32 the minimum holds 64 KiB of state
  *     scratch per (sequence, head), which limits that path to about 200 of them.
  *   - The first call on each device looks up the array's device address
  *     (cudaGetSymbolAddress, with the calling thread's current device).  Make that first call
@@ -159,13 +159,11 @@ kda_status_t kda_chunk_fwd_static(const void *q, const void *k, const void *v,
  *
  * The normalisation, the decay function and the sigmoid of beta are computed inside the
  * intra-chunk kernel from the half-precision pre-activations (no fp32 gate tensor and no
- * normalised copy of q and k ever exists in memory).  The output stage runs inside the inter-chunk
- * kernel: the CTAs that hold the column slices of one (sequence, head) are launched as a thread-block
- * cluster and exchange each row's sums of squares through distributed shared memory.  Where the
- * device cannot keep as many clusters resident as the call has work for (or after
- * kda_layer_set_fused_output(0)), the stage runs as a separate pass over the bf16 output, in place;
- * the results of the two forms differ by rounding only (the separate pass normalises the rounded
- * bf16 output).
+ * normalised copy of q and k ever exists in memory).  The output stage is a kernel behind the
+ * inter-chunk one.  With up to 37 (sequence, head) pairs it starts from fp32 output rows, which the
+ * inter-chunk kernel leaves in the workspace; with more (or after kda_layer_set_fused_output(0)) it
+ * runs over the bf16 output, in place.  The results of the two forms differ by rounding only (the
+ * second normalises the rounded bf16 output).
  *
  *   q_c, k_c, g_a [T_total,H,dk], v, g_o, y [T_total,H,dv]   bf16 device
  *   b_pre [T_total,H]                                        fp32 device
@@ -177,7 +175,7 @@ kda_status_t kda_chunk_fwd_static(const void *q, const void *k, const void *v,
  * Only dk = dv = 128 and chunk = 64.  Asynchronous; nothing is allocated; errors and the status
  * word as for kda_chunk_fwd.
  */
-/* Process-wide switch (default 1): 0 makes kda_layer_fwd always run its output stage as a pass of its own. */
+/* Process-wide switch (default 1): 0 makes kda_layer_fwd always run its output stage on the bf16 output. */
 kda_status_t kda_layer_set_fused_output(int on);
 size_t kda_layer_fwd_workspace_bytes(int64_t total_tokens, int n_seqs, int H, int dk, int dv, int chunk);
 size_t kda_layer_fwd_min_workspace_bytes(int64_t total_tokens, int n_seqs, int H, int dk, int dv, int chunk);
@@ -215,8 +213,9 @@ kda_status_t kda_layer_decode_step(const void *q_c, const void *k_c, const void 
  * recomputed inside (nothing has to be kept from kda_chunk_fwd), in the chunkwise form of Section 3.1:
  * per-chunk quantities of all chunks at once, the recurrences of the state and of its adjoint over
  * the chunks, then the gradients of all chunks at once.  Heads in which some chunk's log decay
- * leaves [-40, 1] run token by token instead (any decay is exact there).  Inputs of the matrix
- * products keep 22 significant bits, sums are fp32.
+ * leaves [-40, 1], or some token is not finite, run token by token instead (any decay is exact there).
+ * Inputs of the matrix products keep 24 significant bits, sums are fp32: relative errors of 1.3e-7 to
+ * 6e-7 where a chunk decays by e^-4, up to 7.6e-7 (dlog_alpha) near e^-40; token by token 1e-7 to 1.5e-7 there.
  *
  *   q, k [T_total,H,dk], v, d_o [T_total,H,dv]   device, element type `dt` (KDA_F32 or KDA_BF16)
  *   log_alpha [T_total,H,dk], beta [T_total,H]   fp32 device

@@ -284,8 +284,8 @@ def kda_chunk_bwd(q, k, v, log_alpha, beta, S0, d_o, dS_T, dq, dk_out, dv_out, d
 
 
 def kda_layer_set_fused_output(on: bool) -> None:
-    """False: ``kda_layer_fwd`` runs its output stage as a separate pass (default: inside the
-    inter-chunk kernel when the device can hold the clusters this needs)."""
+    """False: ``kda_layer_fwd`` always runs its output stage on the bf16 output (default: from fp32 rows with up to
+    37 (sequence, head) pairs)."""
     _check(load().kda_layer_set_fused_output(1 if on else 0))
 
 

@@ -211,7 +211,7 @@ bool fused_shape(FusedArgs& f, const std::vector<int64_t>& chunk_cu, int64_t ava
     return true;
 }
 std::atomic<int> g_chunk_path{0};
-std::atomic<int> g_fuse_output{1};  // kda_layer_fwd: 1 = output stage inside the chains, 0 = a pass of its own
+std::atomic<int> g_fuse_output{1};  // kda_layer_fwd: 1 = output stage from fp32 rows where the chains are few, 0 = from bf16 rows
 
 }  // namespace
 }  // namespace kda

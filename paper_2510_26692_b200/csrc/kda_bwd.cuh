@@ -1,4 +1,4 @@
-// What the two translation units of the backward pass share: the arguments and the per-(chunk, head)
+// What the translation units of the backward pass share: the arguments and the per-(chunk, head)
 // scratch tile of the chunkwise form (kda_bwd_chunk.cu); kda_bwd.cu holds the entry point and the
 // token-sequential form.
 #pragma once

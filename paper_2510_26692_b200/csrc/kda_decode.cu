@@ -6,8 +6,8 @@
 // registers, and the state is written back exactly once.  HBM-bound: 64 KiB read + 64 KiB written
 // per (sequence, head).
 //
-// One CTA of 256 threads owns one state.  Thread (warp w, lane l) holds rows w, w+8, ... and the
-// four columns 4l..4l+3 of each: every warp-level access is one fully coalesced 512-byte row, and
+// One CTA of 256 threads owns one state, or half of its columns (decode_cols).  Of a whole state thread (warp w,
+// lane l) holds rows w, w+8, ... and the four columns 4l..4l+3 of each: every warp-level access is one fully coalesced 512-byte row, and
 // all 16 loads of a thread are issued before the first use (64 KiB in flight per CTA).
 #include "kda_common.cuh"
 #include "kda_ptx.cuh"
@@ -28,7 +28,7 @@ __device__ __forceinline__ void st_stream(float* p, float4 x) {
                  : "memory");
 }
 // packed fp32 arithmetic (two independent round-to-nearest operations per instruction on sm_100):
-// the multi-token kernel is bound by instruction issue, not by HBM
+// in the multi-token kernel's loop
 __device__ __forceinline__ void mul4(float4& x, float a) {
     const float2 aa = make_float2(a, a);
     const float2 lo = __fmul2_rn(make_float2(x.x, x.y), aa), hi = __fmul2_rn(make_float2(x.z, x.w), aa);
@@ -218,7 +218,7 @@ kda_decode_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __r
 // finer first and last wave; whole states win where one wave of two per SM holds the call (n_sm * 2 items)
 // and, by the fewer barriers per byte, in long streams.  Measured (us a step, whole / half): 32 states 3.4 /
 // 3.1, 96: 4.3 / 3.8, 160: 6.0 / 5.4, 288: 5.8 / 6.0, 512: 14.0 / 13.2, 1184: 27.8 / 26.4, 2048: 44.6 / 42.9,
-// 8192: 165.1 / 165.9.
+// 8192: 165.1 / 165.9 (the line at 40 n_sm lies between these two without a point of its own).
 inline int decode_cols(int64_t items, int n_sm)
 {
     if (items <= n_sm + n_sm / 2) return 64;
@@ -236,7 +236,7 @@ inline int decode_cols(int64_t items, int n_sm)
 // butterfly shuffles.  No shared-memory reduction and no CTA-wide barrier per token (the
 // single-token kernel keeps its fully coalesced row layout: it has no token loop to protect).
 //
-// The token loop is bound by instruction issue, so a CTA that only started to fetch its state when
+// The tokens of a state depend on each other, so a CTA that only started to fetch its state when
 // it began would leave HBM idle while it computes.  CTAs are therefore persistent (two per SM) and
 // fetch the NEXT state into shared memory with asynchronous 16-byte copies while they work on the
 // current one; every thread copies exactly the elements it will own into its own slots, so the
@@ -246,9 +246,10 @@ __device__ __forceinline__ void cp_async16(void* dst_smem, const void* src_gmem)
                  "l"(src_gmem)
                  : "memory");
 }
-// Dynamic shared memory of the multi-token kernel.  Its token loop is bound by the shared-memory pipe (0.9 us a token
-// and state): vectors in four arrays that a thread reads 16 bytes at a time and sums exchanged by halves take 16
-// loads and 11 shuffles a token and warp, where packed (alpha, k, q, beta k) and a butterfly took 32 and 24:
+// Dynamic shared memory of the multi-token kernel.  Its token loop takes 0.76 us a token and state on an SM (128 x 32
+// states, 8 tokens); 128 packed FMAs a thread and what follows fill no pipe for as long, so it is the chain of loads, sums
+// and shuffles that each token ends in.  Vectors in four arrays that a thread reads 16 bytes at a time and sums exchanged
+// by halves take 16 loads and 11 shuffles a token and warp, where packed (alpha, k, q, beta k) and a butterfly took 32 and 24:
 // 64 x 32 states, 4 tokens 64.2 -> 60.9 us; 128 x 32, 8 tokens 185 -> 169.
 template <typename T> struct MultiSmem {
     static constexpr int GT = 8;                        // tokens staged together
