@@ -315,7 +315,7 @@ struct LayerMode {
 };
 
 // Into how many segments the chains of a bf16 call are cut (kda_segments.cu), 1 = none.  All runs of a stage must
-// be resident at once.  Times in us, measured: a chain step 1.33 without, 1.4 (maps) and 1.5 (outputs) with all SMs
+// be resident at once.  Times in us, measured: a chain step 1.62 in the fused kernel, 1.4 (maps) and 1.5 (outputs) with all SMs
 // at it, a tile of the intra-chunk kernel 8 over two CTAs per SM, launches 22 and a border 1.5.
 // Prefill, 8 heads x 4096 tokens 101 -> 72 us, 8 x 30000: 627 -> 256, 16 x 131072: 2720 -> 1830; 16 x 65536 for the
 // final state 1246 -> 656.  Modes 1 and 2 of kda_set_chunk_path never cut.

@@ -19,7 +19,7 @@
 // A call of this path is small (256 tokens x 2 heads: eight tiles), so what bounds it is the length of a tile's
 // chain of phases and of a chain step, not any throughput: 512 threads per tile, the substitution as
 // blocks, the operands of a chain phase fetched during the other; a tile in three CTAs and a chain of 8 columns
-// where SMs would be idle.  Measured at 256 tokens x 2 heads: 29.7 us a call (intra 17, inter 16, overlapping),
+// where SMs would be idle.  Measured at 256 tokens x 2 heads: 30.3 us a call (intra 17, inter 16, overlapping),
 // 39.5 with one CTA per tile and 16 columns per chain, 104 us with FMA products and a substitution of one
 // thread per column; 2048 tokens x 8 heads: 155 us, 185 before.
 #include <type_traits>

@@ -74,7 +74,7 @@ constexpr uint32_t E_KI_HALF = 8192;
 constexpr uint32_t E_V = 49152;         // V [2 column blocks][64 tokens][64] bf16 (token-major)
 constexpr uint32_t E_V_BLOCK = 8192;
 constexpr uint32_t E_A = 65536;         // fp32 [64][LDT]: L, X below the diagonal, T above it (transposed block
-                                        // positions); then the U staging (four [64][32] bf16 blocks)
+                                        // positions); then the U^T staging
 constexpr uint32_t E_TD = E_A + 64 * LDT * 4;     // fp32 4 x [16][LDD]: diagonal blocks of T; scan exchange [8][128] before
 constexpr uint32_t E_TD_BYTES = 4096;
 constexpr uint32_t E_BETA = E_TD + E_TD_BYTES;    // 64 fp32
