@@ -106,6 +106,9 @@ constexpr uint32_t B_KI = 0, B_AQ = tc::OFF_AQ - tc::OFF_KI, B_GV = tc::OFF_GV -
 constexpr uint32_t kSmemBytes = 2 * E_BYTES > C_BYTES ? 2 * E_BYTES : C_BYTES;
 static_assert(E_BYTES % 1024 == 0, "operand images stay 1024-byte aligned");
 static_assert(kSmemBytes <= 232448, "fits the shared memory of one SM");
+// Registers of the chain kernel's compute warps: the fp32 state takes 64 of them, an accumulator another 32 (at 128, the
+// share of each of 512 threads, some spilled: 1.33 instead of 1.25 us a step).  The other half of the warps gives up as many.
+constexpr int kChainRegs = 160;
 constexpr uint32_t kTmemCols = 512;                // two engines of 256 columns, or one chain
 // TMEM columns of a chain: D1 of two chunks, D3, the bf16 state and V_new (A operands, two values a column)
 constexpr uint32_t T_D1 = 0, T_D3 = 256, T_S = 384, T_VN = 448;
@@ -1013,126 +1016,8 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
     JobInfo J;
     auto next_job = [&](int r) { return kRing ? job_info(f, cid, r, J) : pass_job<kSeg>(f, cid, r, J); };
 
-    if (warp == 9) {
-        // ================= loader =================
-        if (lane == 0) {
-            uint32_t g = 0;
-            KT_DECL(4);
-            for (int r = 0; next_job(r) && !*abort_flag; ++r)
-                for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
-                    const uint32_t e = g % (uint32_t)f.n_eng, m = g / (uint32_t)f.n_eng;
-                    const uint32_t slot = m % (uint32_t)f.depth, sa = g % kStagesA, s = g % kStagesB;
-                    const char* tile = kRing ? f.ring + (size_t)(((uint32_t)cid * f.n_eng + e) * f.depth + slot) * tc::TILE_BYTES
-                                             : f.ring + (size_t)(J.tile0 + (int64_t)c * a.H) * tc::TILE_BYTES;
-                    KT_MARK(true, 0);
-                    if (kRing) {
-                        wait_cluster(&ready[e * (uint32_t)f.depth + slot], (m / (uint32_t)f.depth) & 1u, 30);
-                        ptx::fence_async_global();
-                    }
-                    KT_MARK(true, 1);
-                    if (g >= kStagesB) wait(&emptyB[s], (g / kStagesB - 1) & 1u, 32);
-                    if (*abort_flag) break;
-                    KT_MARK(true, 2);
-                    uint8_t* sB = smem + C_B + s * C_STAGEB;
-                    if (kHasQ) {
-                        ptx::mbar_expect_tx(&fullB[s], kBBytes);
-                        ptx::bulk_g2s(sB, tile + tc::OFF_KI, kBBytes, &fullB[s]);
-                    } else {   // state-only call: only the W rows exist, and no Aqk
-                        ptx::mbar_expect_tx(&fullB[s], kBBytes - 8192);
-                        ptx::bulk_g2s(sB, tile + tc::OFF_KI, 16384, &fullB[s]);
-                        ptx::bulk_g2s(sB + B_GV, tile + tc::OFF_GV, tc::GV_BYTES + 16384, &fullB[s]);
-                    }
-                    if (g >= kStagesA) wait(&emptyA[sa], (g / kStagesA - 1) & 1u, 34);
-                    uint8_t* sA = smem + C_A + sa * kABytes;
-                    if (kHasQ) {
-                        ptx::mbar_expect_tx(&fullA[sa], kABytes);
-                        ptx::bulk_g2s(sA, tile, kABytes, &fullA[sa]);
-                    } else {
-                        ptx::mbar_expect_tx(&fullA[sa], 16384);
-                        ptx::bulk_g2s(sA, tile, 8192, &fullA[sa]);
-                        ptx::bulk_g2s(sA + tc::QW_HALF, tile + tc::QW_HALF, 8192, &fullA[sa]);
-                    }
-                }
-            KT_FLUSH(true, f.hdr, 24, 3);
-            if (*abort_flag) {   // the copies already requested must land before the shared memory goes away
-                for (uint32_t x = g > kStagesB ? g - kStagesB : 0; x < g; ++x)
-                    ptx::mbar_wait(&fullB[x % kStagesB], (x / kStagesB) & 1u, a.wait_limit_ns / 8);
-                for (uint32_t x = g > kStagesA ? g - kStagesA : 0; x < g; ++x)
-                    ptx::mbar_wait(&fullA[x % kStagesA], (x / kStagesA) & 1u, a.wait_limit_ns / 8);
-            }
-        }
-    } else if (kRing && warp == 10) {
-        // ================= gives the ring's positions back =================
-        // (the loader has no time for the release arrivals; it refills a stage only after this warp has seen it)
-        if (lane == 0) {
-            const uint32_t base = ptx::smem_u32(smem);
-            uint32_t g = 0;
-            for (int r = 0; next_job(r) && !*abort_flag; ++r)
-                for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
-                    wait(&fullB[g % kStagesB], (g / kStagesB) & 1u, 31);
-                    wait(&fullA[g % kStagesA], (g / kStagesA) & 1u, 33);
-                    if (*abort_flag) break;
-                    ptx::mbar_arrive(&emptyA[g % kStagesA]);
-                    ptx::mbar_arrive(&emptyB[g % kStagesB]);
-                    const uint32_t e = g % (uint32_t)f.n_eng, slot = (g / (uint32_t)f.n_eng) % (uint32_t)f.depth;
-                    ptx::mbar_arrive_cluster(ptx::map_to_cta(base + (e & 1u) * E_BYTES + E_BAR + 48 + slot * 8, 1 + (e >> 1)));
-                }
-        }
-    } else if (warp == 8) {
-        // ================= MMA issue =================
-        const uint32_t id1 = ptx::umma_idesc_bf16(128, 64);
-        const uint32_t id2 = ptx::umma_idesc_bf16(128, 128) | ptx::kIdescBMajorMN;
-        const uint32_t base = (uint32_t)ptx::warp_uniform((int)ptx::smem_u32(smem));
-        uint32_t g = 0;
-        KT_DECL(8);
-        for (int r = 0; next_job(r) && !*abort_flag; ++r)
-            for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
-                const uint32_t sa = g % kStagesA, s = g % kStagesB;
-                const uint32_t pA = base + C_A + sa * kABytes, pB = base + C_B + s * C_STAGEB;
-                const uint32_t d1 = tm + T_D1 + (g & 1u) * 128u;
-                KT_MARK(lane == 0, 0);
-                wait(&fullA[sa], (g / kStagesA) & 1u, 1);
-                KT_MARK(lane == 0, 1);   // operands
-                if (op && g >= 2) wait(&o_done[g & 1u], ((g >> 1) - 1) & 1u, 2);
-                wait(s_ready, g & 1u, 3);
-                __syncwarp();
-                KT_MARK(lane == 0, 2);   // state
-                ptx::tc_fence_after();
-                // W S first: V_new waits for it alone, Q S runs beside V_new's arithmetic
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    ptx::umma_bf16_ta(d1, tm + T_S + k * 8, ptx::umma_desc_sw128(pA + (k >> 2) * tc::QW_HALF + (k & 3) * 32), id1, k > 0);
-                ptx::umma_commit(m1);
-                if (kHasQ) {
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        ptx::umma_bf16_ta(d1 + 64, tm + T_S + k * 8,
-                                          ptx::umma_desc_sw128(pA + 8192 + (k >> 2) * tc::QW_HALF + (k & 3) * 32), id1, k > 0);
-                }
-                ptx::umma_commit(&emptyA[sa]);
-                KT_MARK(lane == 0, 3);   // MMA1 issue
-                wait(&fullB[s], (g / kStagesB) & 1u, 11);
-                wait(vn_ready, g & 1u, 4);
-                __syncwarp();
-                KT_MARK(lane == 0, 4);   // V_new
-                ptx::tc_fence_after();
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    ptx::umma_bf16_ta(tm + T_D3, tm + T_VN + k * 8, ptx::umma_desc_sw128_mn(pB + B_KI + k * 2048, tc::KI_HALF), id2, k > 0);
-                ptx::umma_commit(m2);
-                if (op) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        ptx::umma_bf16_ta(d1 + 64, tm + T_VN + k * 8, ptx::umma_desc_sw128(pB + B_AQ + k * 32), id1, 1);
-                    ptx::umma_commit(&out_bar[g & 1u]);
-                }
-                ptx::umma_commit(&emptyB[s]);
-                KT_MARK(lane == 0, 5);   // MMA2 + output issue
-            }
-        KT_FLUSH(lane == 0, f.hdr, 16, 6);
-        // every MMA has completed before the TMEM goes away
-        if (g > 0) wait(&emptyB[(g - 1) % kStagesB], ((g - 1) / kStagesB) & 1u, 5);
-    } else if (warp < 8) {
+    if (warp < 8) {
+        if (!kRing) ptx::reg_inc<kChainRegs>();
         // ================= compute warps =================
         const int quad = warp & 3, half = warp >> 2, dv = quad * 32 + lane, dk0 = half * 64;
         const uint32_t tq = tm + ((uint32_t)(quad * 32) << 16);
@@ -1248,83 +1133,205 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                 for (int i = 0; i < 64; ++i) s_out[s_at + i * kD] = S[i];
         }
         KT_FLUSH(t == 0, f.hdr, 28, 7);
-    } else if (warp >= 12 && op) {
-        // ================= output rows =================
-        // The accumulator has a lane per column and a TMEM column per token; read as 8 x 8 fragments and stored with
-        // stmatrix.trans it becomes rows of the output, which leave by two tiled TMA stores.  (Straight from the lanes, 64 two-byte stores a thread, the stores
-        // crowded out the loads of the compute warps: 2.6 instead of 1.6 us a step.)
-        const int quad = warp & 3, ot = t - 384;
-        const uint32_t tq = tm + ((uint32_t)(quad * 32) << 16);
-        // this lane's row of the four 8 x 8 matrices of token block 0, in the swizzled [2][64 tokens][64] image
-        const uint32_t mrow = (uint32_t)(lane & 7), mcol = (uint32_t)((quad & 1) * 32 + (lane >> 3) * 8);
-        const uint32_t moff = (uint32_t)(quad >> 1) * 8192u + ptx::sw128_off(mrow, mcol);
-        uint32_t g = 0;
-        for (int r = 0; next_job(r) && !*abort_flag; ++r)
-            for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
-                const int64_t tok0 = J.tok_begin + (int64_t)c * kC;
-                const int len = (J.tok_end - tok0) < kC ? (int)(J.tok_end - tok0) : kC;
-                wait(&out_bar[g & 1u], (g >> 1) & 1u, 10);
-                __syncwarp();
-                ptx::tc_fence_after();
-                if (kRows32) {     // lane = column, four tokens a piece
+    } else {
+        if (!kRing) ptx::reg_dec<256 - kChainRegs>();
+        if (warp == 9) {
+            // ================= loader =================
+            if (lane == 0) {
+                uint32_t g = 0;
+                KT_DECL(4);
+                for (int r = 0; next_job(r) && !*abort_flag; ++r)
+                    for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
+                        const uint32_t e = g % (uint32_t)f.n_eng, m = g / (uint32_t)f.n_eng;
+                        const uint32_t slot = m % (uint32_t)f.depth, sa = g % kStagesA, s = g % kStagesB;
+                        const char* tile = kRing ? f.ring + (size_t)(((uint32_t)cid * f.n_eng + e) * f.depth + slot) * tc::TILE_BYTES
+                                                 : f.ring + (size_t)(J.tile0 + (int64_t)c * a.H) * tc::TILE_BYTES;
+                        KT_MARK(true, 0);
+                        if (kRing) {
+                            wait_cluster(&ready[e * (uint32_t)f.depth + slot], (m / (uint32_t)f.depth) & 1u, 30);
+                            ptx::fence_async_global();
+                        }
+                        KT_MARK(true, 1);
+                        if (g >= kStagesB) wait(&emptyB[s], (g / kStagesB - 1) & 1u, 32);
+                        if (*abort_flag) break;
+                        KT_MARK(true, 2);
+                        uint8_t* sB = smem + C_B + s * C_STAGEB;
+                        if (kHasQ) {
+                            ptx::mbar_expect_tx(&fullB[s], kBBytes);
+                            ptx::bulk_g2s(sB, tile + tc::OFF_KI, kBBytes, &fullB[s]);
+                        } else {   // state-only call: only the W rows exist, and no Aqk
+                            ptx::mbar_expect_tx(&fullB[s], kBBytes - 8192);
+                            ptx::bulk_g2s(sB, tile + tc::OFF_KI, 16384, &fullB[s]);
+                            ptx::bulk_g2s(sB + B_GV, tile + tc::OFF_GV, tc::GV_BYTES + 16384, &fullB[s]);
+                        }
+                        if (g >= kStagesA) wait(&emptyA[sa], (g / kStagesA - 1) & 1u, 34);
+                        uint8_t* sA = smem + C_A + sa * kABytes;
+                        if (kHasQ) {
+                            ptx::mbar_expect_tx(&fullA[sa], kABytes);
+                            ptx::bulk_g2s(sA, tile, kABytes, &fullA[sa]);
+                        } else {
+                            ptx::mbar_expect_tx(&fullA[sa], 16384);
+                            ptx::bulk_g2s(sA, tile, 8192, &fullA[sa]);
+                            ptx::bulk_g2s(sA + tc::QW_HALF, tile + tc::QW_HALF, 8192, &fullA[sa]);
+                        }
+                    }
+                KT_FLUSH(true, f.hdr, 24, 3);
+                if (*abort_flag) {   // the copies already requested must land before the shared memory goes away
+                    for (uint32_t x = g > kStagesB ? g - kStagesB : 0; x < g; ++x)
+                        ptx::mbar_wait(&fullB[x % kStagesB], (x / kStagesB) & 1u, a.wait_limit_ns / 8);
+                    for (uint32_t x = g > kStagesA ? g - kStagesA : 0; x < g; ++x)
+                        ptx::mbar_wait(&fullA[x % kStagesA], (x / kStagesA) & 1u, a.wait_limit_ns / 8);
+                }
+            }
+        } else if (kRing && warp == 10) {
+            // ================= gives the ring's positions back =================
+            // (the loader has no time for the release arrivals; it refills a stage only after this warp has seen it)
+            if (lane == 0) {
+                const uint32_t base = ptx::smem_u32(smem);
+                uint32_t g = 0;
+                for (int r = 0; next_job(r) && !*abort_flag; ++r)
+                    for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
+                        wait(&fullB[g % kStagesB], (g / kStagesB) & 1u, 31);
+                        wait(&fullA[g % kStagesA], (g / kStagesA) & 1u, 33);
+                        if (*abort_flag) break;
+                        ptx::mbar_arrive(&emptyA[g % kStagesA]);
+                        ptx::mbar_arrive(&emptyB[g % kStagesB]);
+                        const uint32_t e = g % (uint32_t)f.n_eng, slot = (g / (uint32_t)f.n_eng) % (uint32_t)f.depth;
+                        ptx::mbar_arrive_cluster(ptx::map_to_cta(base + (e & 1u) * E_BYTES + E_BAR + 48 + slot * 8, 1 + (e >> 1)));
+                    }
+            }
+        } else if (warp == 8) {
+            // ================= MMA issue =================
+            const uint32_t id1 = ptx::umma_idesc_bf16(128, 64);
+            const uint32_t id2 = ptx::umma_idesc_bf16(128, 128) | ptx::kIdescBMajorMN;
+            const uint32_t base = (uint32_t)ptx::warp_uniform((int)ptx::smem_u32(smem));
+            uint32_t g = 0;
+            KT_DECL(8);
+            for (int r = 0; next_job(r) && !*abort_flag; ++r)
+                for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
+                    const uint32_t sa = g % kStagesA, s = g % kStagesB;
+                    const uint32_t pA = base + C_A + sa * kABytes, pB = base + C_B + s * C_STAGEB;
+                    const uint32_t d1 = tm + T_D1 + (g & 1u) * 128u;
+                    KT_MARK(lane == 0, 0);
+                    wait(&fullA[sa], (g / kStagesA) & 1u, 1);
+                    KT_MARK(lane == 0, 1);   // operands
+                    if (op && g >= 2) wait(&o_done[g & 1u], ((g >> 1) - 1) & 1u, 2);
+                    wait(s_ready, g & 1u, 3);
+                    __syncwarp();
+                    KT_MARK(lane == 0, 2);   // state
+                    ptx::tc_fence_after();
+                    // W S first: V_new waits for it alone, Q S runs beside V_new's arithmetic
+    #pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        ptx::umma_bf16_ta(d1, tm + T_S + k * 8, ptx::umma_desc_sw128(pA + (k >> 2) * tc::QW_HALF + (k & 3) * 32), id1, k > 0);
+                    ptx::umma_commit(m1);
+                    if (kHasQ) {
+    #pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            ptx::umma_bf16_ta(d1 + 64, tm + T_S + k * 8,
+                                              ptx::umma_desc_sw128(pA + 8192 + (k >> 2) * tc::QW_HALF + (k & 3) * 32), id1, k > 0);
+                    }
+                    ptx::umma_commit(&emptyA[sa]);
+                    KT_MARK(lane == 0, 3);   // MMA1 issue
+                    wait(&fullB[s], (g / kStagesB) & 1u, 11);
+                    wait(vn_ready, g & 1u, 4);
+                    __syncwarp();
+                    KT_MARK(lane == 0, 4);   // V_new
+                    ptx::tc_fence_after();
+    #pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        ptx::umma_bf16_ta(tm + T_D3, tm + T_VN + k * 8, ptx::umma_desc_sw128_mn(pB + B_KI + k * 2048, tc::KI_HALF), id2, k > 0);
+                    ptx::umma_commit(m2);
+                    if (op) {
+    #pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            ptx::umma_bf16_ta(d1 + 64, tm + T_VN + k * 8, ptx::umma_desc_sw128(pB + B_AQ + k * 32), id1, 1);
+                        ptx::umma_commit(&out_bar[g & 1u]);
+                    }
+                    ptx::umma_commit(&emptyB[s]);
+                    KT_MARK(lane == 0, 5);   // MMA2 + output issue
+                }
+            KT_FLUSH(lane == 0, f.hdr, 16, 6);
+            // every MMA has completed before the TMEM goes away
+            if (g > 0) wait(&emptyB[(g - 1) % kStagesB], ((g - 1) / kStagesB) & 1u, 5);
+        } else if (warp >= 12 && op) {
+            // ================= output rows =================
+            // The accumulator has a lane per column and a TMEM column per token; read as 8 x 8 fragments and stored with
+            // stmatrix.trans it becomes rows of the output, which leave by two tiled TMA stores.  (Straight from the lanes, 64 two-byte stores a thread, the stores
+            // crowded out the loads of the compute warps: 2.6 instead of 1.6 us a step.)
+            const int quad = warp & 3, ot = t - 384;
+            const uint32_t tq = tm + ((uint32_t)(quad * 32) << 16);
+            // this lane's row of the four 8 x 8 matrices of token block 0, in the swizzled [2][64 tokens][64] image
+            const uint32_t mrow = (uint32_t)(lane & 7), mcol = (uint32_t)((quad & 1) * 32 + (lane >> 3) * 8);
+            const uint32_t moff = (uint32_t)(quad >> 1) * 8192u + ptx::sw128_off(mrow, mcol);
+            uint32_t g = 0;
+            for (int r = 0; next_job(r) && !*abort_flag; ++r)
+                for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
+                    const int64_t tok0 = J.tok_begin + (int64_t)c * kC;
+                    const int len = (J.tok_end - tok0) < kC ? (int)(J.tok_end - tok0) : kC;
+                    wait(&out_bar[g & 1u], (g >> 1) & 1u, 10);
+                    __syncwarp();
+                    ptx::tc_fence_after();
+                    if (kRows32) {     // lane = column, four tokens a piece
+                        uint32_t y[2][32];
+                        ptx::tmem_ld_32x32b_x32(tq + T_D1 + (g & 1u) * 128u + 64, y[0]);
+                        ptx::tmem_ld_32x32b_x32(tq + T_D1 + (g & 1u) * 128u + 96, y[1]);
+                        ptx::tmem_ld_wait();
+                        ptx::tc_fence_before();
+                        warp_arrive(&o_done[g & 1u]);
+                        if (ot == 0) ptx::bulk_wait_read0();      // the previous block has been read out of its buffer
+                        ptx::named_bar_sync(6, 128);
+                        uint4* rows = reinterpret_cast<uint4*>(smem + C_OUT) + ot;
+    #pragma unroll
+                        for (int q = 0; q < 16; ++q)
+                            rows[q * 128] = make_uint4(y[q >> 3][4 * (q & 7)], y[q >> 3][4 * (q & 7) + 1], y[q >> 3][4 * (q & 7) + 2],
+                                                       y[q >> 3][4 * (q & 7) + 3]);
+                        ptx::fence_async_smem();
+                        ptx::named_bar_sync(6, 128);
+                        if (ot == 0 && !*abort_flag) {
+                            ptx::bulk_s2g(f.ring + (size_t)(J.tile0 + (int64_t)c * a.H) * tc::TILE_BYTES + tc::OFF_O32, smem + C_OUT, 32768);
+                            ptx::bulk_commit();
+                        }
+                        continue;
+                    }
+                    // y[b >> 1][4 j + 2 (b & 1) + e]: column 8 b + lane / 4 of the quadrant, token 8 j + 2 (lane % 4) + e
                     uint32_t y[2][32];
-                    ptx::tmem_ld_32x32b_x32(tq + T_D1 + (g & 1u) * 128u + 64, y[0]);
-                    ptx::tmem_ld_32x32b_x32(tq + T_D1 + (g & 1u) * 128u + 96, y[1]);
+                    ptx::tmem_ld_16x256b_x8(tq + T_D1 + (g & 1u) * 128u + 64, y[0]);
+                    ptx::tmem_ld_16x256b_x8(tq + (16u << 16) + T_D1 + (g & 1u) * 128u + 64, y[1]);
                     ptx::tmem_ld_wait();
                     ptx::tc_fence_before();
                     warp_arrive(&o_done[g & 1u]);
-                    if (ot == 0) ptx::bulk_wait_read0();      // the previous block has been read out of its buffer
+                    // the previous block has been read out of its buffer
+                    uint8_t* sb = smem + C_OUT;
+                    if (ot == 0) ptx::bulk_wait_read0();
                     ptx::named_bar_sync(6, 128);
-                    uint4* rows = reinterpret_cast<uint4*>(smem + C_OUT) + ot;
-#pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        rows[q * 128] = make_uint4(y[q >> 3][4 * (q & 7)], y[q >> 3][4 * (q & 7) + 1], y[q >> 3][4 * (q & 7) + 2],
-                                                   y[q >> 3][4 * (q & 7) + 3]);
+    #pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        uint32_t z[4];
+    #pragma unroll
+                        for (int b = 0; b < 4; ++b)
+                            z[b] = pack_bf16(__uint_as_float(y[b >> 1][4 * j + 2 * (b & 1)]), __uint_as_float(y[b >> 1][4 * j + 2 * (b & 1) + 1]));
+                        ptx::stmatrix_x4_trans(sb + moff + j * 1024, z);
+                    }
                     ptx::fence_async_smem();
                     ptx::named_bar_sync(6, 128);
-                    if (ot == 0 && !*abort_flag) {
-                        ptx::bulk_s2g(f.ring + (size_t)(J.tile0 + (int64_t)c * a.H) * tc::TILE_BYTES + tc::OFF_O32, smem + C_OUT, 32768);
-                        ptx::bulk_commit();
-                    }
-                    continue;
-                }
-                // y[b >> 1][4 j + 2 (b & 1) + e]: column 8 b + lane / 4 of the quadrant, token 8 j + 2 (lane % 4) + e
-                uint32_t y[2][32];
-                ptx::tmem_ld_16x256b_x8(tq + T_D1 + (g & 1u) * 128u + 64, y[0]);
-                ptx::tmem_ld_16x256b_x8(tq + (16u << 16) + T_D1 + (g & 1u) * 128u + 64, y[1]);
-                ptx::tmem_ld_wait();
-                ptx::tc_fence_before();
-                warp_arrive(&o_done[g & 1u]);
-                // the previous block has been read out of its buffer
-                uint8_t* sb = smem + C_OUT;
-                if (ot == 0) ptx::bulk_wait_read0();
-                ptx::named_bar_sync(6, 128);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    uint32_t z[4];
-#pragma unroll
-                    for (int b = 0; b < 4; ++b)
-                        z[b] = pack_bf16(__uint_as_float(y[b >> 1][4 * j + 2 * (b & 1)]), __uint_as_float(y[b >> 1][4 * j + 2 * (b & 1) + 1]));
-                    ptx::stmatrix_x4_trans(sb + moff + j * 1024, z);
-                }
-                ptx::fence_async_smem();
-                ptx::named_bar_sync(6, 128);
-                if (len == kC) {
-                    if (ot == 0 && !*abort_flag) {
-                        ptx::tma_store_2d(tm_o, sb, J.h * kD, (int)tok0);
-                        ptx::tma_store_2d(tm_o, sb + 8192, J.h * kD + 64, (int)tok0);
-                        ptx::bulk_commit();
-                    }
-                } else {       // the rows past the end of the sequence belong to the next one
-                    if (!*abort_flag)
-                        for (int idx = ot; idx < len * 16; idx += 128) {
-                            const int row = idx >> 4, ch = idx & 15;
-                            *reinterpret_cast<uint4*>(op + ((size_t)(tok0 + row) * a.H + J.h) * kD + ch * 8) =
-                                *reinterpret_cast<const uint4*>(sb + (ch >> 3) * 8192 + ptx::sw128_off((uint32_t)row, (uint32_t)(ch & 7) * 8));
+                    if (len == kC) {
+                        if (ot == 0 && !*abort_flag) {
+                            ptx::tma_store_2d(tm_o, sb, J.h * kD, (int)tok0);
+                            ptx::tma_store_2d(tm_o, sb + 8192, J.h * kD + 64, (int)tok0);
+                            ptx::bulk_commit();
                         }
+                    } else {       // the rows past the end of the sequence belong to the next one
+                        if (!*abort_flag)
+                            for (int idx = ot; idx < len * 16; idx += 128) {
+                                const int row = idx >> 4, ch = idx & 15;
+                                *reinterpret_cast<uint4*>(op + ((size_t)(tok0 + row) * a.H + J.h) * kD + ch * 8) =
+                                    *reinterpret_cast<const uint4*>(sb + (ch >> 3) * 8192 + ptx::sw128_off((uint32_t)row, (uint32_t)(ch & 7) * 8));
+                            }
+                    }
                 }
-            }
-        if (ot == 0) ptx::bulk_wait_all0();
+            if (ot == 0) ptx::bulk_wait_all0();
+        }
     }
     ptx::tc_fence_before();
     __syncthreads();
