@@ -87,19 +87,14 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
         __syncthreads();
         ptx::tc_fence_after();
     };
-    if (t < 64) {
-        sBeta[t] = t < loc.len ? a.beta[(size_t)(loc.tok0 + t) * a.H + h] : 0.f;
+    if (t < 64) sBeta[t] = t < loc.len ? a.beta[(size_t)(loc.tok0 + t) * a.H + h] : 0.f;
+    {
         int64_t ng; int nh;
         if (bwd_next(a, ng, nh)) {   // see prefetch_l2
             const BwdLoc nl = bwd_locate(a, ng);
-            if (t < nl.len) {
-                const size_t off = ((size_t)(nl.tok0 + t) * a.H + nh) * kD;
-                prefetch_l2(a.log_alpha + off, kD * 4);
-                prefetch_l2(static_cast<const T*>(a.k) + off, kD * sizeof(T));
-                prefetch_l2(static_cast<const T*>(a.q) + off, kD * sizeof(T));
-                prefetch_l2(static_cast<const T*>(a.v) + off, kD * sizeof(T));
-                if (a.d_o) prefetch_l2(static_cast<const T*>(a.d_o) + off, kD * sizeof(T));
-            }
+            prefetch_rows<kT, float, 1>(nl, a.H, nh, t, {a.log_alpha});
+            prefetch_rows<kT, T, 4>(nl, a.H, nh, t, {static_cast<const T*>(a.k), static_cast<const T*>(a.q), static_cast<const T*>(a.v),
+                                               static_cast<const T*>(a.d_o)});
         }
     }
     bool out_of_form;

@@ -126,20 +126,13 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
 #pragma unroll
     for (int j = 0; j < 2; ++j)
         ldraw(dd[j], static_cast<const T*>(a.d_o) + tok_off(row0 + 32 * j) + c8, row0 + 32 * j < loc.len && a.d_o);
-    {   // see prefetch_l2; the token vectors by 64 threads, a row each
+    {   // see prefetch_l2
         int64_t ng; int nh;
-        if ((t & ~63) == 448 && bwd_next(a, ng, nh)) {
+        if (bwd_next(a, ng, nh)) {
             const float* nt = a.tiles + ((size_t)ng * a.H + nh) * bt::kFloats;
-            const int r = t & 63;
-            if (r == 0) prefetch_l2(nt + bt::R, 2 * 64 * kD * 4);
-            if (r == 1) prefetch_l2(nt + bt::S, (bt::kFloats - bt::S) * 4);
-            const BwdLoc nl = bwd_locate(a, ng);
-            if (r < nl.len) {
-                const size_t off = ((size_t)(nl.tok0 + r) * a.H + nh) * kD;
-                prefetch_l2(static_cast<const T*>(a.k) + off, kD * sizeof(T));
-                prefetch_l2(static_cast<const T*>(a.q) + off, kD * sizeof(T));
-                if (a.d_o) prefetch_l2(static_cast<const T*>(a.d_o) + off, kD * sizeof(T));
-            }
+            if (t == kT - 32) prefetch_l2(nt + bt::R, 2 * 64 * kD * 4);
+            if (t == kT - 64) prefetch_l2(nt + bt::S, (bt::kFloats - bt::S) * 4);
+            prefetch_rows<kT, T, 3>(bwd_locate(a, ng), a.H, nh, t, {static_cast<const T*>(a.k), static_cast<const T*>(a.q), static_cast<const T*>(a.d_o)});
         }
     }
     publish();
