@@ -77,8 +77,18 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
     if (w == 9) {
         if (lane == 0) {
             int64_t i = 0;
+            // what a step reads into registers, asked into L2 two steps ahead: 64 rows of R or X, 128 of N, the vectors
+            auto ahead = [&](int64_t j) {
+                if (j >= nc) return;
+                const float* p = tile_of(j);
+                prefetch_l2(p + (kFwd ? bt::R : bt::X) + rf(64, 0, col0), 64 * NS * 4);
+                if (!kFwd) prefetch_l2(p + bt::N + rf(128, 0, col0), 128 * NS * 4);
+                prefetch_l2(p + bt::GC, 256 * 4);
+            };
+            ahead(1);
             for (; i < nc; ++i) {
                 const float* tile = tile_of(i);
+                ahead(i + 2);
                 // (i >= 2: the second product of chunk i - 2 has been waited for below, and with it the first, which
                 // read this buffer.  The barrier of the first may be a phase further on by now.)
                 ptx::mbar_expect_tx(&fullA[i & 1], kImg);
