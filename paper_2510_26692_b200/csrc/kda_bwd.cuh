@@ -98,10 +98,10 @@ __device__ __forceinline__ void bwd_tile(const BwdChunkArgs& a, int64_t id, int6
     g = (int64_t)((uint32_t)id / (uint32_t)a.H);
     h = (int)(id - g * a.H);
 }
-// tile of the CTA n_sm places further on; false if there is none
-__device__ __forceinline__ bool bwd_next(const BwdChunkArgs& a, int64_t& g, int& h) {
-    const int64_t id = (int64_t)blockIdx.x + a.n_sm;
-    if (id >= gridDim.x) return false;
+// the tile n_sm places behind tile `id`; false if there is none
+__device__ __forceinline__ bool bwd_next(const BwdChunkArgs& a, int64_t id, int64_t& g, int& h) {
+    id += a.n_sm;
+    if (id >= a.n_chunks * a.H) return false;
     bwd_tile(a, id, g, h);
     return true;
 }

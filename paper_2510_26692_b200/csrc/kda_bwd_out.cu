@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         ldraw(dd[j], static_cast<const T*>(a.d_o) + tok_off(row0 + 32 * j) + c8, row0 + 32 * j < loc.len && a.d_o);
     {   // see prefetch_l2
         int64_t ng; int nh;
-        if (bwd_next(a, ng, nh)) {
+        if (bwd_next(a, blockIdx.x, ng, nh)) {
             const float* nt = a.tiles + ((size_t)ng * a.H + nh) * bt::kFloats;
             if (t == kT - 32) prefetch_l2(nt + bt::R, 2 * 64 * kD * 4);
             if (t == kT - 64) prefetch_l2(nt + bt::S, (bt::kFloats - bt::S) * 4);

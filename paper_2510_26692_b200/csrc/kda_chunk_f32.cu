@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kT1, 1) kda_intra_f32(ChunkArgs a, float* __re
         }
         return;
     }
-    invert_unit_lower<LM>(sB, sT, t);      // a3
+    invert_unit_lower<LM>(sB, sT, t, [] { __syncthreads(); });      // a3
 
     // a4: warps 2 x 8, 32 x 16 entries each; the triangle bounds the sums
     {

@@ -123,10 +123,10 @@ __device__ __forceinline__ void st2(float* p, float x, float y) { *reinterpret_c
 // T = (I + L)^-1 of a strictly lower triangular 64 x 64 L (row pitch LD, its upper triangle is overwritten), by
 // at least 4 warps; T has to be zero above the diagonal blocks on entry.  16 x 16 diagonal blocks by substitution
 // (one column per thread, fp32 FMA), then two doublings [T11 0; T21 T22], T21 = -T22 (L21 T11), as warp-level
-// products whose inner factor sits in the empty upper triangle of L.  Ends with a barrier.  (With the
+// products whose inner factor sits in the empty upper triangle of L.  `barrier` is one of all calling threads; ends with it.  (With the
 // doublings as FMA products over all threads: 11.1k cycles instead of 8.0k.)
-template <int LD>
-__device__ __forceinline__ void invert_unit_lower(float* __restrict__ L, float* __restrict__ T, int t) {
+template <int LD, typename Barrier>
+__device__ __forceinline__ void invert_unit_lower(float* __restrict__ L, float* __restrict__ T, int t, Barrier barrier) {
     const int lane = t & 31, w = t >> 5;
     if (t < 64) {
         const int b0 = t & 48, j = t & 15;
@@ -144,7 +144,7 @@ __device__ __forceinline__ void invert_unit_lower(float* __restrict__ L, float* 
 #pragma unroll
         for (int i = 0; i < 16; ++i) T[(b0 + i) * LD + b0 + j] = x[i];
     }
-    __syncthreads();
+    barrier();
 #pragma unroll
     for (int s = 16; s < 64; s *= 2) {
         // 16 x 16 block (i0, j0) of the pair at c0: two warps for s = 16, four for s = 32
@@ -156,14 +156,14 @@ __device__ __forceinline__ void invert_unit_lower(float* __restrict__ L, float* 
             gemm<0, 2, false, false, false, false>(acc, L + (c0 + s + i0) * LD + c0, LD, T + c0 * LD + c0 + j0, LD, j0, s, lane);
             each_pair(acc, lane, [&](int i, int j, float x, float y) { st2(L + (c0 + i0 + i) * LD + c0 + s + j0 + j, x, y); });
         }
-        __syncthreads();
+        barrier();
         if (mine) {
             zero(acc);
             gemm<0, 2, false, false, false, false>(acc, T + (c0 + s + i0) * LD + c0 + s, LD, L + c0 * LD + c0 + s + j0, LD, 0,
                                                    i0 + 16, lane);
             each_pair(acc, lane, [&](int i, int j, float x, float y) { st2(T + (c0 + s + i0 + i) * LD + c0 + j0 + j, -x, -y); });
         }
-        __syncthreads();
+        barrier();
     }
 }
 
