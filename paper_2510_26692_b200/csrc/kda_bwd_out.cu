@@ -1,16 +1,20 @@
 // Gradients stage of the chunkwise backward pass (equations in kda_bwd_chunk.cu): one CTA per (chunk, head),
 // every product on tcgen05 with split operands (kda_split3.cuh), accumulators in TMEM.
 //
-// The products of a tile and where their operand images live (RA, RB: 96 KB each; rows x columns):
-//   P1  dV  = (beta T')^T dX              T' 64x64, dX 64x128 in RA
-//   P2  e^(G_m) [dO ; -dV] S^T            [dO ; -dV] 128x128 in RA, e^(G_m) S 128x128 in RB
-//   P4  [dO ; -dV] r^T                    r 64x128 in RB (over S)
-//   P3  r Lam^T                           Lam's column halves: in RB beside r, then in RA
-//   P5  P2 += [dP ; dB] K_                [dP ; dB] 128x64 and K_ 64x128 in RA
-//   P6  [dP ; dB]^T [Q ; K^]              [Q ; K^] 128x128 in RB
-// While the tensor core works on one product the threads fetch and split the operands of the next.
+// The products of a tile (M x N x K) and where their operands live: D and X are regions of shared memory of 96 KB each, A
+// the 192 TMEM columns of an A operand.
+//   P1  dV = (beta T')^T dX                 T' 64x64 and dX 64x128 in X
+//   P2  e^(G_m) S [dO ; -dV]^T              S in A, [dO ; -dV] 128x128 in D
+//   P4  [dO ; -dV] r^T                      r 64x128 in X
+//   P3  Lam r^T                             Lam in A
+//   P5  P2 += K_^T [dP ; dB]^T              [dP ; dB] 128x64 and K_ 64x128 in X
+//   P6  [Q ; K^]^T [dP ; dB]                [Q ; K^] 128x128 in D
+// P2, P3, P5 and P6 have the channels in the TMEM lanes, so that the pass over the columns (a thread per channel) reads them
+// there.  Operands in shared memory are what these products are bound by: a product of 128 x 128 x 16 reads 8 KB of it
+// in the 64 clocks that it takes, all there is, and with A in TMEM half of that.
 //
-// T=4096, H=32: warp-level tf32 products 784 us, 473 in this form.
+// T=4096, H=32: warp-level tf32 products 784 us; all operands in shared memory and accumulators staged there 418; 341 in
+// this form.
 #include "kda_bwd.cuh"
 #include "kda_split3.cuh"
 
@@ -19,18 +23,16 @@ namespace {
 
 using namespace split3;
 constexpr int kT = 512;
-constexpr int LR = 132;
-constexpr uint32_t O_RA = 0, O_RB = 98304, O_VEC = 196608;
-constexpr uint32_t O_DX = O_RA + 3 * 8192;                    // dX beside T'
-constexpr uint32_t O_LAM0 = O_RB + 3 * 16384;                 // Lam, v columns 0-63, beside r
-constexpr uint32_t O_LAM1 = O_RA;                             // Lam, v columns 64-127; then K_
-constexpr uint32_t O_DPB = O_RA + 3 * 16384;                  // [dP ; dB]
-// fp32 vectors (floats from O_VEC): beta[64] em[128] dbeta[8][64] sGC[4][128] colsum[2][64] seg[4][128], then barriers
-constexpr int V_BETA = 0, V_EM = 64, V_DB = 192, V_GC = 704, V_CS = 1216, V_SEG = 1344, V_BAR = 1856;
+constexpr int kIssue = 15;                                    // the warp that issues the MMAs
+constexpr uint32_t O_D = 0, O_X = 98304, O_VEC = 196608;
+constexpr uint32_t O_T = O_X, O_DX = O_X + 24576;             // T', dX
+constexpr uint32_t O_R = O_X, O_DPB = O_X + 49152;            // r, later K_; [dP ; dB]
+// fp32 vectors (floats from O_VEC): beta[64] dbeta[8][64] sGC[4][128] colsum[2][64] seg[4][128] sum[4][128], then barriers
+constexpr int V_BETA = 0, V_DB = 64, V_GC = 576, V_CS = 1088, V_SEG = 1216, V_SUM = 1728, V_BAR = 2240;
 constexpr uint32_t kSmem = O_VEC + V_BAR * 4 + 64 + 1024;     // + alignment slack
-static_assert(4 * 64 * LR * 4 <= O_VEC, "the staged accumulators fit over the images");
 static_assert(kSmem <= 232448, "fits the shared memory of one SM");
-constexpr uint32_t C_P2 = 0, C_P4 = 128, C_P1 = 192, C_P6 = 256, C_P3 = 384;   // TMEM columns (P1: 192-319, read before P6)
+// TMEM columns; P1 (128) lies where P3 and P6 come to lie
+constexpr uint32_t C_A = 0, kAParts = 64, C_P2 = 192, C_P4 = 320, C_P1 = 384, C_P3 = 384, C_P6 = 448;
 
 __device__ __forceinline__ float ldv(const float* p, bool in) {
     float x = 0.f;
@@ -53,8 +55,8 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     if (a.seq_heads[h]) return;
     uint8_t* sm = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
     float* vec = reinterpret_cast<float*>(sm + O_VEC);
-    float* sBeta = vec + V_BETA; float* sDb = vec + V_DB; float* sEm = vec + V_EM; float* sGC = vec + V_GC;
-    float* sCs = vec + V_CS; float* sSeg = vec + V_SEG;
+    float* sBeta = vec + V_BETA; float* sDb = vec + V_DB; float* sGC = vec + V_GC;
+    float* sCs = vec + V_CS; float* sSeg = vec + V_SEG; float* sSum = vec + V_SUM;
     uint64_t* bar = reinterpret_cast<uint64_t*>(vec + V_BAR);   // one per group of MMAs, each used once
     uint32_t* slot = reinterpret_cast<uint32_t*>(bar + 6);
     const BwdLoc loc = bwd_locate(a, chunk);
@@ -84,11 +86,12 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     // unit u of a matrix with 128 columns: row u >> 4, columns 8 (u & 15) .. + 7
     const int c8 = (t & 15) * 8, row0 = t >> 4;      // token tensors: rows row0 + 32 j
     const int ra = t & 63, ca = (t >> 6) * 8;        // rf matrices of 64 rows: columns ca + 64 j
-    const int rs = t & 127, cs = (t >> 7) * 8;       // and of 128 rows: columns cs + 32 j
+    const int rs = t & 127, cs = (t >> 7) * 32;      // and of 128 rows (TMEM lane rs): columns cs + 8 j
     auto tok_off = [&](int r) { return ((size_t)(loc.tok0 + r) * a.H + h) * kD; };
 
     // ---- P1: dV -----------------------------------------------------------------------------------------
-    Raw8<float> xs[4], rr[2];     // S now, Lam later; r
+    Raw8<float> xs[4], rr[2];     // S, r
+    const float em = tile[bt::EM + rs];      // of row rs of S, and of channel rs in the pass over the columns
     {
         Raw8<float> xt, xx[2];
         const int r = t >> 3, x = (t & 7) * 8;
@@ -98,16 +101,14 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
 #pragma unroll
         for (int j = 0; j < 2; ++j) ldraw_rf(rr[j], tile + bt::R, 64, ra, ca + 64 * j);
         const float b = r < loc.len ? a.beta[(size_t)(loc.tok0 + r) * a.H + h] : 0.f;
-        const float em = tile[bt::EM + (t & 127)];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) ldraw_rf(xs[j], tile + bt::S, 128, rs, cs + 32 * j);
+        for (int j = 0; j < 4; ++j) ldraw_rf(xs[j], tile + bt::S, 128, rs, cs + 8 * j);
         float v[8], u[8];
         to_f(xt, v);
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] *= b;
-        put8<64, 1>(sm + O_RA, r, x, v);
+        put8<64, 1>(sm + O_T, r, x, v);
         if (x == 0) sBeta[r] = b;
-        if (t < 128) sEm[t] = em;
         float s = 0.f;      // share of r_j . dX_j
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -122,7 +123,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     Raw8<float> lam[4];
     Raw8<T> dd[2];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) ldraw_rf(lam[j], tile + bt::L, 128, rs, cs + 32 * j);
+    for (int j = 0; j < 4; ++j) ldraw_rf(lam[j], tile + bt::L, 128, rs, cs + 8 * j);
 #pragma unroll
     for (int j = 0; j < 2; ++j)
         ldraw(dd[j], static_cast<const T*>(a.d_o) + tok_off(row0 + 32 * j) + c8, row0 + 32 * j < loc.len && a.d_o);
@@ -137,15 +138,16 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     }
     publish();
     const uint32_t tm = (uint32_t)ptx::warp_uniform((int)*slot);
-    const uint32_t mnA = ptx::kIdescAMajorMN, mnB = ptx::kIdescBMajorMN;
-    if (w == 0) {
-        mma6<4>(tm + C_P1, mn_major<64, 1>(sm + O_RA), mn_major<64, 2>(sm + O_DX), ptx::umma_idesc_bf16(128, 128) | mnA | mnB, false);
+    const uint32_t mnA = ptx::kIdescAMajorMN, mnB = ptx::kIdescBMajorMN, id = ptx::umma_idesc_bf16(128, 128);
+    const int quad = w & 3, seg = w >> 2;
+    const uint32_t tq = tm + ((uint32_t)(quad * 32) << 16);
+    if (w == kIssue) {
+        mma6<4>(tm + C_P1, mn_major<64, 1>(sm + O_T, 0, true), mn_major<64, 2>(sm + O_DX), id | mnA | mnB, false);
         ptx::umma_commit(&bar[0]);
     }
-    // meanwhile: e^(G_m) S, and its dot products with Lam
+    // meanwhile: e^(G_m) S, and its dot products with Lam; dO
     {
-        const float em = sEm[rs];
-        float s = 0.f;
+        float s = 0.f, x[32];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             float v[8], l[8];
@@ -154,47 +156,52 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 s = fmaf(v[e], l[e], s);
-                v[e] *= em;
+                x[8 * j + e] = v[e] * em;
             }
-            put8<128, 2>(sm + O_RB, rs, cs + 32 * j, v);
         }
+        put32_tmem<kAParts>(tq + C_A + seg * 16, x);
         sGC[t] = s * em * em;      // [4][128]; (G_m = G_C / 2)
-    }
-    wait(0);
-    // dV: rows = TMEM lanes 0-63 (warps of quadrants 0 and 1), 32 columns each
-    const int quad = w & 3, cg = (w >> 2) * 32;
-    const uint32_t tq = tm + ((uint32_t)(quad * 32) << 16);
-    if (quad < 2) {
-        const int i = quad * 32 + lane;
-        uint32_t y[32];
-        ptx::tmem_ld_32x32b_x32(tq + C_P1 + cg, y);
-        ptx::tmem_ld_wait();
-        if (i < loc.len) {
-            float* p = a.dv + tok_off(i) + cg;
-#pragma unroll
-            for (int e = 0; e < 32; e += 4)
-                *reinterpret_cast<uint4*>(p + e) = make_uint4(y[e], y[e + 1], y[e + 2], y[e + 3]);
-        }
-#pragma unroll
-        for (int q8 = 0; q8 < 4; ++q8) {
-            float v[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = -__uint_as_float(y[8 * q8 + e]);
-            put8<128, 2>(sm + O_RA, 64 + i, cg + 8 * q8, v);
-        }
     }
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
         float v[8];
         to_f(dd[j], v);
-        put8<128, 2>(sm + O_RA, row0 + 32 * j, c8, v);
+        put8<128, 2>(sm + O_D, row0 + 32 * j, c8, v);
+    }
+    ptx::tmem_st_wait();
+    wait(0);
+    {   // dV: rows = TMEM lanes 0-63, repeated in lanes 64-127; 16 columns a thread.  r over T' and dX
+        const int i = (quad & 1) * 32 + lane, c0 = seg * 32 + (quad >> 1) * 16;
+        uint32_t y[16];
+        ptx::tmem_ld_32x32b_x16(tq + C_P1 + c0, y);
+        ptx::tmem_ld_wait();
+        if (i < loc.len) {
+            float* p = a.dv + tok_off(i) + c0;
+#pragma unroll
+            for (int e = 0; e < 16; e += 4)
+                *reinterpret_cast<uint4*>(p + e) = make_uint4(y[e], y[e + 1], y[e + 2], y[e + 3]);
+        }
+        float v[8];
+#pragma unroll
+        for (int q8 = 0; q8 < 2; ++q8) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = -__uint_as_float(y[8 * q8 + e]);
+            put8<128, 2>(sm + O_D, 64 + i, c0 + 8 * q8, v);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            to_f(rr[j], v);
+            put8<64, 2>(sm + O_R, ra, ca + 64 * j, v);
+        }
     }
     publish();
 
-    // ---- P2, then P4 and the first half of P3 ---------------------------------------------------------------
-    if (w == 0) {
-        mma6<8>(tm + C_P2, k_major<128, 2>(sm + O_RA), k_major<128, 2>(sm + O_RB), ptx::umma_idesc_bf16(128, 128), false);
+    // ---- P2, P4 ---------------------------------------------------------------------------------------------
+    if (w == kIssue) {
+        mma6_ta<8, kAParts>(tm + C_P2, tm + C_A, k_major<128, 2>(sm + O_D), id, false);
         ptx::umma_commit(&bar[1]);
+        mma6<8>(tm + C_P4, k_major<128, 2>(sm + O_D), k_major<64, 2>(sm + O_R), ptx::umma_idesc_bf16(128, 64), false);
+        ptx::umma_commit(&bar[2]);
     }
     // the gated operands' inputs, requested while the tensor core works
     Raw8<T> kr[2], qr[2];
@@ -207,31 +214,24 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         ldraw(gr[j], tile + bt::F + r * kD + c8);
     }
     wait(1);
+    {   // Lam over S
+        float x[32];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        float v[8];
-        to_f(rr[j], v);
-        put8<64, 2>(sm + O_RB, ra, ca + 64 * j, v);
-    }
+        for (int j = 0; j < 4; ++j) {
+            float v[8];
+            to_f(lam[j], v);
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        float v[8];
-        to_f(lam[j], v);
-        put8<128, 1>(sm + O_LAM0, rs, cs + 32 * j, v);
+            for (int e = 0; e < 8; ++e) x[8 * j + e] = v[e];
+        }
+        put32_tmem<kAParts>(tq + C_A + seg * 16, x);
+        ptx::tmem_st_wait();
     }
     publish();
-    if (w == 0) {
-        mma6<8>(tm + C_P4, k_major<128, 2>(sm + O_RA), k_major<64, 2>(sm + O_RB), ptx::umma_idesc_bf16(128, 64), false);
-        ptx::umma_commit(&bar[2]);
-        mma6<4>(tm + C_P3, k_major<64, 2>(sm + O_RB), k_major<128, 1>(sm + O_LAM0), ptx::umma_idesc_bf16(128, 128), false);
+    if (w == kIssue) {
+        mma6_ta<8, kAParts>(tm + C_P3, tm + C_A, k_major<64, 2>(sm + O_R), ptx::umma_idesc_bf16(128, 64), false);
+        ptx::umma_commit(&bar[3]);
     }
     wait(2);
-#pragma unroll
-    for (int j = 2; j < 4; ++j) {
-        float v[8];
-        to_f(lam[j], v);
-        put8<128, 1>(sm + O_LAM1, rs, cs + 32 * j - 64, v);
-    }
     {   // masked and scaled Gram matrices; columns j0 .. j0 + 15 of row lane + 32 quad of [dP ; dB]
         const int R = quad * 32 + lane, i = R & 63, j0 = (w >> 2) * 16;
         const bool isB = quad >= 2;
@@ -272,17 +272,6 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
             if (lane < 16) sCs[(quad - 2) * 64 + j0 + lane] = bb[0];
         }
     }
-    publish();
-    if (w == 0) {
-        mma6<4>(tm + C_P3, k_major<64, 2>(sm + O_RB + 8192), k_major<128, 1>(sm + O_LAM1), ptx::umma_idesc_bf16(128, 128), true);
-        ptx::umma_commit(&bar[3]);
-    }
-    if (t < loc.len) {
-        float s = sCs[t] + sCs[64 + t];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) s += sDb[j * 64 + t];
-        a.db[(size_t)(loc.tok0 + t) * a.H + h] = s;
-    }
     // gated operands: exp(G - G_m), exp(G_m - G)
     float kk[2][8], qq[2][8], gg[2][8];
 #pragma unroll
@@ -298,32 +287,32 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
             qq[j][e] *= a.scale * f1;                // Q
         }
     }
-    wait(3);
-
-    // ---- P5, P6 -------------------------------------------------------------------------------------------
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
         const int r = row0 + 32 * j;
-        put8<64, 2>(sm + O_LAM1, r, c8, gg[j]);
-        put8<128, 2>(sm + O_RB, r, c8, qq[j]);
-        put8<128, 2>(sm + O_RB, 64 + r, c8, kk[j]);
+        put8<128, 2>(sm + O_D, r, c8, qq[j]);
+        put8<128, 2>(sm + O_D, 64 + r, c8, kk[j]);
     }
+    wait(3);              // r has been read: K_ over it
+#pragma unroll
+    for (int j = 0; j < 2; ++j) put8<64, 2>(sm + O_R, row0 + 32 * j, c8, gg[j]);
     publish();
-    if (w == 0) {
-        mma6<4>(tm + C_P2, k_major<128, 1>(sm + O_DPB), mn_major<64, 2>(sm + O_LAM1), ptx::umma_idesc_bf16(128, 128) | mnB, true);
-        mma6<8>(tm + C_P6, mn_major<128, 1>(sm + O_DPB), mn_major<128, 2>(sm + O_RB), ptx::umma_idesc_bf16(128, 128) | mnA | mnB, false);
+
+    // ---- P5, P6 -------------------------------------------------------------------------------------------
+    if (w == kIssue) {
+        mma6<4>(tm + C_P2, mn_major<64, 2>(sm + O_R), k_major<128, 1>(sm + O_DPB), id | mnA, true);
+        mma6<8>(tm + C_P6, mn_major<128, 2>(sm + O_D), mn_major<128, 1>(sm + O_DPB), ptx::umma_idesc_bf16(128, 64) | mnA | mnB, false);
         ptx::umma_commit(&bar[4]);
     }
-    // accumulators to shared memory: [0] dQ, [1] dK^, [2] dK_, [3] beta r Lam^T, rows = tokens.  P3 first: it is complete.
-    float* stage = reinterpret_cast<float*>(sm);
-    uint32_t y3[32];
-    if (quad < 2) {
-        ptx::tmem_ld_32x32b_x32(tq + C_P3 + cg, y3);
-        ptx::tmem_ld_wait();
+    if (t < loc.len) {
+        float s = sCs[t] + sCs[64 + t];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s += sDb[j * 64 + t];
+        a.db[(size_t)(loc.tok0 + t) * a.H + h] = s;
     }
     // the column pass's inputs: thread = channel c of 16 consecutive tokens
-    const int c = t & 127, seg = t >> 7;
-    const float ec = sEm[c];          // e^(G_C - G_m): G_m = G_C / 2
+    const int c = rs;
+    const float ec = em;              // e^(G_C - G_m): G_m = G_C / 2
     const T* kp = static_cast<const T*>(a.k);
     const T* qp = static_cast<const T*>(a.q);
     float kv[16], qv[16], gv[16];
@@ -336,51 +325,34 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         gv[i] = ldv(tile + bt::F + r * kD + c, true);
     }
     wait(4);
-    {
-        uint32_t y[32];
-        ptx::tmem_ld_32x32b_x32(tq + C_P2 + cg, y);
-        ptx::tmem_ld_wait();
-        float* p = stage + (quad * 32 + lane) * LR + cg;
-#pragma unroll
-        for (int e = 0; e < 32; e += 4) *reinterpret_cast<uint4*>(p + e) = make_uint4(y[e], y[e + 1], y[e + 2], y[e + 3]);
-    }
-    if (quad < 2) {
-        const int i = quad * 32 + lane;
-        uint32_t y[32];
-        ptx::tmem_ld_32x32b_x32(tq + C_P6 + cg, y);
-        ptx::tmem_ld_wait();
-        float* p = stage + (128 + i) * LR + cg;
-        const float b = sBeta[i];
-#pragma unroll
-        for (int e = 0; e < 32; e += 4) {
-            *reinterpret_cast<uint4*>(p + e) = make_uint4(y[e], y[e + 1], y[e + 2], y[e + 3]);
-            *reinterpret_cast<float4*>(p + 64 * LR + e) =
-                make_float4(b * __uint_as_float(y3[e]), b * __uint_as_float(y3[e + 1]), b * __uint_as_float(y3[e + 2]),
-                            b * __uint_as_float(y3[e + 3]));
-        }
-    }
-    ptx::tc_fence_before();
-    __syncthreads();
     float dG[16], run = 0.f, gsum = 0.f;
 #pragma unroll
-    for (int i = 15; i >= 0; --i) {
-        const int r = seg * 16 + i;
-        const size_t off = tok_off(r) + c;
-        const bool in = r < loc.len;
-        const float f1 = gv[i], f2 = reciprocal(f1);
-        const float dq = a.scale * f1 * stage[r * LR + c];
-        const float p3 = ec * f2 * stage[(192 + r) * LR + c];       // e^(G_C - G) (beta r Lam^T)
-        const float dk1 = f1 * stage[(64 + r) * LR + c], dk2 = fmaf(f2, stage[(128 + r) * LR + c], p3);
-        if (in) {
-            a.dq[off] = dq;
-            a.dk[off] = dk1 + dk2;
+    for (int half = 1; half >= 0; --half) {
+        uint32_t yq[8], yk[8], y6[8], y3[8];      // dQ, dK^, dK_, Lam r^T before the gates
+        const uint32_t at = tq + seg * 16 + half * 8;
+        ptx::tmem_ld_32x32b_x8(at + C_P2, yq);
+        ptx::tmem_ld_32x32b_x8(at + C_P2 + 64, yk);
+        ptx::tmem_ld_32x32b_x8(at + C_P6, y6);
+        ptx::tmem_ld_32x32b_x8(at + C_P3, y3);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int x = 7; x >= 0; --x) {
+            const int i = half * 8 + x, r = seg * 16 + i;
+            const size_t off = tok_off(r) + c;
+            const float f1 = gv[i], f2 = reciprocal(f1);
+            const float dq = a.scale * f1 * __uint_as_float(yq[x]);
+            const float p3 = ec * f2 * (sBeta[r] * __uint_as_float(y3[x]));       // e^(G_C - G) (beta r Lam^T)
+            const float dk1 = f1 * __uint_as_float(yk[x]), dk2 = fmaf(f2, __uint_as_float(y6[x]), p3);
+            if (r < loc.len) {
+                a.dq[off] = dq;
+                a.dk[off] = dk1 + dk2;
+            }
+            gsum = fmaf(kv[i], p3, gsum);
+            run += fmaf(qv[i], dq, kv[i] * (dk1 - dk2));
+            dG[i] = run;
         }
-        gsum = fmaf(kv[i], p3, gsum);
-        run += fmaf(qv[i], dq, kv[i] * (dk1 - dk2));
-        dG[i] = run;
     }
     // d G_C: all segments' sums of K~ dK~ and e^(G_C) rowsum(S Lam)
-    float* sSum = stage + 256 * LR;      // [4][128], behind the staged accumulators
     sSeg[seg * 128 + c] = run;
     sSum[seg * 128 + c] = gsum;
     __syncthreads();
@@ -392,6 +364,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         if (r < loc.len) a.dg[tok_off(r) + c] = dG[i] + base;
     }
     if (!ok && atomicCAS(&a.hdr->status, 0, (int)KDA_ERR_TIMEOUT) == 0) a.hdr->where = 30;
+    ptx::tc_fence_before();
     __syncthreads();
     if (w == 0) ptx::tmem_dealloc(tm, 512);
 }

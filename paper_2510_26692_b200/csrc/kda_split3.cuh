@@ -46,6 +46,25 @@ __device__ __forceinline__ void put8(uint8_t* img, int row, int col, const float
     }
 }
 
+// Splits 32 consecutive columns of this lane's row into the A operand in TMEM (two bf16 values a column, kParts columns from
+// one split to the next): no pass over shared memory, and the product reads only its B operand there.
+template <int kParts>
+__device__ __forceinline__ void put32_tmem(uint32_t taddr, float (&x)[32]) {
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        uint32_t w[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            w[e] = pack2(x[2 * e], x[2 * e + 1]);
+            if (s < 2) {
+                x[2 * e] -= __uint_as_float(w[e] << 16);
+                x[2 * e + 1] -= __uint_as_float(w[e] & 0xffff0000u);
+            }
+        }
+        ptx::tmem_st_32x32b_x16(taddr + s * kParts, w);
+    }
+}
+
 // One operand of a product: descriptor of split 0 at K = 0, and the distances between splits and of 16 in K
 // (in descriptor units of 16 bytes).  KH: distance of the second 64 of K (K-major operands).
 struct Operand {
@@ -76,6 +95,24 @@ __device__ __forceinline__ void mma6(uint32_t d_tmem, const Operand& A, const Op
             const uint32_t oa = A.k16 == 2u ? (uint32_t)(k >> 2) * A.khalf + (k & 3) * 2u : (uint32_t)k * A.k16;
             const uint32_t ob = B.k16 == 2u ? (uint32_t)(k >> 2) * B.khalf + (k & 3) * 2u : (uint32_t)k * B.k16;
             ptx::umma_bf16(d_tmem, da + oa, db + ob, idesc, acc);
+            acc = 1u;
+        }
+    }
+}
+
+// the same with A in TMEM (put32_tmem)
+template <int KS, int kParts>
+__device__ __forceinline__ void mma6_ta(uint32_t d_tmem, uint32_t a_tmem, const Operand& B, uint32_t idesc, bool accumulate) {
+    uint32_t acc = accumulate ? 1u : 0u;
+#pragma unroll 1
+    for (int p = 0; p < 6; ++p) {
+        const uint32_t sa = p == 0 ? 2u : (p == 2 || p == 3) ? 1u : 0u, sb = p == 1 ? 2u : (p == 2 || p == 4) ? 1u : 0u;
+        const uint32_t ta = a_tmem + sa * kParts;
+        const uint64_t db = B.desc + sb * B.split;
+#pragma unroll
+        for (int k = 0; k < KS; ++k) {
+            const uint32_t ob = B.k16 == 2u ? (uint32_t)(k >> 2) * B.khalf + (k & 3) * 2u : (uint32_t)k * B.k16;
+            ptx::umma_bf16_ta(d_tmem, ta + k * 8, db + ob, idesc, acc);
             acc = 1u;
         }
     }
