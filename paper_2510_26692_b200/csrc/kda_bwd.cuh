@@ -26,23 +26,30 @@ struct BwdChunkArgs {
 // middle G_m of the chunk's log decay (K^ = k e^(G - G_m), K_ = k e^(G_m - G)); the chains restore the true
 // scale on the state.  "rf" = rows fastest: element (row, c) of a matrix with R rows at float
 // ((c / 4) R + row) 4 + c % 4, which a thread per row reads and writes in whole 16-byte pieces beside its
-// neighbours'.
+// neighbours'.  What the chains read and write has the columns of the state in the rows, as they have them in the TMEM
+// lanes; the states that they leave have its rows there (sf), as the gradients stage needs them.
 namespace bt {
-constexpr int WI = 0;                // W' = T' K^ [64][128] as a split image (kda_split3.cuh), T' = (I + B Diag(beta))^-1
+constexpr int WI = 0;                // W'^T [128][64] as a split image (kda_split3.cuh), W' = T' K^, T' = (I + B Diag(beta))^-1
 constexpr int KI = WI + 12288;       // K_ [64][128] as a split image
-constexpr int R = KI + 12288;        // [64][128] rf: U' = T' V, replaced by r = U' - W' S by the forward chain
-constexpr int X = R + 64 * 128;      // [64][128] rf: P^T dO, replaced by dX = P^T dO + K~ Lam by the backward chain
-constexpr int N = X + 64 * 128;      // [128][128] rf: Q^T dO
-constexpr int S = N + 128 * 128;     // [128][128] rf: state entering the chunk (forward chain)
-constexpr int L = S + 128 * 128;     // [128][128] rf: adjoint of the state leaving the chunk (backward chain)
-constexpr int F = L + 128 * 128;     // [64][128] e^(G - G_m)
+constexpr int R = KI + 12288;        // [128][64] rf: U'^T, U' = T' V, replaced by r^T, r = U' - W' S, by the forward chain
+constexpr int X = R + 64 * 128;      // [128][64] rf: dO^T P, replaced by dX^T, dX = P^T dO + K~ Lam, by the backward chain
+constexpr int N = X + 64 * 128;      // [128][128] rf: dO^T Q
+constexpr int kState = 128 * 128;
+constexpr int S = N + 128 * 128;     // [128][128] sf: state entering the chunk (forward chain)
+constexpr int L = S + kState;        // [128][128] sf: adjoint of the state leaving the chunk (backward chain)
+constexpr int F = L + kState;        // [64][128] e^(G - G_m)
 constexpr int T = F + 64 * 128;      // [64][64] T'
 constexpr int B = T + 64 * 64;       // [64][64] B = StrictTril(K^ K_^T)
 constexpr int GC = B + 64 * 64;      // [128] e^(G_C)
 constexpr int EM = GC + 128;         // [128] e^(G_m), also e^(G_C - G_m)
-constexpr int kFloats = EM + 128;
+constexpr int BE = EM + 128;         // [64] beta, zero past the end of the sequence
+constexpr int kFloats = BE + 64;
+constexpr int kVec = kFloats - GC;   // the vectors
 }  // namespace bt
 __device__ __forceinline__ int rf(int rows, int row, int c) { return ((c >> 2) * rows + row) * 4 + (c & 3); }
+// rf of 128 rows with the rows of a group of four columns in another order from group to group: a warp with the columns in its
+// lanes writes a row to shared memory without bank conflicts
+__device__ __forceinline__ int sf(int row, int c) { return (c >> 2) * 512 + ((row ^ ((c >> 2) & 7)) << 2) + (c & 3); }
 
 // Largest decay of a chunk taken in chunk form.
 constexpr float kBwdRange = 40.f;
@@ -136,6 +143,11 @@ __device__ __forceinline__ void ldraw(Raw8<__nv_bfloat16>& r, const __nv_bfloat1
 __device__ __forceinline__ void ldraw_rf(Raw8<float>& r, const float* m, int rows, int row, int c) {
     ldraw4(r.w, m + rf(rows, row, c));
     ldraw4(r.w + 4, m + rf(rows, row, c + 4));
+}
+// (row, c .. c + 7) of an sf matrix
+__device__ __forceinline__ void ldraw_sf(Raw8<float>& r, const float* m, int row, int c) {
+    ldraw4(r.w, m + sf(row, c));
+    ldraw4(r.w + 4, m + sf(row, c + 4));
 }
 __device__ __forceinline__ void to_f(const Raw8<float>& r, float (&x)[8]) {
 #pragma unroll

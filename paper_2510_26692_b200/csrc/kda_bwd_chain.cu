@@ -1,16 +1,23 @@
 // The two state recurrences of the chunkwise backward pass (equations in kda_bwd_chunk.cu), side by side:
 //   forward   r  = U' - W' S            S   <- e^(G_C) S + K~^T (beta r)
 //   backward  dX = P^T dO + K~ Lam      Lam <- e^(G_C) Lam + Q^T dO - W'^T (beta dX)       (W', Q here with e^G)
-// State columns never mix: one CTA per (64-column slice, direction, head, sequence), sequential over the chunks,
-// on tcgen05 with split operands (kda_split3.cuh).  The fp32 state stays in registers (thread = row, half of
-// the columns); its operand image carries the factor e^(G_m) that W' and K_ are relative to.  Bound by the
-// chain: two dependent groups of MMAs (48 and 24 of N = 64) with their read-outs per chunk.
+// One CTA per (direction, head, sequence), sequential over the chunks, on tcgen05 with split operands (kda_split3.cuh).
+// Everything is transposed: the TMEM lanes are the 128 columns of the state, so that the state and r or dX are A operands
+// in TMEM and only what the per-chunk stage left is read from shared memory:
+//   D1[v][token] = state^T (W'^T or K_^T)        48 MMAs of N = 64
+//   D3[v][k]     = (beta r or -beta dX)^T (K_ or W')       24 of N = 128
+// The fp32 state stays in registers (thread = column v, a quarter of k); its operand carries the factor e^(G_m) that W' and K_
+// are relative to.  Bound by the chain: 3072 clocks of MMAs a step at least, and the splitting of two operands between
+// them.
 //
-// Warps 0-7 compute (TMEM lane quadrant = warp & 3, column half = warp >> 2), 8 issues the MMAs, 9 loads.
-// The first product's operand image has two buffers, the second's one: each is requested when the product
-// that read it last is complete, most of a step ahead.
+// Warps 0-15 compute (TMEM lane quadrant = warp & 3, quarter of k and of the tokens = warp >> 2), 16 issues the MMAs, 17 loads.
+// Each product's operand image has one buffer and the vectors two, requested again when what read them last is known to be
+// done.  The state leaves for the tile by way of a buffer of its own.
 //
-// T=4096, H=32 (128 CTAs): 570 us with warp-level tf32 products, 323 in this form.
+// T=4096, H=32: 570 us with warp-level tf32 products; with state and r in shared memory and two CTAs of 64 columns 277 (6 KB of
+// operands for 32 clocks of an MMA of N = 64).  In this form 290 with half the CTAs; six packed sequences of 8 heads, which
+// took two waves then, 75 -> 56.  A step: 2100 clocks of the first product, 1300 to r, 1900 of the second, 2400 to the state;
+// shared memory is half busy all the time, and a wait that read a flag beside its barrier cost 400 clocks of it.
 #include "kda_bwd.cuh"
 #include "kda_split3.cuh"
 
@@ -18,49 +25,48 @@ namespace kda {
 namespace {
 
 using namespace split3;
-constexpr int kT = 320;
-constexpr int NS = 64;
-constexpr uint32_t kImg = 49152;
-constexpr uint32_t O_A = 0, O_B = 2 * kImg, O_S = 3 * kImg, O_X = 4 * kImg, O_BAR = O_X + 24576;
-constexpr uint32_t kSmem = O_BAR + 128 + 1024;
+constexpr int kT = 640, kCompute = 512;
+constexpr int kRegs = 112, kRegsRest = 32;      // of a compute thread and of the others: 512 x 112 + 128 x 32 <= 640 x 96
+constexpr uint32_t kImg = 49152, kStateBytes = bt::kState * 4, kVecBytes = bt::kVec * 4;
+constexpr uint32_t O_A = 0, O_B = kImg, O_ST = 2 * kImg, O_N = O_ST + kStateBytes, O_VEC = O_N + kStateBytes, O_BAR = O_VEC + 2 * kVecBytes;
+constexpr uint32_t kSmem = O_BAR + 160;      // (the images need 1024-byte alignment, and there is no room to align)
 static_assert(kSmem <= 232448, "fits the shared memory of one SM");
-constexpr uint32_t C_1 = 0, C_2 = NS;      // TMEM columns of the two products
+static_assert(kVecBytes % 16 == 0 && kStateBytes % 16 == 0 && O_BAR % 8 == 0, "bulk copies and barriers are aligned");
+// TMEM columns: the operands (three splits each) and the two products
+constexpr uint32_t C_S = 0, kSParts = 64, C_X = 192, kXParts = 32, C_1 = 288, C_3 = 352;
 
 template <bool kFwd>
-__device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, int n, int h, int col0)
+__device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, int n, int h)
 {
-    uint64_t* fullA = reinterpret_cast<uint64_t*>(sm + O_BAR);   // [2]
-    uint64_t* fullB = fullA + 2;
-    uint64_t* m1 = fullB + 1;            // first product of a chunk complete
+    uint64_t* fullA = reinterpret_cast<uint64_t*>(sm + O_BAR);
+    uint64_t* fullB = fullA + 1;
+    uint64_t* fullN = fullB + 1;
+    uint64_t* fullV = fullN + 1;         // [2]
+    uint64_t* m1 = fullV + 2;            // first product of a chunk complete
     uint64_t* m2 = m1 + 1;               // second
-    uint64_t* s_ready = m2 + 1;          // 8 warps: state image written
-    uint64_t* x_ready = s_ready + 1;     // 4 warps: beta r or -beta dX written
-    volatile uint32_t* abort_word = reinterpret_cast<volatile uint32_t*>(x_ready + 1);
+    uint64_t* freed = m2 + 1;            // the state has been read out of the staging buffer
+    uint64_t* done = freed + 1;          // all MMAs complete
+    uint64_t* s_ready = done + 1;        // 16 warps: state operand written
+    uint64_t* x_ready = s_ready + 1;     // 16 warps: beta r or -beta dX written
+    uint64_t* staged = x_ready + 1;      // 16 warps: state written to the staging buffer
+    uint64_t* n_read = staged + 1;       // 16 warps: N read
+    volatile uint32_t* abort_word = reinterpret_cast<volatile uint32_t*>(n_read + 1);
     uint32_t* slot = const_cast<uint32_t*>(abort_word) + 1;
     const int t = threadIdx.x, lane = t & 31, w = ptx::warp_uniform(t >> 5);
-    int64_t g0, nc, tok_begin, tok_end;
+    int64_t g0, nc;
     if (a.cu_seqlens) {
         g0 = a.chunk_cu[n]; nc = a.chunk_cu[n + 1] - g0;
-        tok_begin = a.cu_seqlens[n]; tok_end = a.cu_seqlens[n + 1];
     } else {
         g0 = (int64_t)n * a.chunks_per_seq; nc = a.chunks_per_seq;
-        tok_begin = (int64_t)n * a.seq_len; tok_end = tok_begin + a.seq_len;
     }
-    auto chunk_of = [&](int64_t i) { return kFwd ? i : nc - 1 - i; };
-    auto tile_of = [&](int64_t i) { return a.tiles + ((size_t)(g0 + chunk_of(i)) * a.H + h) * bt::kFloats; };
+    auto tile_of = [&](int64_t i) { return a.tiles + ((size_t)(g0 + (kFwd ? i : nc - 1 - i)) * a.H + h) * bt::kFloats; };
 
     if (w == 0) {
-        ptx::tmem_alloc(slot, 128);
+        ptx::tmem_alloc(slot, 512);
         ptx::tmem_relinquish();
     }
     if (t == 32) {
-        ptx::mbar_init(&fullA[0], 1);
-        ptx::mbar_init(&fullA[1], 1);
-        ptx::mbar_init(fullB, 1);
-        ptx::mbar_init(m1, 1);
-        ptx::mbar_init(m2, 1);
-        ptx::mbar_init(s_ready, 8);
-        ptx::mbar_init(x_ready, 4);
+        for (uint64_t* b = fullA; b <= n_read; ++b) ptx::mbar_init(b, b < s_ready ? 1 : kCompute / 32);
         *abort_word = 0;
         ptx::fence_mbar_init();
     }
@@ -70,160 +76,215 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
     const uint32_t tm = (uint32_t)ptx::warp_uniform((int)*slot);
     // false once any wait of the CTA has run out
     auto wait = [&](uint64_t* bar, int64_t phase) {
+        if (ptx::mbar_try(bar, (uint32_t)phase & 1u)) return true;      // (the shared memory is busy: one access where one will do)
+        if (*abort_word) return false;
         if (!ptx::mbar_wait(bar, (uint32_t)phase & 1u, a.wait_limit_ns)) *abort_word = 1;
         return *abort_word == 0;
     };
 
-    if (w == 9) {
-        if (lane == 0) {
-            int64_t i = 0;
-            // what a step reads into registers, asked into L2 two steps ahead: 64 rows of R or X, 128 of N, the vectors
-            auto ahead = [&](int64_t j) {
-                if (j >= nc) return;
-                const float* p = tile_of(j);
-                prefetch_l2(p + (kFwd ? bt::R : bt::X) + rf(64, 0, col0), 64 * NS * 4);
-                if (!kFwd) prefetch_l2(p + bt::N + rf(128, 0, col0), 128 * NS * 4);
-                prefetch_l2(p + bt::GC, 256 * 4);
-            };
-            ahead(1);
-            for (; i < nc; ++i) {
-                const float* tile = tile_of(i);
-                ahead(i + 2);
-                // (i >= 2: the second product of chunk i - 2 has been waited for below, and with it the first, which
-                // read this buffer.  The barrier of the first may be a phase further on by now.)
-                ptx::mbar_expect_tx(&fullA[i & 1], kImg);
-                ptx::bulk_g2s(sm + O_A + (i & 1) * kImg, tile + (kFwd ? bt::WI : bt::KI), kImg, &fullA[i & 1]);
-                if (i >= 1 && !wait(m2, i - 1)) { ++i; break; }
-                ptx::mbar_expect_tx(fullB, kImg);
-                ptx::bulk_g2s(sm + O_B, tile + (kFwd ? bt::KI : bt::WI), kImg, fullB);
-            }
-            if (*abort_word) {      // nothing may be in flight when the CTA leaves
-                for (int64_t j = i > 2 ? i - 2 : 0; j < i; ++j) ptx::mbar_wait(&fullA[j & 1], (uint32_t)(j >> 1) & 1u, a.wait_limit_ns);
-                for (int64_t j = i > 2 ? i - 2 : 0; j < i; ++j) ptx::mbar_wait(fullB, (uint32_t)j & 1u, a.wait_limit_ns);
-            }
-        }
-    } else if (w == 8) {
-        const uint32_t id1 = ptx::umma_idesc_bf16(128, NS) | ptx::kIdescBMajorMN, id2 = id1 | ptx::kIdescAMajorMN;
-        for (int64_t i = 0; i < nc; ++i) {
-            if (!wait(s_ready, i) || !wait(&fullA[i & 1], i >> 1)) break;
-            __syncwarp();
-            ptx::tc_fence_after();
-            mma6<8>(tm + C_1, k_major<64, 2>(sm + O_A + (i & 1) * kImg), mn_major<128, 1>(sm + O_S), id1, false);
-            ptx::umma_commit(m1);
-            if (!wait(x_ready, i) || !wait(fullB, i)) break;
-            __syncwarp();
-            ptx::tc_fence_after();
-            mma6<4>(tm + C_2, mn_major<64, 2>(sm + O_B), mn_major<64, 1>(sm + O_X), id2, false);
-            ptx::umma_commit(m2);
-        }
-    } else {
-        const int quad = w & 3, row = quad * 32 + lane, ch = (w >> 2) * 32;
+    if (w < kCompute / 32) {
+        ptx::reg_inc<kRegs>();
+        const int quad = w & 3, part = w >> 2, v = quad * 32 + lane, k0 = part * 32, j0 = part * 16;
         const uint32_t tq = tm + ((uint32_t)(quad * 32) << 16);
-        const size_t sbase = (((size_t)n * a.H + h) * kD + row) * (size_t)kD + col0 + ch;
-        const bool rows_x = quad < 2;           // rows 0-63 of the first product are tokens, the rest is not used
-        float S[32];
+        const size_t sbase = (((size_t)n * a.H + h) * kD + k0) * (size_t)kD + v;
+        float* stage = reinterpret_cast<float*>(sm + O_ST);
+        float2 S[16];
         const float* init = kFwd ? a.S0 : a.dS_T;
 #pragma unroll
-        for (int e = 0; e < 32; e += 4) {
-            const float4 v = init ? *reinterpret_cast<const float4*>(init + sbase + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-            S[e] = v.x; S[e + 1] = v.y; S[e + 2] = v.z; S[e + 3] = v.w;
-        }
-        auto put_state = [&](float em) {
-#pragma unroll
-            for (int q8 = 0; q8 < 4; ++q8) {
-                float x[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) x[e] = em * S[8 * q8 + e];
-                put8<128, 1>(sm + O_S, row, ch + 8 * q8, x);
-            }
-            ptx::fence_async_smem();
+        for (int e = 0; e < 16; ++e)
+            S[e] = init ? make_float2(init[sbase + (size_t)(2 * e) * kD], init[sbase + (size_t)(2 * e + 1) * kD]) : make_float2(0.f, 0.f);
+        // a vector of a chunk's step: four values from c on
+        auto vec = [&](int64_t i, int off, int c) {
+            return *reinterpret_cast<const float4*>(sm + O_VEC + (uint32_t)(i & 1) * kVecBytes + (uint32_t)(off - bt::GC + c) * 4);
+        };
+        auto lo = [](const float4& m) { return make_float2(m.x, m.y); };
+        auto hi = [](const float4& m) { return make_float2(m.z, m.w); };
+        auto pair = [](const uint32_t* y) { return make_float2(__uint_as_float(y[0]), __uint_as_float(y[1])); };
+        auto arrive = [&](uint64_t* bar) {
+            ptx::tmem_st_wait();
             ptx::tc_fence_before();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(s_ready);
+            if (lane == 0) ptx::mbar_arrive(bar);
         };
-        float em = nc > 0 ? tile_of(0)[bt::EM + row] : 0.f;
-        if (nc > 0) put_state(em);
+        auto put_state = [&](int64_t i) {
+            wait(&fullV[i & 1], i >> 1);
+            float2 x[16];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float4 m = vec(i, bt::EM, k0 + 4 * e);
+                x[2 * e] = __fmul2_rn(lo(m), S[2 * e]);
+                x[2 * e + 1] = __fmul2_rn(hi(m), S[2 * e + 1]);
+            }
+            put_tmem<kSParts>(tq + C_S + part * 16, x);
+            arrive(s_ready);
+        };
+        if (nc > 0) put_state(0);
         for (int64_t i = 0; i < nc; ++i) {
             float* tile = tile_of(i);
-            const float em_next = i + 1 < nc ? tile_of(i + 1)[bt::EM + row] : 0.f;
-            const float gam = tile[bt::GC + row];
-            uint32_t u[32], nn[kFwd ? 1 : 32];
-            float beta = 0.f;
-            float* ux = tile + (kFwd ? bt::R : bt::X);
-            if (rows_x) {
+            float* ux = tile + (kFwd ? bt::R : bt::X) + rf(128, v, j0);
+            uint32_t u[16];
 #pragma unroll
-                for (int e = 0; e < 32; e += 4) ldraw4_w(u + e, ux + rf(64, row, col0 + ch + e));
-                const int64_t tok = tok_begin + chunk_of(i) * kC + row;
-                if (tok < tok_end) beta = a.beta[(size_t)tok * a.H + h];
+            for (int e = 0; e < 16; e += 4) ldraw4_w(u + e, ux + e * 128);
+            // the state as the gradients stage needs it, by way of shared memory
+            if (i > 0 && !wait(freed, i - 1)) break;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                stage[sf(k0 + 2 * e, v)] = S[e].x;
+                stage[sf(k0 + 2 * e + 1, v)] = S[e].y;
             }
-            if (!kFwd)
-#pragma unroll
-                for (int e = 0; e < (kFwd ? 0 : 32); e += 4) ldraw4(nn + e, tile + bt::N + rf(128, row, col0 + ch + e));
-            {   // the state as the gradients stage needs it
-                float* keep = tile + (kFwd ? bt::S : bt::L);
-#pragma unroll
-                for (int e = 0; e < 32; e += 4)
-                    *reinterpret_cast<float4*>(keep + rf(128, row, col0 + ch + e)) = make_float4(S[e], S[e + 1], S[e + 2], S[e + 3]);
-            }
+            ptx::fence_async_smem();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(staged);
             if (!wait(m1, i)) break;
             __syncwarp();
             ptx::tc_fence_after();
-            if (rows_x) {
-                uint32_t y[32];
-                ptx::tmem_ld_32x32b_x32(tq + C_1 + ch, y);
+            {
+                uint32_t y[16];
+                ptx::tmem_ld_32x32b_x16(tq + C_1 + j0, y);
                 ptx::tmem_ld_wait();
-                float x[32];
+                const float sg = kFwd ? -1.f : 1.f;
+                float2 x[8], z[8];
 #pragma unroll
-                for (int e = 0; e < 32; ++e)
-                    x[e] = kFwd ? __uint_as_float(u[e]) - __uint_as_float(y[e]) : __uint_as_float(u[e]) + __uint_as_float(y[e]);
-                const float f = kFwd ? beta : -beta;
+                for (int e = 0; e < 8; ++e) x[e] = __ffma2_rn(pair(y + 2 * e), make_float2(sg, sg), pair(u + 2 * e));
 #pragma unroll
-                for (int q8 = 0; q8 < 4; ++q8) {
-                    float z[8];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) z[e] = f * x[8 * q8 + e];
-                    put8<64, 1>(sm + O_X, row, ch + 8 * q8, z);
+                for (int e = 0; e < 8; e += 2) {
+                    float4 b = vec(i, bt::BE, j0 + 2 * e);
+                    if (!kFwd) b = make_float4(-b.x, -b.y, -b.z, -b.w);
+                    z[e] = __fmul2_rn(lo(b), x[e]);
+                    z[e + 1] = __fmul2_rn(hi(b), x[e + 1]);
                 }
-                ptx::fence_async_smem();
-                ptx::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(x_ready);
+                put_tmem<kXParts>(tq + C_X + part * 8, z);
+                arrive(x_ready);
 #pragma unroll
-                for (int e = 0; e < 32; e += 4)
-                    *reinterpret_cast<float4*>(ux + rf(64, row, col0 + ch + e)) = make_float4(x[e], x[e + 1], x[e + 2], x[e + 3]);
+                for (int e = 0; e < 16; e += 4)
+                    *reinterpret_cast<float4*>(ux + e * 128) = make_float4(x[e / 2].x, x[e / 2].y, x[e / 2 + 1].x, x[e / 2 + 1].y);
             }
+            // what does not need the second product
+            if (!kFwd && !wait(fullN, i)) break;
+            const float* np = reinterpret_cast<const float*>(sm + O_N) + rf(128, v, k0);
 #pragma unroll
-            for (int e = 0; e < 32; ++e) S[e] = kFwd ? S[e] * gam : fmaf(em, __uint_as_float(nn[kFwd ? 0 : e]), S[e] * gam);
+            for (int e = 0; e < 8; ++e) {
+                const float4 gc = vec(i, bt::GC, k0 + 4 * e);
+                S[2 * e] = __fmul2_rn(lo(gc), S[2 * e]);
+                S[2 * e + 1] = __fmul2_rn(hi(gc), S[2 * e + 1]);
+                if (!kFwd) {
+                    const float4 em = vec(i, bt::EM, k0 + 4 * e), nn = *reinterpret_cast<const float4*>(np + e * 512);
+                    S[2 * e] = __ffma2_rn(lo(em), lo(nn), S[2 * e]);
+                    S[2 * e + 1] = __ffma2_rn(hi(em), hi(nn), S[2 * e + 1]);
+                }
+            }
+            if (!kFwd) {
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(n_read);
+            }
             if (!wait(m2, i)) break;
             __syncwarp();
             ptx::tc_fence_after();
-            uint32_t y[32];
-            ptx::tmem_ld_32x32b_x32(tq + C_2 + ch, y);
-            ptx::tmem_ld_wait();
+            {
+                uint32_t y[32];
+                ptx::tmem_ld_32x32b_x32(tq + C_3 + k0, y);
+                ptx::tmem_ld_wait();
 #pragma unroll
-            for (int e = 0; e < 32; ++e) S[e] = fmaf(em, __uint_as_float(y[e]), S[e]);
-            em = em_next;
-            if (i + 1 < nc) put_state(em);
+                for (int e = 0; e < 8; ++e) {
+                    const float4 em = vec(i, bt::EM, k0 + 4 * e);
+                    S[2 * e] = __ffma2_rn(lo(em), pair(y + 4 * e), S[2 * e]);
+                    S[2 * e + 1] = __ffma2_rn(hi(em), pair(y + 4 * e + 2), S[2 * e + 1]);
+                }
+            }
+            if (i + 1 < nc) put_state(i + 1);
         }
         ptx::tc_fence_before();
         if (!kFwd && a.dS0)
 #pragma unroll
-            for (int e = 0; e < 32; e += 4)
-                *reinterpret_cast<float4*>(a.dS0 + sbase + e) = make_float4(S[e], S[e + 1], S[e + 2], S[e + 3]);
+            for (int e = 0; e < 16; ++e) {
+                a.dS0[sbase + (size_t)(2 * e) * kD] = S[e].x;
+                a.dS0[sbase + (size_t)(2 * e + 1) * kD] = S[e].y;
+            }
+    } else {
+        ptx::reg_dec<kRegsRest>();
+        if (w == kCompute / 32 + 1) {
+            if (lane == 0) {
+                auto get = [&](uint32_t at, int64_t j, int from, uint32_t bytes, uint64_t* bar) {
+                    ptx::mbar_expect_tx(bar, bytes);
+                    ptx::bulk_g2s(sm + at, tile_of(j) + from, bytes, bar);
+                };
+                auto first = [&](int64_t j) { get(O_A, j, kFwd ? bt::WI : bt::KI, kImg, fullA); };
+                auto second = [&](int64_t j) { get(O_B, j, kFwd ? bt::KI : bt::WI, kImg, fullB); };
+                auto vectors = [&](int64_t j) { get(O_VEC + (uint32_t)(j & 1) * kVecBytes, j, bt::GC, kVecBytes, &fullV[j & 1]); };
+                auto n_of = [&](int64_t j) { if (!kFwd) get(O_N, j, bt::N, kStateBytes, fullN); };
+                // what the compute warps read themselves, asked into L2 two steps ahead
+                auto ahead = [&](int64_t j) { if (j < nc) prefetch_l2(tile_of(j) + (kFwd ? bt::R : bt::X), 64 * kD * 4); };
+                int64_t in_a = 0, in_b = 0, in_n = 0;      // requested so far (vectors with the first operand)
+                if (nc > 0) {
+                    vectors(0); first(0); second(0); n_of(0);
+                    in_a = in_b = in_n = 1;
+                }
+                ahead(1);
+                for (int64_t i = 0; i < nc; ++i) {
+                    const bool more = i + 1 < nc;
+                    if (!wait(staged, i)) break;
+                    ptx::bulk_s2g(tile_of(i) + (kFwd ? bt::S : bt::L), sm + O_ST, kStateBytes);
+                    ptx::bulk_commit();
+                    if (!wait(m1, i)) break;
+                    if (more) {        // (the first product's operand is free, and so are the vectors of chunk i - 1)
+                        vectors(i + 1); first(i + 1);
+                        ++in_a;
+                    }
+                    ahead(i + 2);
+                    ptx::bulk_wait_read0();
+                    ptx::mbar_arrive(freed);
+                    if (!kFwd) {
+                        if (!wait(n_read, i)) break;
+                        if (more) { n_of(i + 1); ++in_n; }
+                    }
+                    if (!wait(m2, i)) break;
+                    if (more) { second(i + 1); ++in_b; }
+                }
+                ptx::bulk_wait_all0();
+                if (*abort_word) {      // nothing may be in flight when the CTA leaves
+                    for (int64_t j = in_a > 1 ? in_a - 2 : 0; j < in_a; ++j) ptx::mbar_wait(&fullV[j & 1], (uint32_t)(j >> 1) & 1u, a.wait_limit_ns);
+                    if (in_a > 0) ptx::mbar_wait(fullA, (uint32_t)(in_a - 1) & 1u, a.wait_limit_ns);
+                    if (in_b > 0) ptx::mbar_wait(fullB, (uint32_t)(in_b - 1) & 1u, a.wait_limit_ns);
+                    if (!kFwd && in_n > 0) ptx::mbar_wait(fullN, (uint32_t)(in_n - 1) & 1u, a.wait_limit_ns);
+                }
+            }
+        } else if (w == kCompute / 32) {
+            const uint32_t id64 = ptx::umma_idesc_bf16(128, 64), id128 = ptx::umma_idesc_bf16(128, 128), mnB = ptx::kIdescBMajorMN;
+            for (int64_t i = 0; i < nc; ++i) {
+                if (!wait(fullA, i) || !wait(s_ready, i)) break;
+                __syncwarp();
+                ptx::tc_fence_after();
+                const uint8_t* img = sm + O_A;
+                mma6_ta<8, kSParts>(tm + C_1, tm + C_S, kFwd ? mn_major<128, 1>(img) : k_major<64, 2>(img), kFwd ? id64 | mnB : id64, false);
+                ptx::umma_commit(m1);
+                if (!wait(fullB, i) || !wait(x_ready, i)) break;
+                __syncwarp();
+                ptx::tc_fence_after();
+                mma6_ta<4, kXParts>(tm + C_3, tm + C_X, kFwd ? mn_major<64, 2>(sm + O_B) : k_major<128, 1>(sm + O_B), kFwd ? id128 | mnB : id128, false);
+                ptx::umma_commit(m2);
+            }
+            __syncwarp();
+            ptx::umma_commit(done);        // before the TMEM goes away
+            if (!ptx::mbar_wait(done, 0, a.wait_limit_ns)) *abort_word = 1;
+            __syncwarp();
+        }
     }
     __syncthreads();
     if (t == 0 && *abort_word && atomicCAS(&a.hdr->status, 0, (int)KDA_ERR_TIMEOUT) == 0) a.hdr->where = 32;
-    if (w == 0) ptx::tmem_dealloc(tm, 128);
+    if (w == 0) ptx::tmem_dealloc(tm, 512);
 }
 
 __global__ void __launch_bounds__(kT, 1) kda_bwd_chain(BwdChunkArgs a)
 {
-    extern __shared__ uint8_t smem_raw[];
-    const int h = blockIdx.y, n = blockIdx.z, slice = blockIdx.x >> 1;
+    extern __shared__ __align__(1024) uint8_t sm[];
+    const int h = blockIdx.y, n = blockIdx.z;
     if (a.seq_heads[h]) return;
-    uint8_t* sm = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
-    if (blockIdx.x & 1) chain_run<true>(a, sm, n, h, slice * NS);
-    else chain_run<false>(a, sm, n, h, slice * NS);
+    if ((ptx::smem_u32(sm) & 1023u) != 0) {
+        if (threadIdx.x == 0 && atomicCAS(&a.hdr->status, 0, (int)KDA_ERR_TIMEOUT) == 0) a.hdr->where = 33;
+        return;
+    }
+    if (blockIdx.x & 1) chain_run<true>(a, sm, n, h);
+    else chain_run<false>(a, sm, n, h);
 }
 
 }  // namespace
@@ -239,7 +300,7 @@ kda_status_t launch_bwd_chain(const BwdChunkArgs& a, cudaStream_t st)
         }
     }
     ProfScope ps(PROF_INTER, st);
-    kda_bwd_chain<<<dim3(2 * kD / NS, (unsigned)a.H, (unsigned)a.n_seqs), kT, kSmem, st>>>(a);
+    kda_bwd_chain<<<dim3(2, (unsigned)a.H, (unsigned)a.n_seqs), kT, kSmem, st>>>(a);
     count_launch();
     KDA_CUDA_TRY(cudaGetLastError());
     return KDA_OK;

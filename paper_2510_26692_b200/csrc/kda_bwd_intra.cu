@@ -3,11 +3,14 @@
 // (kda_split3.cuh); the 64 x 64 inverse is fp32 FMA and runs beside the two products that do not need it.
 //
 //   A   [K^ ; Q] K_^T        -> B (masked), P (masked)
-//   C1  Q^T dO               -> N            C2  P^T dO -> X
-//   D1  T' K^                -> W'           D2  T' V   -> U'
-// Shared memory: RQ 96 KB [K^ ; Q], later the W' image; RK 48 KB K_, then dO, then V; L, T' fp32; RP 24 KB P, then T'.
+//   C1  dO^T Q               -> N            C2  dO^T P -> X
+//   D1  K^^T T'^T            -> W'^T         D2  V^T T'^T -> U'^T
+// (the 64-row matrices as the N side: 128 x 64 x 16 takes the tensor core half of 128 x 128 x 16).  dO and V that are stored
+// in bf16 are operands as they are.  Shared memory: RQ 96 KB [K^ ; Q], later the W'^T image; RK 48 KB K_, then V;
+// L, T' fp32; RP 24 KB P, then T'; dO in a place of its own (bf16) or in RK before V.
 //
-// T=4096, H=32: 470 us with warp-level tf32 products, 271 in this form.
+// T=4096, H=32: 470 us with warp-level tf32 products; with all operands split and 64-row products on 128 rows 271; 230
+// in this form.
 #include "kda_bwd.cuh"
 #include "kda_mma3.cuh"
 #include "kda_split3.cuh"
@@ -21,12 +24,12 @@ constexpr int kIssue = 15;              // the warp that issues the MMAs: no par
 constexpr int LM = 68;
 constexpr uint32_t O_RQ = 0, O_RK = 98304, O_RP = O_RK + 49152, O_L = O_RP + 24576, O_T = O_L + 64 * LM * 4,
                    O_G = O_RP,                       // e^(G - G_m) [64][132] fp32 before P, L and T' exist
-                   O_VEC = O_T + 64 * LM * 4;
-static_assert(O_G + 64 * 132 * 4 <= O_VEC, "G fits where P, L and T' come to lie");
+                   O_DO = O_T + 64 * LM * 4, O_VEC = O_DO + 16384;
+static_assert(O_G + 64 * 132 * 4 <= O_DO, "G fits where P, L and T' come to lie");
 constexpr int V_BETA = 0, V_SEG = 64, V_BAR = 1088;     // floats: beta, segment sums [2][4][128], barriers
 constexpr uint32_t kSmem = O_VEC + V_BAR * 4 + 64 + 1024;
 static_assert(kSmem <= 232448, "fits the shared memory of one SM");
-constexpr uint32_t C_N = 0, C_X = 128, C_A = 256, C_W = 256, C_U = 384;   // TMEM columns (A is read before W' is formed)
+constexpr uint32_t C_N = 0, C_X = 128, C_A = 192, C_W = 256, C_U = 320;   // TMEM columns
 
 template <typename T>
 __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
@@ -42,7 +45,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
     // bf16 rows: a CTA per SM goes through the tiles, and the inputs of the next wait in registers while the tensor core
     // works on the last products of this one (4096 x 32 heads 285 -> 271 us).  fp32 rows take twice the registers, and
     // spilled (67 -> 77 us on six packed sequences): a CTA per tile.
-    constexpr bool kLoop = sizeof(T) == 2;
+    constexpr bool kExact = sizeof(T) == 2, kLoop = kExact;
     const int64_t n_tiles = a.n_chunks * a.H;
     int64_t id = blockIdx.x;
     int h;
@@ -93,6 +96,10 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
         if (ok) ok = ptx::mbar_wait(&bar[i], phase, a.wait_limit_ns);
         __syncwarp();
         ptx::tc_fence_after();
+    };
+    // a unit of a bf16 matrix as the first split of its image
+    auto put_exact = [&](uint8_t* img, int r, int col, const Raw8<T>& x) {
+        *reinterpret_cast<uint4*>(img + (col >> 6) * 8192 + ptx::sw128_off((uint32_t)r, (uint32_t)(col & 63))) = make_uint4(x.w[0], x.w[1], x.w[2], x.w[3]);
     };
     auto publish = [&]() {     // shared-memory images written by all threads -> visible to the MMA and the TMA engine
         ptx::fence_async_smem();
@@ -159,6 +166,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
                 tile[bt::GC + c] = exp_of(total);
                 tile[bt::EM + c] = exp_of(gm);
             }
+            if (t < 64) tile[bt::BE + t] = sBeta[t];
         }
         // A head that the sequential kernels do needs no tiles: they are left here (4096 x 32 heads, all of them out of
         // range: the stage 326 us when they went on).
@@ -187,6 +195,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
                 put8<128, 2>(sm + O_RQ, r, c8, kk);
                 put8<128, 2>(sm + O_RQ, 64 + r, c8, qq);
                 put8<64, 2>(sm + O_RK, r, c8, ki);
+                if (kExact) put_exact(sm + O_DO, r, c8, dr[j]);
             }
         }
         publish();
@@ -233,18 +242,20 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
             }
         }
         if (t == kCopy) ptx::bulk_wait_read0();
-        __syncthreads();      // K_ has been read out
+        if (!kExact) {
+            __syncthreads();      // K_ has been read out
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            float x[8];
-            to_f(dr[j], x);
-            put8<64, 2>(sm + O_RK, row0 + 32 * j, c8, x);
+            for (int j = 0; j < 2; ++j) {
+                float x[8];
+                to_f(dr[j], x);
+                put8<64, 2>(sm + O_RK, row0 + 32 * j, c8, x);
+            }
         }
         publish();
         if (w == kIssue) {
-            const uint32_t idesc = ptx::umma_idesc_bf16(128, 128) | mnA | mnB;
-            mma6<4>(tm + C_N, mn_major<128, 2>(sm + O_RQ, 64), mn_major<64, 2>(sm + O_RK), idesc, false);
-            mma6<4>(tm + C_X, mn_major<64, 1>(sm + O_RP), mn_major<64, 2>(sm + O_RK), idesc, false);
+            const Operand dO = mn_major<64, 2>(sm + (kExact ? O_DO : O_RK));
+            mma6<4, kExact>(tm + C_N, dO, mn_major<128, 2>(sm + O_RQ, 64), ptx::umma_idesc_bf16(128, 128) | mnA | mnB, false);
+            mma6<4, kExact>(tm + C_X, dO, mn_major<64, 1>(sm + O_RP), ptx::umma_idesc_bf16(128, 64) | mnA | mnB, false);
             ptx::umma_commit(&bar[1]);
         }
         if (w < 4) mma3::invert_unit_lower<LM>(sL, sT, t, [] { ptx::named_bar_sync(1, 128); });
@@ -260,16 +271,20 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
             put8<64, 1>(sm + O_RP, r, x0, x);
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-                to_f(vr[j], x);
-                put8<64, 2>(sm + O_RK, row0 + 32 * j, c8, x);
+                if (kExact) {
+                    put_exact(sm + O_RK, row0 + 32 * j, c8, vr[j]);
+                } else {
+                    to_f(vr[j], x);
+                    put8<64, 2>(sm + O_RK, row0 + 32 * j, c8, x);
+                }
             }
         }
         publish();
         if (w == kIssue) {
-            const uint32_t idesc = ptx::umma_idesc_bf16(128, 128) | mnB;
-            mma6<4>(tm + C_W, k_major<64, 1>(sm + O_RP), mn_major<128, 2>(sm + O_RQ), idesc, false);
+            const uint32_t idesc = ptx::umma_idesc_bf16(128, 64) | mnA;
+            mma6<4>(tm + C_W, mn_major<128, 2>(sm + O_RQ), k_major<64, 1>(sm + O_RP), idesc, false);
             ptx::umma_commit(&bar[2]);
-            mma6<4>(tm + C_U, k_major<64, 1>(sm + O_RP), mn_major<64, 2>(sm + O_RK), idesc, false);
+            mma6<4, kExact>(tm + C_U, mn_major<64, 2>(sm + O_RK), k_major<64, 1>(sm + O_RP), idesc, false);
             ptx::umma_commit(&bar[3]);
         }
         id += gridDim.x;
@@ -277,32 +292,30 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
             request();
             request_rows();
         }
-        // accumulators out: columns cg .. cg + 31 of this thread's row
-        const int row = quad * 32 + lane, cg = (w >> 2) * 32;
-        auto store_rf = [&](uint32_t col, float* m, int rows) {
-            uint32_t y[32];
-            ptx::tmem_ld_32x32b_x32(tq + col + cg, y);
+        // accumulators out: this thread's row, 16 columns from cg (of N also 64 + cg)
+        const int row = quad * 32 + lane, cg = (w >> 2) * 16;
+        auto store_rf = [&](uint32_t col, float* m, int c0) {
+            uint32_t y[16];
+            ptx::tmem_ld_32x32b_x16(tq + col + c0, y);
             ptx::tmem_ld_wait();
 #pragma unroll
-            for (int e = 0; e < 32; e += 4)
-                *reinterpret_cast<uint4*>(m + rf(rows, row, cg + e)) = make_uint4(y[e], y[e + 1], y[e + 2], y[e + 3]);
+            for (int e = 0; e < 16; e += 4)
+                *reinterpret_cast<uint4*>(m + rf(128, row, c0 + e)) = make_uint4(y[e], y[e + 1], y[e + 2], y[e + 3]);
         };
-        store_rf(C_N, tile + bt::N, 128);
-        if (quad < 2) store_rf(C_X, tile + bt::X, 64);
-        wait(2);
-        uint32_t yw[32];
-        if (quad < 2) {
-            ptx::tmem_ld_32x32b_x32(tq + C_W + cg, yw);
+        store_rf(C_N, tile + bt::N, cg);
+        store_rf(C_N, tile + bt::N, 64 + cg);
+        store_rf(C_X, tile + bt::X, cg);
+        wait(2);              // nothing reads [K^ ; Q] any more: W'^T over it
+        {
+            uint32_t yw[16];
+            ptx::tmem_ld_32x32b_x16(tq + C_W + cg, yw);
             ptx::tmem_ld_wait();
-        }
-        wait(3);              // nothing reads the images any more: W' over [K^ ; Q]
-        if (quad < 2) {
 #pragma unroll
-            for (int q8 = 0; q8 < 4; ++q8) {
+            for (int q8 = 0; q8 < 2; ++q8) {
                 float x[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) x[e] = __uint_as_float(yw[8 * q8 + e]);
-                put8<64, 2>(sm + O_RQ, row, cg + 8 * q8, x);
+                put8<128, 1>(sm + O_RQ, row, cg + 8 * q8, x);
             }
         }
         publish();
@@ -310,7 +323,8 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
             ptx::bulk_s2g(tile + bt::WI, sm + O_RQ, 49152);
             ptx::bulk_commit();
         }
-        if (quad < 2) store_rf(C_U, tile + bt::R, 64);
+        wait(3);
+        store_rf(C_U, tile + bt::R, cg);
         phase ^= 1u;
         if (!kLoop || id >= n_tiles) break;
     }

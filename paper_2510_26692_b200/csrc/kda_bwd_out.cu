@@ -3,9 +3,9 @@
 //
 // The products of a tile (M x N x K) and where their operands live: D and X are regions of shared memory of 96 KB each, A
 // the 192 TMEM columns of an A operand.
-//   P1  dV = (beta T')^T dX                 T' 64x64 and dX 64x128 in X
+//   P1  dV = (beta T')^T dX                 T' 64x64 and dX^T 128x64 in X
 //   P2  e^(G_m) S [dO ; -dV]^T              S in A, [dO ; -dV] 128x128 in D
-//   P4  [dO ; -dV] r^T                      r 64x128 in X
+//   P4  [dO ; -dV] r^T                      r^T 128x64 in X
 //   P3  Lam r^T                             Lam in A
 //   P5  P2 += K_^T [dP ; dB]^T              [dP ; dB] 128x64 and K_ 64x128 in X
 //   P6  [Q ; K^]^T [dP ; dB]                [Q ; K^] 128x128 in D
@@ -27,8 +27,8 @@ constexpr int kIssue = 15;                                    // the warp that i
 constexpr uint32_t O_D = 0, O_X = 98304, O_VEC = 196608;
 constexpr uint32_t O_T = O_X, O_DX = O_X + 24576;             // T', dX
 constexpr uint32_t O_R = O_X, O_DPB = O_X + 49152;            // r, later K_; [dP ; dB]
-// fp32 vectors (floats from O_VEC): beta[64] dbeta[8][64] sGC[4][128] colsum[2][64] seg[4][128] sum[4][128], then barriers
-constexpr int V_BETA = 0, V_DB = 64, V_GC = 576, V_CS = 1088, V_SEG = 1216, V_SUM = 1728, V_BAR = 2240;
+// fp32 vectors (floats from O_VEC): beta[64] dbeta[4][64] sGC[4][128] colsum[2][64] seg[4][128] sum[4][128], then barriers
+constexpr int V_BETA = 0, V_DB = 64, V_GC = 320, V_CS = 832, V_SEG = 960, V_SUM = 1472, V_BAR = 1984;
 constexpr uint32_t kSmem = O_VEC + V_BAR * 4 + 64 + 1024;     // + alignment slack
 static_assert(kSmem <= 232448, "fits the shared memory of one SM");
 // TMEM columns; P1 (128) lies where P3 and P6 come to lie
@@ -43,6 +43,20 @@ __device__ __forceinline__ float ldv(const __nv_bfloat16* p, bool in) {
     unsigned short x = 0;
     if (in) asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(x) : "l"(p));
     return __uint_as_float((uint32_t)x << 16);
+}
+
+// sums of 16 values over the warp; lane l gets number l % 16 in s[0] (each exchange halves the values a lane carries)
+__device__ __forceinline__ void lane_sums(float (&s)[16], int lane) {
+#pragma unroll
+    for (int n = 8; n >= 1; n >>= 1) {
+        const bool up = (lane & n) != 0;
+#pragma unroll
+        for (int e = 0; e < n; ++e) {
+            const float send = up ? s[e] : s[e + n], keep = up ? s[e + n] : s[e];
+            s[e] = keep + __shfl_xor_sync(0xffffffffu, send, n);
+        }
+    }
+    s[0] += __shfl_xor_sync(0xffffffffu, s[0], 16);
 }
 
 template <typename T>
@@ -85,8 +99,8 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     };
     // unit u of a matrix with 128 columns: row u >> 4, columns 8 (u & 15) .. + 7
     const int c8 = (t & 15) * 8, row0 = t >> 4;      // token tensors: rows row0 + 32 j
-    const int ra = t & 63, ca = (t >> 6) * 8;        // rf matrices of 64 rows: columns ca + 64 j
-    const int rs = t & 127, cs = (t >> 7) * 32;      // and of 128 rows (TMEM lane rs): columns cs + 8 j
+    const int rs = t & 127, cs = (t >> 7) * 32;      // matrices of 128 rows (TMEM lane rs): columns cs + 8 j, or ct + 8 j of 64
+    const int ct = (t >> 7) * 16;
     auto tok_off = [&](int r) { return ((size_t)(loc.tok0 + r) * a.H + h) * kD; };
 
     // ---- P1: dV -----------------------------------------------------------------------------------------
@@ -97,33 +111,34 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         const int r = t >> 3, x = (t & 7) * 8;
         ldraw(xt, tile + bt::T + r * 64 + x);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) ldraw_rf(xx[j], tile + bt::X, 64, ra, ca + 64 * j);
+        for (int j = 0; j < 2; ++j) ldraw_rf(xx[j], tile + bt::X, 128, rs, ct + 8 * j);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) ldraw_rf(rr[j], tile + bt::R, 64, ra, ca + 64 * j);
+        for (int j = 0; j < 2; ++j) ldraw_rf(rr[j], tile + bt::R, 128, rs, ct + 8 * j);
         const float b = r < loc.len ? a.beta[(size_t)(loc.tok0 + r) * a.H + h] : 0.f;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) ldraw_rf(xs[j], tile + bt::S, 128, rs, cs + 8 * j);
+        for (int j = 0; j < 4; ++j) ldraw_sf(xs[j], tile + bt::S, rs, cs + 8 * j);
         float v[8], u[8];
         to_f(xt, v);
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] *= b;
         put8<64, 1>(sm + O_T, r, x, v);
         if (x == 0) sBeta[r] = b;
-        float s = 0.f;      // share of r_j . dX_j
+        float s[16];      // shares of r_j . dX_j, j = ct ..: column rs of both
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             to_f(xx[j], v);
             to_f(rr[j], u);
-            put8<64, 2>(sm + O_DX, ra, ca + 64 * j, v);
+            put8<128, 1>(sm + O_DX, rs, ct + 8 * j, v);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) s = fmaf(v[e], u[e], s);
+            for (int e = 0; e < 8; ++e) s[8 * j + e] = v[e] * u[e];
         }
-        sDb[t] = s;         // [8][64]
+        lane_sums(s, lane);
+        if (lane < 16) sDb[(w & 3) * 64 + ct + lane] = s[0];
     }
     Raw8<float> lam[4];
     Raw8<T> dd[2];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) ldraw_rf(lam[j], tile + bt::L, 128, rs, cs + 8 * j);
+    for (int j = 0; j < 4; ++j) ldraw_sf(lam[j], tile + bt::L, rs, cs + 8 * j);
 #pragma unroll
     for (int j = 0; j < 2; ++j)
         ldraw(dd[j], static_cast<const T*>(a.d_o) + tok_off(row0 + 32 * j) + c8, row0 + 32 * j < loc.len && a.d_o);
@@ -142,24 +157,24 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     const int quad = w & 3, seg = w >> 2;
     const uint32_t tq = tm + ((uint32_t)(quad * 32) << 16);
     if (w == kIssue) {
-        mma6<4>(tm + C_P1, mn_major<64, 1>(sm + O_T, 0, true), mn_major<64, 2>(sm + O_DX), id | mnA | mnB, false);
+        mma6<4>(tm + C_P1, mn_major<64, 1>(sm + O_T, 0, true), k_major<128, 1>(sm + O_DX), id | mnA, false);
         ptx::umma_commit(&bar[0]);
     }
     // meanwhile: e^(G_m) S, and its dot products with Lam; dO
     {
-        float s = 0.f, x[32];
+        float s = 0.f;
+        float2 x[16];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             float v[8], l[8];
             to_f(xs[j], v);
             to_f(lam[j], l);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                s = fmaf(v[e], l[e], s);
-                x[8 * j + e] = v[e] * em;
-            }
+            for (int e = 0; e < 8; ++e) s = fmaf(v[e], l[e], s);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[4 * j + e] = make_float2(v[2 * e] * em, v[2 * e + 1] * em);
         }
-        put32_tmem<kAParts>(tq + C_A + seg * 16, x);
+        put_tmem<kAParts>(tq + C_A + seg * 16, x);
         sGC[t] = s * em * em;      // [4][128]; (G_m = G_C / 2)
     }
 #pragma unroll
@@ -191,7 +206,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             to_f(rr[j], v);
-            put8<64, 2>(sm + O_R, ra, ca + 64 * j, v);
+            put8<128, 1>(sm + O_R, rs, ct + 8 * j, v);
         }
     }
     publish();
@@ -200,7 +215,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     if (w == kIssue) {
         mma6_ta<8, kAParts>(tm + C_P2, tm + C_A, k_major<128, 2>(sm + O_D), id, false);
         ptx::umma_commit(&bar[1]);
-        mma6<8>(tm + C_P4, k_major<128, 2>(sm + O_D), k_major<64, 2>(sm + O_R), ptx::umma_idesc_bf16(128, 64), false);
+        mma6<8>(tm + C_P4, k_major<128, 2>(sm + O_D), mn_major<128, 1>(sm + O_R), ptx::umma_idesc_bf16(128, 64) | mnB, false);
         ptx::umma_commit(&bar[2]);
     }
     // the gated operands' inputs, requested while the tensor core works
@@ -215,20 +230,17 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     }
     wait(1);
     {   // Lam over S
-        float x[32];
+        float2 x[16];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            float v[8];
-            to_f(lam[j], v);
+        for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int e = 0; e < 8; ++e) x[8 * j + e] = v[e];
-        }
-        put32_tmem<kAParts>(tq + C_A + seg * 16, x);
+            for (int e = 0; e < 4; ++e) x[4 * j + e] = make_float2(__uint_as_float(lam[j].w[2 * e]), __uint_as_float(lam[j].w[2 * e + 1]));
+        put_tmem<kAParts>(tq + C_A + seg * 16, x);
         ptx::tmem_st_wait();
     }
     publish();
     if (w == kIssue) {
-        mma6_ta<8, kAParts>(tm + C_P3, tm + C_A, k_major<64, 2>(sm + O_R), ptx::umma_idesc_bf16(128, 64), false);
+        mma6_ta<8, kAParts>(tm + C_P3, tm + C_A, mn_major<128, 1>(sm + O_R), ptx::umma_idesc_bf16(128, 64) | mnB, false);
         ptx::umma_commit(&bar[3]);
     }
     wait(2);
@@ -259,16 +271,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         put8<128, 1>(sm + O_DPB, R, j0, lo);
         put8<128, 1>(sm + O_DPB, R, j0 + 8, hi);
         if (isB) {   // column sums over the warp's 32 rows: 16 values over 32 lanes
-#pragma unroll
-            for (int s = 8; s >= 1; s >>= 1) {
-                const bool up = (lane & s) != 0;
-#pragma unroll
-                for (int e = 0; e < s; ++e) {
-                    const float send = up ? bb[e] : bb[e + s], keep = up ? bb[e + s] : bb[e];
-                    bb[e] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-                }
-            }
-            bb[0] += __shfl_xor_sync(0xffffffffu, bb[0], 16);
+            lane_sums(bb, lane);
             if (lane < 16) sCs[(quad - 2) * 64 + j0 + lane] = bb[0];
         }
     }
@@ -307,7 +310,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     if (t < loc.len) {
         float s = sCs[t] + sCs[64 + t];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) s += sDb[j * 64 + t];
+        for (int j = 0; j < 4; ++j) s += sDb[j * 64 + t];
         a.db[(size_t)(loc.tok0 + t) * a.H + h] = s;
     }
     // the column pass's inputs: thread = channel c of 16 consecutive tokens

@@ -24,44 +24,42 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
+// The next split of a pair of values: returns it and leaves the rest in r (one packed operation).
+__device__ __forceinline__ uint32_t take2(float2& r) {
+    const uint32_t w = pack2(r.x, r.y);
+    r = __ffma2_rn(make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)), make_float2(-1.f, -1.f), r);
+    return w;
+}
 // Splits x[0..7] into the 16-byte chunk (row, col .. col+7) of a matrix image, col a multiple of 8.
 template <int R, int NB>
 __device__ __forceinline__ void put8(uint8_t* img, int row, int col, const float (&x)[8]) {
     uint8_t* p = img + (col >> 6) * (R * 128) + ptx::sw128_off((uint32_t)row, (uint32_t)(col & 63));
-    float r[8];
+    float2 r[4];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) r[e] = x[e];
+    for (int e = 0; e < 4; ++e) r[e] = make_float2(x[2 * e], x[2 * e + 1]);
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
         uint32_t w[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            w[e] = pack2(r[2 * e], r[2 * e + 1]);
-            if (s < 2) {
-                r[2 * e] -= __uint_as_float(w[e] << 16);
-                r[2 * e + 1] -= __uint_as_float(w[e] & 0xffff0000u);
-            }
-        }
+        for (int e = 0; e < 4; ++e) w[e] = s < 2 ? take2(r[e]) : pack2(r[e].x, r[e].y);
         *reinterpret_cast<uint4*>(p + s * (NB * R * 128)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
 }
-
-// Splits 32 consecutive columns of this lane's row into the A operand in TMEM (two bf16 values a column, kParts columns from
-// one split to the next): no pass over shared memory, and the product reads only its B operand there.
-template <int kParts>
-__device__ __forceinline__ void put32_tmem(uint32_t taddr, float (&x)[32]) {
+// Splits 16 or 32 consecutive columns of this lane's row into the A operand in TMEM (two bf16 values a column, kParts columns
+// from one split to the next): no pass over shared memory, and the product reads only its B operand there.
+template <int kParts, int N>
+__device__ __forceinline__ void put_tmem(uint32_t taddr, const float2 (&x)[N]) {
+    static_assert(N == 8 || N == 16, "a tcgen05.st of 8 or 16 columns");
+    float2 r[N];
+#pragma unroll
+    for (int e = 0; e < N; ++e) r[e] = x[e];
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
-        uint32_t w[16];
+        uint32_t w[N];
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            w[e] = pack2(x[2 * e], x[2 * e + 1]);
-            if (s < 2) {
-                x[2 * e] -= __uint_as_float(w[e] << 16);
-                x[2 * e + 1] -= __uint_as_float(w[e] & 0xffff0000u);
-            }
-        }
-        ptx::tmem_st_32x32b_x16(taddr + s * kParts, w);
+        for (int e = 0; e < N; ++e) w[e] = s < 2 ? take2(r[e]) : pack2(r[e].x, r[e].y);
+        if constexpr (N == 16) ptx::tmem_st_32x32b_x16(taddr + s * kParts, w);
+        else ptx::tmem_st_32x32b_x8(taddr + s * kParts, w);
     }
 }
 
@@ -81,14 +79,16 @@ __device__ __forceinline__ Operand mn_major(const uint8_t* img, int row0 = 0, bo
     return {ptx::umma_desc_sw128_mn(ptx::smem_u32(img) + row0 * 128, dup ? 0u : R * 128u), NB * R * 8u, 128u, 512u};
 }
 
-// d (+)= A B over KS steps of 16 in K; a whole converged warp.  idesc carries M, N and the majors.
-template <int KS>
+// d (+)= A B over KS steps of 16 in K; a whole converged warp.  idesc carries M, N and the majors.  kExactA: A holds bf16
+// numbers, its image the first split alone (three MMAs).
+template <int KS, bool kExactA = false>
 __device__ __forceinline__ void mma6(uint32_t d_tmem, const Operand& A, const Operand& B, uint32_t idesc, bool accumulate) {
-    // (sa, sb): (2,0) (0,2) (1,1) (1,0) (0,1) (0,0)
+    // (sa, sb): (2,0) (0,2) (1,1) (1,0) (0,1) (0,0); exact: (0,2) (0,1) (0,0)
     uint32_t acc = accumulate ? 1u : 0u;
 #pragma unroll 1
-    for (int p = 0; p < 6; ++p) {
-        const uint32_t sa = p == 0 ? 2u : (p == 2 || p == 3) ? 1u : 0u, sb = p == 1 ? 2u : (p == 2 || p == 4) ? 1u : 0u;
+    for (int p = 0; p < (kExactA ? 3 : 6); ++p) {
+        const uint32_t sa = kExactA ? 0u : p == 0 ? 2u : (p == 2 || p == 3) ? 1u : 0u;
+        const uint32_t sb = kExactA ? 2u - p : p == 1 ? 2u : (p == 2 || p == 4) ? 1u : 0u;
         const uint64_t da = A.desc + sa * A.split, db = B.desc + sb * B.split;
 #pragma unroll
         for (int k = 0; k < KS; ++k) {
@@ -100,7 +100,7 @@ __device__ __forceinline__ void mma6(uint32_t d_tmem, const Operand& A, const Op
     }
 }
 
-// the same with A in TMEM (put32_tmem)
+// the same with A in TMEM (put_tmem)
 template <int KS, int kParts>
 __device__ __forceinline__ void mma6_ta(uint32_t d_tmem, uint32_t a_tmem, const Operand& B, uint32_t idesc, bool accumulate) {
     uint32_t acc = accumulate ? 1u : 0u;
