@@ -987,8 +987,8 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
     __nv_bfloat16* op = kHasQ ? reinterpret_cast<__nv_bfloat16*>(a.o) : nullptr;
 
     auto wait_by = [&](auto attempt, uint64_t* bar, uint32_t parity, int where) {
+        if (attempt(bar, parity)) return;        // (one access to the busy shared memory where one will do)
         if (*abort_flag) return;
-        if (attempt(bar, parity)) return;
         const uint64_t t0 = ptx::globaltimer_ns();
         uint32_t spins = 0;
         while (!attempt(bar, parity)) {
