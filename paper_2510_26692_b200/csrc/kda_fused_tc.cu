@@ -48,7 +48,7 @@ constexpr int kEngThreads = 256;
 // the MMAs); what it can it does during the blocked substitution, which warps 6 and 7 have no part in.
 constexpr int kServiceThread = 224;
 constexpr int LDT = 68;                                   // padded fp32 row of the 64x64 matrix
-constexpr int LDD = 16;                                   // padded fp32 row of a 16x16 diagonal block
+constexpr int LDD = 20;                                   // padded fp32 row of a 16x16 diagonal block
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kClamp2 = 80.f * 1.4426950408889634f;     // the +-80 clamp in the log2 domain
 constexpr float kClampX = kClamp2 + 0.5f;                 // (G_m is rounded to a whole number)
@@ -76,7 +76,7 @@ constexpr uint32_t E_V_BLOCK = 8192;
 constexpr uint32_t E_A = 65536;         // fp32 [64][LDT]: L, X below the diagonal, T above it (transposed block
                                         // positions); then the U^T staging
 constexpr uint32_t E_TD = E_A + 64 * LDT * 4;     // fp32 4 x [16][LDD]: diagonal blocks of T; scan exchange [8][128] before
-constexpr uint32_t E_TD_BYTES = 4096;
+constexpr uint32_t E_TD_BYTES = 4 * 16 * LDD * 4;
 constexpr uint32_t E_BETA = E_TD + E_TD_BYTES;    // 64 fp32
 constexpr uint32_t E_DESC = E_BETA + 256;         // three tile descriptors: this tile, the next, the one after
 constexpr uint32_t E_CUR = E_DESC + 192;          // the service thread's EngineCursor
@@ -176,6 +176,12 @@ __device__ __forceinline__ float lg2(float x) {
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// two values of an array as one operand of the packed fp32 operations (half the instructions of single ones)
+__device__ __forceinline__ float2 pair(const float* x) { return make_float2(x[0], x[1]); }
+__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
+__device__ __forceinline__ void set(float* x, float2 v) { x[0] = v.x; x[1] = v.y; }
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b);
+__device__ __forceinline__ uint32_t pack_bf16(float2 v) { return pack_bf16(v.x, v.y); }
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<uint32_t*>(&p);
@@ -337,7 +343,9 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
                            const CUtensorMap* tm_q, const CUtensorMap* tm_v)
 {
     constexpr bool has_q = kHasQ;
-    constexpr int kNW = 8, kRPT = 8;
+    // rows of the gating loop at once: the fewer, the less code.  4096 x 32 heads, fused, 8 / 4 / 2: 113.6, 113.0, 115.1 us; 128 Ki tokens
+    // for the state, fused: 2800, 2743, 2567; layer call on three prompts: 218.4, 222.8, 223.9
+    constexpr int kNW = 8, kRPT = 8, kGateRows = kLayer ? 8 : kFused && !kHasQ ? 2 : 4;
     constexpr int kInvWarps = 6;       // warps of the blocked substitution
     constexpr int kMma2Warp = 2;       // issues half of the second MMA group (warp 0 the rest)
     const ChunkArgs& a = f.a;
@@ -498,11 +506,11 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         // ---- a1: cumulative log-decay, in the log2 domain (exponentials below are bare ex2) ---------
         if (!kLayer) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) G[0][e] *= kLog2e;
+            for (int e = 0; e < 4; e += 2) set(&G[0][e], __fmul2_rn(pair(&G[0][e]), both(kLog2e)));
 #pragma unroll
             for (int r = 1; r < kRPT; ++r)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) G[r][e] = fmaf(G[r][e], kLog2e, G[r - 1][e]);
+                for (int e = 0; e < 4; e += 2) set(&G[r][e], __ffma2_rn(pair(&G[r][e]), both(kLog2e), pair(&G[r - 1][e])));
         }
         *reinterpret_cast<float4*>(sTot + warp * kD + d0) =
             make_float4(G[kRPT - 1][0], G[kRPT - 1][1], G[kRPT - 1][2], G[kRPT - 1][3]);
@@ -554,8 +562,9 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         pend_k = pend_q = false;
         KT_MARK(te == 0, 2);   // prefix + TMA wait
         // ---- gated operands ---------------------------------------------------------------------------
-        // (two copies of the loop, chosen per warp: without the clamp when no channel of the warp's
-        // share of the tile can reach it, since |G_i - G_m| <= |G_C| / 2)
+        // (the clamp is for channels that reach it, see out_of_range; a second copy of the loop without it, chosen per warp,
+        // cost more in fetched instructions than it saved: packed batch, two kernels, 3053 instead of 2944 us.  Rolled for the
+        // same reason.)
         float* sNorm = reinterpret_cast<float*>(smem + E_NORM);
         if (kLayer) {
             // L2Norm of k and q: the warp owns its eight rows whole (32 lanes x 4 channels)
@@ -592,61 +601,60 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             }
             __syncwarp();
         }
-        auto gate_rows = [&](auto clamp_tag) {
-            constexpr bool kClamp = decltype(clamp_tag)::value;
+        {
             const int hf = c4 >> 4;                       // K-half (channels 0-63 / 64-127)
             float off[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) off[e] = base[e] - gref[e];
+#pragma unroll 1
+            for (int r0 = 0; r0 < kRPT; r0 += kGateRows) {
 #pragma unroll
-            for (int r = 0; r < kRPT; ++r) {
-                const int i = i0 + r;
-                const uint32_t o2 = (uint32_t)(i * 128 + ((((c4 >> 1) & 7) ^ (i & 7)) << 4) + (c4 & 1) * 8);
-                uint8_t* pk = smem + E_KQ + hf * E_KQ_HALF + o2;
-                uint2 k2 = *reinterpret_cast<const uint2*>(smem + E_KS + hf * 8192 + o2);
-                uint2 q2 = make_uint2(0u, 0u);
-                if (has_q) q2 = *reinterpret_cast<const uint2*>(pk + 8192);
-                if (i >= d_len) k2 = q2 = make_uint2(0u, 0u);
-                const float kf[4] = {__uint_as_float(k2.x << 16), __uint_as_float(k2.x & 0xffff0000u),
-                                     __uint_as_float(k2.y << 16), __uint_as_float(k2.y & 0xffff0000u)};
-                const float qf[4] = {__uint_as_float(q2.x << 16), __uint_as_float(q2.x & 0xffff0000u),
-                                     __uint_as_float(q2.y << 16), __uint_as_float(q2.y & 0xffff0000u)};
-                float okg[4], oqg[4], oki[4];
-                float rk = 1.f, rq = a.scale;
-                if (kLayer) {
-                    rk = sNorm[i];
-                    rq = a.scale * sNorm[kC + i];
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    float x = G[r][e] + off[e];
-                    if (kClamp) x = fminf(fmaxf(x, -kClampX), kClampX);
-                    const float e1 = ex2(x);                     // exp(G - G_m)
-                    const float e2 = ex2(-x);                    // exp(G_m - G)
+                for (int r = 0; r < kGateRows; ++r) {
+                    const int i = i0 + r0 + r;
+                    const uint32_t o2 = (uint32_t)(i * 128 + ((((c4 >> 1) & 7) ^ (i & 7)) << 4) + (c4 & 1) * 8);
+                    uint8_t* pk = smem + E_KQ + hf * E_KQ_HALF + o2;
+                    uint2 k2 = *reinterpret_cast<const uint2*>(smem + E_KS + hf * 8192 + o2);
+                    uint2 q2 = make_uint2(0u, 0u);
+                    if (has_q) q2 = *reinterpret_cast<const uint2*>(pk + 8192);
+                    if (i >= d_len) k2 = q2 = make_uint2(0u, 0u);
+                    const float kf[4] = {__uint_as_float(k2.x << 16), __uint_as_float(k2.x & 0xffff0000u),
+                                         __uint_as_float(k2.y << 16), __uint_as_float(k2.y & 0xffff0000u)};
+                    const float qf[4] = {__uint_as_float(q2.x << 16), __uint_as_float(q2.x & 0xffff0000u),
+                                         __uint_as_float(q2.y << 16), __uint_as_float(q2.y & 0xffff0000u)};
+                    float okg[4], oqg[4], oki[4];
+                    float rk = 1.f, rq = a.scale;
                     if (kLayer) {
-                        okg[e] = kf[e] * (e1 * rk);
-                        oki[e] = kf[e] * (e2 * rk);
-                    } else {
-                        okg[e] = kf[e] * e1;
-                        oki[e] = kf[e] * e2;
+                        rk = sNorm[i];
+                        rq = a.scale * sNorm[kC + i];
                     }
-                    oqg[e] = rq * qf[e] * e1;
+#pragma unroll
+                    for (int e = 0; e < 4; e += 2) {
+                        const float2 x2 = __fadd2_rn(pair(&G[r][e]), pair(&off[e]));
+                        const float x0 = fminf(fmaxf(x2.x, -kClampX), kClampX), x1 = fminf(fmaxf(x2.y, -kClampX), kClampX);
+                        float2 e1 = make_float2(ex2(x0), ex2(x1)), e2 = make_float2(ex2(-x0), ex2(-x1));   // exp(G - G_m), exp(G_m - G)
+                        set(&oqg[e], __fmul2_rn(__fmul2_rn(both(rq), pair(&qf[e])), e1));
+                        if (kLayer) {
+                            e1 = __fmul2_rn(e1, both(rk));
+                            e2 = __fmul2_rn(e2, both(rk));
+                        }
+                        set(&okg[e], __fmul2_rn(pair(&kf[e]), e1));
+                        set(&oki[e], __fmul2_rn(pair(&kf[e]), e2));
+                    }
+                    *reinterpret_cast<uint2*>(pk) = make_uint2(pack_bf16(okg[0], okg[1]), pack_bf16(okg[2], okg[3]));
+                    if (has_q)
+                        *reinterpret_cast<uint2*>(pk + 8192) =
+                            make_uint2(pack_bf16(oqg[0], oqg[1]), pack_bf16(oqg[2], oqg[3]));
+                    *reinterpret_cast<uint2*>(smem + E_KI + hf * E_KI_HALF + o2) =
+                        make_uint2(pack_bf16(oki[0], oki[1]), pack_bf16(oki[2], oki[3]));
+                    if (has_q)   // what the chain reads: scale Q exp(G), over the raw k that this thread has just read
+                        *reinterpret_cast<uint2*>(smem + E_KS + hf * 8192 + o2) =
+                            make_uint2(pack_bf16(__fmul2_rn(pair(oqg), pair(em))), pack_bf16(__fmul2_rn(pair(oqg + 2), pair(em + 2))));
                 }
-                *reinterpret_cast<uint2*>(pk) = make_uint2(pack_bf16(okg[0], okg[1]), pack_bf16(okg[2], okg[3]));
-                if (has_q)
-                    *reinterpret_cast<uint2*>(pk + 8192) =
-                        make_uint2(pack_bf16(oqg[0], oqg[1]), pack_bf16(oqg[2], oqg[3]));
-                *reinterpret_cast<uint2*>(smem + E_KI + hf * E_KI_HALF + o2) =
-                    make_uint2(pack_bf16(oki[0], oki[1]), pack_bf16(oki[2], oki[3]));
-                if (has_q)   // what the chain reads: scale Q exp(G), over the raw k that this thread has just read
-                    *reinterpret_cast<uint2*>(smem + E_KS + hf * 8192 + o2) =
-                        make_uint2(pack_bf16(oqg[0] * em[0], oqg[1] * em[1]), pack_bf16(oqg[2] * em[2], oqg[3] * em[3]));
+#pragma unroll
+                for (int r = 0; r + kGateRows < kRPT; ++r)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) G[r][e] = G[r + kGateRows][e];
             }
-        };
-        {
-            const bool may_clamp = fminf(fminf(gref[0], gref[1]), fminf(gref[2], gref[3])) < -kClamp2 + 0.5f;
-            if (__any_sync(0xffffffffu, may_clamp)) gate_rows(std::true_type{});
-            else gate_rows(std::false_type{});
         }
         if (te == kServiceThread) ptx::bulk_wait_read0();   // the previous tile's W and U^T have been read out
         ptx::fence_async_smem();
@@ -706,31 +714,32 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
             const int q4 = warp & 3, c0 = (warp >> 2) * 32;
             const int Rr = q4 * 32 + lane;
             uint32_t r[32];
-            ptx::tmem_ld_32x32b_x32(tmem_e + ((uint32_t)(q4 * 32) << 16) + c0, r);
-            ptx::tmem_ld_wait();
+            // the warp's block of 32 rows lies above the diagonal, below it, or on it: only the last needs masks, the first is
+            // zero (and of L nobody reads it)
+            const int where = (q4 & 1) * 32 - c0;      // > 0: below
+            if (where >= 0) {
+                ptx::tmem_ld_32x32b_x32(tmem_e + ((uint32_t)(q4 * 32) << 16) + c0, r);
+                ptx::tmem_ld_wait();
+            }
             if (Rr < 64) {
-                const int i = Rr;
+                const int i = Rr, lim = where > 0 ? 32 : lane;
                 const float bi = sBeta[i];
+                if (where >= 0) {
 #pragma unroll
-                for (int j4 = 0; j4 < 32; j4 += 4) {
-                    float x[4];
+                    for (int j4 = 0; j4 < 32; j4 += 4) {
+                        float x[4];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int j = c0 + j4 + e;
-                        x[e] = (j < i) ? bi * __uint_as_float(r[j4 + e]) : 0.f;
+                        for (int e = 0; e < 4; ++e) x[e] = j4 + e < lim ? bi * __uint_as_float(r[j4 + e]) : 0.f;
+                        *reinterpret_cast<float4*>(sA + i * LDT + c0 + j4) = make_float4(x[0], x[1], x[2], x[3]);
                     }
-                    *reinterpret_cast<float4*>(sA + i * LDT + c0 + j4) = make_float4(x[0], x[1], x[2], x[3]);
                 }
             } else if (has_q) {
-                const int i = Rr - 64;
+                const int i = Rr - 64, lim = where > 0 ? 32 : where < 0 ? -1 : lane;
 #pragma unroll
                 for (int j8 = 0; j8 < 32; j8 += 8) {
                     float x[8];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int j = c0 + j8 + e;
-                        x[e] = (j <= i) ? __uint_as_float(r[j8 + e]) : 0.f;
-                    }
+                    for (int e = 0; e < 8; ++e) x[e] = j8 + e <= lim ? __uint_as_float(r[j8 + e]) : 0.f;
                     *reinterpret_cast<uint4*>(smem + E_AQ + ptx::sw128_off(i, c0 + j8)) =
                         make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]),
                                    pack_bf16(x[6], x[7]));
@@ -835,7 +844,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
 
         // ---- a4: Mm = T Diag(beta) as the A operand; [W | U] = Mm [Kg | V] ---------------------------------
         {
-            const int i = te >> 2, J = te & 3, I = i >> 4;   // one 16-column block of one row per thread
+            const int i = te & 63, J = te >> 6, I = i >> 4;   // one 16-column block of one row per thread
             const int j0 = J * 16;
             float x[16];
             if (J > I) {
@@ -847,7 +856,8 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
                 for (int e4 = 0; e4 < 16; e4 += 4) {
                     const float4 tv = *reinterpret_cast<const float4*>(src + e4);
                     const float4 bv = *reinterpret_cast<const float4*>(sBeta + j0 + e4);
-                    x[e4] = tv.x * bv.x; x[e4 + 1] = tv.y * bv.y; x[e4 + 2] = tv.z * bv.z; x[e4 + 3] = tv.w * bv.w;
+                    set(x + e4, __fmul2_rn(make_float2(tv.x, tv.y), make_float2(bv.x, bv.y)));
+                    set(x + e4 + 2, __fmul2_rn(make_float2(tv.z, tv.w), make_float2(bv.z, bv.w)));
                 }
             }
 #pragma unroll
@@ -898,10 +908,10 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
                 const float4 e0 = *reinterpret_cast<const float4*>(smem + E_EM + (col0 + j8) * 4);
                 const float4 e1 = *reinterpret_cast<const float4*>(smem + E_EM + (col0 + j8) * 4 + 16);
                 *reinterpret_cast<uint4*>(smem + E_V + (col0 >> 6) * 8192 + ptx::sw128_off(i, (col0 & 63) + j8)) =
-                    make_uint4(pack_bf16(__uint_as_float(r[j8]) * e0.x, __uint_as_float(r[j8 + 1]) * e0.y),
-                               pack_bf16(__uint_as_float(r[j8 + 2]) * e0.z, __uint_as_float(r[j8 + 3]) * e0.w),
-                               pack_bf16(__uint_as_float(r[j8 + 4]) * e1.x, __uint_as_float(r[j8 + 5]) * e1.y),
-                               pack_bf16(__uint_as_float(r[j8 + 6]) * e1.z, __uint_as_float(r[j8 + 7]) * e1.w));
+                    make_uint4(pack_bf16(__fmul2_rn(make_float2(__uint_as_float(r[j8]), __uint_as_float(r[j8 + 1])), make_float2(e0.x, e0.y))),
+                               pack_bf16(__fmul2_rn(make_float2(__uint_as_float(r[j8 + 2]), __uint_as_float(r[j8 + 3])), make_float2(e0.z, e0.w))),
+                               pack_bf16(__fmul2_rn(make_float2(__uint_as_float(r[j8 + 4]), __uint_as_float(r[j8 + 5])), make_float2(e1.x, e1.y))),
+                               pack_bf16(__fmul2_rn(make_float2(__uint_as_float(r[j8 + 6]), __uint_as_float(r[j8 + 7])), make_float2(e1.z, e1.w))));
             }
             ptx::tmem_ld_32x32b_x32(tq + 128 + g * 32, r);
             ptx::tmem_ld_wait();
