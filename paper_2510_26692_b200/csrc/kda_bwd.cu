@@ -17,6 +17,7 @@
 // shared memory (8 decayed states of this slice, 128 KB) and runs the adjoint through it.  All
 // arithmetic is fp32 FMA; q, k, v, d_o may be stored as bf16.
 #include "kda_bwd.cuh"
+#include "kda_ptx.cuh"
 
 namespace kda {
 namespace {
@@ -102,6 +103,8 @@ __global__ void __launch_bounds__(kThreads, 1) kda_bwd_sweep(BwdArgs a)
     extern __shared__ __align__(16) float sm[];
     const int t = threadIdx.x, lane = t & 31, rg = t >> 5;
     const int slice = blockIdx.x, h = blockIdx.y, n = blockIdx.z;
+    ptx::grid_dep_wait();      // (launched before the preceding kernel has ended)
+    ptx::grid_dep_launch();
     if (!a.seq_heads[h]) return;
     const int col = slice * NS + lane;
     const int i0 = rg * kRows;                 // first of this thread's rows
@@ -272,6 +275,8 @@ __global__ void kda_bwd_reduce(const float* __restrict__ part_q, const float* __
                                float* __restrict__ dbeta, size_t n_vec, size_t n_tok,
                                const int* __restrict__ seq_heads, int H)
 {
+    ptx::grid_dep_wait();      // (launched before the preceding kernel has ended)
+    ptx::grid_dep_launch();
     int any = 0;
     for (int h = threadIdx.x; h < H; h += blockDim.x) any |= seq_heads[h];
     if (!__syncthreads_or(any)) return;
@@ -429,18 +434,15 @@ kda_status_t kda_chunk_bwd(const void* q, const void* k, const void* v, const fl
     if (total_tokens > 0 || dS0) {
         dim3 grid(kSlices, (unsigned)H, (unsigned)n_seqs);
         ProfScope ps(PROF_INTER, st);
-        if (dt == KDA_BF16) kda_bwd_sweep<__nv_bfloat16><<<grid, kThreads, kSweepSmem, st>>>(a);
-        else kda_bwd_sweep<float><<<grid, kThreads, kSweepSmem, st>>>(a);
+        KDA_CUDA_TRY(launch_dependent(dt == KDA_BF16 ? kda_bwd_sweep<__nv_bfloat16> : kda_bwd_sweep<float>, grid, kThreads, kSweepSmem, st, a));
         count_launch();
-        KDA_CUDA_TRY(cudaGetLastError());
     }
     if (total_tokens > 0) {
         const size_t n_vec = (size_t)total_tokens * H * kD, n_tok = (size_t)total_tokens * H;
         ProfScope ps(PROF_INTRA, st);
-        kda_bwd_reduce<<<1184, 256, 0, st>>>(a.part_q, a.part_k, a.part_g, a.part_b, dq, dk_out, dlog_alpha,
-                                             dbeta, n_vec, n_tok, a.seq_heads, H);
+        KDA_CUDA_TRY(launch_dependent(kda_bwd_reduce, dim3(1184), 256, 0, st, (const float*)a.part_q, (const float*)a.part_k, (const float*)a.part_g,
+                                      (const float*)a.part_b, dq, dk_out, dlog_alpha, dbeta, n_vec, n_tok, (const int*)a.seq_heads, H));
         count_launch();
-        KDA_CUDA_TRY(cudaGetLastError());
     }
     return KDA_OK;
 }

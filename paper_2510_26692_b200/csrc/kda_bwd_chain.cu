@@ -269,6 +269,7 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
             __syncwarp();
         }
     }
+    ptx::grid_dep_launch();
     __syncthreads();
     if (t == 0 && *abort_word && atomicCAS(&a.hdr->status, 0, (int)KDA_ERR_TIMEOUT) == 0) a.hdr->where = 32;
     if (w == 0) ptx::tmem_dealloc(tm, 512);
@@ -278,6 +279,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_chain(BwdChunkArgs a)
 {
     extern __shared__ __align__(1024) uint8_t sm[];
     const int h = blockIdx.y, n = blockIdx.z;
+    ptx::grid_dep_wait();      // (launched before the preceding kernel has ended)
     if (a.seq_heads[h]) return;
     if ((ptx::smem_u32(sm) & 1023u) != 0) {
         if (threadIdx.x == 0 && atomicCAS(&a.hdr->status, 0, (int)KDA_ERR_TIMEOUT) == 0) a.hdr->where = 33;
@@ -300,9 +302,8 @@ kda_status_t launch_bwd_chain(const BwdChunkArgs& a, cudaStream_t st)
         }
     }
     ProfScope ps(PROF_INTER, st);
-    kda_bwd_chain<<<dim3(2, (unsigned)a.H, (unsigned)a.n_seqs), kT, kSmem, st>>>(a);
+    KDA_CUDA_TRY(launch_dependent(kda_bwd_chain, dim3(2, (unsigned)a.H, (unsigned)a.n_seqs), kT, kSmem, st, a));
     count_launch();
-    KDA_CUDA_TRY(cudaGetLastError());
     return KDA_OK;
 }
 

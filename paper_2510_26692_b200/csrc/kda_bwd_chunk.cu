@@ -18,6 +18,7 @@
 // whose log decay leaves [-kBwdRange, 1], or with a token that is not finite, is left to the token-sequential kernels
 // (kda_bwd.cu).
 #include "kda_bwd.cuh"
+#include "kda_ptx.cuh"
 
 namespace kda {
 namespace {
@@ -26,6 +27,8 @@ namespace {
 __global__ void kda_bwd_prep(WsHeader* hdr, const int32_t* __restrict__ cu, int32_t* __restrict__ chunk_cu, int n_seqs,
                              int* __restrict__ seq_heads, int H)
 {
+    ptx::grid_dep_wait();      // (launched before the preceding kernel has ended)
+    ptx::grid_dep_launch();
     for (int h = threadIdx.x; h < H; h += blockDim.x) seq_heads[h] = 0;
     if (threadIdx.x == 0) {
         hdr->status = 0; hdr->where = 0; hdr->flags = 0;
@@ -54,9 +57,8 @@ kda_status_t launch_bwd_chunk(BwdChunkArgs a, kda_dtype_t dt, int32_t* chunk_cu_
         }
         a.n_sm = lk.st->n_sm;
     }
-    kda_bwd_prep<<<1, 256, 0, st>>>(a.hdr, a.cu_seqlens, chunk_cu_dev, a.n_seqs, a.seq_heads, a.H);
+    KDA_CUDA_TRY(launch_dependent(kda_bwd_prep, dim3(1), 256, 0, st, a.hdr, a.cu_seqlens, chunk_cu_dev, a.n_seqs, a.seq_heads, a.H));
     count_launch();
-    KDA_CUDA_TRY(cudaGetLastError());
     kda_status_t rc = a.n_chunks > 0 ? launch_bwd_intra(a, dt, st) : KDA_OK;
     if (rc == KDA_OK) rc = launch_bwd_chain(a, st);
     if (rc == KDA_OK && a.n_chunks > 0) rc = launch_bwd_out(a, dt, st);

@@ -42,6 +42,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
     uint64_t* bar = reinterpret_cast<uint64_t*>(vec + V_BAR);   // one per group of MMAs, a phase per tile
     uint32_t* slot = reinterpret_cast<uint32_t*>(bar + 4);
 
+    ptx::grid_dep_wait();      // (launched before the preceding kernel has ended)
     // bf16 rows: a CTA per SM goes through the tiles, and the inputs of the next wait in registers while the tensor core
     // works on the last products of this one (4096 x 32 heads 285 -> 271 us).  fp32 rows take twice the registers, and
     // spilled (67 -> 77 us on six packed sequences): a CTA per tile.
@@ -328,6 +329,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
         phase ^= 1u;
         if (!kLoop || id >= n_tiles) break;
     }
+    ptx::grid_dep_launch();
     if (t == kCopy) ptx::bulk_wait_all0();
     if (!ok && atomicCAS(&a.hdr->status, 0, (int)KDA_ERR_TIMEOUT) == 0) a.hdr->where = 31;
     ptx::tc_fence_before();
@@ -350,10 +352,10 @@ kda_status_t launch_bwd_intra(const BwdChunkArgs& a, kda_dtype_t dt, cudaStream_
     }
     const unsigned tiles = (unsigned)(a.n_chunks * a.H);
     ProfScope ps(PROF_INTRA, st);
-    if (dt == KDA_BF16) kda_bwd_intra<__nv_bfloat16><<<tiles < (unsigned)a.n_sm ? tiles : (unsigned)a.n_sm, kT, kSmem, st>>>(a);
-    else kda_bwd_intra<float><<<tiles, kT, kSmem, st>>>(a);
+    const unsigned loop = tiles < (unsigned)a.n_sm ? tiles : (unsigned)a.n_sm;
+    if (dt == KDA_BF16) KDA_CUDA_TRY(launch_dependent(kda_bwd_intra<__nv_bfloat16>, dim3(loop), kT, kSmem, st, a));
+    else KDA_CUDA_TRY(launch_dependent(kda_bwd_intra<float>, dim3(tiles), kT, kSmem, st, a));
     count_launch();
-    KDA_CUDA_TRY(cudaGetLastError());
     return KDA_OK;
 }
 

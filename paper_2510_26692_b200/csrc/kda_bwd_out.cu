@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         __syncwarp();
         ptx::tc_fence_after();
     };
+    ptx::grid_dep_wait();      // (launched before the preceding kernel has ended)
     // tiles of this CTA: id, id + gridDim.x, ... without those of heads that are not in chunk form
     uint32_t id = blockIdx.x;      // (fewer than 2^31 tiles)
     int h = 0;
@@ -440,6 +441,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
         }
         phase ^= 1u;
     }
+    ptx::grid_dep_launch();
     if (!ok && atomicCAS(&a.hdr->status, 0, (int)KDA_ERR_TIMEOUT) == 0) a.hdr->where = 30;
     ptx::tc_fence_before();
     __syncthreads();
@@ -461,10 +463,8 @@ kda_status_t launch_bwd_out(const BwdChunkArgs& a, kda_dtype_t dt, cudaStream_t 
     const int64_t tiles = a.n_chunks * a.H;
     const unsigned grid = (unsigned)(tiles < a.n_sm ? tiles : a.n_sm);
     ProfScope ps(PROF_INTRA, st);
-    if (dt == KDA_BF16) kda_bwd_out<__nv_bfloat16><<<grid, kT, kSmem, st>>>(a);
-    else kda_bwd_out<float><<<grid, kT, kSmem, st>>>(a);
+    KDA_CUDA_TRY(launch_dependent(dt == KDA_BF16 ? kda_bwd_out<__nv_bfloat16> : kda_bwd_out<float>, dim3(grid), kT, kSmem, st, a));
     count_launch();
-    KDA_CUDA_TRY(cudaGetLastError());
     return KDA_OK;
 }
 

@@ -391,23 +391,6 @@ __global__ void kda_prep_kernel(WsHeader* hdr, const int32_t* __restrict__ cu,
     }
 }
 
-// launched as the predecessor's programmatic dependent: the launch overlaps its end
-template <typename... P, typename... A>
-cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 }  // namespace
 
 size_t f32_tile_bytes() { return (size_t)T_FLOATS * sizeof(float); }

@@ -177,6 +177,23 @@ __device__ __forceinline__ LogSum operator-(LogSum a, LogSum b) {
 }
 __device__ __forceinline__ float exp_of(LogSum x) { const float e = expf(x.hi); return fmaf(e, x.lo, e); }
 
+// launched as the predecessor's programmatic dependent: the launch overlaps its end
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // ---- launchers implemented by the kernel translation units --------------------------------------
 kda_status_t launch_decode(const void* q, const void* k, const void* v, const float* log_alpha,
                            const float* beta, float* S, const int32_t* slot, void* o, int n_seqs,
