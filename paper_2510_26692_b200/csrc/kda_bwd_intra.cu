@@ -9,7 +9,7 @@
 // in bf16 are operands as they are.  Shared memory: RQ 96 KB [K^ ; Q], later the W'^T image; RK 48 KB K_, then V;
 // L, T' fp32; RP 24 KB P, then T'; dO in a place of its own (bf16) or in RK before V.
 //
-// T=4096, H=32: 470 us with warp-level tf32 products; with all operands split and 64-row products on 128 rows 271; 230
+// T=4096, H=32: 470 us with warp-level tf32 products; with all operands split and 64-row products on 128 rows 271; 223
 // in this form.
 #include "kda_bwd.cuh"
 #include "kda_mma3.cuh"
@@ -43,8 +43,8 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
     uint32_t* slot = reinterpret_cast<uint32_t*>(bar + 4);
 
     ptx::grid_dep_wait();      // (launched before the preceding kernel has ended)
-    // bf16 rows: a CTA per SM goes through the tiles, and the inputs of the next wait in registers while the tensor core
-    // works on the last products of this one (4096 x 32 heads 285 -> 271 us).  fp32 rows take twice the registers, and
+    // bf16 rows: a CTA per SM goes through the tiles, and the inputs of the next are requested as soon as
+    // their registers are free (4096 x 32 heads 285 -> 271 us; all of them during the last products: 230, now 223).  fp32 rows take twice the registers, and
     // spilled (67 -> 77 us on six packed sequences): a CTA per tile.
     constexpr bool kExact = sizeof(T) == 2, kLoop = kExact;
     const int64_t n_tiles = a.n_chunks * a.H;
@@ -77,11 +77,15 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
             ldraw(kr[j], static_cast<const T*>(a.k) + off, in);
             ldraw(qr[j], static_cast<const T*>(a.q) + off, in);
             ldraw(dr[j], static_cast<const T*>(a.d_o) + off, in && a.d_o);
-            ldraw(vr[j], static_cast<const T*>(a.v) + off, in);
         }
+    };
+    auto request_v = [&]() {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) ldraw(vr[j], static_cast<const T*>(a.v) + tok_off(row0 + 32 * j) + c8, row0 + 32 * j < loc.len);
     };
     request();
     request_rows();
+    request_v();
     if (w == 0) {
         ptx::tmem_alloc(slot, 512);
         ptx::tmem_relinquish();
@@ -176,6 +180,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
             if (!kLoop || id >= n_tiles) break;
             request();
             request_rows();
+            request_v();
             continue;
         }
         {
@@ -207,6 +212,11 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
         if (t == kCopy) {
             ptx::bulk_s2g(tile + bt::KI, sm + O_RK, 49152);
             ptx::bulk_commit();
+        }
+        id += gridDim.x;
+        if (kLoop && id < n_tiles) {       // (all but V of this tile has been read from the registers)
+            request();
+            request_rows();
         }
         float* sL = reinterpret_cast<float*>(sm + O_L);
         float* sT = reinterpret_cast<float*>(sm + O_T);
@@ -288,11 +298,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
             mma6<4, kExact>(tm + C_U, mn_major<64, 2>(sm + O_RK), k_major<64, 1>(sm + O_RP), idesc, false);
             ptx::umma_commit(&bar[3]);
         }
-        id += gridDim.x;
-        if (kLoop && id < n_tiles) {
-            request();
-            request_rows();
-        }
+        if (kLoop && id < n_tiles) request_v();
         // accumulators out: this thread's row, 16 columns from cg (of N also 64 + cg)
         const int row = quad * 32 + lane, cg = (w >> 2) * 16;
         auto store_rf = [&](uint32_t col, float* m, int c0) {
