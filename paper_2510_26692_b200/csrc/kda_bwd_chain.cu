@@ -29,7 +29,7 @@ constexpr int kT = 640, kCompute = 512;
 constexpr int kRegs = 112, kRegsRest = 32;      // of a compute thread and of the others: 512 x 112 + 128 x 32 <= 640 x 96
 constexpr uint32_t kImg = 49152, kStateBytes = bt::kState * 4, kVecBytes = bt::kVec * 4;
 constexpr uint32_t O_A = 0, O_B = kImg, O_ST = 2 * kImg, O_N = O_ST + kStateBytes, O_VEC = O_N + kStateBytes, O_BAR = O_VEC + 2 * kVecBytes;
-constexpr uint32_t kSmem = O_BAR + 160;      // (the images need 1024-byte alignment, and there is no room to align)
+constexpr uint32_t kSmem = O_BAR + 192;      // (the images need 1024-byte alignment, and there is no room to align)
 static_assert(kSmem <= 232448, "fits the shared memory of one SM");
 static_assert(kVecBytes % 16 == 0 && kStateBytes % 16 == 0 && O_BAR % 8 == 0, "bulk copies and barriers are aligned");
 // TMEM columns: the operands (three splits each) and the two products
@@ -46,9 +46,9 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
     uint64_t* m2 = m1 + 1;               // second
     uint64_t* freed = m2 + 1;            // the state has been read out of the staging buffer
     uint64_t* done = freed + 1;          // all MMAs complete
-    uint64_t* s_ready = done + 1;        // 16 warps: state operand written
-    uint64_t* x_ready = s_ready + 1;     // 16 warps: beta r or -beta dX written
-    uint64_t* staged = x_ready + 1;      // 16 warps: state written to the staging buffer
+    uint64_t* s_ready = done + 1;        // [3] 16 warps: a split of the state operand written
+    uint64_t* x_ready = s_ready + 3;     // [3] 16 warps: of beta r or -beta dX
+    uint64_t* staged = x_ready + 3;      // 16 warps: state written to the staging buffer
     uint64_t* n_read = staged + 1;       // 16 warps: N read
     volatile uint32_t* abort_word = reinterpret_cast<volatile uint32_t*>(n_read + 1);
     uint32_t* slot = const_cast<uint32_t*>(abort_word) + 1;
@@ -115,8 +115,7 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
                 x[2 * e] = __fmul2_rn(lo(m), S[2 * e]);
                 x[2 * e + 1] = __fmul2_rn(hi(m), S[2 * e + 1]);
             }
-            put_tmem<kSParts>(tq + C_S + part * 16, x);
-            arrive(s_ready);
+            put_tmem<kSParts>(tq + C_S + part * 16, x, [&](int s) { arrive(&s_ready[s]); });
         };
         if (nc > 0) put_state(0);
         for (int64_t i = 0; i < nc; ++i) {
@@ -153,8 +152,7 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
                     z[e] = __fmul2_rn(lo(b), x[e]);
                     z[e + 1] = __fmul2_rn(hi(b), x[e + 1]);
                 }
-                put_tmem<kXParts>(tq + C_X + part * 8, z);
-                arrive(x_ready);
+                put_tmem<kXParts>(tq + C_X + part * 8, z, [&](int s) { arrive(&x_ready[s]); });
 #pragma unroll
                 for (int e = 0; e < 16; e += 4)
                     *reinterpret_cast<float4*>(ux + e * 128) = make_float4(x[e / 2].x, x[e / 2].y, x[e / 2 + 1].x, x[e / 2 + 1].y);
@@ -250,17 +248,21 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
             }
         } else if (w == kCompute / 32) {
             const uint32_t id64 = ptx::umma_idesc_bf16(128, 64), id128 = ptx::umma_idesc_bf16(128, 128), mnB = ptx::kIdescBMajorMN;
-            for (int64_t i = 0; i < nc; ++i) {
-                if (!wait(fullA, i) || !wait(s_ready, i)) break;
-                __syncwarp();
-                ptx::tc_fence_after();
-                const uint8_t* img = sm + O_A;
-                mma6_ta<8, kSParts>(tm + C_1, tm + C_S, kFwd ? mn_major<128, 1>(img) : k_major<64, 2>(img), kFwd ? id64 | mnB : id64, false);
+            bool go = true;
+            for (int64_t i = 0; i < nc && go; ++i) {
+                // the products with the first splits of an operand run while the others are written
+                auto operand = [&](uint64_t* ready) {
+                    return [&, ready](int s) {
+                        if (!wait(&ready[s], i)) go = false;
+                        __syncwarp();
+                        ptx::tc_fence_after();
+                    };
+                };
+                if (!wait(fullA, i)) break;
+                mma6_ta<8, kSParts>(tm + C_1, tm + C_S, kFwd ? mn_major<128, 1>(sm + O_A) : k_major<64, 2>(sm + O_A), kFwd ? id64 | mnB : id64, false, operand(s_ready));
                 ptx::umma_commit(m1);
-                if (!wait(fullB, i) || !wait(x_ready, i)) break;
-                __syncwarp();
-                ptx::tc_fence_after();
-                mma6_ta<4, kXParts>(tm + C_3, tm + C_X, kFwd ? mn_major<64, 2>(sm + O_B) : k_major<128, 1>(sm + O_B), kFwd ? id128 | mnB : id128, false);
+                if (!go || !wait(fullB, i)) break;
+                mma6_ta<4, kXParts>(tm + C_3, tm + C_X, kFwd ? mn_major<64, 2>(sm + O_B) : k_major<128, 1>(sm + O_B), kFwd ? id128 | mnB : id128, false, operand(x_ready));
                 ptx::umma_commit(m2);
             }
             __syncwarp();

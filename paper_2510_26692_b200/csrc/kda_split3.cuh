@@ -47,8 +47,9 @@ __device__ __forceinline__ void put8(uint8_t* img, int row, int col, const float
 }
 // Splits 16 or 32 consecutive columns of this lane's row into the A operand in TMEM (two bf16 values a column, kParts columns
 // from one split to the next): no pass over shared memory, and the product reads only its B operand there.
-template <int kParts, int N>
-__device__ __forceinline__ void put_tmem(uint32_t taddr, const float2 (&x)[N]) {
+// `written(s)` is called behind the store of split s.
+template <int kParts, int N, typename F>
+__device__ __forceinline__ void put_tmem(uint32_t taddr, const float2 (&x)[N], F written) {
     static_assert(N == 8 || N == 16, "a tcgen05.st of 8 or 16 columns");
     float2 r[N];
 #pragma unroll
@@ -60,7 +61,12 @@ __device__ __forceinline__ void put_tmem(uint32_t taddr, const float2 (&x)[N]) {
         for (int e = 0; e < N; ++e) w[e] = s < 2 ? take2(r[e]) : pack2(r[e].x, r[e].y);
         if constexpr (N == 16) ptx::tmem_st_32x32b_x16(taddr + s * kParts, w);
         else ptx::tmem_st_32x32b_x8(taddr + s * kParts, w);
+        written(s);
     }
+}
+template <int kParts, int N>
+__device__ __forceinline__ void put_tmem(uint32_t taddr, const float2 (&x)[N]) {
+    put_tmem<kParts>(taddr, x, [](int) {});
 }
 
 // One operand of a product: descriptor of split 0 at K = 0, and the distances between splits and of 16 in K
@@ -100,22 +106,33 @@ __device__ __forceinline__ void mma6(uint32_t d_tmem, const Operand& A, const Op
     }
 }
 
-// the same with A in TMEM (put_tmem)
+// one of the six with A in TMEM (put_tmem): split sa of A, split sb of B
 template <int KS, int kParts>
-__device__ __forceinline__ void mma6_ta(uint32_t d_tmem, uint32_t a_tmem, const Operand& B, uint32_t idesc, bool accumulate) {
+__device__ __forceinline__ void mma_ta(uint32_t d_tmem, uint32_t a_tmem, const Operand& B, uint32_t idesc, uint32_t sa, uint32_t sb, bool accumulate) {
     uint32_t acc = accumulate ? 1u : 0u;
+    const uint32_t ta = a_tmem + sa * kParts;
+    const uint64_t db = B.desc + sb * B.split;
+#pragma unroll
+    for (int k = 0; k < KS; ++k) {
+        const uint32_t ob = B.k16 == 2u ? (uint32_t)(k >> 2) * B.khalf + (k & 3) * 2u : (uint32_t)k * B.k16;
+        ptx::umma_bf16_ta(d_tmem, ta + k * 8, db + ob, idesc, acc);
+        acc = 1u;
+    }
+}
+// all six, those with the splits of A that are written first at the start: (0,2) (1,1) (2,0) (1,0) (0,1) (0,0); `ready(s)`
+// comes before the first that needs split s
+template <int KS, int kParts, typename F>
+__device__ __forceinline__ void mma6_ta(uint32_t d_tmem, uint32_t a_tmem, const Operand& B, uint32_t idesc, bool accumulate, F ready) {
 #pragma unroll 1
     for (int p = 0; p < 6; ++p) {
-        const uint32_t sa = p == 0 ? 2u : (p == 2 || p == 3) ? 1u : 0u, sb = p == 1 ? 2u : (p == 2 || p == 4) ? 1u : 0u;
-        const uint32_t ta = a_tmem + sa * kParts;
-        const uint64_t db = B.desc + sb * B.split;
-#pragma unroll
-        for (int k = 0; k < KS; ++k) {
-            const uint32_t ob = B.k16 == 2u ? (uint32_t)(k >> 2) * B.khalf + (k & 3) * 2u : (uint32_t)k * B.k16;
-            ptx::umma_bf16_ta(d_tmem, ta + k * 8, db + ob, idesc, acc);
-            acc = 1u;
-        }
+        if (p < 3) ready(p);
+        const uint32_t sa = p < 3 ? p : p == 3 ? 1u : 0u, sb = p < 3 ? 2u - p : p == 4 ? 1u : 0u;
+        mma_ta<KS, kParts>(d_tmem, a_tmem, B, idesc, sa, sb, accumulate || p > 0);
     }
+}
+template <int KS, int kParts>
+__device__ __forceinline__ void mma6_ta(uint32_t d_tmem, uint32_t a_tmem, const Operand& B, uint32_t idesc, bool accumulate) {
+    mma6_ta<KS, kParts>(d_tmem, a_tmem, B, idesc, accumulate, [](int) {});
 }
 
 }  // namespace split3
