@@ -148,3 +148,19 @@ def test_backward_chains_of_every_length(oracle_mod):
     for _ in range(10):
         out = run_bwd(d, d_o, dS_T)
         assert all(torch.equal(out[n], first[n]) for n in NAMES)
+
+
+@pytest.mark.parametrize("lens,H,dtype,harsh", [([9477, 0, 3], 1, torch.bfloat16, None), ([2117, 0, 1, 400], 7, torch.bfloat16, 3),
+                                                ([1500, 700], 9, torch.bfloat16, 0), ([1500, 700], 9, torch.float32, 8)])
+def test_backward_several_tiles_per_cta(oracle_mod, lens, H, dtype, harsh):
+    """More tiles than multiprocessors (150, 294, 315): CTAs go through several, ragged and short ones among them, past the
+    tiles of a head that leaves the chunk form in its last chunk, and the last round is not full."""
+    d = inputs.chunk_inputs(lens, H=H, dtype=dtype, seed=35, s0_std=0.02)
+    if harsh is not None:
+        d["log_alpha"][-1, harsh, 5] = -45.0
+    d_o, dS_T = cotangents(d, 35, dtype)
+    out, ref = run_bwd(d, d_o, dS_T), oracle_bwd(oracle_mod, d, d_o, dS_T)
+    for n in NAMES:
+        assert rel_l2(to_np32(out[n]), ref[n]) <= 1e-5, n
+    again = run_bwd(d, d_o, dS_T)
+    assert all(torch.equal(out[n], again[n]) for n in NAMES)
