@@ -317,8 +317,8 @@ struct LayerMode {
 // Into how many segments the chains of a bf16 call are cut (kda_segments.cu), 1 = none.  All runs of a stage must
 // be resident at once.  Times in us, measured: a chain step 1.62 in the fused kernel, 1.4 (maps) and 1.5 (outputs) with all SMs
 // at it, a tile of the intra-chunk kernel 8 over two CTAs per SM, launches 22 and a border 1.5.
-// Prefill, 8 heads x 4096 tokens 101 -> 72 us, 8 x 30000: 627 -> 256, 16 x 131072: 2720 -> 1830; 16 x 65536 for the
-// final state 1246 -> 656.  Modes 1 and 2 of kda_set_chunk_path never cut.
+// Prefill, whole / cut: 8 heads x 4096 tokens 89 -> 62 us, 8 x 30000: 604 -> 252, 16 x 65536: 1367 -> 939, for the final
+// state 1270 -> 658.  Modes 1 and 2 of kda_set_chunk_path never cut.
 // Below 48 chunks it gains at most a tenth, and a short sequence keeps the same bits however it is handed over.
 int segments(int64_t J, int64_t longest, int64_t tiles, bool out, bool layer, int n_sm)
 {
@@ -350,10 +350,11 @@ kda_status_t fused_schedule(FusedArgs& f, const std::vector<int64_t>& chunk_cu, 
 // Whether a bf16 call without the layer's functions runs as the fused kernel (kda_set_chunk_path): always where the
 // tiles of all chunks do not fit the workspace, else by the time of both in us.  Fused: 17, and per tile of the most
 // loaded cluster 1.62 with one chain to a cluster; with several 1.5 where the others idle beside a few long chains, up
-// to 1.9 where all are loaded alike.  Two kernels: a tile 8 with two per SM, a chain step 1.4, 8 for the launches.
-// Measured, fused / two: 32 heads x 1000 tokens 44 / 44, x 1500 58 / 64, x 4096 121 / 148; 16 x 2000 64 / 62;
-// 37 x 900 48 / 43; 8 heads, 7 sequences of 813 .. 5057 tokens 144 / 184, one of 4000 and six of 600 111 / 121, of
-// 100 .. 12000 296 / 345; 32 heads, 2 x 2048 124 / 113; 16 heads, 7 of 500 .. 10000 481 / 432.  Layer calls: never faster.
+// to 1.9 where all are loaded alike.  Two kernels: a tile 8 with two per SM, a chain step 1.4, 8 for the launches
+// (all of them 5 to 8 per cent less by now, alike on both sides, and shorter steps where few chains run: their ratio decides).
+// Measured, fused / two: 32 heads x 1000 tokens 40 / 40, x 1500 54 / 59, x 4096 113 / 135; 16 x 2000 60 / 56;
+// 37 x 900 45 / 41; 8 heads, 7 sequences, 19620 tokens, the longest 4679: 148 / 161, 31108 and 6677: 223 / 235; 3 of up to
+// 16632: 370 / 423; 32 heads, 2 x 2048 117 / 109; 16 heads, 7 of up to 9948 441 / 426, 8 of up to 2735 224 / 201.  Layer calls: never faster.
 kda_status_t use_fused(FusedArgs& f, const std::vector<int64_t>& chunk_cu, const void* workspace, size_t bytes, bool has_q, bool* fused)
 {
     const int mode = g_chunk_path.load(std::memory_order_relaxed);

@@ -18,12 +18,13 @@
 //     a4   Mm = T Diag(beta) (bf16);  second MMA group  [Mm ; Mm] x [Kg | V]  ->  W' = Mm Kg, U = Mm V
 //   The tile (operand images of kda_tiles.cuh) goes to global memory; in the fused kernel to a ring of a few tiles per
 //   engine that stays in L2.
-//   Two kernels: 8.1 us a tile with two in flight per SM, where reading its inputs and writing it takes 7.2 at the copy
-//   bandwidth.  Fused (3.8 without the write): the chain of its phases, of which shared memory lets no third one overlap.
+//   Two kernels: 7.7 us a tile with two in flight per SM, where reading its inputs and writing it takes 7.2 at the copy
+//   bandwidth.  Fused 9 (without outputs 7.5): the chain of its phases, of which shared memory lets no third one overlap, and
+//   the shared memory itself.
 //
 //   inter-chunk chain (a CTA; roles and products: see chain_run): all 128 columns of the state of one (sequence,
-//   head), walked over the chunks in order -- a6 V_new = U - W S, a8 the state, a7 the outputs.  1.23 us a step for
-//   the final state alone, 1.33 with outputs: two dependent round trips tensor core - registers - tensor core.
+//   head), walked over the chunks in order -- a6 V_new = U - W S, a8 the state, a7 the outputs.  1.02 us a step for
+//   the final state alone, 1.2 with outputs: two dependent round trips tensor core - registers - tensor core.
 //   Tiles arrive by 1-D bulk copies (TMA engine).
 //
 // Every wait (mbarrier, flag word) is bounded by a wall-clock limit; when one runs out the role
@@ -107,7 +108,7 @@ constexpr uint32_t kSmemBytes = 2 * E_BYTES > C_BYTES ? 2 * E_BYTES : C_BYTES;
 static_assert(E_BYTES % 1024 == 0, "operand images stay 1024-byte aligned");
 static_assert(kSmemBytes <= 232448, "fits the shared memory of one SM");
 // Registers of the chain kernel's compute warps: the fp32 state takes 64 of them, an accumulator another 32 (at 128, the
-// share of each of 512 threads, some spilled: 1.33 instead of 1.25 us a step).  The other half of the warps gives up as many.
+// share of each of 512 threads, some spilled: 1.33 instead of 1.25 us a step then).  The other half of the warps gives up as many.
 constexpr int kChainRegs = 160;
 constexpr uint32_t kTmemCols = 512;                // two engines of 256 columns, or one chain
 // TMEM columns of a chain: D1 of two chunks, D3, the bf16 state and V_new (A operands, two values a column)
@@ -1370,8 +1371,8 @@ __device__ void chain_init(uint8_t* smem, int ring)
 // announces a tile once its copies have completed, the chain gives a position back once its copy has landed; both
 // by release arrivals, taken up by acquire waits and a proxy fence before the next bulk copy.  The arrivals are made where
 // nothing waits for the thread, during the substitution and by a warp of their own: 4096 x 32 heads 120.7 us, 1 Mi tokens
-// for the state 20.6 ms (made by the loader, and by the service thread ahead of its copies: 141 us and 28.9 ms; relaxed,
-// which orders nothing: 112.5 and 20.2).
+// for the state 20.6 ms, 113 and 20.35 now (made by the loader, and by the service thread ahead of its copies, then: 141 us and
+// 28.9 ms; relaxed, which orders nothing: 112.5 and 20.2).
 template <bool kHasQ>
 __global__ void __launch_bounds__(kThreads, 1)
 kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtensorMap tm_k,
