@@ -37,11 +37,11 @@ STATE_BYTES = 2 * D * D * 4
 DEC_BYTES_PER_STATE = 2 * D * D * 4 + 4 * D * 2 + D * 4 + 4
 FLOPS_PER_TOKEN_HEAD = 6 * D * D + 3 * CHUNK * D + CHUNK * CHUNK   # the paper's FLOPs model
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised under
-# profiles/ (prefill, which runs as the fused kernel: 171.8 + 106.7 MB;
+# profiles/ (prefill, which runs as the fused kernel: 173.1 + 106.5 MB;
 # decode: 547.4 + 484.7 MB)
-PREFILL_DRAM_TRAFFIC = {"fused": 278.6e6}
+PREFILL_DRAM_TRAFFIC = {"fused": 279.7e6}
 DECODE_DRAM_TRAFFIC = 1032.1e6
-FUSED_DRAM_TRAFFIC = 278.6e6
+FUSED_DRAM_TRAFFIC = 279.7e6
 TRAFFIC_SOURCE = "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch, copied from the summaries under profiles/ (not measured in this run)"
 MIN_TIMED_S = 0.5      # the timed region is extended (whole blocks of `steps` calls) to at least this
 MAX_BLOCKS = 2000
