@@ -80,9 +80,8 @@ __device__ __forceinline__ BwdLoc bwd_locate(const BwdChunkArgs& a, int64_t g) {
 }
 
 // The per-chunk kernels hold one CTA per SM whose loads, products and stores take turns, so HBM idles while
-// the tensor core works and the other way round.  Each CTA therefore asks for what the CTA n_sm places
-// further on will read (likely the next on its SM) to come into L2 while it works itself: 148 tiles are
-// 45 MB of the 126 MB.
+// the tensor core works and the other way round.  Each CTA therefore asks for the tile n_sm places further on
+// (likely the next on its SM) to come into L2 while it works itself: 148 tiles are 45 MB of the 126 MB.
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {   // 16-byte aligned, multiple of 16
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
@@ -138,16 +137,6 @@ __device__ __forceinline__ void ldraw(Raw8<__nv_bfloat16>& r, const __nv_bfloat1
 #pragma unroll
     for (int e = 0; e < 4; ++e) r.w[e] = 0u;
     if (in) ldraw4(r.w, p);
-}
-// (row, c .. c + 7) of an rf matrix
-__device__ __forceinline__ void ldraw_rf(Raw8<float>& r, const float* m, int rows, int row, int c) {
-    ldraw4(r.w, m + rf(rows, row, c));
-    ldraw4(r.w + 4, m + rf(rows, row, c + 4));
-}
-// (row, c .. c + 7) of an sf matrix
-__device__ __forceinline__ void ldraw_sf(Raw8<float>& r, const float* m, int row, int c) {
-    ldraw4(r.w, m + sf(row, c));
-    ldraw4(r.w + 4, m + sf(row, c + 4));
 }
 __device__ __forceinline__ void to_f(const Raw8<float>& r, float (&x)[8]) {
 #pragma unroll

@@ -16,7 +16,8 @@
 //
 // T=4096, H=32: 570 us with warp-level tf32 products; with state and r in shared memory and two CTAs of 64 columns 277 (6 KB of
 // operands for 32 clocks of an MMA of N = 64).  In this form 290 with half the CTAs; six packed sequences of 8 heads, which
-// took two waves then, 75 -> 56.  A step: 2100 clocks of the first product, 1300 to r, 1900 of the second, 2400 to the state;
+// took two waves then, 75 -> 56.  The products with an operand's first splits run while the others are written (296 -> 291 on
+// one machine).  A step: 2100 clocks of the first product, 1300 to r, 1900 of the second, 2400 to the state;
 // shared memory is half busy all the time, and a wait that read a flag beside its barrier cost 400 clocks of it.
 #include "kda_bwd.cuh"
 #include "kda_split3.cuh"

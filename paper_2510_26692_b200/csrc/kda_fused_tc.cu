@@ -34,8 +34,6 @@
 // k = q = v = 0).
 #include <cuda.h>
 
-#include <type_traits>
-
 #include "kda_common.cuh"
 #include "kda_ptx.cuh"
 #include "kda_tiles.cuh"
