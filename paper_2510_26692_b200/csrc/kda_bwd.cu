@@ -269,11 +269,9 @@ __global__ void __launch_bounds__(kThreads, 1) kda_bwd_sweep(BwdArgs a)
 }
 
 // adds the four slices' shares, in slice order
-__global__ void kda_bwd_reduce(const float* __restrict__ part_q, const float* __restrict__ part_k,
-                               const float* __restrict__ part_g, const float* __restrict__ part_b,
-                               float* __restrict__ dq, float* __restrict__ dk, float* __restrict__ dg,
-                               float* __restrict__ dbeta, size_t n_vec, size_t n_tok,
-                               const int* __restrict__ seq_heads, int H)
+__global__ void kda_bwd_reduce(const float* part_q, const float* part_k, const float* part_g, const float* part_b,
+                               float* dq, float* dk, float* dg, float* dbeta, size_t n_vec, size_t n_tok,
+                               const int* seq_heads, int H)
 {
     ptx::grid_dep_wait();      // (launched before the preceding kernel has ended)
     ptx::grid_dep_launch();

@@ -24,8 +24,8 @@ namespace kda {
 namespace {
 
 // clears the status word and the per-head marks, builds the chunk table of a packed batch
-__global__ void kda_bwd_prep(WsHeader* hdr, const int32_t* __restrict__ cu, int32_t* __restrict__ chunk_cu, int n_seqs,
-                             int* __restrict__ seq_heads, int H)
+__global__ void kda_bwd_prep(WsHeader* hdr, const int32_t* cu, int32_t* chunk_cu, int n_seqs,
+                             int* seq_heads, int H)
 {
     ptx::grid_dep_wait();      // (launched before the preceding kernel has ended)
     ptx::grid_dep_launch();

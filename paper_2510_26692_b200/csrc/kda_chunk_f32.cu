@@ -252,7 +252,7 @@ template <int NS> struct s2 {                           // NS = dv columns per i
 // of warps 4-7, and the state's 128 rows, which stay in the accumulator fragments of all warps (copy in
 // shared memory as B operand).  The operands of each phase arrive by cp.async during the other.
 template <int NS>
-__global__ void __launch_bounds__(kT2, 1) kda_inter_f32(ChunkArgs a, const float* __restrict__ tiles, int n_begin)
+__global__ void __launch_bounds__(kT2, 1) kda_inter_f32(ChunkArgs a, const float* tiles, int n_begin)
 {
     using L = s2<NS>;
     constexpr int LS = L::LS, NT = NS / 8;
@@ -371,8 +371,7 @@ __global__ void __launch_bounds__(kT2, 1) kda_inter_f32(ChunkArgs a, const float
     each_pair(S, lane, [&](int i, int j, float x, float y) { st2(a.S_out + sbase + (size_t)(16 * w + i) * kD + j, x, y); });
 }
 
-__global__ void kda_prep_kernel(WsHeader* hdr, const int32_t* __restrict__ cu,
-                                int32_t* __restrict__ chunk_cu, int n_seqs)
+__global__ void kda_prep_kernel(WsHeader* hdr, const int32_t* cu, int32_t* chunk_cu, int n_seqs)
 {
     ptx::grid_dep_wait();        // (launched before the preceding kernel has ended)
     ptx::grid_dep_launch();

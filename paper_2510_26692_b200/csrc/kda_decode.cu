@@ -67,9 +67,8 @@ struct DecodeLayer {
 // RMSNorm needs the whole output row, so it keeps whole states.
 template <typename T, bool kLayer, int NC>
 __global__ void __launch_bounds__(256, kD / NC * 2)
-kda_decode_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-                  const float* __restrict__ log_alpha, const float* __restrict__ beta, float* S,
-                  const int32_t* __restrict__ slot, T* __restrict__ o, int H, float scale, DecodeLayer lay)
+kda_decode_kernel(const T* q, const T* k, const T* v, const float* log_alpha, const float* beta, float* S,
+                  const int32_t* slot, T* o, int H, float scale, DecodeLayer lay)
 {
     static_assert(!kLayer || NC == kD, "the output stage needs the whole row");
     constexpr int kSlices = kD / NC;
@@ -273,9 +272,8 @@ __device__ __forceinline__ void cp_async4b(void* dst_smem, const void* src_gmem)
 
 template <typename T>
 __global__ void __launch_bounds__(256, 2)
-kda_decode_multi_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-                        const float* __restrict__ log_alpha, const float* __restrict__ beta, float* S,
-                        const int32_t* __restrict__ slot, T* __restrict__ o, int H, int n_tok, float scale,
+kda_decode_multi_kernel(const T* q, const T* k, const T* v, const float* log_alpha, const float* beta, float* S,
+                        const int32_t* slot, T* o, int H, int n_tok, float scale,
                         int n_items)
 {
     using L = MultiSmem<T>;

@@ -113,8 +113,8 @@ constexpr uint32_t kTmemCols = 512;                // two engines of 256 columns
 constexpr uint32_t T_D1 = 0, T_D3 = 256, T_S = 384, T_VN = 448;
 
 // loads that the compiler may not sink below their issue point (register prefetch of the next tile)
-__device__ __forceinline__ void ld_nc_f4(const float* p, float& a, float& b, float& c, float& d) {
-    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
+__device__ __forceinline__ void ld_f4(const float* p, float& a, float& b, float& c, float& d) {
+    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
                  : "=f"(a), "=f"(b), "=f"(c), "=f"(d)
                  : "l"(p));
 }
@@ -379,7 +379,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
                 const int i = i0 + r;
                 uint32_t lo = 0u, hi = 0u;
                 if (i < D.len)
-                    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];"
+                    asm volatile("ld.global.L1::no_allocate.v2.u32 {%0,%1}, [%2];"
                                  : "=r"(lo), "=r"(hi)
                                  : "l"(gp + (size_t)i * a.H * kD));
                 G[r][0] = __uint_as_float(lo);    // (unpacked when they are used: nothing here waits for the loads)
@@ -395,7 +395,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         for (int r = 0; r < kRPT; ++r) {
             const int i = i0 + r;
             if (i < D.len) {
-                ld_nc_f4(gp + (size_t)i * a.H * kD, G[r][0], G[r][1], G[r][2], G[r][3]);
+                ld_f4(gp + (size_t)i * a.H * kD, G[r][0], G[r][1], G[r][2], G[r][3]);
             } else {
                 G[r][0] = G[r][1] = G[r][2] = G[r][3] = 0.f;
             }

@@ -25,10 +25,8 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
 // kRows consecutive pairs of rows, all of whose loads are issued before the first is used.
 constexpr int kRows = 4;
 
-__global__ void __launch_bounds__(256) kda_layer_epilogue_kernel(__nv_bfloat16* __restrict__ y,
-                                                                 const __nv_bfloat16* __restrict__ g_o,
-                                                                 const float* __restrict__ w, float eps,
-                                                                 int64_t n_rows)
+__global__ void __launch_bounds__(256) kda_layer_epilogue_kernel(__nv_bfloat16* y, const __nv_bfloat16* g_o, const float* w,
+                                                                 float eps, int64_t n_rows)
 {
     ptx::grid_dep_wait();      // (launched while the chains end)
     ptx::grid_dep_launch();
@@ -74,10 +72,8 @@ __global__ void __launch_bounds__(256) kda_layer_epilogue_kernel(__nv_bfloat16* 
 // The same from the fp32 rows that the chains left in the scratch tiles: one CTA per (chunk, head), a warp per
 // four tokens, four columns a lane.  The caller's tensors are fetched before the chains have ended
 // (kda_chain_tc allows this launch only once everything before it is complete).
-__global__ void __launch_bounds__(512) kda_layer_rows_kernel(ChunkArgs a, const char* __restrict__ tiles,
-                                                             __nv_bfloat16* __restrict__ y,
-                                                             const __nv_bfloat16* __restrict__ g_o,
-                                                             const float* __restrict__ w, float eps)
+__global__ void __launch_bounds__(512) kda_layer_rows_kernel(ChunkArgs a, const char* tiles, __nv_bfloat16* y,
+                                                             const __nv_bfloat16* g_o, const float* w, float eps)
 {
     const int lane = threadIdx.x & 31, quad = threadIdx.x >> 5;
     const int64_t gl = blockIdx.x / (unsigned)a.H;

@@ -150,6 +150,9 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // attribute may begin before its predecessor in the stream has finished; grid_dep_wait() blocks
 // until the predecessor has completed and its writes are visible.  grid_dep_launch() in the
 // predecessor allows the dependent grid to be scheduled as soon as resources free up.
+// A kernel that begins early shares part of its life with the writes of the one before: what may come from that one is not
+// read-only for its duration, so it is read through pointers without __restrict__ and by loads without .nc, which the
+// compiler could also move ahead of the wait.  (The kernel before that one is complete, if its successor waited first.)
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
