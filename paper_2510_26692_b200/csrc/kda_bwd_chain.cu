@@ -75,12 +75,20 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tm = (uint32_t)ptx::warp_uniform((int)*slot);
-    // false once any wait of the CTA has run out
+    // Once any wait of the CTA has run out nobody waits any more, but every warp goes through all of its steps: lanes that
+    // find out apart must not part, or some would wait for the others in the next warp-wide instruction without a bound.
+    // (A vote of the lanes at each wait instead cost the kernel 5 per cent.)  The shared memory is busy: one access to it where
+    // one will do.
+    bool ok = true;
     auto wait = [&](uint64_t* bar, int64_t phase) {
-        if (ptx::mbar_try(bar, (uint32_t)phase & 1u)) return true;      // (the shared memory is busy: one access where one will do)
-        if (*abort_word) return false;
-        if (!ptx::mbar_wait(bar, (uint32_t)phase & 1u, a.wait_limit_ns)) *abort_word = 1;
-        return *abort_word == 0;
+        if (ok && !ptx::mbar_try(bar, (uint32_t)phase & 1u)) {
+            ok = *abort_word == 0 && ptx::mbar_wait(bar, (uint32_t)phase & 1u, a.wait_limit_ns);
+            if (!ok) *abort_word = 1;
+        }
+    };
+    auto wait_warp = [&](uint64_t* bar, int64_t phase) {
+        wait(bar, phase);
+        __syncwarp();
     };
 
     if (w < kCompute / 32) {
@@ -108,7 +116,7 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
             if (lane == 0) ptx::mbar_arrive(bar);
         };
         auto put_state = [&](int64_t i) {
-            wait(&fullV[i & 1], i >> 1);
+            wait_warp(&fullV[i & 1], i >> 1);
             float2 x[16];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -126,7 +134,7 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
 #pragma unroll
             for (int e = 0; e < 16; e += 4) ldraw4_w(u + e, ux + e * 128);
             // the state as the gradients stage needs it, by way of shared memory
-            if (i > 0 && !wait(freed, i - 1)) break;
+            if (i > 0) wait_warp(freed, i - 1);
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
                 stage[sf(k0 + 2 * e, v)] = S[e].x;
@@ -135,8 +143,7 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
             ptx::fence_async_smem();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(staged);
-            if (!wait(m1, i)) break;
-            __syncwarp();
+            wait_warp(m1, i);
             ptx::tc_fence_after();
             {
                 uint32_t y[16];
@@ -159,7 +166,7 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
                     *reinterpret_cast<float4*>(ux + e * 128) = make_float4(x[e / 2].x, x[e / 2].y, x[e / 2 + 1].x, x[e / 2 + 1].y);
             }
             // what does not need the second product
-            if (!kFwd && !wait(fullN, i)) break;
+            if (!kFwd) wait_warp(fullN, i);
             const float* np = reinterpret_cast<const float*>(sm + O_N) + rf(128, v, k0);
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -176,8 +183,7 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(n_read);
             }
-            if (!wait(m2, i)) break;
-            __syncwarp();
+            wait_warp(m2, i);
             ptx::tc_fence_after();
             {
                 uint32_t y[32];
@@ -221,10 +227,12 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
                 ahead(1);
                 for (int64_t i = 0; i < nc; ++i) {
                     const bool more = i + 1 < nc;
-                    if (!wait(staged, i)) break;
+                    wait(staged, i);
+                    if (!ok) break;
                     ptx::bulk_s2g(tile_of(i) + (kFwd ? bt::S : bt::L), sm + O_ST, kStateBytes);
                     ptx::bulk_commit();
-                    if (!wait(m1, i)) break;
+                    wait(m1, i);
+                    if (!ok) break;
                     if (more) {        // (the first product's operand is free, and so are the vectors of chunk i - 1)
                         vectors(i + 1); first(i + 1);
                         ++in_a;
@@ -233,10 +241,12 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
                     ptx::bulk_wait_read0();
                     ptx::mbar_arrive(freed);
                     if (!kFwd) {
-                        if (!wait(n_read, i)) break;
+                        wait(n_read, i);
+                        if (!ok) break;
                         if (more) { n_of(i + 1); ++in_n; }
                     }
-                    if (!wait(m2, i)) break;
+                    wait(m2, i);
+                    if (!ok) break;
                     if (more) { second(i + 1); ++in_b; }
                 }
                 ptx::bulk_wait_all0();
@@ -249,20 +259,18 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
             }
         } else if (w == kCompute / 32) {
             const uint32_t id64 = ptx::umma_idesc_bf16(128, 64), id128 = ptx::umma_idesc_bf16(128, 128), mnB = ptx::kIdescBMajorMN;
-            bool go = true;
-            for (int64_t i = 0; i < nc && go; ++i) {
+            for (int64_t i = 0; i < nc; ++i) {
                 // the products with the first splits of an operand run while the others are written
                 auto operand = [&](uint64_t* ready) {
                     return [&, ready](int s) {
-                        if (!wait(&ready[s], i)) go = false;
-                        __syncwarp();
+                        wait_warp(&ready[s], i);
                         ptx::tc_fence_after();
                     };
                 };
-                if (!wait(fullA, i)) break;
+                wait_warp(fullA, i);
                 mma6_ta<8, kSParts>(tm + C_1, tm + C_S, kFwd ? mn_major<128, 1>(sm + O_A) : k_major<64, 2>(sm + O_A), kFwd ? id64 | mnB : id64, false, operand(s_ready));
                 ptx::umma_commit(m1);
-                if (!go || !wait(fullB, i)) break;
+                wait_warp(fullB, i);
                 mma6_ta<4, kXParts>(tm + C_3, tm + C_X, kFwd ? mn_major<64, 2>(sm + O_B) : k_major<128, 1>(sm + O_B), kFwd ? id128 | mnB : id128, false, operand(x_ready));
                 ptx::umma_commit(m2);
             }

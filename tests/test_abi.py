@@ -281,22 +281,3 @@ def test_marshalling_of_another_torch_is_refused(lib, monkeypatch, tmp_path):
     monkeypatch.setattr(build, "_build_marshal", lambda: built.append(1))
     build.build()
     assert built
-
-
-def test_overlapping_kernels_read_coherently():
-    """A kernel that starts while its predecessor still writes (grid_dep_wait) may not declare its inputs read-only for its
-    whole duration: no const __restrict__ parameters, and .nc loads only in the backward stages whose inputs come from
-    kernels that were complete before they began."""
-    src = os.path.join(ROOT, "paper_2510_26692_b200", "csrc")
-    seen = 0
-    for name in sorted(os.listdir(src)):
-        text = open(os.path.join(src, name)).read()
-        text = re.sub(r"//[^\n]*", "", text)
-        assert "ld.global.nc" not in text or name in ("kda_bwd.cuh", "kda_bwd_intra.cu", "kda_bwd_out.cu"), name
-        for kernel in re.split(r"(?=__global__)", text)[1:]:
-            if "grid_dep_wait" not in kernel:
-                continue
-            head = kernel[:kernel.index("{")]
-            seen += 1
-            assert not re.search(r"const[^,]*__restrict__", head), (name, head)
-    assert seen >= 15

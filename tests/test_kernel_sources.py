@@ -1,0 +1,37 @@
+"""Rules that the kernels' sources keep and that no run on a GPU shows: what breaks one goes wrong by timing only, or by a
+hang after a wait has run out."""
+import os
+import re
+
+SRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2510_26692_b200", "csrc")
+
+
+def source(name):
+    return re.sub(r"//[^\n]*", "", open(os.path.join(SRC, name)).read())
+
+
+def test_overlapping_kernels_read_coherently():
+    """A kernel that starts while its predecessor still writes (grid_dep_wait) may not declare its inputs read-only for its
+    whole duration: no const __restrict__ parameters, and .nc loads only in the backward stages whose inputs come from
+    kernels that were complete before they began."""
+    seen = 0
+    for name in sorted(os.listdir(SRC)):
+        text = source(name)
+        assert "ld.global.nc" not in text or name in ("kda_bwd.cuh", "kda_bwd_intra.cu", "kda_bwd_out.cu"), name
+        for kernel in re.split(r"(?=__global__)", text)[1:]:
+            if "grid_dep_wait" not in kernel:
+                continue
+            head = kernel[:kernel.index("{")]
+            seen += 1
+            assert not re.search(r"const[^,]*__restrict__", head), (name, head)
+    assert seen >= 15
+
+
+def test_backward_chain_waits_do_not_part_a_warp():
+    """The lanes of a warp may find out apart that a wait has run out, so no warp-wide role branches on a wait's answer: the
+    ones that do would leave the others in the next warp-wide instruction.  Only the loader, one lane, leaves its loop."""
+    text = source("kda_bwd_chain.cu")
+    assert not re.search(r"if \([^{;]*!\s*wait", text)
+    loader = text[text.index("if (lane == 0) {\n                auto get"):text.index("} else if (w == kCompute / 32) {")]
+    rest = text.replace(loader, "")
+    assert "if (!ok) break;" in loader and "break" not in rest and not re.search(r"for \([^;{]*;[^;{]*\b(ok|abort_word)\b", rest)
