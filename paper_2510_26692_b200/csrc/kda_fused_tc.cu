@@ -1018,6 +1018,9 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
     auto wait_cluster = [&](uint64_t* bar, uint32_t parity, int where) {
         wait_by([](uint64_t* b, uint32_t p) { return ptx::mbar_try_cluster(b, p); }, bar, parity, where);
     };
+    // The flag may change between two lanes' looks at it.  Who goes on together leaves together: a warp by a vote, the output
+    // warps by their barrier.
+    auto aborted = [&]() { return __any_sync(0xffffffffu, *abort_flag != 0) != 0; };
     auto warp_arrive = [&](uint64_t* bar) {
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(bar);
@@ -1136,7 +1139,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                 }
                 KT_MARK(t == 0, 6);
             }
-            if (*abort_flag) break;
+            if (aborted()) break;
             if (float* s_out = state_out<kSeg>(f, s_off, cid))
 #pragma unroll
                 for (int i = 0; i < 64; ++i) s_out[s_at + i * kD] = S[i];
@@ -1216,8 +1219,8 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
             const uint32_t base = (uint32_t)ptx::warp_uniform((int)ptx::smem_u32(smem));
             uint32_t g = 0;
             KT_DECL(8);
-            for (int r = 0; next_job(r) && !*abort_flag; ++r)
-                for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
+            for (int r = 0; next_job(r) && !aborted(); ++r)
+                for (int c = 0; c < J.nch && !aborted(); ++c, ++g) {
                     const uint32_t sa = g % kStagesA, s = g % kStagesB;
                     const uint32_t pA = base + C_A + sa * kABytes, pB = base + C_B + s * C_STAGEB;
                     const uint32_t d1 = tm + T_D1 + (g & 1u) * 128u;
@@ -1274,8 +1277,9 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
             const uint32_t mrow = (uint32_t)(lane & 7), mcol = (uint32_t)((quad & 1) * 32 + (lane >> 3) * 8);
             const uint32_t moff = (uint32_t)(quad >> 1) * 8192u + ptx::sw128_off(mrow, mcol);
             uint32_t g = 0;
-            for (int r = 0; next_job(r) && !*abort_flag; ++r)
-                for (int c = 0; c < J.nch && !*abort_flag; ++c, ++g) {
+            bool stop = false;
+            for (int r = 0; !stop && next_job(r); ++r)
+                for (int c = 0; c < J.nch && !stop; ++c, ++g) {
                     const int64_t tok0 = J.tok_begin + (int64_t)c * kC;
                     const int len = (J.tok_end - tok0) < kC ? (int)(J.tok_end - tok0) : kC;
                     wait(&out_bar[g & 1u], (g >> 1) & 1u, 10);
@@ -1289,7 +1293,8 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                         ptx::tc_fence_before();
                         warp_arrive(&o_done[g & 1u]);
                         if (ot == 0) ptx::bulk_wait_read0();      // the previous block has been read out of its buffer
-                        ptx::named_bar_sync(6, 128);
+                        stop = ptx::named_bar_or(6, 128, *abort_flag != 0);
+                        if (stop) break;
                         uint4* rows = reinterpret_cast<uint4*>(smem + C_OUT) + ot;
     #pragma unroll
                         for (int q = 0; q < 16; ++q)
@@ -1313,7 +1318,8 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                     // the previous block has been read out of its buffer
                     uint8_t* sb = smem + C_OUT;
                     if (ot == 0) ptx::bulk_wait_read0();
-                    ptx::named_bar_sync(6, 128);
+                    stop = ptx::named_bar_or(6, 128, *abort_flag != 0);
+                    if (stop) break;
     #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         uint32_t z[4];

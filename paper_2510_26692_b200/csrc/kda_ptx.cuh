@@ -165,6 +165,20 @@ __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
     __syncwarp();
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
+// the same barrier; every thread gets whether `x` holds for any of them
+__device__ __forceinline__ bool named_bar_or(int id, int nthreads, bool x) {
+    __syncwarp();
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %3, 0;\n\t"
+        "bar.red.or.pred q, %1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(id), "r"(nthreads), "r"((uint32_t)x)
+        : "memory");
+    return r != 0;
+}
 // all bulk stores of this thread have completed (their writes are performed), not only read out
 __device__ __forceinline__ void bulk_wait_all0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // the same for all but the kPending groups committed last

@@ -35,3 +35,18 @@ def test_backward_chain_waits_do_not_part_a_warp():
     loader = text[text.index("if (lane == 0) {\n                auto get"):text.index("} else if (w == kCompute / 32) {")]
     rest = text.replace(loader, "")
     assert "if (!ok) break;" in loader and "break" not in rest and not re.search(r"for \([^;{]*;[^;{]*\b(ok|abort_word)\b", rest)
+
+
+def test_prefill_chain_roles_leave_together():
+    """The abort flag may change between two looks at it.  The roles of kda_fused_tc.cu's chain that are whole warps leave on
+    a vote, those that share a barrier on the barrier's own answer; only single lanes go by the flag as they see it."""
+    text = source("kda_fused_tc.cu")
+    chain = text[text.index("__device__ void chain_run("):text.index("__device__ void chain_init(")]
+    compute, loader, giver, mma, out = re.split(r"reg_inc<kChainRegs>|if \(warp == 9\)|if \(kRing && warp == 10\)|if \(warp == 8\)|if \(warp >= 12 && op\)",
+                                                chain)[1:]
+    for single in (loader, giver):
+        assert re.search(r"for \([^{;]*;[^;{]*!\*abort_flag", single) and single.lstrip(" {\n").startswith("if (lane == 0)")
+    for together in (compute, mma, out):
+        assert not re.search(r"for \([^{;]*;[^;{]*\*abort_flag", together)
+        assert not re.search(r"if \(\*abort_flag\)\s*\{?\s*(break|return)", together)
+    assert out.count("named_bar_or(6, 128, *abort_flag != 0)") == 2 and out.count("if (stop) break;") == 2
