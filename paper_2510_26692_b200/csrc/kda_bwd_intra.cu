@@ -40,7 +40,8 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
     float* vec = reinterpret_cast<float*>(sm + O_VEC);
     float* sBeta = vec + V_BETA; float* sSeg = vec + V_SEG;
     uint64_t* bar = reinterpret_cast<uint64_t*>(vec + V_BAR);   // one per group of MMAs, a phase per tile
-    uint32_t* slot = reinterpret_cast<uint32_t*>(bar + 4);
+    uint64_t* done = bar + 4;      // all MMAs complete, where a wait has run out
+    uint32_t* slot = reinterpret_cast<uint32_t*>(done + 1);
 
     ptx::grid_dep_wait();      // (launched before the preceding kernel has ended)
     // bf16 rows: a CTA per SM goes through the tiles, and the inputs of the next are requested as soon as
@@ -92,7 +93,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
     }
     if (t == 32) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) ptx::mbar_init(&bar[i], 1);
+        for (int i = 0; i < 5; ++i) ptx::mbar_init(&bar[i], 1);
         ptx::fence_mbar_init();
     }
     bool ok = true;
@@ -336,6 +337,11 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_intra(BwdChunkArgs a)
         if (!kLoop || id >= n_tiles) break;
     }
     ptx::grid_dep_launch();
+    if (w == kIssue && __any_sync(0xffffffffu, !ok)) {      // (not all of the groups issued since have been waited for)
+        ptx::umma_commit(done);
+        ptx::mbar_wait(done, 0, a.wait_limit_ns);
+        __syncwarp();
+    }
     if (t == kCopy) ptx::bulk_wait_all0();
     if (!ok && atomicCAS(&a.hdr->status, 0, (int)KDA_ERR_TIMEOUT) == 0) a.hdr->where = 31;
     ptx::tc_fence_before();

@@ -105,13 +105,14 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
     uint64_t* bar = reinterpret_cast<uint64_t*>(vec + V_BAR);
     uint64_t* ready = bar + 5;
     uint64_t* landed = ready + 4;
-    uint32_t* slot = reinterpret_cast<uint32_t*>(landed + 1);
+    uint64_t* done = landed + 1;       // (once) all MMAs complete
+    uint32_t* slot = reinterpret_cast<uint32_t*>(done + 1);
     if (w == kCompute / 32) {
         ptx::tmem_alloc(slot, 512);
         ptx::tmem_relinquish();
         if (lane == 0) {
 #pragma unroll
-            for (int i = 0; i < 10; ++i) ptx::mbar_init(&bar[i], i >= 5 && i < 9 ? kCompute / 32 : 1);
+            for (int i = 0; i < 11; ++i) ptx::mbar_init(&bar[i], i >= 5 && i < 9 ? kCompute / 32 : 1);
             ptx::fence_mbar_init();
         }
     }
@@ -161,6 +162,9 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_out(BwdChunkArgs a)
                 ptx::umma_commit(&bar[4]);
                 phase ^= 1u;
             }
+            ptx::umma_commit(done);        // before the TMEM goes away, also where a wait has run out
+            if (!ptx::mbar_wait(done, 0, a.wait_limit_ns)) ok = false;
+            __syncwarp();
         } else if (w == kCompute / 32 + 1) {
             // ================= loads =================
             while (find()) {

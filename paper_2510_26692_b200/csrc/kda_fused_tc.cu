@@ -991,7 +991,8 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
     uint64_t* o_done = out_bar + 2;          // [2] and read (4 warps)
     uint64_t* s_ready = o_done + 2;          // state operand written (8 warps)
     uint64_t* vn_ready = s_ready + 1;        // V_new operand written (8 warps)
-    volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(vn_ready + 1);
+    uint64_t* done = vn_ready + 1;           // all MMAs complete, where a wait has run out
+    volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(done + 1);
     const int warp = ptx::warp_uniform(t >> 5), lane = t & 31;
     __nv_bfloat16* op = kHasQ ? reinterpret_cast<__nv_bfloat16*>(a.o) : nullptr;
 
@@ -1266,6 +1267,11 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
             KT_FLUSH(lane == 0, f.hdr, 16, 6);
             // every MMA has completed before the TMEM goes away
             if (g > 0) wait(&emptyB[(g - 1) % kStagesB], ((g - 1) / kStagesB) & 1u, 5);
+            if (aborted()) {
+                ptx::umma_commit(done);
+                ptx::mbar_wait(done, 0, a.wait_limit_ns);
+                __syncwarp();
+            }
         } else if (warp >= 12 && op) {
             // ================= output rows =================
             // The accumulator has a lane per column and a TMEM column per token; read as 8 x 8 fragments and stored with
@@ -1366,6 +1372,7 @@ __device__ void chain_init(uint8_t* smem, int ring)
     for (int i = 0; i < 2; ++i) ptx::mbar_init(b++, 4);               // o_done
     ptx::mbar_init(b++, 8);                                           // s_ready
     ptx::mbar_init(b++, 8);                                           // vn_ready
+    ptx::mbar_init(b++, 1);                                           // done
     *reinterpret_cast<volatile uint32_t*>(b) = 0;                     // abort flag
     ptx::fence_mbar_init();
 }

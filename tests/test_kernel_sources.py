@@ -50,3 +50,13 @@ def test_prefill_chain_roles_leave_together():
         assert not re.search(r"for \([^{;]*;[^;{]*\*abort_flag", together)
         assert not re.search(r"if \(\*abort_flag\)\s*\{?\s*(break|return)", together)
     assert out.count("named_bar_or(6, 128, *abort_flag != 0)") == 2 and out.count("if (stop) break;") == 2
+
+
+def test_matrix_products_end_before_their_memory_does():
+    """After a wait has run out products may be under way that nobody waited for.  The warp that issued them commits once more
+    and waits for that, with the limit of every wait, before its CTA gives its TMEM and shared memory back."""
+    for name in ("kda_bwd_intra.cu", "kda_bwd_chain.cu", "kda_bwd_out.cu", "kda_fused_tc.cu"):
+        text = source(name)
+        at = [m.end() for m in re.finditer(r"umma_commit\(done\);", text)]
+        assert len(at) == 1 and re.match(r"\s*(if \(!)?ptx::mbar_wait\(done, 0, a\.wait_limit_ns\)", text[at[0]:]), name
+        assert re.search(r"tmem_dealloc", text[at[0]:]), name
