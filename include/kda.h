@@ -56,7 +56,8 @@ typedef enum {
     KDA_ERR_INVALID_ARG = 1, /* NULL/misaligned pointer, bad size, non-monotone cu_seqlens */
     KDA_ERR_UNSUPPORTED = 2, /* shape or dtype outside the supported set */
     KDA_ERR_WORKSPACE = 3,   /* workspace NULL or smaller than the minimum */
-    KDA_ERR_CUDA = 4,        /* a CUDA runtime call or launch failed */
+    KDA_ERR_CUDA = 4,        /* a CUDA runtime call or launch failed, or gave a kernel shared memory that is
+                                not aligned as it must be (the latter reported by kda_check_status) */
     KDA_ERR_TIMEOUT = 5,     /* a bounded device-side wait ran out (reported by kda_check_status) */
     KDA_ERR_GATE_RANGE = 6   /* a channel decayed by more than e^-160 inside one chunk: results are
                                 finite but not exact (reported by kda_check_status) */
@@ -345,7 +346,8 @@ kda_status_t kda_decode_step_host(const void *q_host, const void *k_host, const 
  * Reads back (synchronising the stream) the status word that device code sets when one of its
  * bounded waits runs out, and the flag that marks a decay outside the supported range (see the
  * conventions at the top), and clears both.  They live at the start of the workspace passed to
- * kda_chunk_fwd.  Returns KDA_OK, KDA_ERR_TIMEOUT or KDA_ERR_GATE_RANGE (a timeout wins).
+ * kda_chunk_fwd.  Returns KDA_OK, KDA_ERR_TIMEOUT, KDA_ERR_CUDA (see there) or KDA_ERR_GATE_RANGE
+ * (which the others win over).
  */
 kda_status_t kda_check_status(void *workspace, void *cuda_stream);
 

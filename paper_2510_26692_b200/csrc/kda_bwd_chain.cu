@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kT, 1) kda_bwd_chain(BwdChunkArgs a)
     ptx::grid_dep_wait();      // (launched before the preceding kernel has ended)
     if (a.seq_heads[h]) return;
     if ((ptx::smem_u32(sm) & 1023u) != 0) {
-        if (threadIdx.x == 0 && atomicCAS(&a.hdr->status, 0, (int)KDA_ERR_TIMEOUT) == 0) a.hdr->where = 33;
+        if (threadIdx.x == 0 && atomicCAS(&a.hdr->status, 0, (int)KDA_ERR_CUDA) == 0) a.hdr->where = 33;
         return;
     }
     if (blockIdx.x & 1) chain_run<true>(a, sm, n, h);

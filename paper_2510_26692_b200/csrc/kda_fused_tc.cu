@@ -273,8 +273,8 @@ __device__ __forceinline__ bool pass_job(const FusedArgs& f, int id, int r, JobI
 __device__ __forceinline__ bool call_aborted(const FusedArgs& f) {
     return *reinterpret_cast<volatile unsigned int*>(&f.hdr->abort_epoch) == f.epoch;
 }
-__device__ __forceinline__ void report_timeout(const FusedArgs& f, int where) {
-    if (atomicCAS(&f.hdr->status, 0, (int)KDA_ERR_TIMEOUT) == 0) f.hdr->where = where;
+__device__ __forceinline__ void report(const FusedArgs& f, kda_status_t code, int where) {
+    if (atomicCAS(&f.hdr->status, 0, (int)code) == 0) f.hdr->where = where;
     *reinterpret_cast<volatile unsigned int*>(&f.hdr->abort_epoch) = f.epoch;
     __threadfence();
 }
@@ -939,7 +939,7 @@ __device__ void engine_run(const FusedArgs& f, uint8_t* smem, uint32_t tmem_e, i
         const int last = cur == 0 ? 2 : cur - 1;
         store_staged(desc[last].tile);
     }
-    if (timed_out) report_timeout(f, 10);
+    if (timed_out) report(f, KDA_ERR_TIMEOUT, 10);
     if (out_of_range) atomicOr(&f.hdr->flags, 1);
     if (te == kServiceThread) {
         ptx::bulk_wait_all0();   // shared memory must outlive the reads of every bulk store
@@ -1007,7 +1007,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                 if (call_aborted(f)) { *abort_flag = 1; return; }
                 if (ptx::globaltimer_ns() - t0 > a.wait_limit_ns) {
                     *abort_flag = 1;
-                    report_timeout(f, where);
+                    report(f, KDA_ERR_TIMEOUT, where);
                     return;
                 }
             }
@@ -1431,7 +1431,7 @@ kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     }
     const uint32_t tmem_base = (uint32_t)ptx::warp_uniform((int)*tmem_slot);
     if ((ptx::smem_u32(smem) & 1023u) != 0) {   // the operand images need 1024-byte alignment
-        if (t == 0) report_timeout(f, 90);
+        if (t == 0) report(f, KDA_ERR_CUDA, 90);
     } else if (chain_cta) {
         chain_run<kHasQ, false, true>(f, smem, tmem_base, t, cid, &tm_o);
     } else {
@@ -1468,7 +1468,7 @@ kda_chain_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     ptx::tc_fence_after();
     const uint32_t tmem_base = (uint32_t)ptx::warp_uniform((int)*tmem_slot);
     if ((ptx::smem_u32(smem) & 1023u) != 0) {
-        if (t == 0) report_timeout(f, 90);
+        if (t == 0) report(f, KDA_ERR_CUDA, 90);
     } else {
         // The tiles, the chunk table and S0 come from kernels before this one.  Only then the next may start: what
         // that reads before its own wait (the gates of kda_layer_rows_kernel) is older than this kernel's inputs.
@@ -1513,7 +1513,7 @@ kda_intra_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtens
     ptx::tc_fence_after();
     const uint32_t tmem_base = (uint32_t)ptx::warp_uniform((int)*tmem_slot);
     if ((ptx::smem_u32(smem) & 1023u) != 0) {
-        if (t == 0) report_timeout(f, 90);   // the operand images need 1024-byte alignment
+        if (t == 0) report(f, KDA_ERR_CUDA, 90);   // the operand images need 1024-byte alignment
     } else {
         ptx::grid_dep_wait();     // (launched before the preceding kernel has ended)
         ptx::grid_dep_launch();   // the chains may set themselves up while this one drains

@@ -60,3 +60,14 @@ def test_matrix_products_end_before_their_memory_does():
         at = [m.end() for m in re.finditer(r"umma_commit\(done\);", text)]
         assert len(at) == 1 and re.match(r"\s*(if \(!)?ptx::mbar_wait\(done, 0, a\.wait_limit_ns\)", text[at[0]:]), name
         assert re.search(r"tmem_dealloc", text[at[0]:]), name
+
+
+def test_misaligned_shared_memory_is_not_called_a_timeout():
+    """A kernel that finds its dynamic shared memory not aligned says so by a code of its own."""
+    seen = 0
+    for name in sorted(os.listdir(SRC)):
+        text = source(name)
+        for m in re.finditer(r"& 1023u\) != 0\) \{([^}]*)\}", text):
+            seen += 1
+            assert "KDA_ERR_CUDA" in m.group(1) and "TIMEOUT" not in m.group(1) and "timeout" not in m.group(1), name
+    assert seen == 4
