@@ -28,13 +28,14 @@ def test_overlapping_kernels_read_coherently():
 
 
 def test_backward_chain_waits_do_not_part_a_warp():
-    """The lanes of a warp may find out apart that a wait has run out, so no warp-wide role branches on a wait's answer: the
-    ones that do would leave the others in the next warp-wide instruction.  Only the loader, one lane, leaves its loop."""
+    """The lanes of a warp may find out apart that a wait has run out, so no warp-wide role branches on a lane's own answer: the
+    ones that do would leave the others in the next warp-wide instruction.  They leave on a vote; only the loader, one lane,
+    leaves on its own."""
     text = source("kda_bwd_chain.cu")
-    assert not re.search(r"if \([^{;]*!\s*wait", text)
     loader = text[text.index("if (lane == 0) {\n                auto get"):text.index("} else if (w == kCompute / 32) {")]
-    rest = text.replace(loader, "")
-    assert "if (!ok) break;" in loader and "break" not in rest and not re.search(r"for \([^;{]*;[^;{]*\b(ok|abort_word)\b", rest)
+    rest = re.sub(r"!__all_sync\(0xffffffffu, wait\(\w+, i\)\)\) break;", "", text.replace(loader, ""))
+    assert "if (!wait(" in loader and "break" not in rest and not re.search(r"if \([^{;]*!\s*wait", rest)
+    assert not re.search(r"for \([^;{]*;[^;{]*\b(ok|abort_word)\b", rest)
 
 
 def test_prefill_chain_roles_leave_together():
