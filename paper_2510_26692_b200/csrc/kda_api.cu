@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <limits>
 #include <mutex>
 #include <random>
 #include <vector>
@@ -314,28 +315,6 @@ struct LayerMode {
     float rms_eps = 0.f;
 };
 
-// Into how many segments the chains of a bf16 call are cut (kda_segments.cu), 1 = none.  All runs of a stage must
-// be resident at once.  Times in us, measured: a chain step 1.62 in the fused kernel, 1.4 (maps) and 1.5 (outputs) with all SMs
-// at it, a tile of the intra-chunk kernel 8 over two CTAs per SM, launches 22 and a border 1.5.
-// Prefill, whole / cut: 8 heads x 4096 tokens 89 -> 62 us, 8 x 30000: 604 -> 252, 16 x 65536: 1367 -> 939, for the final
-// state 1270 -> 658.  Modes 1 and 2 of kda_set_chunk_path never cut.
-// Below 48 chunks it gains at most a tenth, and a short sequence keeps the same bits however it is handed over.
-int segments(int64_t J, int64_t longest, int64_t tiles, bool out, bool layer, int n_sm)
-{
-    if (g_chunk_path.load(std::memory_order_relaxed) != 0) return 1;
-    const int64_t runs = (n_sm < kMaxRuns ? n_sm : kMaxRuns) / J;
-    const int64_t most = out ? (runs + 3) / 2 : (runs + 1) / 2;     // maps of P - 1 and P - 2 segments, or of P and P - 1
-    const double intra = 8. * tiles / (2 * n_sm), two = intra + 1.4 * longest + 4.;
-    const double fused = 1.62 * longest + 17.;
-    double best = 0.95 * (layer ? two : std::min(two, fused));      // (layer calls never run fused)
-    int P = 1;
-    for (int64_t p = 3; p <= most && 4 * p <= longest; ++p) {
-        const double us = intra + (double)((longest + p - 1) / p) * (out ? 1.4 + 1.5 : 1.4) + 1.5 * p + 22.;
-        if (us < best) { best = us; P = (int)p; }
-    }
-    return P;
-}
-
 // fused_shape for the current device
 kda_status_t fused_schedule(FusedArgs& f, const std::vector<int64_t>& chunk_cu, int64_t avail, bool has_q, int64_t* load)
 {
@@ -347,32 +326,96 @@ kda_status_t fused_schedule(FusedArgs& f, const std::vector<int64_t>& chunk_cu, 
     return KDA_OK;
 }
 
-// Whether a bf16 call without the layer's functions runs as the fused kernel (kda_set_chunk_path): always where the
-// tiles of all chunks do not fit the workspace, else by the time of both in us.  Fused: 17, and per tile of the most
-// loaded cluster 1.62 with one chain to a cluster; with several 1.5 where the others idle beside a few long chains, up
-// to 1.9 where all are loaded alike.  Two kernels: a tile 8 with two per SM, a chain step 1.4, 8 for the launches
-// (all of them 5 to 8 per cent less by now, alike on both sides, and shorter steps where few chains run: their ratio decides).
-// Measured, fused / two: 32 heads x 1000 tokens 40 / 40, x 1500 54 / 59, x 4096 113 / 135; 16 x 2000 60 / 56;
-// 37 x 900 45 / 41; 8 heads, 7 sequences, 19620 tokens, the longest 4679: 148 / 161, 31108 and 6677: 223 / 235; 3 of up to
-// 16632: 370 / 423; 32 heads, 2 x 2048 117 / 109; 16 heads, 7 of up to 9948 441 / 426, 8 of up to 2735 224 / 201.  Layer calls: never faster.
-kda_status_t use_fused(FusedArgs& f, const std::vector<int64_t>& chunk_cu, const void* workspace, size_t bytes, bool has_q, bool* fused)
+// ---- schedule of a bf16 call, by estimated times in us --------------------------------------------------------
+// Fitted to 526 calls of 1 to 512 chains and 1 to 768 chunks, each run every way it can, the ways in turn (with outputs; for the
+// final state): the way taken costs 0.22 per cent more than the fastest on the mean, at worst 11 (chains of 768 chunks, where a step
+// of the fused kernel is longer).  0.89 and 17 with the times that stood here before the steps of the chains became shorter.
+struct Estimate {
+    double tiles;      // the intra-chunk kernel, two tiles per SM
+    double two;        // both kernels
+    double fused;      // the fused kernel; infinite where it cannot run
+    double table;      // the chunk table of a packed batch, a kernel ahead of the two
+};
+Estimate estimate(const FusedArgs& f, int64_t tiles, int64_t longest, int64_t load, bool out, int n_sm)
+{
+    Estimate e;
+    e.table = f.a.cu_seqlens ? 5. : 0.;
+    e.tiles = (out ? 9.5 : 7.3) * (double)tiles / (2 * n_sm);
+    e.two = e.tiles + 0.97 * std::max((double)longest, (double)tiles / n_sm) + 9. + e.table;
+    e.fused = std::numeric_limits<double>::infinity();
+    if (load == 0) return e;
+    // per tile of the most loaded cluster: of four CTAs 1.3 to 1.5 (more clusters wait more for memory; final state 1.25 to 1.35),
+    // of three 2.0 (1.83: four engines are too few for a chain); where a cluster goes through several chains, more the less the
+    // others idle
+    const bool three = f.cluster_size == 3;
+    const int rounds = (f.J + f.n_clusters - 1) / f.n_clusters;
+    double per = out ? 1.34 : 1.3;
+    if (rounds > 1) {
+        const double busy = (double)tiles / ((double)f.n_clusters * (double)load);
+        per = (per + (out ? 0.5 : 0.2) * std::max(0., busy - 0.45)) * (three ? 1.5 : 1.);
+    } else {
+        per = three ? (out ? 2.0 : 1.83) : per + (out ? 0.01 : 0.004) * std::max(0, f.J - 16);
+    }
+    e.fused = per * (double)load + 2. * (rounds - 1) + 17.;
+    return e;
+}
+
+// Into how many segments the chains are cut (kda_segments.cu), 1 = none; `whole`: the time without.  All runs of a stage must
+// be resident at once.  A step of the maps and of the outputs together 1.9, more as the runs take all SMs (final state: maps
+// alone, 0.9), a border 2.1 (1.5), launches 23 (15).
+// Measured, whole (two kernels, fused) / cut, with outputs, 64 chunks: 8 chains 89, 100 / 62, 16 chains 108, 102 / 88, 24 chains 120, 106 / 117;
+// 160 chunks: 34 chains 326, 334 / 305, 36 chains 336, 335 / 318, 40 chains 355, 336 / 347; 48 chains of 96 chunks 241, 286 / 258, of
+// 320 chunks 783, 1003 / 771.  Final state, 48 chunks: 10 chains 67, 77 / 44, 24 chains 84, 80 / 68.  Modes 1 and 2 of
+// kda_set_chunk_path never cut.
+// Below 48 chunks it gains at most a tenth, and a short sequence keeps the same bits however it is handed over.
+int segments(int64_t J, int64_t longest, const Estimate& e, double whole, bool out, int n_sm)
+{
+    const int64_t runs = (n_sm < kMaxRuns ? n_sm : kMaxRuns) / J;
+    const int64_t most = out ? (runs + 3) / 2 : (runs + 1) / 2;     // maps of P - 1 and P - 2 segments, or of P and P - 1
+    double best = whole;
+    int P = 1;
+    for (int64_t p = 3; p <= most && 4 * p <= longest; ++p) {
+        const double step = out ? 1.9 + 1.2 * std::max(0., (double)(J * p) / n_sm - 0.6) : 0.9;
+        const double us = e.tiles + (double)((longest + p - 1) / p) * step + (out ? 2.1 : 1.5) * (double)p + (out ? 23. : 15.) + e.table;
+        if (us < best) { best = us; P = (int)p; }
+    }
+    return P;
+}
+
+// Schedule of a bf16 call: P segments, or the fused kernel, or (neither) the two kernels.  `seg_bytes`: workspace that
+// segments need, given P.  The fused kernel always where the tiles of all chunks do not fit the workspace; never for
+// layer calls, where it was never faster.
+// Measured, fused / two, heads x tokens: 32 x 1024 41 / 41, x 2048 67 / 75, x 4096 113 / 136; 16 x 2048 60 / 57; 38 x 1024 47 / 46, x 2048
+// 81 / 81; 40 x 4096 146 / 151; 56 x 1536 90 / 79, x 4096 205 / 180; 8 heads, sequences of 4000 and six of 600 105 / 111, seven of 1100
+// 73 / 65, five of 500 to 8000 188 / 201; 32 heads, 4000 and 2000 164 / 166.  Final state: 32 x 1024 40 / 37, x 2048 61 / 67; 38 x 2048
+// 74 / 72, x 4096 133 / 131; 8 heads, 4000 and six of 600 99 / 98; 32 heads, 3000 and 200 91 / 98.
+template <typename SegBytes>
+kda_status_t choose_schedule(const FusedArgs& call, const std::vector<int64_t>& chunk_cu, const void* workspace, size_t bytes, bool out,
+                             bool layer, bool may_cut, SegBytes seg_bytes, int* P, bool* fused)
 {
     const int mode = g_chunk_path.load(std::memory_order_relaxed);
+    FusedArgs f = call;      // (the shape of its clusters is filled in here)
     const size_t fixed = ws_layout(f.a.n_seqs, f.a.H).fixed, row = (size_t)f.a.H * tc_tile_bytes();
     const int64_t chunks = chunk_cu[f.a.n_seqs];
-    *fused = mode == 2 || (mode == 0 && (bytes < fixed || (int64_t)((bytes - fixed) / row) < chunks));
-    if (mode != 0 || *fused || f.J > kMaxRuns || chunks == 0 || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1))) return KDA_OK;
+    const bool all_fit = bytes >= fixed && (int64_t)((bytes - fixed) / row) >= chunks;
+    *P = 1;
+    *fused = !layer && (mode == 2 || (mode == 0 && !all_fit));
+    may_cut = may_cut && mode == 0;
+    const bool may_fuse = !layer && mode == 0 && f.J <= kMaxRuns && bytes >= kFusedRing + 2 * tc_tile_bytes();
+    if (chunks == 0 || !(may_cut || (may_fuse && !*fused)) || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1))) return KDA_OK;
     int n_sm = 0;
     int64_t load = 0, longest = 0;
     kda_status_t rc = sm_count(&n_sm);
-    if (rc == KDA_OK) rc = fused_schedule(f, chunk_cu, (int64_t)((bytes - kFusedRing) / tc_tile_bytes()), has_q, &load);
+    if (rc == KDA_OK && may_fuse) rc = fused_schedule(f, chunk_cu, (int64_t)((bytes - kFusedRing) / tc_tile_bytes()), out, &load);
     if (rc != KDA_OK) return rc;
-    if (load == 0) return KDA_OK;
     for (int n = 0; n < f.a.n_seqs; ++n) longest = std::max(longest, chunk_cu[n + 1] - chunk_cu[n]);
-    const double tiles = (double)chunks * f.a.H, busy = tiles / ((double)f.n_clusters * load);
-    const double per = (f.J <= f.n_clusters ? 1.62 : 1.5 + std::max(0., busy - 0.5)) * (has_q ? 1. : 0.8);
-    const double two = (has_q ? 8. : 7.5) * tiles / (2 * n_sm) + (has_q ? 1.4 : 1.3) * std::max((double)longest, tiles / n_sm) + 8.;
-    *fused = per * load + 17. < 0.93 * two;
+    const Estimate e = estimate(f, chunks * f.a.H, longest, load, out, n_sm);
+    if (may_cut && longest >= kMinCut && f.J <= kMaxRuns / 3) {
+        *P = segments(f.J, longest, e, *fused ? e.fused : std::min(e.two, e.fused), out, n_sm);
+        if (*P > 1 && bytes < seg_bytes(*P)) *P = 1;
+    }
+    if (*P > 1) *fused = false;
+    else if (may_fuse && all_fit) *fused = e.fused < e.two;
     return KDA_OK;
 }
 
@@ -442,22 +485,20 @@ kda_status_t chunk_fwd_impl(const void* q, const void* k, const void* v, const f
         f.epoch = next_epoch();
     }
     int P = 1;
-    int64_t longest = 0;
-    for (int n = 0; n < n_seqs; ++n) longest = std::max(longest, chunk_cu[n + 1] - chunk_cu[n]);
-    if (dt == KDA_BF16 && (o || S_T) && workspace && longest >= kMinCut && (int64_t)n_seqs * H <= kMaxRuns / 3) {
-        int n_sm = 0;
-        if (const kda_status_t rc = sm_count(&n_sm)) return rc;
-        P = segments((int64_t)n_seqs * H, longest, total_chunks * H, q && o, lm.rate != nullptr, n_sm);
-        // Their scratch lies behind the tiles, which should all fit; one sequence without outputs may also go in passes.
+    bool fused = false;
+    if (dt == KDA_BF16) {
+        // The segments' scratch lies behind the tiles, which should all fit; one sequence without outputs may also go in passes.
         // With outputs the last segment writes the final state while the first may not have read S0 yet.
         const bool out = q && o, passes = n_seqs == 1 && !out;
-        const size_t need = ws_layout(n_seqs, H).fixed + kSegScratch + kAlign +
-                            (size_t)H * tc_tile_bytes() * (size_t)(passes ? std::min<int64_t>(64 * P, total_chunks) : total_chunks);
-        if (P > 1 && (workspace_bytes < need || (out && S0 && S0 == S_T))) P = 1;
+        const kda_status_t rc = choose_schedule(
+            f, chunk_cu, workspace, workspace_bytes, out, lm.rate != nullptr, (o || S_T) && workspace && !(out && S0 && S0 == S_T),
+            [&](int p) {
+                return ws_layout(n_seqs, H).fixed + kSegScratch + kAlign +
+                       (size_t)H * tc_tile_bytes() * (size_t)(passes ? std::min<int64_t>(64 * p, total_chunks) : total_chunks);
+            },
+            &P, &fused);
+        if (rc != KDA_OK) return rc;
     }
-    bool fused = false;
-    if (dt == KDA_BF16 && P == 1 && !lm.rate)
-        if (const kda_status_t rc = use_fused(f, chunk_cu, workspace, workspace_bytes, q && o, &fused)) return rc;
     if (fused) {
         const size_t tbf = tc_tile_bytes();
         if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) || workspace_bytes < kFusedRing + 2 * tbf)
