@@ -164,3 +164,62 @@ def test_backward_several_tiles_per_cta(oracle_mod, lens, H, dtype, harsh):
         assert rel_l2(to_np32(out[n]), ref[n]) <= 1e-5, n
     again = run_bwd(d, d_o, dS_T)
     assert all(torch.equal(out[n], again[n]) for n in NAMES)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_calls_queued_without_a_wait(dtype):
+    """Launches overlap the end of the call before.  Backward, forward and decode calls queued on one stream and one workspace,
+    some on the others' outputs, one with a head out of the chunk form's range: the same bits as with a wait after each."""
+    dt = K.KDA_BF16 if dtype == torch.bfloat16 else K.KDA_F32
+    T, N, H = 900, 3, 8
+    d = [inputs.chunk_inputs([300, 17, 583], H=H, dtype=dtype, seed=s, s0_std=0.02, device="cuda:0") for s in (36, 37)]
+    d[1]["log_alpha"][-1, 3, 5] = -45.0
+    cot = [[x.cuda() for x in cotangents(d[i], 36 + i, dtype)] for i in range(2)]
+    cu = d[0]["cu_seqlens"].cpu()
+    cu_dev = cu.cuda()
+    nb = max(K.kda_chunk_bwd_workspace_bytes(T, N, H), K.kda_chunk_fwd_workspace_bytes(T, N, H, 128, 128, 64, dt))
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda:0")
+
+    def calls(wait):
+        done = []
+        after = torch.cuda.synchronize if wait else (lambda: None)
+
+        def backward(x, c, d_o):
+            g = {n: torch.full((T, H, 128), float("nan"), device="cuda:0") for n in ("dq", "dk", "dv", "dlog_alpha")}
+            g["dbeta"] = torch.full((T, H), float("nan"), device="cuda:0")
+            g["dS0"] = torch.full((N, H, 128, 128), float("nan"), device="cuda:0")
+            K.kda_chunk_bwd(x["q"], x["k"], x["v"], x["log_alpha"], x["beta"], x["S0"], d_o, c[1], *(g[n] for n in NAMES), cu_dev, cu,
+                            N, T, H, 128, 128, 64, 1.0, dt, ws)
+            after()
+            done.extend(g[n] for n in NAMES)
+            return g
+
+        def forward(x, q):
+            o, S = torch.empty_like(x["v"]), torch.empty((N, H, 128, 128), device="cuda:0")
+            K.kda_chunk_fwd(q, x["k"], x["v"], x["log_alpha"], x["beta"], x["S0"], o, S, cu_dev, cu, N, T, H, 128, 128, 64, 1.0, dt, ws)
+            after()
+            done.extend((o, S))
+            return o, S
+
+        g = backward(d[0], cot[0], cot[0][0])
+        o, S = forward(d[1], d[1]["q"])
+        backward(d[1], cot[1], o)                       # the forward's outputs, and a head that runs token by token
+        o, S = forward(d[0], g["dq"] if dtype == torch.float32 else o)
+        x = d[1]
+        for t in range(3):                              # the states that have just been written, the row before as q and v
+            o1 = torch.empty((N, H, 128), dtype=dtype, device="cuda:0")
+            q = x["q"][:N].contiguous() if t == 0 else prev
+            K.kda_decode_step(q, x["k"][:N], q, x["log_alpha"][:N], x["beta"][:N], S, None, o1, N, H, 128, 128, 1.0, dt)
+            after()
+            done.append(o1)
+            prev = o1
+        backward(d[0], cot[0], cot[0][0])
+        torch.cuda.synchronize()
+        K.kda_check_status(ws)
+        return done
+
+    apart = calls(True)
+    assert all(torch.isfinite(x.float()).all() for x in apart)
+    for _ in range(5):
+        for x, y in zip(calls(False), apart):
+            assert torch.equal(x, y)
