@@ -1291,6 +1291,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                     wait(&out_bar[g & 1u], (g >> 1) & 1u, 10);
                     __syncwarp();
                     ptx::tc_fence_after();
+                    const uint32_t seen = *abort_flag;      // (looked at beside the read-out: at the barrier it cost a layer call on 24 chains 3 per cent)
                     if (kRows32) {     // lane = column, four tokens a piece
                         uint32_t y[2][32];
                         ptx::tmem_ld_32x32b_x32(tq + T_D1 + (g & 1u) * 128u + 64, y[0]);
@@ -1299,8 +1300,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                         ptx::tc_fence_before();
                         warp_arrive(&o_done[g & 1u]);
                         if (ot == 0) ptx::bulk_wait_read0();      // the previous block has been read out of its buffer
-                        stop = ptx::named_bar_or(6, 128, *abort_flag != 0);
-                        if (stop) break;
+                        stop = ptx::named_bar_or(6, 128, seen != 0);
                         uint4* rows = reinterpret_cast<uint4*>(smem + C_OUT) + ot;
     #pragma unroll
                         for (int q = 0; q < 16; ++q)
@@ -1324,8 +1324,7 @@ __device__ void chain_run(const FusedArgs& f, uint8_t* smem, uint32_t tm, int t,
                     // the previous block has been read out of its buffer
                     uint8_t* sb = smem + C_OUT;
                     if (ot == 0) ptx::bulk_wait_read0();
-                    stop = ptx::named_bar_or(6, 128, *abort_flag != 0);
-                    if (stop) break;
+                    stop = ptx::named_bar_or(6, 128, seen != 0);
     #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         uint32_t z[4];
@@ -1381,9 +1380,9 @@ __device__ void chain_init(uint8_t* smem, int ring)
 // mbarriers in each other's shared memory.  The ring is written and read by bulk copies alone: an engine
 // announces a tile once its copies have completed, the chain gives a position back once its copy has landed; both
 // by release arrivals, taken up by acquire waits and a proxy fence before the next bulk copy.  The arrivals are made where
-// nothing waits for the thread, during the substitution and by a warp of their own: 4096 x 32 heads 120.7 us, 1 Mi tokens
-// for the state 20.6 ms, 113 and 20.35 now (made by the loader, and by the service thread ahead of its copies, then: 141 us and
-// 28.9 ms; relaxed, which orders nothing: 112.5 and 20.2).
+// nothing waits for the thread, during the substitution and by a warp of their own: 4096 x 32 heads 120.7 us when they were
+// added, 1 Mi tokens for the state 20.6 ms, 114 and 20.1 now (made by the loader, and by the service thread ahead of its copies, then: 141 us
+// and 28.9 ms; relaxed, which orders nothing, then: 112.5 and 20.2).
 template <bool kHasQ>
 __global__ void __launch_bounds__(kThreads, 1)
 kda_fused_tc(const __grid_constant__ FusedArgs f, const __grid_constant__ CUtensorMap tm_k,

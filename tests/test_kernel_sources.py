@@ -50,7 +50,7 @@ def test_prefill_chain_roles_leave_together():
     for together in (compute, mma, out):
         assert not re.search(r"for \([^{;]*;[^;{]*\*abort_flag", together)
         assert not re.search(r"if \(\*abort_flag\)\s*\{?\s*(break|return)", together)
-    assert out.count("named_bar_or(6, 128, *abort_flag != 0)") == 2 and out.count("if (stop) break;") == 2
+    assert out.count("stop = ptx::named_bar_or(6, 128, seen != 0);") == 2 and len(re.findall(r"for \([^{;]*;[^;{]*!stop", out)) == 2
 
 
 def test_matrix_products_end_before_their_memory_does():
