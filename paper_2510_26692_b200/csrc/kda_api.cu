@@ -172,8 +172,8 @@ void order_sequences(FusedArgs& f, const std::vector<int64_t>& chunk_cu, bool pa
 bool fused_shape(FusedArgs& f, const std::vector<int64_t>& chunk_cu, int64_t avail, bool has_q, const int (&most)[2], int64_t* load)
 {
     const int H = f.a.H, n_seqs = f.a.n_seqs;
-    // Two or three engine CTAs per chain: microseconds a tile costs the chain and an engine (measured), times the
-    // tiles of the most loaded cluster.
+    // Two or three engine CTAs per chain: microseconds a tile costs the chain and an engine, times the tiles of the most loaded
+    // cluster (a step measured, with outputs and without: of four CTAs 1.3 to 1.5 and 1.2 to 1.34, of three 2.0 and 1.83).
     const double chain = has_q ? 1.5 : 1.3, engine = has_q ? 8.0 : 7.5;
     double best = 0.;
     f.n_clusters = 0;
@@ -400,17 +400,17 @@ kda_status_t choose_schedule(const FusedArgs& call, const std::vector<int64_t>& 
     const bool all_fit = bytes >= fixed && (int64_t)((bytes - fixed) / row) >= chunks;
     *P = 1;
     *fused = !layer && (mode == 2 || (mode == 0 && !all_fit));
-    may_cut = may_cut && mode == 0;
+    int64_t load = 0, longest = 0;
+    for (int n = 0; n < f.a.n_seqs; ++n) longest = std::max(longest, chunk_cu[n + 1] - chunk_cu[n]);
+    may_cut = may_cut && mode == 0 && longest >= kMinCut && f.J <= kMaxRuns / 3 && bytes >= seg_bytes(3);
     const bool may_fuse = !layer && mode == 0 && f.J <= kMaxRuns && bytes >= kFusedRing + 2 * tc_tile_bytes();
     if (chunks == 0 || !(may_cut || (may_fuse && !*fused)) || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1))) return KDA_OK;
     int n_sm = 0;
-    int64_t load = 0, longest = 0;
     kda_status_t rc = sm_count(&n_sm);
     if (rc == KDA_OK && may_fuse) rc = fused_schedule(f, chunk_cu, (int64_t)((bytes - kFusedRing) / tc_tile_bytes()), out, &load);
     if (rc != KDA_OK) return rc;
-    for (int n = 0; n < f.a.n_seqs; ++n) longest = std::max(longest, chunk_cu[n + 1] - chunk_cu[n]);
     const Estimate e = estimate(f, chunks * f.a.H, longest, load, out, n_sm);
-    if (may_cut && longest >= kMinCut && f.J <= kMaxRuns / 3) {
+    if (may_cut) {
         *P = segments(f.J, longest, e, *fused ? e.fused : std::min(e.two, e.fused), out, n_sm);
         if (*P > 1 && bytes < seg_bytes(*P)) *P = 1;
     }
