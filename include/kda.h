@@ -216,7 +216,8 @@ kda_status_t kda_layer_decode_step(const void *q_c, const void *k_c, const void 
  * the chunks, then the gradients of all chunks at once.  Heads in which some chunk's log decay
  * leaves [-40, 1], or some token is not finite, run token by token instead (any decay is exact there).
  * Inputs of the matrix products keep 24 significant bits, sums are fp32: relative errors of 1.3e-7 to
- * 6e-7 where a chunk decays by e^-4, up to 7.6e-7 (dlog_alpha) near e^-40; token by token 1e-7 to 1.5e-7 there.
+ * 4.1e-7 where a chunk decays by e^-2; where it decays by e^-20 3.1e-7 but for dlog_alpha, 8.3e-7, and near
+ * e^-40 2.8e-7 and 1.2e-6; token by token 0.8e-7 to 1.3e-7.
  *
  *   q, k [T_total,H,dk], v, d_o [T_total,H,dv]   device, element type `dt` (KDA_F32 or KDA_BF16)
  *   log_alpha [T_total,H,dk], beta [T_total,H]   fp32 device

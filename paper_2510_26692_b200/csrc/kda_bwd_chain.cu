@@ -17,8 +17,9 @@
 // T=4096, H=32: 570 us with warp-level tf32 products; with state and r in shared memory and two CTAs of 64 columns 277 (6 KB of
 // operands for 32 clocks of an MMA of N = 64).  In this form 290 with half the CTAs; six packed sequences of 8 heads, which
 // took two waves then, 75 -> 56.  The products with an operand's first splits run while the others are written (296 -> 291 on
-// one machine).  A step: 2100 clocks of the first product, 1300 to r, 1900 of the second, 2400 to the state;
-// shared memory is half busy all the time, and a wait that read a flag beside its barrier cost 400 clocks of it.
+// one machine).  A step: 4.05 us (8000 clocks) with 8 CTAs, 4.25 with 32, 4.6 with 64; of 7700 clocks in a build that took times, 2100 for
+// the first product, 1300 to r, 1900 for the second, 2400 to the state.  The tensor pipe is active 40 per cent of the time, shared memory
+// half busy all the time; a wait that read a flag beside its barrier cost 400 clocks of it.
 #include "kda_bwd.cuh"
 #include "kda_split3.cuh"
 
@@ -78,8 +79,8 @@ __device__ __forceinline__ void chain_run(const BwdChunkArgs& a, uint8_t* sm, in
     // Once any wait of the CTA has run out nobody waits any more.  The lanes of a warp may find that out apart, and must not part
     // on it, or some would wait for the others in the next warp-wide instruction without a bound: warps that go on together
     // ignore the answer, and leave by votes ahead of the state's update.  (Where the votes stand decides more than that they are
-    // there: at every wait 305 us at 4096 x 32 heads against 290, at none 295.)  The shared memory is busy: one access to it where one
-    // will do.
+    // there.  4096 x 32 heads, this kernel: at every wait 305 us, at none 297, here 294; 7074 x 4, the call: none 620, here 608.  With
+    // lanes leaving on their own it was 288 and 607.)  The shared memory is busy: one access to it where one will do.
     auto wait = [&](uint64_t* bar, int64_t phase) {
         if (ptx::mbar_try(bar, (uint32_t)phase & 1u)) return true;
         if (*abort_word == 0 && ptx::mbar_wait(bar, (uint32_t)phase & 1u, a.wait_limit_ns)) return true;

@@ -1,6 +1,7 @@
 // First stage of the chunkwise backward pass (equations in kda_bwd_chunk.cu): everything of a (chunk, head) tile
 // that depends on neither state.  Products on tcgen05 with split operands
-// (kda_split3.cuh); the 64 x 64 inverse is fp32 FMA and runs beside the two products that do not need it.
+// (kda_split3.cuh); the 64 x 64 inverse (16 x 16 blocks by fp32 substitution, joined by split tf32 products, kda_mma3.cuh) runs
+// beside the two products that do not need it.
 //
 //   A   [K^ ; Q] K_^T        -> B (masked), P (masked)
 //   C1  dO^T Q               -> N            C2  dO^T P -> X
@@ -20,7 +21,7 @@ namespace {
 
 using namespace split3;
 constexpr int kT = 512;
-constexpr int kIssue = 15;              // the warp that issues the MMAs: no part in the inverse, and only N to store
+constexpr int kIssue = 15;              // the warp that issues the MMAs (it has no part in the inverse)
 constexpr int LM = 68;
 constexpr uint32_t O_RQ = 0, O_RK = 98304, O_RP = O_RK + 49152, O_L = O_RP + 24576, O_T = O_L + 64 * LM * 4,
                    O_G = O_RP,                       // e^(G - G_m) [64][132] fp32 before P, L and T' exist

@@ -1,8 +1,8 @@
 // fp32 matrix products on tcgen05: every fp32 operand is stored as three bf16 images in shared memory,
 // x = x1 + x2 + x3 with each part rounded to nearest (24 significant bits together), and a product takes
 // the six MMAs x1 y1, x1 y2, x2 y1, x2 y2, x1 y3, x3 y1 into one fp32 accumulator in TMEM, small ones
-// first, so that the accumulator is truncated at full size by the last group alone.  The dropped terms are
-// below 2^-25 of a product.
+// first, so that the accumulator is truncated at full size by the last group alone (by all six where a product is added
+// to one that is complete).  The dropped terms are below 2^-25 of a product.
 //
 // An image is a sequence of blocks [R rows][64 columns] bf16 with 128-byte rows and the 128-byte swizzle;
 // split s, column block b of a matrix with NB column blocks start at (s * NB + b) * R * 128 bytes.  The
